@@ -3,23 +3,25 @@
 // over column slices instead of the merge of Section 4.1.
 //
 // B's columns are cut into K slices of W columns (W a multiple of 32, at most
-// DENSE_W_MAX, K W >= ncols).  A slice of a row is one CTA.  The counting pass marks
+// DENSE_W_MAX, K W >= ncols).  A slice of a row is one CTA's item.  The counting pass marks
 // the columns of the row's products in the slice in a shared bitmap and counts its
 // bits, and may leave the bitmap in device memory.  The fill pass reads it back (or marks
 // the columns again when it was not kept), ranks the bitmap (set bits before each word),
-// and adds every product into a compact buffer of sums, one per column of the result,
-// at its column's rank: clearing and writing out cost the slice's entries, not its
-// width, and the sums come out in column order.  There are no misses, no merges and no
-// capacity to outgrow (a slice with more entries than the buffer is done in pieces).
-// The part of each B row that falls in slice s is read from a table of per-row slice
-// boundaries, built once per call, and is cut into chunks of consecutive entries that
-// the warps share out.
+// and adds every product into the sum at its column's rank: clearing and writing out cost
+// the slice's entries, not its width, and the sums come out in column order.  There are no
+// misses, no merges and no capacity to outgrow.  The part of each B row that falls in slice
+// s is read from a table of per-row slice boundaries, built once per call.
 //
 // Because the rows are counted first, they need no temporary result rows: their sizes
 // go into the row counts of C with the other rows', and the values are written
 // straight into C once its row pointers exist (the kept bitmaps, W / 8 bytes per
 // (row, slice), are the only temporary, and an optional one).  The same launch recomputes the values
 // for a values-only replay.
+//
+// Measured (count + fill launches of C = A*A, double, one GB300, before -> after the product
+// walk below replaced a search per product and the sums moved from shared memory into C):
+// R-MAT 2^18 x 8, every bin-37 row, bitmaps not kept: 24.4 -> 11.9 ms; R-MAT 2^20 x 8 with
+// u_i >= 8,192, kept: 129.8 -> 75.9 ms (14.6 -> 25 G B-entries/s through both passes).
 #include "internal.h"
 #include "common.cuh"
 
@@ -165,157 +167,102 @@ cudaError_t launch_dense_select(const int32_t *bin_rows, int64_t m, BinSummary *
     return cudaGetLastError();
 }
 
-// ---- the product expansion shared by the count and fill kernels ----
-// Walks the A entries of `row` in windows of WIN (<= NT); wbs holds 2 WIN entries (the
-// parts' starts, then their lengths).  Where the window's parts -- the selected B rows'
-// entries inside slice s -- average DENSE_FLAT_BELOW products or more, they are cut into
-// chunks of DENSE_CH entries and warp w takes the w-th contiguous range of the chunks, its
-// lanes a chunk's entries 32 at a time.  Shorter parts (the slices of a wide B cut most
-// sparse rows into parts of a few entries, which would leave most lanes idle) form one
-// flat sequence of products: the threads take consecutive products and find each one's
-// part by a binary search of the window's scan.  Either way consecutive lanes read
-// consecutive entries of one B row (coalesced, distinct ascending columns).
-// f(p, ok) gets DENSE_UN entry positions p[] of B and which of them are valid; every lane
-// of a warp makes the same calls (so f may use warp-wide intrinsics).  Ends with a barrier.
-constexpr int DENSE_CH = 256;
-constexpr int DENSE_UN = 4;
-constexpr int DENSE_FLAT_BELOW = 32;  // windows whose parts average fewer products go flat
+// ---- the products of a (row, slice) ----
+// The A entries of the row are taken NT at a time.  The entries of one window that select a
+// non-empty part of a B row (its entries inside slice s) are compacted into a table: each
+// part's first product in the window's sequence of products, and its place in B.  Every warp
+// then takes one contiguous range of that sequence, 32 products at a time, without a barrier:
+// the lanes look at the next 32 part starts, the starts that fall into the 32 products become
+// a bit mask (one warp-wide OR), and a lane's part is the number of mask bits at or below it.
+// So parts of any length -- most are a few entries long, a hub's has thousands -- keep all
+// lanes busy, and a product costs no search.  (A binary search per product, and whole-CTA
+// passes with a barrier per part for the long parts, held the 2^16-row R-MAT to a quarter of
+// the rate of the shared-memory atomics.)
+constexpr int DENSE_UN = 4;  // groups of 32 products in flight per warp
 
-template <int NT, int WIN, typename F>
-SPG_DEV void dense_expand(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int row, int s, int64_t *wbs,
-                          int64_t *cscan, int64_t *scan64, F f) {
-    const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
-    const int K1 = D.K + 1;
-    for (int64_t e = a0; e < a1; e += WIN) {
-        const int nW = (int)min((int64_t)WIN, a1 - e);
-        int64_t len = 0;
-        if (threadIdx.x < nW) {
-            const int32_t k = A.col[e + threadIdx.x];
-            const int64_t rs = B.rp[k];
-            int64_t bs, be;
-            if (D.K > 1) {
-                const int32_t *bk = D.bnd + (int64_t)k * K1 + s;
-                bs = rs + bk[0];
-                be = rs + bk[1];
-            } else {
-                bs = rs;
-                be = B.rp[k + 1];
-            }
-            wbs[threadIdx.x] = bs;
-            wbs[WIN + threadIdx.x] = be - bs;
-            len = be - bs;
-        }
-        int64_t tot;
-        const int64_t ex = block_exclusive_scan<NT, int64_t, false>(len, scan64, tot);
-        if (threadIdx.x < nW) cscan[threadIdx.x] = ex;
-        __syncthreads();
-        if (tot >= (int64_t)DENSE_FLAT_BELOW * nW) {
-            // long parts on average: warp w takes the w-th contiguous range of the window's
-            // chunks of DENSE_CH entries, its lanes a chunk's entries 32 at a time
-            constexpr int NW = NT / 32;
-            const int lane = lane_id(), wid = warp_id();
-            const int64_t nch = threadIdx.x < nW ? (wbs[WIN + threadIdx.x] + DENSE_CH - 1) / DENSE_CH : 0;
-            int64_t tc;
-            const int64_t exc = block_exclusive_scan<NT, int64_t, false>(nch, scan64, tc);
-            if (threadIdx.x < nW) cscan[threadIdx.x] = exc;  // now the first chunk of each part
-            __syncthreads();
-            const int64_t c0 = tc * wid / NW, c1 = tc * (wid + 1) / NW;
-            int t = 0;
-            if (c0 < c1) t = find_segment_i64(cscan, nW, c0);
-            for (int64_t c = c0; c < c1; ++c) {
-                while (t + 1 < nW && cscan[t + 1] <= c) ++t;  // warp-uniform: skips parts without chunks
-                const int64_t off = (c - cscan[t]) * DENSE_CH;
-                const int64_t p0 = wbs[t] + off;
-                const int n = (int)min((int64_t)DENSE_CH, wbs[WIN + t] - off);
-                // the trip count is the same for every lane (f may be warp-collective)
-                for (int i0 = 0; i0 < n; i0 += 32 * DENSE_UN) {
-                    const int i = i0 + lane;
-                    int64_t p[DENSE_UN];
-                    bool ok[DENSE_UN];
-#pragma unroll
-                    for (int u = 0; u < DENSE_UN; ++u) {
-                        ok[u] = i + 32 * u < n;
-                        p[u] = p0 + i + 32 * u;
-                    }
-                    f(p, ok);
-                }
-            }
+template <int NT>
+struct DenseWin {
+    int64_t base[NT];        // place in B of the part's first entry, minus start
+    int64_t scan[NT / 32 + 1];
+    val_t av[NT];            // a_ik
+    int32_t start[NT + 32];  // first product of the part; INT_MAX past the last part
+};
+
+// Builds the table of the entries [e, min(e + NT, a1)); returns the number of products (a
+// part has at most DENSE_W_MAX entries, so the window's products fit 32 bits).  Its first
+// barrier ends the use of the previous window; the table is ready when it returns.
+template <int NT, bool VALS>
+SPG_DEV int dense_window(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int s, int64_t e, int64_t a1,
+                         DenseWin<NT> &w) {
+    static_assert((int64_t)NT * DENSE_W_MAX < INT32_MAX, "products of a window");
+    int64_t bs = 0;
+    int len = 0;
+    val_t av = val_t(0);
+    const int64_t i = e + threadIdx.x;
+    if (i < a1) {
+        const int32_t k = A.col[i];
+        if (VALS) av = A.val[i];
+        const int64_t rs = B.rp[k];
+        if (D.K > 1) {
+            const int32_t *bk = D.bnd + (int64_t)k * (D.K + 1) + s;
+            const int32_t b0 = bk[0];
+            bs = rs + b0;
+            len = bk[1] - b0;
         } else {
-            // short parts on average: one flat sequence of products; the trip count is the
-            // same for every lane (f may be warp-collective)
-            for (int64_t q0 = 0; q0 < tot; q0 += (int64_t)NT * DENSE_UN) {
-                int64_t p[DENSE_UN];
-                bool ok[DENSE_UN];
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u) {
-                    const int64_t q = q0 + (int64_t)u * NT + threadIdx.x;
-                    ok[u] = q < tot;
-                    p[u] = 0;
-                    if (ok[u]) {
-                        const int t = find_segment_i64(cscan, nW, q);  // the last part starting at or before q
-                        p[u] = wbs[t] + (q - cscan[t]);
-                    }
-                }
-                f(p, ok);
-            }
+            bs = rs;
+            len = (int)(B.rp[k + 1] - rs);
         }
-        __syncthreads();  // the window's tables are reused
+    }
+    int64_t tot;
+    const int64_t ex = block_exclusive_scan<NT, int64_t, false>(len > 0 ? (int64_t(1) << 32) | len : 0, w.scan, tot);
+    const int np = (int)(tot >> 32);
+    if (len > 0) {
+        const int q = (int)(ex >> 32), st = (int)(ex & 0xffffffff);
+        w.start[q] = st;
+        w.base[q] = bs - st;
+        if (VALS) w.av[q] = av;
+    }
+    if ((int)threadIdx.x >= np) w.start[threadIdx.x] = INT_MAX;
+    if (threadIdx.x < 32) w.start[NT + threadIdx.x] = INT_MAX;
+    __syncthreads();
+    return (int)(tot & 0xffffffff);
+}
+
+// f(p, a, ok): DENSE_UN entry positions p[] of B, the a_ik that multiply them (VALS) and which
+// are valid, called by whole warps.  Each access of a warp reads consecutive entries of few
+// B rows.
+template <int NT, bool VALS, typename F>
+SPG_DEV void dense_walk(const DenseWin<NT> &w, int T, F f) {
+    constexpr int NW = NT / 32, ST = NT / 32;
+    const int lane = lane_id(), wid = warp_id();
+    const int64_t G = (T + 31) >> 5;
+    const int g0 = (int)(G * wid / NW), g1 = (int)(G * (wid + 1) / NW);
+    if (g0 >= g1) return;
+    // the part of product 32 g0: among every ST-th start, then among the ST after it
+    const int c = __popc(__ballot_sync(SPG_FULL, w.start[lane * ST] <= (g0 << 5))) - 1;
+    int t = c * ST - 1 + __popc(__ballot_sync(SPG_FULL, lane < ST && w.start[c * ST + (lane < ST ? lane : 0)] <= (g0 << 5)));
+    const unsigned le = (2u << lane) - 1u;  // the lanes up to this one
+    for (int g = g0; g < g1; g += DENSE_UN) {
+        int64_t p[DENSE_UN];
+        val_t a[DENSE_UN];
+        bool ok[DENSE_UN];
+#pragma unroll
+        for (int u = 0; u < DENSE_UN; ++u) {
+            const int q = (g + u) << 5;
+            const bool on = g + u < g1;
+            const unsigned d = (unsigned)(w.start[t + 1 + lane] - q);
+            const unsigned m = __reduce_or_sync(SPG_FULL, (on && d < 32u) ? 1u << d : 0u);
+            const int pt = t + __popc(m & le);
+            ok[u] = on && q + lane < T;
+            p[u] = w.base[pt] + (q + lane);
+            if (VALS) a[u] = w.av[pt];
+            t += __popc(m);
+        }
+        f(p, a, ok);
     }
 }
 
 // ---- the column bitmap of a (row, slice) ----
-// Sets bit x - lo of Bm for every column x of the row's products in the slice.  The 32
-// lanes of an access read consecutive entries of one B row (ascending columns), so lanes
-// whose columns share a word are neighbours: an OR over each such run of lanes leaves one
-// shared atomic per word touched instead of one per product.  Ends with a barrier.
-
-SPG_DEV void bitmap_set_warp(uint32_t *Bm, int x, bool ok) {
-    const int lane = lane_id();
-    const int w = ok ? (x >> 5) : -1 - lane;  // invalid lanes form runs of their own
-    uint32_t bits = ok ? (1u << (x & 31)) : 0u;
-    // sparse columns (no two neighbours in one word): one atomic per lane, no combining
-    const int prev_w = __shfl_up_sync(SPG_FULL, w, 1);  // every lane takes part in the shuffle
-    const bool shared_word = lane > 0 && prev_w == w;
-    if (!__any_sync(SPG_FULL, shared_word)) {
-        if (ok) atomicOr(&Bm[w], bits);
-        return;
-    }
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t nb = __shfl_down_sync(SPG_FULL, bits, d);
-        const int nw = __shfl_down_sync(SPG_FULL, w, d);
-        if (lane + d < 32 && nw == w) bits |= nb;
-    }
-    const int pw = __shfl_up_sync(SPG_FULL, w, 1);
-    if (ok && (lane == 0 || pw != w)) atomicOr(&Bm[w], bits);
-}
-
-template <int NT>
-SPG_DEV bool dense_bitmap(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int row, int s, int64_t lo,
-                          int span, uint32_t *Bm, int64_t *wbs, int64_t *cscan, int64_t *scan64) {
-    const int nq = (((span + 31) >> 5) + 3) >> 2;  // 16-byte groups of bitmap words
-    uint4 *b4 = reinterpret_cast<uint4 *>(Bm);
-    for (int q = threadIdx.x; q < nq; q += NT) b4[q] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
-    bool bad = false;
-    dense_expand<NT, NT>(A, B, D, row, s, wbs, cscan, scan64, [&](const int64_t *p, const bool *ok) {
-        int32_t c[DENSE_UN];
-#pragma unroll
-        for (int u = 0; u < DENSE_UN; ++u)
-            if (ok[u]) c[u] = __ldg(B.col + p[u]);
-#pragma unroll
-        for (int u = 0; u < DENSE_UN; ++u) {
-            const int x = ok[u] ? (int)(c[u] - lo) : 0;
-            const bool in = ok[u] && (unsigned)x < (unsigned)span;
-            if (ok[u] && !in) bad = true;  // cannot happen: the slice boundaries select the columns
-            bitmap_set_warp(Bm, x, in);
-        }
-    });
-    return bad;
-}
-
-// ---- pass 1: the number of columns of every (row, slice) ----
-// Shared memory: the slice's column bitmap (one bit per column), then its popcount.
 
 // The next (item, slice) of a CTA: blockIdx.x, then + gridDim.x (a grid that covers the
 // items takes one each), or, with a work counter, the counter's next ticket (a persistent
@@ -343,12 +290,40 @@ SPG_DEV int dense_span(const DevCSR &B, const DenseArgs &D, int64_t d, int s, in
     return (int)(min(min((int64_t)(s + 1) * D.W, B.ncols), (int64_t)D.chi[d]) - lo);
 }
 
-// FLAGS: narrow slices count with one flag byte per column (a plain store of 1 per product:
-// every writer stores the same value, so no atomics are needed); wide ones with the bitmap.
-template <int NT, bool FLAGS>
+// Marks the column offset x of every product of the row in the slice with mark(x).  Returns
+// whether a column lay outside [lo, lo + span) (cannot happen: the slice boundaries select
+// the columns); a barrier must follow before the marks are read.
+template <int NT, typename M>
+SPG_DEV bool dense_mark_columns(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int row, int s, int64_t lo,
+                                int span, DenseWin<NT> &win, M mark) {
+    bool bad = false;
+    const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
+    for (int64_t e = a0; e < a1; e += NT) {
+        const int T = dense_window<NT, false>(A, B, D, s, e, a1, win);
+        dense_walk<NT, false>(win, T, [&](const int64_t *p, const val_t *, const bool *ok) {
+            int32_t c[DENSE_UN];
+#pragma unroll
+            for (int u = 0; u < DENSE_UN; ++u)
+                if (ok[u]) c[u] = __ldg(B.col + p[u]);
+#pragma unroll
+            for (int u = 0; u < DENSE_UN; ++u) {
+                if (!ok[u]) continue;
+                const int x = (int)(c[u] - lo);
+                if ((unsigned)x < (unsigned)span) mark(x);
+                else bad = true;
+            }
+        });
+    }
+    return bad;
+}
+
+// ---- pass 1: the number of columns of every (row, slice) ----
+// Shared memory: the slice's column bitmap (one bit per column), then its popcount.  Bound by
+// the gather of B's columns and the shared atomics on the bitmap.
+template <int NT>
 SPG_DEV void dense_count_item(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t b, int64_t *err) {
     extern __shared__ __align__(16) uint32_t dc_bm[];
-    __shared__ int64_t wbs[2 * NT], cscan[NT], scan64[NT / 32 + 1];  // part starts, then part lengths
+    __shared__ DenseWin<NT> win;
     __shared__ int32_t scan32[NT / 32 + 1];
     const int64_t d = b / D.K;
     const int s = (int)(b - d * D.K);
@@ -358,77 +333,33 @@ SPG_DEV void dense_count_item(const DevCSR &A, const DevCSR &B, const DenseArgs 
         if (threadIdx.x == 0) D.cnt[b] = 0;
         return;
     }
-    bool bad = false;
+    const int ng = (((span + 31) >> 5) + 3) >> 2;  // 16-byte groups of bitmap words
+    uint4 *b4 = reinterpret_cast<uint4 *>(dc_bm);
+    for (int q = threadIdx.x; q < ng; q += NT) b4[q] = make_uint4(0u, 0u, 0u, 0u);
+    // (the first window's barriers come before the first mark)
+    const bool bad = dense_mark_columns<NT>(A, B, D, D.rows[d], s, lo, span, win,
+                                            [&](int x) { atomicOr(&dc_bm[x >> 5], 1u << (x & 31)); });
+    __syncthreads();
     int n = 0;
-    if constexpr (FLAGS) {
-        const int nq = ((span + 31) >> 5) << 1;  // 16-byte groups of flags, whole 32-column words
-        uint4 *f4 = reinterpret_cast<uint4 *>(dc_bm);
-        for (int q = threadIdx.x; q < nq; q += NT) f4[q] = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-        volatile uint8_t *fl = reinterpret_cast<uint8_t *>(dc_bm);
-        dense_expand<NT, NT>(A, B, D, D.rows[d], s, wbs, cscan, scan64, [&](const int64_t *p, const bool *ok) {
-            int32_t c[DENSE_UN];
-#pragma unroll
-            for (int u = 0; u < DENSE_UN; ++u)
-                if (ok[u]) c[u] = __ldg(B.col + p[u]);
-#pragma unroll
-            for (int u = 0; u < DENSE_UN; ++u) {
-                if (!ok[u]) continue;
-                const int x = (int)(c[u] - lo);
-                if ((unsigned)x >= (unsigned)span) {  // cannot happen: the slice boundaries select the columns
-                    bad = true;
-                    continue;
-                }
-                fl[x] = 1;
-            }
-        });
-        for (int q = threadIdx.x; q < nq; q += NT) {
-            const uint4 v = f4[q];
-            n += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
-        }
-        if (D.keep != nullptr) {
-            // the flags as a bitmap (32 columns per word, whole 16-byte groups), for the fill
-            uint32_t *kb = D.keep + b * (int64_t)D.keep_words;
-            const int nw = (span + 31) >> 5;
-            for (int w = threadIdx.x; w < ((nw + 3) & ~3); w += NT) {
-                uint32_t m = 0;
-                if (w < nw) {
-                    const uint4 lo4 = f4[2 * w], hi4 = f4[2 * w + 1];
-                    const uint32_t q[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        // byte j of q[k] (0 or 1) is column 4k + j
-                        const uint32_t y = q[k];
-                        m |= ((y & 1u) | ((y >> 7) & 2u) | ((y >> 14) & 4u) | ((y >> 21) & 8u)) << (4 * k);
-                    }
-                }
-                kb[w] = m;
-            }
-        }
-    } else {
-        bad = dense_bitmap<NT>(A, B, D, D.rows[d], s, lo, span, dc_bm, wbs, cscan, scan64);
-        const int nw = (span + 31) >> 5;
-        for (int w = threadIdx.x; w < nw; w += NT) n += __popc(dc_bm[w]);
-        if (D.keep != nullptr) {
-            // the bitmap, in whole 16-byte groups (the words past the span were cleared), for the fill
-            const uint4 *b4 = reinterpret_cast<const uint4 *>(dc_bm);
-            uint4 *k4 = reinterpret_cast<uint4 *>(D.keep + b * (int64_t)D.keep_words);
-            for (int q = threadIdx.x; q < (nw + 3) >> 2; q += NT) k4[q] = b4[q];
-        }
+    uint4 *k4 = D.keep != nullptr ? reinterpret_cast<uint4 *>(D.keep + b * (int64_t)D.keep_words) : nullptr;
+    for (int q = threadIdx.x; q < ng; q += NT) {
+        const uint4 v = b4[q];
+        n += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+        if (k4 != nullptr) k4[q] = v;  // for the fill (whole groups: the words past the span are clear)
     }
     n = block_reduce_sum<NT, int>(n, scan32);
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicExch((unsigned long long *)err, 5ull);
     if (threadIdx.x == 0) D.cnt[b] = n;
 }
 
-template <int NT, bool FLAGS>
-__global__ void __launch_bounds__(NT)
+template <int NT>
+__global__ void __launch_bounds__(NT, 1536 / NT)
 k_dense_count(DevCSR A, DevCSR B, DenseArgs D, int64_t *err) {
     __shared__ int64_t s_b;
     unsigned long long *q = D.dev_n != nullptr ? D.queue : nullptr;
     const int64_t nb = dense_items(D);
     for (int64_t b = dense_next(q, 0, true, &s_b); b < nb; b = dense_next(q, b, false, &s_b))
-        dense_count_item<NT, FLAGS>(A, B, D, b, err);
+        dense_count_item<NT>(A, B, D, b, err);
 }
 
 // One thread per dense item: the slices' offsets inside the row and the row's length.
@@ -450,224 +381,75 @@ __global__ void k_dense_rows(MergeItems it, DenseArgs D) {
 }
 
 // ---- pass 2: the values, written into C ----
-// Shared memory: the slice's column bitmap Bm and its rank directory Rd (Rd[w] = set bits
-// in the words before w), then a compact buffer V of vcap sums.  A product's column x has
-// the position Rd[x >> 5] + popc(bits of its word below x) among the slice's columns, so
-// V holds one sum per column of the result, in column order: clearing and writing out
-// cost the slice's entries, not its width.  When a slice has more entries than V holds,
-// its word range is cut into pieces of at most vcap entries (the rank directory gives
-// the cuts) and the products are gone through once per piece.
-//
-// The columns of one B row are distinct, so while the whole CTA works on a single B-row
-// part no two threads add into the same sum and plain adds suffice; parts of at least
-// DENSE_LONG products are done that way, one after another (a barrier between two
-// parts), each product one fused multiply-add.  The shorter parts are shared out to the
-// warps in chunks and added with shared fp64 atomics, before the long ones.
-constexpr int DENSE_FILL_WIN = 512;  // A entries per window
-constexpr int DENSE_LONG = 512;
+// Shared memory: per 32-column word of the slice the pair (bits, set bits in the words before
+// it).  A product's column x has the position rank + popc(bits below x) among the slice's
+// columns, i.e. its place in the row of C, so one 8-byte shared load leads from a column to
+// its sum.  The columns are written and the sums cleared first, straight in C; in double
+// precision every product is then added in C itself (an atomic add performed in L2, which
+// holds the slice just cleared): no buffer of sums, so a CTA needs 32 KB for the widest slice,
+// five CTAs share an SM and any number of entries takes one pass.  Measured over the chip
+// with random addresses: 214-280 G adds/s in L2 against 288-372 G/s for fp64 atomics in shared
+// memory, which would leave one or two CTAs per SM.  In single precision the sums are kept in
+// shared memory (SHV: 786-1,171 G adds/s, and global float atomics flush denormals), one per
+// column of the result, in pieces when a slice has more entries than the buffer holds.
 
 __host__ __device__ inline int dense_nw4(int W) { return ((W + 31) / 32 + 4) & ~3; }
 
-// The product loop of a fill: every product of row `row` in slice s whose column offset x
-// lies in [x0, x1) is passed to add(x, a * b) (short parts, by the warps) or add_plain
-// (long parts, the whole CTA on one part).  Ends with a barrier.
-template <int NT, typename Fa, typename Fp>
-SPG_DEV bool dense_products(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int row, int s, int64_t lo,
-                            int x0, int x1, int64_t *wbs, int64_t *cscan, val_t *wa, int32_t *wlen, int32_t *lidx,
-                            int64_t *scan64, Fa add, Fp add_plain) {
-    constexpr int WIN = DENSE_FILL_WIN;
-    bool bad = false;
-    const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
-    const int K1 = D.K + 1;
-    for (int64_t e = a0; e < a1; e += WIN) {
-        const int nW = (int)min((int64_t)WIN, a1 - e);
-        // products of the short parts (low 40 bits) and the count of long parts (above)
-        int64_t packed = 0;
-        if (threadIdx.x < nW) {
-            const int32_t k = A.col[e + threadIdx.x];
-            const int64_t rs = B.rp[k];
-            int64_t bs, be;
-            if (D.K > 1) {
-                const int32_t *bk = D.bnd + (int64_t)k * K1 + s;
-                bs = rs + bk[0];
-                be = rs + bk[1];
-            } else {
-                bs = rs;
-                be = B.rp[k + 1];
-            }
-            const int64_t len = be - bs;
-            wbs[threadIdx.x] = bs;
-            wlen[threadIdx.x] = (int32_t)len;  // a B row has at most ncols < 2^31 entries
-            wa[threadIdx.x] = A.val[e + threadIdx.x];
-            packed = len >= DENSE_LONG ? (int64_t(1) << 40) : len;
-        }
-        int64_t ptot;
-        const int64_t ex = block_exclusive_scan<NT, int64_t, false>(packed, scan64, ptot);
-        if (threadIdx.x < nW) {
-            cscan[threadIdx.x] = ex & ((int64_t(1) << 40) - 1);
-            if (packed >> 40) lidx[ex >> 40] = threadIdx.x;
-        }
-        const int64_t tshort = ptot & ((int64_t(1) << 40) - 1);
-        const int nlong = (int)(ptot >> 40);
-        __syncthreads();
-        const int nshort = nW - nlong;
-        if (tshort >= (int64_t)DENSE_FLAT_BELOW * (nshort > 0 ? nshort : 1)) {
-            // short parts averaging DENSE_FLAT_BELOW products or more: warp w takes the w-th
-            // contiguous range of their chunks of DENSE_CH entries, shared atomics
-            constexpr int NW = NT / 32;
-            const int lane = lane_id(), wid = warp_id();
-            const int64_t nch = (threadIdx.x < nW && wlen[threadIdx.x] < DENSE_LONG)
-                                    ? ((int64_t)wlen[threadIdx.x] + DENSE_CH - 1) / DENSE_CH : 0;
-            int64_t tc;
-            const int64_t exc = block_exclusive_scan<NT, int64_t, false>(nch, scan64, tc);
-            if (threadIdx.x < nW) cscan[threadIdx.x] = exc;  // now the first chunk of each part
-            __syncthreads();
-            const int64_t c0 = tc * wid / NW, c1 = tc * (wid + 1) / NW;
-            int t = 0;
-            if (c0 < c1) t = find_segment_i64(cscan, nW, c0);
-            for (int64_t c = c0; c < c1; ++c) {
-                while (t + 1 < nW && cscan[t + 1] <= c) ++t;  // warp-uniform: skips parts without chunks
-                const int64_t off = (c - cscan[t]) * DENSE_CH;
-                const int64_t p0 = wbs[t] + off;
-                const int n = (int)min((int64_t)DENSE_CH, (int64_t)wlen[t] - off);
-                const val_t av = wa[t];
-                for (int i = lane; i < n; i += 32 * DENSE_UN) {
-                    int32_t cc[DENSE_UN];
-                    val_t v[DENSE_UN];
+// Turns the words of a slice's bitmap into the index: the groups of four words from src(g)
+// are counted, ranked and written as pairs.  Returns the number of set bits; put(g, bits,
+// rank) is called for every group by the thread that ranked it, after `enter(total)` was
+// true (else the caller must return).  The index is complete after the caller's next barrier.
+template <int NT, typename S, typename E, typename P>
+SPG_DEV bool dense_index(uint2 *idx, int nwords, int32_t *scan32, S src, E enter, P put) {
+    constexpr int NW = NT / 32, RG = (DENSE_W_MAX / 128 + NT - 1) / NT;
+    const int lane = lane_id(), wid = warp_id();
+    const int ng = (nwords + 3) >> 2;
+    const int per = (ng + NT - 1) / NT;  // at most RG: each warp takes per * 32 consecutive groups
+    uint4 b[RG];
+    int mine = 0;
 #pragma unroll
-                    for (int u = 0; u < DENSE_UN; ++u)
-                        if (i + 32 * u < n) cc[u] = __ldg(B.col + p0 + i + 32 * u);
-#pragma unroll
-                    for (int u = 0; u < DENSE_UN; ++u)
-                        if (i + 32 * u < n) v[u] = __ldg(B.val + p0 + i + 32 * u);
-#pragma unroll
-                    for (int u = 0; u < DENSE_UN; ++u) {
-                        if (i + 32 * u >= n) continue;
-                        const int x = (int)(cc[u] - lo);
-                        if (x < x0 || x >= x1) continue;
-                        if (!add(x, av * v[u])) bad = true;
-                    }
-                }
-            }
-        } else {
-            // shorter ones: one flat sequence of their products (long parts add none to the
-            // scan), consecutive threads on consecutive products, shared atomics
-            for (int64_t q0 = 0; q0 < tshort; q0 += (int64_t)NT * DENSE_UN) {
-                int64_t pp[DENSE_UN];
-                int tt[DENSE_UN];
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u) {
-                    const int64_t q = q0 + (int64_t)u * NT + threadIdx.x;
-                    tt[u] = -1;
-                    if (q < tshort) {
-                        const int t = find_segment_i64(cscan, nW, q);  // the last part starting at or before q
-                        tt[u] = t;
-                        pp[u] = wbs[t] + (q - cscan[t]);
-                    }
-                }
-                int32_t cc[DENSE_UN];
-                val_t v[DENSE_UN];
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u)
-                    if (tt[u] >= 0) cc[u] = __ldg(B.col + pp[u]);
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u)
-                    if (tt[u] >= 0) v[u] = __ldg(B.val + pp[u]);
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u) {
-                    if (tt[u] < 0) continue;
-                    const int x = (int)(cc[u] - lo);
-                    if (x < x0 || x >= x1) continue;
-                    if (!add(x, wa[tt[u]] * v[u])) bad = true;
-                }
-            }
-        }
-        __syncthreads();
-        // long parts: one at a time, the whole CTA, plain adds.  A round is NT * DENSE_UN
-        // consecutive entries of one part; the loads of the next two rounds are in flight
-        // while a round is added (they touch no shared memory, so they may cross the
-        // barrier between two parts)
-        if (nlong > 0) {
-            constexpr int RND = NT * DENSE_UN;
-            int32_t c0[DENSE_UN], c1[DENSE_UN], c2[DENSE_UN];
-            val_t v0[DENSE_UN], v1[DENSE_UN], v2[DENSE_UN];
-            int j0 = 0, o0 = 0, j1, o1, j2, o2;
-            auto load = [&](int32_t (&cc)[DENSE_UN], val_t (&vv)[DENSE_UN], int j, int i0) {
-                if (j >= nlong) return;
-                const int t = lidx[j];
-                const int64_t p0 = wbs[t] + i0;
-                const int n = wlen[t] - i0;
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u)
-                    if ((int)threadIdx.x + NT * u < n) cc[u] = __ldg(B.col + p0 + threadIdx.x + NT * u);
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u)
-                    if ((int)threadIdx.x + NT * u < n) vv[u] = __ldg(B.val + p0 + threadIdx.x + NT * u);
-            };
-            auto after = [&](int j, int i0, int &nj, int &ni) {
-                if (j >= nlong) {
-                    nj = nlong;
-                    ni = 0;
-                } else if (i0 + RND < wlen[lidx[j]]) {
-                    nj = j;
-                    ni = i0 + RND;
-                } else {
-                    nj = j + 1;
-                    ni = 0;
-                }
-            };
-            load(c0, v0, j0, o0);
-            after(j0, o0, j1, o1);
-            load(c1, v1, j1, o1);
-            while (j0 < nlong) {
-                after(j1, o1, j2, o2);
-                load(c2, v2, j2, o2);
-                {
-                    const int t = lidx[j0];
-                    const int n = wlen[t] - o0;
-                    const val_t av = wa[t];
-#pragma unroll
-                    for (int u = 0; u < DENSE_UN; ++u) {
-                        if ((int)threadIdx.x + NT * u >= n) continue;
-                        const int x = (int)(c0[u] - lo);
-                        if (x < x0 || x >= x1) continue;
-                        if (!add_plain(x, av * v0[u])) bad = true;
-                    }
-                }
-                if (j1 != j0) __syncthreads();  // the next part may add into the same columns
-#pragma unroll
-                for (int u = 0; u < DENSE_UN; ++u) {
-                    c0[u] = c1[u];
-                    v0[u] = v1[u];
-                    c1[u] = c2[u];
-                    v1[u] = v2[u];
-                }
-                j0 = j1;
-                o0 = o1;
-                j1 = j2;
-                o1 = o2;
-            }
-        }
-        __syncthreads();  // the window's tables are reused
+    for (int i = 0; i < RG; ++i) {
+        const int g = (wid * per + i) * 32 + lane;
+        b[i] = (i < per && g < ng) ? src(g) : make_uint4(0u, 0u, 0u, 0u);
+        mine += __popc(b[i].x) + __popc(b[i].y) + __popc(b[i].z) + __popc(b[i].w);
     }
-    return bad;
+    mine = warp_reduce_sum(mine);
+    if (lane == 0) scan32[wid] = mine;
+    __syncthreads();
+    int run = 0, tot = 0;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        const int c = scan32[k];
+        if (k < wid) run += c;
+        tot += c;
+    }
+    if (!enter(tot)) return false;
+#pragma unroll
+    for (int i = 0; i < RG; ++i) {
+        if (i >= per) break;
+        const int g = (wid * per + i) * 32 + lane;
+        const int c0 = __popc(b[i].x), c1 = c0 + __popc(b[i].y), c2 = c1 + __popc(b[i].z), c3 = c2 + __popc(b[i].w);
+        const int inc = warp_inclusive_scan(c3);
+        const int ex = run + inc - c3;
+        run += __shfl_sync(SPG_FULL, inc, 31);
+        if (g < ng) {
+            uint4 *o4 = reinterpret_cast<uint4 *>(idx + 4 * g);
+            o4[0] = make_uint4(b[i].x, (unsigned)ex, b[i].y, (unsigned)(ex + c0));
+            o4[1] = make_uint4(b[i].z, (unsigned)(ex + c1), b[i].w, (unsigned)(ex + c2));
+            put(g, b[i], ex);
+        }
+    }
+    return true;
 }
 
 // REPLAY: values-only replay; C's columns are already in place, so the bitmap is built
 // from the slice's known entries of C and only the values are written.
-// WIDE: the single-pass form for slices narrow enough to hold one sum per column of the
-// slice (W sums, W flag bytes, then the flags as a bitmap with its rank directory for the
-// write-out): every product adds into its column's sum and marks its flag in one pass,
-// and the write-out walks the slice's columns.  It reads the products once instead of
-// twice, which pays where slices are dense (products well above their width).
-template <int NT, bool REPLAY, bool WIDE>
+template <int NT, bool REPLAY, bool SHV>
 SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t b, const int64_t *c_rp,
                              int32_t *c_col, val_t *c_val, int64_t *err, int vcap, int cmin, int cmax) {
-    constexpr int WIN = DENSE_FILL_WIN;
     extern __shared__ __align__(16) unsigned char df_smem[];
-    __shared__ int64_t wbs[2 * WIN], cscan[WIN], scan64[NT / 32 + 1];  // part starts, then part lengths
-    __shared__ val_t wa[WIN];
-    __shared__ int32_t wlen[WIN], lidx[WIN], scan32[NT / 32 + 1];
+    __shared__ DenseWin<NT> win;
+    __shared__ int32_t scan32[NT / 32 + 1];
     const int expected = D.cnt[b];
     if (expected <= cmin || expected > cmax) return;  // empty, or another launch's item
     const int64_t d = b / D.K;
@@ -677,187 +459,122 @@ SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &
     int64_t lo;
     const int span = dense_span(B, D, d, s, lo);
     const int nwords = (span + 31) >> 5;
-    const int nw4 = dense_nw4(D.W);
     const int64_t o = c_rp[row] + D.soff[b];  // the slice's first entry in C
+    uint2 *idx = reinterpret_cast<uint2 *>(df_smem);
+    val_t *V = reinterpret_cast<val_t *>(idx + dense_nw4(D.W));
     bool bad = false;
-    if constexpr (WIDE) {
-        val_t *V = reinterpret_cast<val_t *>(df_smem);
-        uint8_t *flag = reinterpret_cast<uint8_t *>(V + D.W);
-        uint32_t *Bm = reinterpret_cast<uint32_t *>(flag + D.W);  // D.W is a multiple of 32
-        int32_t *Rd = reinterpret_cast<int32_t *>(Bm + nw4);
-        {
-            // V's first span sums, in whole 16-byte groups (W sums fill a multiple of 16 bytes)
-            uint4 *z4 = reinterpret_cast<uint4 *>(V);
-            const int nz = (int)((span * sizeof(val_t) + 15) / 16);
-            for (int q = threadIdx.x; q < nz; q += NT) z4[q] = make_uint4(0u, 0u, 0u, 0u);
-            uint4 *f4 = reinterpret_cast<uint4 *>(flag);  // whole 32-column words, as read below
-            if (!REPLAY)
-                for (int q = threadIdx.x; q < 2 * nwords; q += NT) f4[q] = make_uint4(0u, 0u, 0u, 0u);
-        }
-        __syncthreads();
-        volatile uint8_t *fl = flag;
-        bad = dense_products<NT>(
-            A, B, D, row, s, lo, 0, span, wbs, cscan, wa, wlen, lidx, scan64,
-            [&](int x, val_t v) {
-                atomicAdd(&V[x], v);
-                if (!REPLAY) fl[x] = 1;
-                return true;
-            },
-            [&](int x, val_t v) {
-                V[x] += v;
-                if (!REPLAY) fl[x] = 1;
-                return true;
-            });
+    // ---- the slice's columns ----
+    const bool kept = !REPLAY && D.keep != nullptr;
+    if (!kept) {
+        uint4 *i4 = reinterpret_cast<uint4 *>(idx);
+        for (int q = threadIdx.x; q < 2 * ((nwords + 3) >> 2); q += NT) i4[q] = make_uint4(0u, 0u, 0u, 0u);
+        auto mark = [&](int x) { atomicOr(&idx[x >> 5].x, 1u << (x & 31)); };
         if (REPLAY) {
-            // the slice's entries of C, in place since the product: their values
+            __syncthreads();
             for (int t = threadIdx.x; t < expected; t += NT) {
                 const int x = (int)(c_col[o + t] - lo);
-                if ((unsigned)x < (unsigned)span) c_val[o + t] = V[x];
+                if ((unsigned)x < (unsigned)span) mark(x);
                 else bad = true;  // C's columns were changed since the product
             }
-            if (__syncthreads_or(bad) && threadIdx.x == 0) atomicExch((unsigned long long *)err, 6ull);
-            return;
+        } else {
+            bad = dense_mark_columns<NT>(A, B, D, row, s, lo, span, win, mark);
         }
-        // flags -> bitmap (32 columns per word), then its rank directory
-        for (int w = threadIdx.x; w < nwords; w += NT) {
-            const uint4 *f4 = reinterpret_cast<const uint4 *>(flag + 32 * w);
-            const uint4 lo4 = f4[0], hi4 = f4[1];
-            const uint32_t q[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
-            uint32_t m = 0;
+        __syncthreads();
+    }
+    const uint4 *k4 = kept ? reinterpret_cast<const uint4 *>(D.keep + b * (int64_t)D.keep_words) : nullptr;
+    const uint4 *i4 = reinterpret_cast<const uint4 *>(idx);
+    const bool match = dense_index<NT>(
+        idx, nwords, scan32,
+        [&](int g) {
+            if (kept) return __ldg(k4 + g);
+            const uint4 p = i4[2 * g], q = i4[2 * g + 1];
+            return make_uint4(p.x, p.z, q.x, q.z);
+        },
+        [&](int tot) { return tot == expected; },
+        [&](int g, const uint4 &w, int r) {
+            if (REPLAY) return;
+            const uint32_t wd[4] = {w.x, w.y, w.z, w.w};
+            int64_t q = o + r;
+            int32_t base = (int32_t)(lo + ((int64_t)g << 7));
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                // byte j of q[k] (0 or 1) is column 4k + j
-                const uint32_t y = q[k];
-                m |= ((y & 1u) | ((y >> 7) & 2u) | ((y >> 14) & 4u) | ((y >> 21) & 8u)) << (4 * k);
-            }
-            Bm[w] = m;
-        }
-        __syncthreads();
-        const int tot = bitmap_rank<NT>(Bm, Rd, nwords, scan32);
-        if (__syncthreads_or(bad || tot != expected)) {  // the counting pass saw other columns: cannot happen
-            if (threadIdx.x == 0) atomicExch((unsigned long long *)err, 6ull);
-            return;
-        }
-        // column order: consecutive threads take consecutive columns, so a warp's stores
-        // land in one contiguous run of C
-        for (int x = threadIdx.x; x < span; x += NT) {
-            const uint32_t wd = Bm[x >> 5];  // the same word for the whole warp
-            if (wd == 0u) continue;
-            if ((wd >> (x & 31)) & 1u) {
-                const int64_t pos = o + Rd[x >> 5] + __popc(wd & ((1u << (x & 31)) - 1u));
-                if (!SPG_IN(pos < o + expected, 112)) continue;  // the slice's entries of C
-                c_col[pos] = (int32_t)(lo + x);
-                c_val[pos] = V[x];
-            }
-        }
-        return;
-    }
-    uint32_t *Bm = reinterpret_cast<uint32_t *>(df_smem);
-    int32_t *Rd = reinterpret_cast<int32_t *>(Bm + nw4);
-    val_t *V = reinterpret_cast<val_t *>(Rd + nw4);
-    // ---- the slice's columns: bitmap and rank directory ----
-    if (REPLAY) {
-        uint4 *b4 = reinterpret_cast<uint4 *>(Bm);
-        for (int q = threadIdx.x; q < (nwords + 3) >> 2; q += NT) b4[q] = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-        for (int t0 = 0; t0 < expected; t0 += NT) {  // whole warps: the bitmap update is warp-wide
-            const int t = t0 + (int)threadIdx.x;
-            const int x = t < expected ? (int)(c_col[o + t] - lo) : 0;
-            const bool in = t < expected && (unsigned)x < (unsigned)span;
-            if (t < expected && !in) bad = true;  // C's columns were changed since the product
-            bitmap_set_warp(Bm, x, in);
-        }
-        __syncthreads();
-    } else if (D.keep != nullptr) {
-        // the bitmap the counting pass left for this (row, slice)
-        const uint4 *k4 = reinterpret_cast<const uint4 *>(D.keep + b * (int64_t)D.keep_words);
-        uint4 *b4 = reinterpret_cast<uint4 *>(Bm);
-        for (int q = threadIdx.x; q < (nwords + 3) >> 2; q += NT) b4[q] = __ldg(k4 + q);
-        __syncthreads();
-    } else {
-        bad = dense_bitmap<NT>(A, B, D, row, s, lo, span, Bm, wbs, cscan, scan64);
-    }
-    const int tot = bitmap_rank<NT>(Bm, Rd, nwords, scan32);
-    if (__syncthreads_or(bad || tot != expected)) {  // the counting pass saw other columns: cannot happen
-        if (threadIdx.x == 0) atomicExch((unsigned long long *)err, 6ull);
-        return;
-    }
-    auto rank_at = [&](int w) { return w < nwords ? Rd[w] : tot; };
-    // ---- pieces of at most vcap entries, each summed in V and written out ----
-    for (int w0 = 0; w0 < nwords;) {
-        // the last word end w1 with rank_at(w1) - Rd[w0] <= vcap (a word holds <= 32 <= vcap entries)
-        const int e0 = Rd[w0];
-        int w1 = nwords;  // the rest of the slice, when it fits
-        if (tot - e0 > vcap) {
-            int lo_ = w0 + 1, hi = nwords;
-            while (lo_ < hi) {
-                const int mid = (lo_ + hi + 1) >> 1;
-                if (rank_at(mid) - e0 <= vcap) lo_ = mid; else hi = mid - 1;
-            }
-            w1 = lo_;
-        }
-        const int n = rank_at(w1) - e0;
-        const int x0 = w0 << 5, x1 = min(span, w1 << 5);
-        for (int k = threadIdx.x; k < n; k += NT) V[k] = val_t(0);
-        __syncthreads();
-        auto pos_of = [&](int x) {
-            const uint32_t wd = Bm[x >> 5];
-            return ((wd >> (x & 31)) & 1u) ? Rd[x >> 5] + __popc(wd & ((1u << (x & 31)) - 1u)) - e0 : -1;
-        };
-        bad = dense_products<NT>(
-            A, B, D, row, s, lo, x0, x1, wbs, cscan, wa, wlen, lidx, scan64,
-            [&](int x, val_t v) {
-                const int q = pos_of(x);
-                if (q < 0) return false;  // a column the bitmap does not hold: cannot happen
-                if (SPG_IN(q < n, 109)) atomicAdd(&V[q], v);
-                return true;
-            },
-            [&](int x, val_t v) {
-                const int q = pos_of(x);
-                if (q < 0) return false;
-                if (SPG_IN(q < n, 109)) V[q] += v;
-                return true;
-            });
-        if (__syncthreads_or(bad)) {
-            if (threadIdx.x == 0) atomicExch((unsigned long long *)err, 6ull);
-            return;
-        }
-        // write-out: the sums in column order (contiguous), and the columns word by word
-        // (a thread takes a 16-byte group of words when the piece starts on one)
-        if (SPG_IN(e0 + n <= expected, 111))
-            for (int k = threadIdx.x; k < n; k += NT) c_val[o + e0 + k] = V[k];
-        if (!REPLAY) {
-            auto put = [&](int w, uint32_t bits, int r) {
-                if (!SPG_IN(r + __popc(bits) <= expected, 110)) return;  // the slice's entries of C
-                int64_t q = o + r;
+            for (int k = 0; k < 4; ++k, base += 32) {
+                uint32_t bits = wd[k];
+                if (!SPG_IN(q + __popc(bits) <= o + expected, 110)) return;  // the slice's entries of C
                 while (bits) {
                     const int t = __ffs(bits) - 1;
                     bits &= bits - 1u;
-                    c_col[q++] = (int32_t)(lo + ((int64_t)w << 5) + t);
+                    c_col[q++] = base + t;
                 }
-            };
-            if ((w0 & 3) == 0) {
-                for (int g = (w0 >> 2) + (int)threadIdx.x; g < (w1 + 3) >> 2; g += NT) {
-                    const int w = g << 2;
-                    const uint4 bv = *reinterpret_cast<const uint4 *>(Bm + w);
-                    if ((bv.x | bv.y | bv.z | bv.w) == 0u) continue;
-                    const int4 rv = *reinterpret_cast<const int4 *>(Rd + w);  // entries past w1 are not used
-                    put(w, bv.x, rv.x);
-                    if (w + 1 < w1) put(w + 1, bv.y, rv.y);
-                    if (w + 2 < w1) put(w + 2, bv.z, rv.z);
-                    if (w + 3 < w1) put(w + 3, bv.w, rv.w);
-                }
-            } else {
-                for (int w = w0 + (int)threadIdx.x; w < w1; w += NT) put(w, Bm[w], Rd[w]);
             }
+        });
+    if (!match) {  // the counting pass saw other columns: cannot happen
+        if (threadIdx.x == 0) atomicExch((unsigned long long *)err, 6ull);
+        return;
+    }
+    if (!SHV)
+        for (int t = threadIdx.x; t < expected; t += NT) c_val[o + t] = val_t(0);
+    // ---- the sums: in C at once, or in pieces of at most vcap entries in V ----
+    const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
+    for (int w0 = 0; w0 < nwords;) {
+        int w1 = nwords, e0 = 0, n = expected;
+        if (SHV) {
+            __syncthreads();  // the index is complete, and V is free
+            auto rank_at = [&](int w) { return w < nwords ? (int)idx[w].y : expected; };
+            // the last word end w1 with rank_at(w1) - e0 <= vcap (a word holds <= 32 <= vcap entries)
+            e0 = rank_at(w0);
+            if (expected - e0 > vcap) {
+                int l = w0 + 1, h = nwords;
+                while (l < h) {
+                    const int mid = (l + h + 1) >> 1;
+                    if (rank_at(mid) - e0 <= vcap) l = mid; else h = mid - 1;
+                }
+                w1 = l;
+            }
+            n = rank_at(w1) - e0;
+            for (int k = threadIdx.x; k < n; k += NT) V[k] = val_t(0);
         }
-        __syncthreads();  // V is reused by the next piece
+        const int x0 = w0 << 5, x1 = min(span, w1 << 5);
+        for (int64_t e = a0; e < a1; e += NT) {
+            const int T = dense_window<NT, true>(A, B, D, s, e, a1, win);
+            dense_walk<NT, true>(win, T, [&](const int64_t *p, const val_t *a, const bool *ok) {
+                int32_t c[DENSE_UN];
+                val_t v[DENSE_UN];
+#pragma unroll
+                for (int u = 0; u < DENSE_UN; ++u)
+                    if (ok[u]) c[u] = __ldg(B.col + p[u]);
+#pragma unroll
+                for (int u = 0; u < DENSE_UN; ++u)
+                    if (ok[u]) v[u] = __ldg(B.val + p[u]);
+#pragma unroll
+                for (int u = 0; u < DENSE_UN; ++u) {
+                    if (!ok[u]) continue;
+                    const int x = (int)(c[u] - lo);
+                    if (SHV && (x < x0 || x >= x1)) continue;  // another piece's
+                    const bool in = (unsigned)x < (unsigned)span;
+                    const uint2 wd = in ? idx[x >> 5] : make_uint2(0u, 0u);
+                    if (!((wd.x >> (x & 31)) & 1u)) {
+                        bad = true;  // a column the bitmap does not hold (the structure changed)
+                        continue;
+                    }
+                    const int q = (int)wd.y + __popc(wd.x & ((1u << (x & 31)) - 1u));
+                    if (!SPG_IN(q >= e0 && q - e0 < n, 109)) continue;
+                    if (SHV) atomicAdd(&V[q - e0], a[u] * v[u]);
+                    else atomicAdd(&c_val[o + q], a[u] * v[u]);
+                }
+            });
+        }
+        if (SHV) {
+            __syncthreads();
+            if (SPG_IN(e0 + n <= expected, 111))
+                for (int k = threadIdx.x; k < n; k += NT) c_val[o + e0 + k] = V[k];
+        }
         w0 = w1;
     }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicExch((unsigned long long *)err, 6ull);
 }
 
-// Items whose count lies in (cmin, cmax]; with a work counter the grid is persistent.
-template <int NT, int MINB, bool REPLAY, bool WIDE>
+// A persistent grid that takes the items whose count lies in (cmin, cmax] from a work counter.
+template <int NT, int MINB, bool REPLAY, bool SHV>
 __global__ void __launch_bounds__(NT, MINB)
 k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_col, val_t *c_val, int64_t *err,
              const int64_t *gate, int vcap, unsigned long long *counter, int cmin, int cmax) {
@@ -869,14 +586,14 @@ k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_co
         // the CTA's next item is taken one item ahead, so that its kept bitmap (written by the
         // counting pass, long out of L2) is on its way into L2 while this item is filled
         if (threadIdx.x == 0) {
-            const int64_t nx = counter != nullptr ? (int64_t)atomicAdd(counter, 1ull) : b + gridDim.x;
+            const int64_t nx = (int64_t)atomicAdd(counter, 1ull);
             s_nx = nx;
             if (!REPLAY && D.keep != nullptr && nx < nb) {
                 const int c = D.cnt[nx];
                 if (c > cmin && c <= cmax) prefetch_l2(D.keep + nx * (int64_t)D.keep_words, 4u * (uint32_t)D.keep_words);
             }
         }
-        dense_fill_item<NT, REPLAY, WIDE>(A, B, D, b, c_rp, c_col, c_val, err, vcap, cmin, cmax);
+        dense_fill_item<NT, REPLAY, SHV>(A, B, D, b, c_rp, c_col, c_val, err, vcap, cmin, cmax);
         __syncthreads();  // s_nx is visible and the item's shared memory is free
         b = s_nx;
         __syncthreads();  // every thread has read s_nx before thread 0 overwrites it
@@ -897,60 +614,34 @@ __global__ void k_dense_rowsum(DenseArgs D, int32_t *nnzc) {
     nnzc[D.rows[d]] = acc;
 }
 
-constexpr int DENSE_COUNT_NT = 256;
-constexpr int DENSE_COUNT_FLAGS_MAX = 32768;
-constexpr int DENSE_FILL_NT = 512;
-constexpr int DENSE_FILL_TWO_MIN = 4096;  // smallest sum buffer worth a second CTA per SM
+constexpr int DENSE_NT = 256;
 
-// Bytes of a fill CTA's bitmap and rank directory for slices of W columns.
-static int dense_index_bytes(int W) { return (int)(2 * sizeof(int32_t) * (size_t)dense_nw4(W)); }
+int dense_keep_words(int W) { return dense_nw4(W); }  // a multiple of 4: every item's bitmap starts on a 16-byte boundary
 
-int dense_fill_smem_bytes(int W) {
-    // the index, and room for at least one word's entries in V
-    return dense_index_bytes(W) + 32 * (int)sizeof(val_t);
-}
-
-// The single-pass form: one sum and one flag byte per column of the slice, and the index.
-int dense_fill_wide_bytes(int W) { return (int)((sizeof(val_t) + 1) * (size_t)W) + dense_index_bytes(W); }
-
-// Largest dynamic shared memory of a fill CTA when `per_sm` of them share an SM
-// (228 KB per SM, 1 KB of it reserved per CTA, at most 227 KB per CTA).
-int dense_fill_max_dynamic(int per_sm) {
-    const int per_cta = std::min(227 * 1024, 228 * 1024 / per_sm - 1024);
-    return per_cta - dense_fill_static_smem();
-}
-
-int dense_fill_static_smem() {
-    return (int)(DENSE_FILL_WIN * (3 * sizeof(int64_t) + sizeof(val_t) + 2 * sizeof(int32_t)) +
-                 (DENSE_FILL_NT / 32 + 1) * 12 + 64);
-}
-
-int dense_keep_words(int W) {
-    if (dense_fill_wide_bytes(W) <= dense_fill_max_dynamic(1)) return 0;
-    return dense_nw4(W);  // a multiple of 4: every item's bitmap starts on a 16-byte boundary
+static cudaError_t dense_check(const DevCSR &B, const DenseArgs &D) {
+    if (D.n * D.K > INT32_MAX || D.W % 32 != 0 || D.W > DENSE_W_MAX || (int64_t)D.K * D.W < B.ncols || D.queue == nullptr)
+        return cudaErrorInvalidValue;
+    if (D.keep != nullptr && (D.keep_words < dense_nw4(D.W) || D.keep_words % 4 != 0)) return cudaErrorInvalidValue;
+    return cudaSuccess;
 }
 
 cudaError_t launch_dense_count(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t *err, cudaStream_t st) {
     if (D.n <= 0) return cudaSuccess;
     const int64_t nb = D.n * D.K;
-    if (nb > INT32_MAX || D.W % 32 != 0 || (int64_t)D.K * D.W < B.ncols) return cudaErrorInvalidValue;
-    // flag bytes for slices of up to DENSE_COUNT_FLAGS_MAX columns, else the bitmap
-    const bool flags = D.W <= DENSE_COUNT_FLAGS_MAX;
-    if (D.keep != nullptr && (D.keep_words < dense_nw4(D.W) || D.keep_words % 4 != 0))
-        return cudaErrorInvalidValue;
-    const int smem = flags ? D.W : (int)(sizeof(uint32_t) * dense_nw4(D.W));
-    auto kern = flags ? k_dense_count<DENSE_COUNT_NT, true> : k_dense_count<DENSE_COUNT_NT, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = dense_check(B, D);
+    if (e != cudaSuccess) return e;
+    const int smem = (int)(sizeof(uint32_t) * dense_nw4(D.W));
+    auto kern = k_dense_count<DENSE_NT>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     int64_t grid = nb;
     if (D.dev_n != nullptr) {  // persistent grid over the items counted on the device
-        if (D.queue == nullptr) return cudaErrorInvalidValue;
         e = cudaMemsetAsync(D.queue, 0, sizeof(unsigned long long), st);
         if (e != cudaSuccess) return e;
-        grid = persistent_blocks((const void *)kern, DENSE_COUNT_NT, smem, nb);
+        grid = persistent_blocks((const void *)kern, DENSE_NT, smem, nb);
         if (grid <= 0) return cudaErrorInvalidValue;
     }
-    kern<<<(unsigned)grid, DENSE_COUNT_NT, smem, st>>>(A, B, D, err);
+    kern<<<(unsigned)grid, DENSE_NT, smem, st>>>(A, B, D, err);
     return cudaGetLastError();
 }
 
@@ -970,55 +661,44 @@ cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs 
                               int32_t *c_col, val_t *c_val, int64_t *err, cudaStream_t st, bool replay,
                               const int64_t *gate) {
     if (D.n <= 0) return cudaSuccess;
-    const int64_t nb = D.n * D.K;
-    if (nb > INT32_MAX || D.W % 32 != 0 || (int64_t)D.K * D.W < B.ncols) return cudaErrorInvalidValue;
-    if (D.keep != nullptr && (D.keep_words < dense_nw4(D.W) || D.keep_words % 4 != 0)) return cudaErrorInvalidValue;
-    // one launch: a grid over the items, or a persistent grid taking them from counter q
-    auto go = [&](auto kern, int smem, int vcap, unsigned long long *q, int cmin, int cmax) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (e != cudaSuccess) return e;
-        int64_t grid = nb;
-        if (q != nullptr) {
-            e = cudaMemsetAsync(q, 0, sizeof(unsigned long long), st);
-            if (e != cudaSuccess) return e;
-            grid = persistent_blocks((const void *)kern, DENSE_FILL_NT, smem, nb);
-            if (grid <= 0) return cudaErrorInvalidValue;
-        }
-        kern<<<(unsigned)grid, DENSE_FILL_NT, smem, st>>>(A, B, D, c_rp, c_col, c_val, err, gate, vcap, q, cmin,
-                                                           cmax);
+    cudaError_t e = dense_check(B, D);
+    if (e != cudaSuccess) return e;
+    // a persistent grid of nt threads per CTA over the items with counts in (cmin, cmax]
+    auto go = [&](auto kern, int nt, int smem, int vcap, unsigned long long *q, int cmin, int cmax) -> cudaError_t {
+        cudaError_t x = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (x == cudaSuccess) x = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        if (x == cudaSuccess) x = cudaMemsetAsync(q, 0, sizeof(unsigned long long), st);
+        if (x != cudaSuccess) return x;
+        const int grid = persistent_blocks((const void *)kern, nt, smem, D.n * D.K);
+        if (grid <= 0) return cudaErrorInvalidValue;
+        kern<<<(unsigned)grid, nt, smem, st>>>(A, B, D, c_rp, c_col, c_val, err, gate, vcap, q, cmin, cmax);
         return cudaGetLastError();
     };
-    if (D.dev_n != nullptr && D.queue == nullptr) return cudaErrorInvalidValue;
-    const int index = dense_index_bytes(D.W);
-    if (dense_fill_wide_bytes(D.W) <= dense_fill_max_dynamic(1)) {
-        // single-pass form (two CTAs per SM when two slices fit an SM's shared memory)
-        const int smem = dense_fill_wide_bytes(D.W);
-        const int vcap = (smem - index) / (int)sizeof(val_t);
-        unsigned long long *q = D.dev_n != nullptr ? D.queue + 1 : nullptr;
-        if (smem <= dense_fill_max_dynamic(2))
-            return replay ? go(k_dense_fill<DENSE_FILL_NT, 2, true, true>, smem, vcap, q, 0, INT32_MAX)
-                          : go(k_dense_fill<DENSE_FILL_NT, 2, false, true>, smem, vcap, q, 0, INT32_MAX);
-        return replay ? go(k_dense_fill<DENSE_FILL_NT, 1, true, true>, smem, vcap, q, 0, INT32_MAX)
-                      : go(k_dense_fill<DENSE_FILL_NT, 1, false, true>, smem, vcap, q, 0, INT32_MAX);
-    }
-    // compact form: the index, then as many sums as the rest of the CTA's shared memory holds.
-    // With work counters, the items whose slices have at most vcap2 entries run at two CTAs per
-    // SM (half the shared memory each), the others at one
-    const int smem1 = dense_fill_max_dynamic(1) & ~15, smem2 = dense_fill_max_dynamic(2) & ~15;
-    const int vcap1 = (smem1 - index) / (int)sizeof(val_t), vcap2 = (smem2 - index) / (int)sizeof(val_t);
-    if (vcap1 < 32) return cudaErrorInvalidValue;
-    if (D.queue != nullptr && vcap2 >= DENSE_FILL_TWO_MIN) {
-        cudaError_t e = replay ? go(k_dense_fill<DENSE_FILL_NT, 2, true, false>, smem2, vcap2, D.queue + 1, 0, vcap2)
-                               : go(k_dense_fill<DENSE_FILL_NT, 2, false, false>, smem2, vcap2, D.queue + 1, 0, vcap2);
+    const int index = (int)(sizeof(uint2) * (size_t)dense_nw4(D.W));
+    if constexpr (sizeof(val_t) == 8) {
+        return replay ? go(k_dense_fill<DENSE_NT, 5, true, false>, DENSE_NT, index, 0, D.queue + 1, 0, INT32_MAX)
+                      : go(k_dense_fill<DENSE_NT, 5, false, false>, DENSE_NT, index, 0, D.queue + 1, 0, INT32_MAX);
+    } else {
+        // sums in shared memory: the items whose entries fit a quarter of an SM's shared memory at
+        // four CTAs of 256 threads per SM, those that fit a half at two of 512, the rest at one of 1,024
+        auto room = [&](int per_sm, int nt) {  // sums that fit beside the index
+            const int fixed = 1024 + 512 + nt * (int)(sizeof(int64_t) + sizeof(val_t) + sizeof(int32_t)) + nt / 4;
+            return (std::min(227 * 1024, 228 * 1024 / per_sm) - fixed - index) / (int)sizeof(val_t) & ~31;
+        };
+        const int v4 = room(4, 256), v2 = room(2, 512), v1 = room(1, 1024);
+        if (v4 < 32) return cudaErrorInvalidValue;
+        const int fs = (int)sizeof(val_t);
+        e = replay ? go(k_dense_fill<256, 4, true, true>, 256, index + v4 * fs, v4, D.queue + 1, 0, v4)
+                   : go(k_dense_fill<256, 4, false, true>, 256, index + v4 * fs, v4, D.queue + 1, 0, v4);
         if (e != cudaSuccess) return e;
-        return replay ? go(k_dense_fill<DENSE_FILL_NT, 1, true, false>, smem1, vcap1, D.queue + 2, vcap2, INT32_MAX)
-                      : go(k_dense_fill<DENSE_FILL_NT, 1, false, false>, smem1, vcap1, D.queue + 2, vcap2, INT32_MAX);
+        if (D.W <= v4) return e;  // a slice has at most W entries
+        e = replay ? go(k_dense_fill<512, 2, true, true>, 512, index + v2 * fs, v2, D.queue + 2, v4, v2)
+                   : go(k_dense_fill<512, 2, false, true>, 512, index + v2 * fs, v2, D.queue + 2, v4, v2);
+        if (e != cudaSuccess) return e;
+        if (D.W <= v2) return e;
+        return replay ? go(k_dense_fill<1024, 1, true, true>, 1024, index + v1 * fs, v1, D.queue + 3, v2, INT32_MAX)
+                      : go(k_dense_fill<1024, 1, false, true>, 1024, index + v1 * fs, v1, D.queue + 3, v2, INT32_MAX);
     }
-    unsigned long long *q = D.dev_n != nullptr ? D.queue + 1 : nullptr;
-    return replay ? go(k_dense_fill<DENSE_FILL_NT, 1, true, false>, smem1, vcap1, q, 0, INT32_MAX)
-                  : go(k_dense_fill<DENSE_FILL_NT, 1, false, false>, smem1, vcap1, q, 0, INT32_MAX);
 }
 
 }  // namespace spg

@@ -204,6 +204,7 @@ cudaError_t launch_level1_sizes(const MergeItems &it, const int32_t *work, int64
 constexpr int32_t ITEM_DENSE = -2;  // MergeItems.child of a row computed by the dense-slice kernels
 constexpr int DENSE_MAX_SLICES = 64;
 constexpr int DENSE_W_MAX = 131072;  // widest slice: its bitmap and rank directory take 32 KB
+constexpr int DENSE_QUEUES = 4;      // work counters of the slice kernels
 struct DenseArgs {
     const int32_t *items;  // dense items (indices into MergeItems), larger rows first
     const int32_t *rows;   // their rows of A
@@ -217,11 +218,11 @@ struct DenseArgs {
     int32_t *soff;         // n K offsets of the slices inside their row of C
     const int64_t *dev_n = nullptr;  // when set: the number of dense items is *dev_n (<= n), read on
                                      // the device; the kernels run persistent grids over (item, slice)
-    unsigned long long *queue = nullptr;  // three work counters (count, fill, fill of the heavy items),
-                                          // zeroed by the launchers; needed with dev_n
-    uint32_t *keep = nullptr;  // when set (bitmap counts, compact fills only): keep_words words per
-    int keep_words = 0;        // (row, slice), where the count leaves the slice's column bitmap and
-                               // the fill reads it back instead of marking the columns again
+    unsigned long long *queue = nullptr;  // DENSE_QUEUES work counters (count, fills by size), zeroed
+                                          // by the launchers
+    uint32_t *keep = nullptr;  // when set: keep_words words per (row, slice), where the count leaves
+    int keep_words = 0;        // the slice's column bitmap and the fill reads it back instead of
+                               // marking the columns again
 };
 cudaError_t launch_dense_bounds(const DevCSR &B, int K, int W, int32_t *bnd, cudaStream_t st);
 // per row: flag (1 = dense-slice row: bin 37, and u_i >= dmin if dmin > 0, else div u_i >= the
@@ -237,8 +238,7 @@ cudaError_t launch_dense_select(const int32_t *bin_rows, int64_t m, BinSummary *
 // counts the columns of every (row, slice) into D.cnt (reads no work-item table, so it
 // may run beside the merge launches)
 cudaError_t launch_dense_count(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t *err, cudaStream_t st);
-// Words per (row, slice) of a kept column bitmap for slices of W columns, or 0 when the count
-// does not build bitmaps for such slices or the fill does not read them (the single-pass form).
+// Words per (row, slice) of a kept column bitmap for slices of W columns.
 int dense_keep_words(int W);
 // slice offsets inside the rows, and the dense items' lengths in the work-item table
 cudaError_t launch_dense_rows(const MergeItems &it, const DenseArgs &D, cudaStream_t st);
@@ -249,10 +249,6 @@ cudaError_t launch_dense_rowsum(const DenseArgs &D, int32_t *nnzc, cudaStream_t 
 cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs &D, const int64_t *c_rp,
                               int32_t *c_col, val_t *c_val, int64_t *err, cudaStream_t st, bool replay = false,
                               const int64_t *gate = nullptr);
-int dense_fill_smem_bytes(int W);
-int dense_fill_wide_bytes(int W);  // the single-pass form (fits for narrow slices only)
-int dense_fill_static_smem();
-int dense_fill_max_dynamic(int per_sm);
 
 // ---- the merge evaluation of Section 4.2 (merge_micro.cu) ----
 // method 0 ranking merge, 1 merge path, 2 bitonic merge; groups of 2l keys (two sorted runs)

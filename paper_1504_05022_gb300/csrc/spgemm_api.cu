@@ -401,7 +401,7 @@ static void merge_limits(spgemm_plan *p) {
         int wmax = DENSE_W_MAX;
         if (p->opts.dense_span > 0) wmax = std::min(wmax, std::max(1024, p->opts.dense_span & ~31));
         const int64_t k0 = (n + wmax - 1) / wmax;
-        if (k0 <= DENSE_MAX_SLICES && dense_fill_smem_bytes(wmax) <= dense_fill_max_dynamic(1)) {
+        if (k0 <= DENSE_MAX_SLICES) {
             const int64_t w = ((n + k0 - 1) / k0 + 31) & ~int64_t(31);
             p->dense_W = (int)w;
             p->dense_K = (int)((n + w - 1) / w);
@@ -696,7 +696,7 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
             }
             SPG_TRY(p->alloc_n(&p->dense_cnt, p->dense_n * p->dense_K));
             SPG_TRY(p->alloc_n(&p->dense_soff, p->dense_n * p->dense_K));
-            SPG_TRY(p->alloc_n(&p->d_queue, 3));  // work counters of the fill launches
+            SPG_TRY(p->alloc_n(&p->d_queue, DENSE_QUEUES));  // work counters of the fill launches
         }
         // C~ (hybrid: u_i for bins 0..36, 256 for bin 37)
         SPG_TRY(p->alloc_n(&p->ctil_col, p->h_summary.sum_cap, LIFE_NUMERIC));
@@ -960,7 +960,7 @@ static void alloc_dense_keep(spgemm_plan *p) {
     p->dense_keep_words = 0;
     const int want = p->opts.dense_keep;
     const int kw = p->dense_K > 0 ? dense_keep_words(p->dense_W) : 0;
-    if (p->dense_n == 0 || kw == 0 || want < 0 || (want == 0 && p->opts.alloc_policy == SPGEMM_ALLOC_PRECISE))
+    if (p->dense_n == 0 || want < 0 || (want == 0 && p->opts.alloc_policy == SPGEMM_ALLOC_PRECISE))
         return;
     const int64_t words = p->dense_n * p->dense_K * (int64_t)kw;
     size_t free_b = 0, total_b = 0;
@@ -1998,7 +1998,7 @@ static spgemm_status dplan_buffers(spgemm_dplan *d) {
         SPG_TRY(p->alloc_n(&p->d_summary, 1));
         SPG_TRY(p->alloc_n(&p->d_err, 1));
         SPG_TRY(p->alloc_n(&d->gate, 1));
-        SPG_TRY(p->alloc_n(&p->d_queue, 3));
+        SPG_TRY(p->alloc_n(&p->d_queue, DENSE_QUEUES));
         SPG_TRY(p->alloc_n(&p->S, nnzA + 1));
         SPG_TRY(p->alloc_n(&p->scan_partial, std::max(bound_partial_size(nnzA), bin_blocks(m) + 1) + 1));
         SPG_TRY(p->alloc_n(&p->u, m));
