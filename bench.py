@@ -670,7 +670,7 @@ def roofline(args, pairs, m):
         elif dom in ("bound", "bin", "scan"):
             bytes_dom += A.nnz * 12 + 16 * u.shape[0]
         else:
-            hmax = m.get("heap_max_u") or 32  # bins above it (up to 36) run the bitmap ESC kernel
+            hmax = m.get("heap_max_u") or 1  # bins above it (up to 36) run the bitonic ESC kernel
             sel = {"merge": bins == 37, "esc": (bins > hmax) & (bins <= 36), "heap": (bins >= 2) & (bins <= hmax)}.get(
                 dom, np.ones(u.shape[0], dtype=bool))
             bytes_dom += algorithmic_bytes(A, B, u, np.nonzero(sel)[0], rn)

@@ -5,7 +5,7 @@ on the architecture (Section 4.1).  This tuner searches, by coordinate descent o
 measured device time, over the parameters the library exposes for that choice:
 
 * heap_max_u   - the longest rows (u_i) given to the heap kernel; the rest of
-                 bins 2..32 go to the bitonic ESC kernel with 32 slots;
+                 bins 2..36 go to the bitonic ESC kernel;
 * heap_block   - threads per block of the heap kernel;
 * merge_batch  - products absorbed per batch by the bin-37 merge kernel;
 * smem_cap_max - the largest result held in shared memory by the merge kernel
@@ -54,7 +54,7 @@ if _ROOT not in sys.path:
 TUNED = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned.json")
 
 SPACE = {
-    "heap_max_u": [32, 24, 16, 8],
+    "heap_max_u": [0, 32, 16, 8],          # 0 = no row uses the heap kernel
     "heap_block": [128, 64, 256],
     "merge_batch": [2048, 1024, 512],
     "smem_cap_max": [0, 8192, 6144, 4096],

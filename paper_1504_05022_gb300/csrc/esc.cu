@@ -1,129 +1,176 @@
-// Stage 3, bin group 4 (u_i = 33..512): the bitonic ESC method of Section 4.1
-// (expand, sort, compress).  With N = 32 it also serves rows of the heap bins
-// (u_i <= 32) when the heap kernel is limited to shorter rows (heap_max_u).
+// Stage 3, bin groups 3 and 4 (u_i = 2..512): the expand-sort-compress method of Section 4.1
+// with a bitonic network, on packed keys.
 //
-// One warp per row.  The warp expands the row's u_i products into a per-warp
-// shared-memory array padded to N = 32*E entries (64, 128, 256 or 512, the bin's
-// upper edge) with the sentinel column INT_MAX, loads E consecutive entries per
-// lane into registers, and sorts the N entries with a bitonic network: element
-// i = lane*E + e, so compare-exchange distances below E stay inside a thread
-// and larger ones are one __shfl_xor_sync per key and value.  Compression is a
-// segmented inclusive scan over equal columns (in registers, then across lanes
-// with shuffles); the last entry of each run carries the run's sum and is
-// written to C~ at the position given by a warp scan of run ends.
+// A group of G lanes takes a row of at most N = G*E products.  It expands the products into
+// shared memory, sorts them by column and sums equal columns.  The network moves one word per
+// product: the column and the product's number among the N, packed into 32 bits when B has
+// fewer than 2^(32 - log2 N) columns and into 64 bits otherwise.  The values stay where they
+// were expanded and are fetched once, by that number, after the sort.  (A network that carries
+// the value along needs three shuffles per step instead of one; A*A of an Erdos-Renyi matrix
+// with 100,003 rows of 16 spent 0.76 ms in it.)  Element i = lane*E + e, so compare-exchange
+// distances below E stay inside a thread and the others are one shuffle.
+//
+// A product's part is found without a search: the starts of the next G
+// parts (non-empty B rows) that fall into the G products at hand become a bit mask, and a
+// lane's part is the number of mask bits at or below it.  Rows of at most 8, 16 and 32
+// products take groups of 8, 8 and 16 lanes, so that a warp has four or two rows' dependent
+// loads in flight; longer ones take a warp.  Latency and issue slots bound it.
+//
+// Measured (one GB300, kernel time, double; before -> after): A*A of that Erdos-Renyi matrix (25.6 M
+// products, bin 35) 764 -> 265 us; A*P of the 27-point operator on 64^3 (6.9 M products, bins
+// 2..27), the heap kernel with one thread per row 262 us -> 152 us, and a values-only replay of
+// R*(A*P) 234 -> 157 us; A*A of a 64 x 64 5-point Laplacian, heap 63 us -> 13 us.  The heap kernel
+// runs only where opts.heap_max_u asks for it.
 #include "internal.h"
 #include "common.cuh"
 
 namespace spg {
 
-constexpr int ESC_WARPS = 4;
+constexpr int ESC_NT = 128;
+
+template <int G, typename T>
+SPG_DEV T group_inclusive_scan(unsigned gm, int gl, T v) {
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) {
+        const T n = __shfl_up_sync(gm, v, d, G);
+        if (gl >= d) v += n;
+    }
+    return v;
+}
+
+template <int G>
+SPG_DEV unsigned group_or(unsigned gm, unsigned v) {
+    if constexpr (G == 32) {
+        return __reduce_or_sync(gm, v);
+    } else {
+#pragma unroll
+        for (int d = 1; d < G; d <<= 1) v |= __shfl_xor_sync(gm, v, d, G);
+        return v;
+    }
+}
+
+template <int G, int E, typename K, bool COUNT>
+struct EscSmem {
+    static constexpr int N = G * E;
+    K key[N];
+    val_t val[COUNT ? 1 : N];
+    int64_t base[G];        // place in B of the part's first entry, minus start
+    val_t av[COUNT ? 1 : G];
+    int32_t start[2 * G];   // first product of the part; INT_MAX past the last part
+};
 
 // COUNT: the counting pass of the precise method (Section 3.1): the same expansion and sort
 // on the columns alone, and nnz(c_i) = the number of distinct columns, written to a.nnzc.
-// The warps stride over the rows (one pass when the grid covers them).
-template <int E, bool COUNT>
-__global__ void __launch_bounds__(ESC_WARPS * 32)
+// The groups stride over the rows (one pass when the grid covers them).
+template <int G, int E, typename K, bool COUNT>
+__global__ void __launch_bounds__(ESC_NT)
 k_esc(StageArgs a, RowSet R) {
-    constexpr int N = 32 * E;
-    __shared__ int32_t sk[ESC_WARPS][N];
-    __shared__ val_t sv[ESC_WARPS][COUNT ? 1 : N];
-    __shared__ int64_t sbs[ESC_WARPS][32];
-    __shared__ int32_t soff[ESC_WARPS][33];
-    __shared__ val_t sa[ESC_WARPS][32];
-    const int lane = lane_id(), w = warp_id();
+    constexpr int N = G * E, GROUPS = ESC_NT / G;
+    // bits of a product's number below its column
+    constexpr int LB = COUNT ? 0 : (sizeof(K) == 8 ? 32 : (N == 8 ? 3 : N == 16 ? 4 : N == 32 ? 5 : N == 64 ? 6 : N == 128 ? 7 : N == 256 ? 8 : 9));
+    static_assert(N <= 512 && (COUNT || sizeof(K) == 8 || (1 << LB) == N), "N is a power of two");
+    constexpr K PAD = ~K(0);
+    constexpr int U = E < 4 ? E : 4;  // groups of G products in flight
+    using Smem = EscSmem<G, E, K, COUNT>;
+    __shared__ Smem smem[GROUPS];
     if (!COUNT && gated(a.gate)) return;
     const int32_t *rows;
     int64_t nrows;
     rowset_range(R, rows, nrows);
-    int32_t *wk = sk[w];
-    val_t *wv = sv[w];
-    for (int64_t t = (int64_t)blockIdx.x * ESC_WARPS + w; t < nrows; t += (int64_t)gridDim.x * ESC_WARPS) {
-        const int row = rows[t];  // the whole warp takes the same rows
-
+    const int gl = threadIdx.x & (G - 1);
+    const unsigned gm = G == 32 ? SPG_FULL : ((1u << (G & 31)) - 1u) << (lane_id() & ~(G - 1));
+    const unsigned le = (2u << gl) - 1u;
+    Smem &S = smem[threadIdx.x / G];
+    for (int64_t t = (int64_t)blockIdx.x * GROUPS + threadIdx.x / G; t < nrows; t += (int64_t)gridDim.x * GROUPS) {
+        const int row = rows[t];
         // ---- expand ----
         int filled = 0;
         const int64_t a0 = a.A.rp[row], a1 = a.A.rp[row + 1];
-        for (int64_t base = a0; base < a1; base += 32) {
-            const int64_t p = base + lane;
+        for (int64_t ch = a0; ch < a1; ch += G) {
+            const int64_t p = ch + gl;
             int32_t len = 0;
             int64_t bs = 0;
-            val_t av = 0.0;
+            val_t av = val_t(0);
             if (p < a1) {
                 const int32_t j = a.A.col[p];
                 bs = a.B.rp[j];
                 len = (int32_t)(a.B.rp[j + 1] - bs);
                 if (!COUNT) av = a.A.val[p];
             }
-            const int32_t inc = warp_inclusive_scan(len);
-            sbs[w][lane] = bs;
-            sa[w][lane] = av;
-            soff[w][lane] = inc - len;
-            if (lane == 31) soff[w][32] = inc;
-            __syncwarp();
-            const int total = soff[w][32];
-            for (int pos = lane; pos < total; pos += 32) {
-                const int e = find_segment_i32(soff[w], 32, pos);
-                const int64_t q = sbs[w][e] + (pos - soff[w][e]);
-                const int dst = filled + pos;
-                if (dst < N) {
-                    wk[dst] = a.B.col[q];
-                    if (!COUNT) wv[dst] = sa[w][e] * a.B.val[q];
+            const int32_t inc = group_inclusive_scan<G>(gm, gl, len);
+            const int total = __shfl_sync(gm, inc, G - 1, G);
+            const unsigned nz = __ballot_sync(gm, len > 0) >> (lane_id() & ~(G - 1));
+            const int np = __popc(G == 32 ? nz : nz & ((1u << (G & 31)) - 1u));
+            if (len > 0) {
+                const int q = __popc(nz & (le >> 1));
+                S.start[q] = inc - len;
+                S.base[q] = bs - (inc - len);
+                if (!COUNT) S.av[q] = av;
+            }
+            if (gl >= np) S.start[gl] = INT_MAX;
+            S.start[G + gl] = INT_MAX;
+            __syncwarp(gm);
+            int part = 0;
+            for (int q0 = 0; q0 < total; q0 += U * G) {
+                int64_t pos[U];
+                int pt[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int q = q0 + u * G;
+                    const unsigned d = (unsigned)(S.start[part + 1 + gl] - q);
+                    const unsigned m = group_or<G>(gm, (q < total && d < (unsigned)G) ? 1u << d : 0u);
+                    pt[u] = part + __popc(m & le);
+                    part += __popc(m);
+                    pos[u] = S.base[pt[u]] + (q + gl);
+                }
+                int32_t c[U];
+                val_t v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (q0 + u * G + gl < total) c[u] = __ldg(a.B.col + pos[u]);
+                if (!COUNT) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (q0 + u * G + gl < total) v[u] = __ldg(a.B.val + pos[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int dst = filled + q0 + u * G + gl;
+                    if (q0 + u * G + gl < total && dst < N) {
+                        S.key[dst] = COUNT ? (K)(uint32_t)c[u] : ((K)(uint32_t)c[u] << (LB & (8 * sizeof(K) - 1))) | (K)dst;
+                        if (!COUNT) S.val[dst] = S.av[pt[u]] * v[u];
+                    }
                 }
             }
             filled += total;
-            __syncwarp();
+            __syncwarp(gm);  // the part table is free again, and the products are visible
         }
-        for (int pos = filled + lane; pos < N; pos += 32) {
-            wk[pos] = KEY_PAD;
-            if (!COUNT) wv[pos] = 0.0;
-        }
-        __syncwarp();
-
-        int32_t key[E];
-        val_t val[E];
+        K key[E];
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-            key[e] = wk[lane * E + e];
-            val[e] = COUNT ? val_t(0) : wv[lane * E + e];
-        }
-        __syncwarp();  // the next row's expansion reuses the warp's arrays
+        for (int e = 0; e < E; ++e) key[e] = e * G + gl < filled ? S.key[e * G + gl] : PAD;
 
-        // ---- bitonic sort, ascending on i = lane*E + e ----
+        // ---- bitonic sort, ascending on i = gl*E + e ----
 #pragma unroll
         for (int k = 2; k <= N; k <<= 1) {
 #pragma unroll
             for (int j = k >> 1; j > 0; j >>= 1) {
                 if (j >= E) {
-                    const int lj = j / E;
-                    const bool lower = (lane & lj) == 0;
+                    const bool lower = (gl & (j / E)) == 0;
 #pragma unroll
                     for (int e = 0; e < E; ++e) {
-                        const int32_t pk = __shfl_xor_sync(SPG_FULL, key[e], lj);
-                        const val_t pv = COUNT ? val_t(0) : __shfl_xor_sync(SPG_FULL, val[e], lj);
-                        const bool up = ((lane * E + e) & k) == 0;
-                        const bool take = (lower == up) ? (pk < key[e]) : (pk > key[e]);
-                        if (take) {
-                            key[e] = pk;
-                            if (!COUNT) val[e] = pv;
-                        }
+                        const K pk = __shfl_xor_sync(gm, key[e], j / E, G);
+                        const bool up = ((gl * E + e) & k) == 0;
+                        key[e] = (lower == up) ? (pk < key[e] ? pk : key[e]) : (pk > key[e] ? pk : key[e]);
                     }
                 } else {
 #pragma unroll
                     for (int e = 0; e < E; ++e) {
                         if ((e & j) == 0) {
-                            const int e2 = e | j;
-                            const bool up = ((lane * E + e) & k) == 0;
-                            const bool sw = up ? (key[e] > key[e2]) : (key[e] < key[e2]);
-                            if (sw) {
-                                const int32_t tk = key[e];
-                                key[e] = key[e2];
-                                key[e2] = tk;
-                                if (!COUNT) {
-                                    const val_t tv = val[e];
-                                    val[e] = val[e2];
-                                    val[e2] = tv;
-                                }
-                            }
+                            const bool up = ((gl * E + e) & k) == 0;
+                            const K x = key[e], y = key[e | j];
+                            const K mn = x < y ? x : y, mx = x < y ? y : x;
+                            key[e] = up ? mn : mx;
+                            key[e | j] = up ? mx : mn;
                         }
                     }
                 }
@@ -132,96 +179,120 @@ k_esc(StageArgs a, RowSet R) {
 
         if constexpr (COUNT) {
             // distinct columns: entries that differ from their predecessor (the pad excluded)
-            const int32_t prev_last_c = __shfl_up_sync(SPG_FULL, key[E - 1], 1);
+            const K before = __shfl_up_sync(gm, key[E - 1], 1, G);
             int cnt = 0;
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int32_t pk = e > 0 ? key[e - 1] : (lane > 0 ? prev_last_c : -1);
-                cnt += (key[e] != KEY_PAD && key[e] != pk) ? 1 : 0;
-            }
-            cnt = warp_reduce_sum(cnt);
-            if (lane == 0) a.nnzc[row] = cnt;
+            for (int e = 0; e < E; ++e)
+                cnt += (key[e] != PAD && (e > 0 ? key[e] != key[e > 0 ? e - 1 : 0] : (gl == 0 || key[e] != before))) ? 1 : 0;
+#pragma unroll
+            for (int d = 1; d < G; d <<= 1) cnt += __shfl_xor_sync(gm, cnt, d, G);
+            if (gl == 0) a.nnzc[row] = cnt;
+            __syncwarp(gm);  // the next row's expansion reuses the keys
         } else {
             // ---- compress: segmented sums over runs of equal columns ----
+            uint32_t col[E];
+            val_t val[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                // the pad's column (all ones) is beyond every real one
+                col[e] = key[e] == PAD ? ~0u : (uint32_t)(key[e] >> (LB & (8 * sizeof(K) - 1)));
+                val[e] = key[e] == PAD ? val_t(0) : S.val[(int)(key[e] & (K)(N - 1))];
+            }
 #pragma unroll
             for (int e = 1; e < E; ++e)
-                if (key[e] == key[e - 1]) val[e] += val[e - 1];
-            const int32_t first = key[0], last = key[E - 1];
-            int32_t prev_last = __shfl_up_sync(SPG_FULL, last, 1);
-            const bool cont = (lane > 0) && (prev_last == first);
-            // R = running sum of the run that ends this lane; flag = a run starts in this lane
-            val_t R = val[E - 1];
-            bool f = !((first == last) && cont);
+                if (col[e] == col[e - 1]) val[e] += val[e - 1];
+            const uint32_t first = col[0], last = col[E - 1];
+            const uint32_t prev_last = __shfl_up_sync(gm, last, 1, G);
+            const bool cont = gl > 0 && prev_last == first && first != ~0u;
+            if (__any_sync(gm, cont)) {
+                // R = running sum of the run that ends this lane; f = a run starts in this lane
+                val_t Rs = val[E - 1];
+                bool f = !((first == last) && cont);
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const val_t Rn = __shfl_up_sync(SPG_FULL, R, d);
-                const bool fn = __shfl_up_sync(SPG_FULL, (int)f, d) != 0;
-                if (lane >= d && !f) {
-                    R += Rn;
-                    f = fn;
+                for (int d = 1; d < G; d <<= 1) {
+                    const val_t Rn = __shfl_up_sync(gm, Rs, d, G);
+                    const bool fn = __shfl_up_sync(gm, (int)f, d, G) != 0;
+                    if (gl >= d && !f) {
+                        Rs += Rn;
+                        f = fn;
+                    }
+                }
+                const val_t carry = __shfl_up_sync(gm, Rs, 1, G);
+                if (cont) {
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (col[e] == first) val[e] += carry;
                 }
             }
-            const val_t carry = __shfl_up_sync(SPG_FULL, R, 1);
-            if (cont) {
-#pragma unroll
-                for (int e = 0; e < E; ++e)
-                    if (key[e] == first) val[e] += carry;
-            }
-            int32_t next_first = __shfl_down_sync(SPG_FULL, first, 1);
-            if (lane == 31) next_first = KEY_PAD;  // nothing follows; the pad never ends a run
+            uint32_t next_first = __shfl_down_sync(gm, first, 1, G);
+            if (gl == G - 1) next_first = ~0u;  // nothing follows; the pad never ends a run
             int cnt = 0;
             unsigned tails = 0;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                const int32_t nk = (e + 1 < E) ? key[e + 1] : next_first;
-                const bool tail = (key[e] != KEY_PAD) && (key[e] != nk || (e == E - 1 && lane == 31));
-                if (tail) {
+                const uint32_t nk = (e + 1 < E) ? col[e + 1 < E ? e + 1 : 0] : next_first;
+                if (col[e] != ~0u && col[e] != nk) {
                     tails |= 1u << e;
                     ++cnt;
                 }
             }
-            const int inc = warp_inclusive_scan(cnt);
-            const int total = __shfl_sync(SPG_FULL, inc, 31);
-            int o = inc - cnt;
-            const int64_t base = a.ctil_rp[row];
-            if (!SPG_IN(base + total <= a.ctil_rp[row + 1], 102)) tails = 0;  // the row's space in C~ (or C)
+            const int inc = group_inclusive_scan<G>(gm, gl, cnt);
+            const int total = __shfl_sync(gm, inc, G - 1, G);
+            const int64_t o = a.ctil_rp[row];
+            const bool fits = SPG_IN(o + total <= a.ctil_rp[row + 1], 102);  // the row's space in C~ (or C)
+            // through shared memory, so that the row leaves in one contiguous run
+            __syncwarp(gm);
+            int q = inc - cnt;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 if (tails & (1u << e)) {
-                    a.ctil_col[base + o] = key[e];
-                    a.ctil_val[base + o] = val[e];
-                    ++o;
+                    S.key[q] = (K)col[e];
+                    S.val[q] = val[e];
+                    ++q;
                 }
             }
-            if (lane == 0) a.nnzc[row] = total;
+            __syncwarp(gm);
+            if (fits) {
+                for (int r = gl; r < total; r += G) {
+                    a.ctil_col[o + r] = (int32_t)S.key[r];
+                    a.ctil_val[o + r] = S.val[r];
+                }
+            }
+            if (gl == 0) a.nnzc[row] = total;
+            __syncwarp(gm);  // the next row's expansion reuses the arrays
         }
     }
 }
 
-cudaError_t launch_esc(const StageArgs &a, const int32_t *rows, int64_t nrows, int bin,
-                       cudaStream_t st) {
-    return launch_esc_set(a, host_rows(rows, nrows), bin, false, st);
-}
-
-template <int E, bool COUNT>
+template <int G, int E, typename K, bool COUNT>
 static cudaError_t esc_go(const StageArgs &a, const RowSet &R, cudaStream_t st) {
-    const int64_t need = (R.n + ESC_WARPS - 1) / ESC_WARPS;
-    const int64_t grid = R.dev_lo ? persistent_blocks((const void *)k_esc<E, COUNT>, ESC_WARPS * 32, 0, need) : need;
+    constexpr int GROUPS = ESC_NT / G;
+    const int64_t need = (R.n + GROUPS - 1) / GROUPS;
+    const int64_t grid = R.dev_lo ? persistent_blocks((const void *)k_esc<G, E, K, COUNT>, ESC_NT, 0, need) : need;
     if (grid <= 0) return cudaErrorInvalidValue;
-    k_esc<E, COUNT><<<(unsigned)grid, ESC_WARPS * 32, 0, st>>>(a, R);
+    k_esc<G, E, K, COUNT><<<(unsigned)grid, ESC_NT, 0, st>>>(a, R);
     return cudaGetLastError();
 }
 
-cudaError_t launch_esc_set(const StageArgs &a, const RowSet &R, int bin, bool count_only, cudaStream_t st) {
+// The counting pass sorts plain columns; else the packed key must hold column and number, and
+// stay below the pad.
+template <int G, int E>
+static cudaError_t esc_pick(const StageArgs &a, const RowSet &R, bool count_only, cudaStream_t st) {
+    if (count_only) return esc_go<G, E, uint32_t, true>(a, R, st);
+    if (a.B.ncols * (G * E) < (int64_t(1) << 32)) return esc_go<G, E, uint32_t, false>(a, R, st);
+    return esc_go<G, E, uint64_t, false>(a, R, st);
+}
+
+cudaError_t launch_esc_set(const StageArgs &a, const RowSet &R, int max_u, bool count_only, cudaStream_t st) {
     if (R.n <= 0) return cudaSuccess;
-    switch (bin) {
-        case 32: return count_only ? esc_go<1, true>(a, R, st) : esc_go<1, false>(a, R, st);  // u <= 32
-        case 33: return count_only ? esc_go<2, true>(a, R, st) : esc_go<2, false>(a, R, st);
-        case 34: return count_only ? esc_go<4, true>(a, R, st) : esc_go<4, false>(a, R, st);
-        case 35: return count_only ? esc_go<8, true>(a, R, st) : esc_go<8, false>(a, R, st);
-        case 36: return count_only ? esc_go<16, true>(a, R, st) : esc_go<16, false>(a, R, st);
-        default: return cudaErrorInvalidValue;
-    }
+    if (max_u <= 8) return esc_pick<8, 1>(a, R, count_only, st);
+    if (max_u <= 16) return esc_pick<8, 2>(a, R, count_only, st);
+    if (max_u <= 32) return esc_pick<16, 2>(a, R, count_only, st);
+    if (max_u <= 64) return esc_pick<32, 2>(a, R, count_only, st);
+    if (max_u <= 128) return esc_pick<32, 4>(a, R, count_only, st);
+    if (max_u <= 256) return esc_pick<32, 8>(a, R, count_only, st);
+    if (max_u <= 512) return esc_pick<32, 16>(a, R, count_only, st);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace spg

@@ -103,11 +103,6 @@ k_heap(StageArgs a, RowSet R, int slots) {
 #undef HV
 }
 
-cudaError_t launch_heap(const StageArgs &a, const int32_t *rows, int64_t nrows, int slots, int nt,
-                        cudaStream_t st) {
-    return launch_heap_set(a, host_rows(rows, nrows), slots, nt, st);
-}
-
 cudaError_t launch_heap_set(const StageArgs &a, const RowSet &R, int slots, int nt, cudaStream_t st) {
     if (R.n <= 0) return cudaSuccess;
     const size_t smem = (size_t)slots * nt * (sizeof(val_t) + sizeof(int32_t));

@@ -122,14 +122,10 @@ struct StageArgs {
     const int64_t *gate = nullptr;  // when set and *gate != 0, the kernels write nothing (C too small)
 };
 
-cudaError_t launch_heap(const StageArgs &a, const int32_t *rows, int64_t nrows, int slots, int nt,
-                        cudaStream_t st);
 cudaError_t launch_heap_set(const StageArgs &a, const RowSet &R, int slots, int nt, cudaStream_t st);
-cudaError_t launch_esc(const StageArgs &a, const int32_t *rows, int64_t nrows, int bin,
-                       cudaStream_t st);
-// count_only: nnz(c_i) of every row into a.nnzc and nothing else (the counting pass of the
-// precise method, Section 3.1); bin 32 stands for any u_i <= 32
-cudaError_t launch_esc_set(const StageArgs &a, const RowSet &R, int bin, bool count_only, cudaStream_t st);
+// rows of at most max_u (<= 512) products.  count_only: nnz(c_i) of every row into a.nnzc and
+// nothing else (the counting pass of the precise method, Section 3.1)
+cudaError_t launch_esc_set(const StageArgs &a, const RowSet &R, int max_u, bool count_only, cudaStream_t st);
 
 // Bin-37 work items.  Item j < n37 is the j-th row of bin 37 with the full
 // column range.  An item whose sequence outgrows the largest shared-memory

@@ -145,6 +145,11 @@ struct Timer {
 // Heap-kernel launches: bins 2..32 split into ranges sized to their widest heap.
 const int kHeapRanges[][2] = {{2, 8}, {9, 16}, {17, 24}, {25, 32}};
 
+// Bitonic ESC launches: ranges of bins by the width of the network.
+const struct {
+    int lo, hi, max_u;
+} kEscRanges[] = {{2, 8, 8}, {9, 16, 16}, {17, 32, 32}, {33, 33, 64}, {34, 34, 128}, {35, 35, 256}, {36, 36, 512}};
+
 // Bytes of one stored entry (int32 column + value).
 constexpr int64_t ENTRY_BYTES = sizeof(int32_t) + sizeof(val_t);
 
@@ -483,13 +488,13 @@ RowSet bin_range(const spgemm_plan *p, int lo, int hi, bool dev) {
     return host_rows(p->bin_rows + p->bin_start[lo], p->bin_start[hi + 1] - p->bin_start[lo]);
 }
 
-// Stage 3, bins 2..36 (bin groups 3 and 4): the heap kernel for bins 2..heap_max_u
-// (one launch per range, sized to the range's widest heap), the bitonic ESC kernel
-// with 32 slots for the rest of bins up to 32, and ESC for bins 33..36.  With dev the
-// bin sizes are read on the device (persistent grids; every launch is made).
+// Stage 3, bins 2..36 (bin groups 3 and 4): the bitonic ESC kernel, one launch per width of
+// its network; with opts.heap_max_u, the heap kernel for bins 2..heap_max_u (one launch per
+// range, sized to the range's widest heap).  With dev the bin sizes are read on the device
+// (persistent grids; every launch is made).
 cudaError_t launch_short_bins(spgemm_plan *p, const StageArgs &a, bool account, bool dev = false) {
     cudaError_t e = cudaSuccess;
-    const int hmax = (p->opts.heap_max_u >= 2 && p->opts.heap_max_u <= 32) ? p->opts.heap_max_u : 32;
+    const int hmax = (p->opts.heap_max_u >= 2 && p->opts.heap_max_u <= 32) ? p->opts.heap_max_u : 1;
     const int heap_nt = p->opts.heap_block > 0 ? p->opts.heap_block : 128;
     auto run = [&](int kind, auto &&launch) {
         if (account) p->time_begin(kind);
@@ -507,14 +512,11 @@ cudaError_t launch_short_bins(spgemm_plan *p, const StageArgs &a, bool account, 
         if (R.n > 0 && run(SPGEMM_K_HEAP, [&] { return launch_heap_set(a, R, hi, heap_nt, p->st); }) != cudaSuccess)
             return e;
     }
-    if (hmax < 32) {
-        const RowSet R = bin_range(p, hmax + 1, 32, dev);
-        if (R.n > 0 && run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, 32, false, p->st); }) != cudaSuccess)
-            return e;
-    }
-    for (int b = BIN_ESC_LO; b <= BIN_ESC_HI; ++b) {
-        const RowSet R = bin_range(p, b, b, dev);
-        if (R.n > 0 && run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, b, false, p->st); }) != cudaSuccess)
+    for (auto &r : kEscRanges) {
+        const int lo = std::max(r.lo, hmax + 1), hi = r.hi;
+        if (lo > hi) continue;
+        const RowSet R = bin_range(p, lo, hi, dev);
+        if (R.n > 0 && run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, r.max_u, false, p->st); }) != cudaSuccess)
             return e;
     }
     return cudaSuccess;
@@ -1886,12 +1888,9 @@ static cudaError_t precise_count(spgemm_plan *p, bool dev) {
         return e;
     };
     cudaError_t e;
-    const RowSet r32 = bin_range(p, BIN_HEAP_LO, BIN_HEAP_HI, dev);
-    if (r32.n > 0 && (e = run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, r32, 32, true, p->st); })) != cudaSuccess)
-        return e;
-    for (int b = BIN_ESC_LO; b <= BIN_ESC_HI; ++b) {
-        const RowSet R = bin_range(p, b, b, dev);
-        if (R.n > 0 && (e = run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, b, true, p->st); })) != cudaSuccess)
+    for (auto &r : kEscRanges) {
+        const RowSet R = bin_range(p, r.lo, r.hi, dev);
+        if (R.n > 0 && (e = run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, r.max_u, true, p->st); })) != cudaSuccess)
             return e;
     }
     if (p->dense_K > 0 && (dev || p->dense_n > 0)) {
