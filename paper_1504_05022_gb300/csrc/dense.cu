@@ -52,54 +52,6 @@ cudaError_t launch_dense_bounds(const DevCSR &B, int K, int W, int32_t *bnd, cud
     return cudaGetLastError();
 }
 
-// ---- which bin-37 rows are dense ----
-// One warp per row: u_i from the stage-1 prefix, and for u_i > 512 the row's column
-// range [lo, hi) (first and last column of every touched B row).  The row is dense when
-// u_i >= dmin (dmin > 0), else when div u_i >= hi - lo: its products cover at least a
-// div-th of the columns they can reach, so the dense accumulator's O(hi - lo) clearing
-// and write-out are small beside them.
-__global__ void k_dense_mark(DevCSR A, DevCSR B, const int64_t *__restrict__ S, int64_t dmin, int div,
-                             uint8_t *flag, int32_t *lo, int32_t *hi) {
-    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (row >= A.nrows) return;
-    const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
-    const int64_t u = S[a1] - S[a0];
-    if (u <= BIN_MERGE_MIN_U) {
-        if (lane == 0) flag[row] = 0;
-        return;
-    }
-    int32_t cmin = INT32_MAX, cmax = -1;
-    for (int64_t e = a0 + lane; e < a1; e += 32) {
-        const int32_t k = A.col[e];
-        const int64_t rs = B.rp[k], re = B.rp[k + 1];
-        if (re > rs) {
-            cmin = min(cmin, B.col[rs]);
-            cmax = max(cmax, B.col[re - 1]);
-        }
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        cmin = min(cmin, __shfl_xor_sync(SPG_FULL, cmin, d));
-        cmax = max(cmax, __shfl_xor_sync(SPG_FULL, cmax, d));
-    }
-    if (lane == 0) {
-        const int64_t span = (int64_t)cmax - cmin + 1;  // u > 0, so some B row is not empty
-        flag[row] = (uint8_t)(dmin > 0 ? u >= dmin : (int64_t)div * u >= span);
-        lo[row] = cmin;
-        hi[row] = cmax + 1;
-    }
-}
-
-cudaError_t launch_dense_mark(const DevCSR &A, const DevCSR &B, const int64_t *S, int64_t dmin, int div,
-                              uint8_t *flag, int32_t *lo, int32_t *hi, cudaStream_t st) {
-    if (A.nrows <= 0) return cudaSuccess;
-    if (div < 1) return cudaErrorInvalidValue;
-    const int64_t threads = A.nrows * 32;
-    k_dense_mark<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(A, B, S, dmin, div, flag, lo, hi);
-    return cudaGetLastError();
-}
-
 // ---- selection of the dense rows among the bin-37 rows ----
 // Bucket g = 63 - floor(log2 u) (the leading zeros of u) for a dense row, so that
 // larger rows come first; DENSE_BUCKETS for the others.  order[0..nd) lists the

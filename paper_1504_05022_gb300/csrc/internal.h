@@ -70,35 +70,48 @@ struct CapPolicy {
 };
 
 // ---- stage 0/1/2 (stage12.cu) ----
-cudaError_t launch_widen_rowptr(const int32_t *in, int64_t *out, int64_t n, cudaStream_t st);
+// widens in[0..n) and, with the same launch, in2[0..n2)
+cudaError_t launch_widen_rowptr(const int32_t *in, int64_t *out, int64_t n, cudaStream_t st,
+                                const int32_t *in2 = nullptr, int64_t *out2 = nullptr, int64_t n2 = 0);
 cudaError_t launch_validate(const DevCSR &M, int64_t *status, cudaStream_t st);
-// S[j] = sum_{t<j} nnz(b_{A.col[t]*}), S[nnzA] = sum u (Algorithm 2 as a prefix sum).
-cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, int64_t *S, int64_t *partial,
-                         cudaStream_t st);
-int64_t bound_partial_size(int64_t nnzA);
-// Binning scratch sizes for m rows.
-int64_t bin_blocks(int64_t m);
-cudaError_t launch_binning(int64_t m, const int64_t *arp, const int64_t *S,
-                           const int64_t *sum_u_ptr, CapPolicy P, int64_t *u, uint8_t *bin, int32_t *nnzc, int32_t *bin_rows,
-                           int64_t *ctil_rp, int32_t *hist, int64_t *cap_partial,
-                           BinSummary *summary, cudaStream_t st);
+// What stage 1 writes: per row u_i (Algorithm 2), its bin, nnz(c_i) where the bound is exact
+// (bins 0 and 1), and with CapPolicy::dense set the dense-slice flag (the same array) and the
+// column range of the bin-37 rows; per block of rows (bin_blocks(m, nnzA) of them) the bin
+// histogram (NUM_BINS x blocks) and the sums of C~ entries and of u_i (2 x blocks).  *err = 0.
+struct BoundOut {
+    int64_t *u;
+    uint8_t *bin;
+    int32_t *nnzc;
+    uint8_t *flag;
+    int32_t *lo, *hi;
+    int64_t dmin;  // a bin-37 row is dense when u_i >= dmin (dmin > 0),
+    int div;       // else when div u_i >= the width of its column range
+    int32_t *hist;
+    int64_t *part;
+    int64_t *err;
+};
+int64_t bin_blocks(int64_t m, int64_t nnzA);
+cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, const BoundOut &O, cudaStream_t st);
+// Stage 2: the rows grouped by bin, C~'s row offsets, and the summary (also into `host`, pinned
+// memory mapped into the device's address space, when given).
+cudaError_t launch_binning(int64_t m, int64_t nnzA, const CapPolicy &P, const BoundOut &O, int32_t *bin_rows,
+                           int64_t *ctil_rp, BinSummary *summary, BinSummary *host, cudaStream_t st);
 
 // C~ row offsets again from u and the bins under P (ctil_rp[0..m]; the total into *total)
 cudaError_t launch_cap_rescan(int64_t m, const int64_t *u, const uint8_t *bin, CapPolicy P, int64_t *ctil_rp,
                               int64_t *partial, int64_t *total, cudaStream_t st);
 
 // ---- learned preallocation (predictor.cu) ----
-// Row features (warp per row).  With the stage-1 prefix S, rows with u_i <= u_min are
+// Row features (warp per row).  With u given, rows with u_i <= u_min are
 // skipped, and so are the rows flagged in `skip` (when given).
 cudaError_t launch_row_features(const DevCSR &A, const DevCSR &B, float *X, cudaStream_t st,
-                                const int64_t *S = nullptr, int64_t u_min = 0, const uint8_t *skip = nullptr);
-// Predicted temporary size per row (0 for rows skipped through arp/S/u_min/skip).  With
+                                const int64_t *u = nullptr, int64_t u_min = 0, const uint8_t *skip = nullptr);
+// Predicted temporary size per row (0 for rows with u_i <= u_min or flagged in `skip`).  With
 // promote_min > 0, a row whose predicted nnz(c_i) is at least promote_min is flagged in
 // skip (a dense-slice row) instead.
 cudaError_t launch_predict_caps(const float *params, const float *X, int64_t m, const int64_t *u, float margin,
-                                int32_t min_cap, int32_t *pred_cap, cudaStream_t st, const int64_t *arp = nullptr,
-                                const int64_t *S = nullptr, int64_t u_min = 0, uint8_t *skip = nullptr,
-                                int64_t promote_min = 0);
+                                int32_t min_cap, int32_t *pred_cap, cudaStream_t st, int64_t u_min = 0,
+                                uint8_t *skip = nullptr, int64_t promote_min = 0);
 // Groups the bin-37 items (tail of bin_rows, size read from summary) by launch
 // class; items of flagged (dense-slice) rows go after the last class; scratch: 96 + m
 // int32; order: item indices grouped by class; counts go to summary->class_count.
@@ -221,10 +234,6 @@ struct DenseArgs {
                                // marking the columns again
 };
 cudaError_t launch_dense_bounds(const DevCSR &B, int K, int W, int32_t *bnd, cudaStream_t st);
-// per row: flag (1 = dense-slice row: bin 37, and u_i >= dmin if dmin > 0, else div u_i >= the
-// width of its column range) and, for bin-37 rows, the column range [lo, hi)
-cudaError_t launch_dense_mark(const DevCSR &A, const DevCSR &B, const int64_t *S, int64_t dmin, int div,
-                              uint8_t *flag, int32_t *lo, int32_t *hi, cudaStream_t st);
 int64_t dense_select_scratch(int64_t m);
 // order[0..nd) = items of the flagged bin-37 rows (larger u first), order[nd..n37) = the rest;
 // rows, rlo, rhi [0..nd) = their rows and column ranges; nd goes to summary->dense_count
@@ -289,13 +298,15 @@ cudaError_t launch_split_out(const PairDesc *d, int64_t npairs, const int64_t *c
                              cudaStream_t st);
 
 // ---- stage 4 (arrange.cu) ----
+// c_rp = the prefix sum of nnzc (m + 1 entries); with host (two words of pinned memory mapped
+// into the device's address space), also host[0] = c_rp[m] and host[1] = *err
+int row_scan_launches(int64_t m);
+int64_t row_scan_partials(int64_t m);  // int64 words of `partial`
 cudaError_t launch_row_scan(int64_t m, const int32_t *nnzc, int64_t *c_rp, int64_t *partial,
-                            cudaStream_t st);
-cudaError_t launch_arrange_short(const StageArgs &a, const int32_t *rows, int64_t nrows,
-                                 const uint8_t *bin, const int64_t *c_rp, int32_t *c_col,
-                                 val_t *c_val, cudaStream_t st);
-cudaError_t launch_arrange_short_set(const StageArgs &a, const RowSet &R, const uint8_t *bin, const int64_t *c_rp,
-                                     int32_t *c_col, val_t *c_val, cudaStream_t st);
+                            cudaStream_t st, int64_t *host = nullptr, const int64_t *err = nullptr);
+// copies the rows of C~ into C; avg_nnz: entries of an average row of C (sets the lanes per row)
+cudaError_t launch_arrange_short(const StageArgs &a, const RowSet &R, const uint8_t *bin, const int64_t *c_rp,
+                                 int32_t *c_col, val_t *c_val, int64_t avg_nnz, cudaStream_t st);
 // *gate = 1, *err = 8 and every c_rp[0..m] = 0 (C empty) when the result of m rows (c_rp[m]
 // entries) exceeds cap entries, else *gate = 0
 cudaError_t launch_gate(int64_t *c_rp, int64_t m, int64_t cap, int64_t *gate, int64_t *err, cudaStream_t st);

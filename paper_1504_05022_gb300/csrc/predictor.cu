@@ -38,16 +38,16 @@ constexpr int R_XH = 0, R_H1 = MLP_IN, R_H2 = R_H1 + MLP_HID, R_DZ1 = R_H2 + MLP
 
 // One warp per row: the 8 features (log2(1+.) of nnz(a_i*), u_i, min/max/mean/std
 // of the selected B-row lengths, the column span of the selected B rows, ncols(B)).
-__global__ void k_row_features(DevCSR A, DevCSR B, const int64_t *__restrict__ S, int64_t u_min,
+__global__ void k_row_features(DevCSR A, DevCSR B, const int64_t *__restrict__ u, int64_t u_min,
                                const uint8_t *__restrict__ skip, float *__restrict__ X) {
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (row >= A.nrows) return;
-    const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
-    // with the stage-1 prefix S given, only rows with u_i > u_min (bin 37) need features, and
+    // with the bounds u given, only rows with u_i > u_min (bin 37) need features, and
     // not the dense-slice rows
-    if (S != nullptr && S[a1] - S[a0] <= u_min) return;
+    if (u != nullptr && u[row] <= u_min) return;
     if (skip != nullptr && skip[row]) return;
+    const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
     double sum_len = 0.0, sg = 0.0, sg2 = 0.0;
     float gmin = 3.4e38f, gmax = -3.4e38f;
     int32_t cmin = INT_MAX, cmax = -1;
@@ -95,11 +95,11 @@ __global__ void k_row_features(DevCSR A, DevCSR B, const int64_t *__restrict__ S
     }
 }
 
-cudaError_t launch_row_features(const DevCSR &A, const DevCSR &B, float *X, cudaStream_t st, const int64_t *S,
+cudaError_t launch_row_features(const DevCSR &A, const DevCSR &B, float *X, cudaStream_t st, const int64_t *u,
                                 int64_t u_min, const uint8_t *skip) {
     if (A.nrows <= 0) return cudaSuccess;
     const int64_t threads = A.nrows * 32;
-    k_row_features<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(A, B, S, u_min, skip, X);
+    k_row_features<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(A, B, u, u_min, skip, X);
     return cudaGetLastError();
 }
 
@@ -268,8 +268,7 @@ __global__ void k_mlp_adam(float *__restrict__ params, const float *__restrict__
 // from the regression head, times `margin`, rounded up to 32; u_i itself when it is
 // within a factor `margin` of that size.
 __global__ void k_mlp_predict_caps(const float *__restrict__ params, const float *__restrict__ X, int64_t m,
-                                   const int64_t *__restrict__ u, const int64_t *__restrict__ arp,
-                                   const int64_t *__restrict__ S, int64_t u_min, uint8_t *__restrict__ skip,
+                                   const int64_t *__restrict__ u, int64_t u_min, uint8_t *__restrict__ skip,
                                    float margin, int32_t min_cap, int32_t *__restrict__ pred_cap,
                                    int64_t promote_min) {
     __shared__ float P[SPGEMM_MLP_NUM_TOTAL];
@@ -277,10 +276,10 @@ __global__ void k_mlp_predict_caps(const float *__restrict__ params, const float
     __syncthreads();
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= m) return;
-    // the row's bound u_i (Algorithm 2), when known
-    const int64_t uu = S != nullptr ? S[arp[s + 1]] - S[arp[s]] : (u != nullptr ? u[s] : -1);
+    // the row's bound u_i (Algorithm 2)
+    const int64_t uu = u[s];
     // outside bin 37, or a dense-slice row: no prediction needed
-    if ((S != nullptr && uu <= u_min) || (skip != nullptr && skip[s])) {
+    if (uu <= u_min || (skip != nullptr && skip[s])) {
         pred_cap[s] = 0;
         return;
     }
@@ -297,21 +296,19 @@ __global__ void k_mlp_predict_caps(const float *__restrict__ params, const float
     double c = ceil(nnz * (double)margin / 32.0) * 32.0;
     int64_t cap = (int64_t)c;
     if (cap < min_cap) cap = min_cap;
-    if (uu >= 0) {
-        // a bound within a factor `margin` of the sized prediction is taken instead: the row
-        // can then never outgrow its slot, for at most `margin` times the prediction's space
-        if ((double)uu <= (double)cap * (double)margin) cap = uu;
-        if (cap > uu) cap = uu;
-    }
+    // a bound within a factor `margin` of the sized prediction is taken instead: the row
+    // can then never outgrow its slot, for at most `margin` times the prediction's space
+    if ((double)uu <= (double)cap * (double)margin) cap = uu;
+    if (cap > uu) cap = uu;
     if (cap > INT32_MAX) cap = INT32_MAX;
     pred_cap[s] = (int32_t)cap;
 }
 
 cudaError_t launch_predict_caps(const float *params, const float *X, int64_t m, const int64_t *u, float margin,
-                                int32_t min_cap, int32_t *pred_cap, cudaStream_t st, const int64_t *arp,
-                                const int64_t *S, int64_t u_min, uint8_t *skip, int64_t promote_min) {
+                                int32_t min_cap, int32_t *pred_cap, cudaStream_t st, int64_t u_min, uint8_t *skip,
+                                int64_t promote_min) {
     if (m <= 0) return cudaSuccess;
-    k_mlp_predict_caps<<<(unsigned)((m + 127) / 128), 128, 0, st>>>(params, X, m, u, arp, S, u_min, skip, margin,
+    k_mlp_predict_caps<<<(unsigned)((m + 127) / 128), 128, 0, st>>>(params, X, m, u, u_min, skip, margin,
                                                                      min_cap, pred_cap, promote_min);
     return cudaGetLastError();
 }

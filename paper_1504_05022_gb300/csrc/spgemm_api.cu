@@ -179,7 +179,7 @@ struct spgemm_plan {
     int64_t bytes_held = 0;  // device bytes the plan holds now
     int64_t bytes_peak = 0;  // largest bytes_held so far
     // stage 1-2 buffers
-    int64_t *S = nullptr, *u = nullptr, *ctil_rp = nullptr, *scan_partial = nullptr;
+    int64_t *u = nullptr, *ctil_rp = nullptr, *scan_partial = nullptr;
     uint8_t *bin = nullptr;
     int32_t *bin_rows = nullptr, *nnzc = nullptr, *ctil_col_i = nullptr;
     int32_t *ctil_col = nullptr;
@@ -560,6 +560,23 @@ static void plan_abort(spgemm_plan *p) {
     delete p;
 }
 
+// Where stage 1 writes (merge_limits and the allocations come first).
+static BoundOut bound_out(const spgemm_plan *p) {
+    BoundOut o{};
+    o.u = p->u;
+    o.bin = p->bin;
+    o.nnzc = p->nnzc;
+    o.flag = p->dense_flag;
+    o.lo = p->dense_lo;
+    o.hi = p->dense_hi;
+    o.dmin = p->dense_min_u;
+    o.div = p->opts.dense_span_div > 0 ? p->opts.dense_span_div : 8;
+    o.hist = p->d_hist;
+    o.part = p->d_capp;
+    o.err = p->d_err;
+    return o;
+}
+
 // Stages 1 and 2 on the plan's A and B (int64 row pointers on the device).
 static spgemm_status plan_symbolic_core(spgemm_plan *p) {
     spgemm_status status = SPGEMM_OK;
@@ -570,10 +587,9 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
     {
         SPG_TRY(p->alloc_n(&p->d_summary, 1));
         SPG_TRY(p->alloc_n(&p->d_err, 1));
-        SPG_TRY(cudaMemsetAsync(p->d_summary, 0, sizeof(BinSummary), p->st));
-        SPG_TRY(cudaMemsetAsync(p->d_err, 0, sizeof(int64_t), p->st));
         if (o.check_inputs) {
             // the check's result is read before any kernel indexes B through A's columns
+            SPG_TRY(cudaMemsetAsync(p->d_summary, 0, sizeof(BinSummary), p->st));
             p->time_begin(SPGEMM_K_OTHER);
             SPG_TRY(launch_validate(p->A, &p->d_summary->status, p->st));
             SPG_TRY(launch_validate(p->B, &p->d_summary->status, p->st));
@@ -586,16 +602,7 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
                 goto fail;
             }
         }
-        // ---- stage 1: upper bound ----
-        SPG_TRY(p->alloc_n(&p->S, nnzA + 1, LIFE_SYMBOLIC));
-        {
-            int64_t nb = std::max<int64_t>(bound_partial_size(nnzA), bin_blocks(m) + 1);
-            SPG_TRY(p->alloc_n(&p->scan_partial, nb + 1));
-        }
-        p->time_begin(SPGEMM_K_BOUND);
-        SPG_TRY(launch_bound(p->A, p->B, p->S, p->scan_partial, p->st));
-        p->time_end();
-        p->count(SPGEMM_K_BOUND, 3);
+        SPG_TRY(p->alloc_n(&p->scan_partial, row_scan_partials(m)));
         merge_limits(p);
         if (o.alloc_policy == SPGEMM_ALLOC_PRECISE && p->dense_K == 0 && p->B.ncols > 0) {
             status = SPGEMM_ERR_SHAPE;  // B too wide for the column slices of the precise method
@@ -606,37 +613,40 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
             SPG_TRY(p->alloc_n(&p->dense_flag, m, LIFE_SYMBOLIC));
             SPG_TRY(p->alloc_n(&p->dense_lo, m, LIFE_SYMBOLIC));
             SPG_TRY(p->alloc_n(&p->dense_hi, m, LIFE_SYMBOLIC));
-            SPG_TRY(launch_dense_mark(p->A, p->B, p->S, p->dense_min_u,
-                                      o.dense_span_div > 0 ? o.dense_span_div : 8, p->dense_flag, p->dense_lo,
-                                      p->dense_hi, p->st));
-            p->count(SPGEMM_K_OTHER);
         }
-        // ---- stage 2: binning ----
-        nblk = bin_blocks(m);
+        nblk = bin_blocks(m, nnzA);
         SPG_TRY(p->alloc_n(&p->u, m));
         SPG_TRY(p->alloc_n(&p->bin, m));
         SPG_TRY(p->alloc_n(&p->nnzc, m));
         SPG_TRY(p->alloc_n(&p->bin_rows, m));
         SPG_TRY(p->alloc_n(&p->ctil_rp, m + 1));
         {
-            int32_t *hist = nullptr;
-            int64_t *capp = nullptr;
-            SPG_TRY(p->alloc_n(&hist, (int64_t)NUM_BINS * nblk, LIFE_SYMBOLIC));
-            SPG_TRY(p->alloc_n(&capp, nblk, LIFE_SYMBOLIC));
+            SPG_TRY(p->alloc_n(&p->d_hist, (int64_t)NUM_BINS * nblk, LIFE_SYMBOLIC));
+            SPG_TRY(p->alloc_n(&p->d_capp, 2 * nblk, LIFE_SYMBOLIC));
             pol.policy = o.alloc_policy;
             pol.initial_cap = o.initial_cap;
             pol.pred_cap = nullptr;  // learned: bin-37 sizes are set after the prediction below
             pol.cap_max = p->capmax;
             pol.dense = p->dense_flag;
-            p->time_begin(SPGEMM_K_BIN);
-            SPG_TRY(launch_binning(m, p->A.rp, p->S, p->S + nnzA, pol, p->u, p->bin, p->nnzc, p->bin_rows,
-                                   p->ctil_rp, hist, capp, p->d_summary, p->st));
+            const BoundOut out = bound_out(p);
+            void *host = nullptr;
+            SPG_TRY(cudaHostGetDevicePointer(&host, p->pinned, 0));
+            // ---- stage 1: upper bound ----
+            p->time_begin(SPGEMM_K_BOUND);
+            SPG_TRY(launch_bound(p->A, p->B, pol, out, p->st));
             p->time_end();
-            p->count(SPGEMM_K_BIN, nblk > 0 ? 3 : 1);
+            p->count(SPGEMM_K_BOUND, nblk > 0 ? 1 : 0);
+            // ---- stage 2: binning ----
+            p->time_begin(SPGEMM_K_BIN);
+            SPG_TRY(launch_binning(m, nnzA, pol, out, p->bin_rows, p->ctil_rp, p->d_summary,
+                                   static_cast<BinSummary *>(host), p->st));
+            p->time_end();
+            p->count(SPGEMM_K_BIN, nblk > 0 ? 2 : 1);
+            SPG_TRY(cudaStreamSynchronize(p->st));
+            std::memcpy(&p->h_summary, p->pinned, sizeof(BinSummary));
         }
-        // the bin sizes first: without bin-37 rows the learned launch classes and the slice
-        // selection have nothing to do, and their launches are skipped
-        SPG_TRY(p->d2h(&p->h_summary, p->d_summary, sizeof(BinSummary)));
+        // without bin-37 rows the learned launch classes and the slice selection have nothing to
+        // do, and their launches are skipped
         if (p->h_summary.bin_count[BIN_MERGE] > 0 && (o.alloc_policy == SPGEMM_ALLOC_LEARNED || p->dense_K > 0)) {
             if (o.alloc_policy == SPGEMM_ALLOC_LEARNED) {
                 // features and predicted temporary sizes of the bin-37 rows, then the rows of C~
@@ -645,11 +655,11 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
                 SPG_TRY(p->alloc_n(&X, m * SPGEMM_MLP_FEATURES, LIFE_SYMBOLIC));
                 SPG_TRY(p->alloc_n(&p->pred_cap, m, LIFE_SYMBOLIC));
                 p->time_begin(SPGEMM_K_OTHER);
-                SPG_TRY(launch_row_features(p->A, p->B, X, p->st, p->S, BIN_MERGE_MIN_U, p->dense_flag));
-                SPG_TRY(launch_predict_caps(predictor_params(o.predictor), X, m, nullptr,
+                SPG_TRY(launch_row_features(p->A, p->B, X, p->st, p->u, BIN_MERGE_MIN_U, p->dense_flag));
+                SPG_TRY(launch_predict_caps(predictor_params(o.predictor), X, m, p->u,
                                             (float)(o.predictor_margin > 0 ? o.predictor_margin : 1.0),
-                                            o.initial_cap, p->pred_cap, p->st, p->A.rp, p->S, BIN_MERGE_MIN_U,
-                                            p->dense_flag, p->dense_K > 0 ? (int64_t)o.dense_pred_min : 0));
+                                            o.initial_cap, p->pred_cap, p->st, BIN_MERGE_MIN_U, p->dense_flag,
+                                            p->dense_K > 0 ? (int64_t)o.dense_pred_min : 0));
                 pol.pred_cap = p->pred_cap;
                 SPG_TRY(launch_cap_rescan(m, p->u, p->bin, pol, p->ctil_rp, p->scan_partial, &p->d_summary->sum_cap,
                                           p->st));
@@ -707,30 +717,39 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
         p->release_temps(LIFE_SYMBOLIC);
         p->dense_flag = nullptr;
         p->dense_lo = p->dense_hi = nullptr;
+        p->d_hist = nullptr;
+        p->d_capp = nullptr;
     }
     return SPGEMM_OK;
 fail:
     return status;
 }
 
-// Widens an int32 row-pointer array into a plan-owned int64 copy when needed.
-static cudaError_t plan_widen(spgemm_plan *p, const spgemm_csr_in *M, DevCSR &D) {
-    D.nrows = M->nrows;
-    D.ncols = M->ncols;
-    D.nnz = M->nnz;
-    D.col = M->col_idx;
-    D.val = M->val;
-    if (M->rowptr_bits == 64) {
-        D.rp = static_cast<const int64_t *>(M->row_ptr);
-        return cudaSuccess;
+// The device matrices of A and B; int32 row pointers are widened into plan-owned int64 copies
+// (one copy when both are the same array).
+static cudaError_t plan_inputs(spgemm_plan *p, const spgemm_csr_in *A, const spgemm_csr_in *B) {
+    const spgemm_csr_in *in[2] = {A, B};
+    DevCSR *D[2] = {&p->A, &p->B};
+    const bool shared = A->row_ptr == B->row_ptr && A->rowptr_bits == B->rowptr_bits && A->nrows == B->nrows;
+    const int32_t *src[2] = {nullptr, nullptr};
+    int64_t *dst[2] = {nullptr, nullptr}, n[2] = {0, 0};
+    for (int k = 0; k < 2; ++k) {
+        const spgemm_csr_in *M = in[k];
+        *D[k] = DevCSR{M->nrows, M->ncols, M->nnz, static_cast<const int64_t *>(M->row_ptr), M->col_idx, M->val};
+        if (M->rowptr_bits == 64) continue;
+        if (k == 1 && shared) {
+            D[1]->rp = D[0]->rp;
+            continue;
+        }
+        cudaError_t e = p->alloc_n(&dst[k], M->nrows + 1);
+        if (e != cudaSuccess) return e;
+        src[k] = static_cast<const int32_t *>(M->row_ptr);
+        n[k] = M->nrows + 1;
+        D[k]->rp = dst[k];
     }
-    int64_t *rp = nullptr;
-    cudaError_t e = p->alloc_n(&rp, M->nrows + 1);
-    if (e != cudaSuccess) return e;
-    e = launch_widen_rowptr(static_cast<const int32_t *>(M->row_ptr), rp, M->nrows + 1, p->st);
+    if (n[0] + n[1] == 0) return cudaSuccess;
     p->count(SPGEMM_K_OTHER);
-    D.rp = rp;
-    return e;
+    return launch_widen_rowptr(src[0], dst[0], n[0], p->st, src[1], dst[1], n[1]);
 }
 
 extern "C" spgemm_status spgemm_symbolic(const spgemm_csr_in *A_in, const spgemm_csr_in *B_in,
@@ -747,8 +766,7 @@ extern "C" spgemm_status spgemm_symbolic(const spgemm_csr_in *A_in, const spgemm
     status = plan_begin(opts, stream, &p);
     if (status != SPGEMM_OK) return status;
     {
-        SPG_TRY(plan_widen(p, A_in, p->A));
-        SPG_TRY(plan_widen(p, B_in, p->B));
+        SPG_TRY(plan_inputs(p, A_in, B_in));
         status = plan_symbolic_core(p);
         if (status != SPGEMM_OK) goto fail;
     }
@@ -1207,20 +1225,18 @@ extern "C" spgemm_status spgemm_numeric(spgemm_plan *p, spgemm_csr_out *C_out) {
         if (status != SPGEMM_OK) goto fail;
         // ---- stage 4: arrange ----
         SPG_TRY(p->alloc_n(&p->C.row_ptr, m + 1));
+        void *host = nullptr;
+        SPG_TRY(cudaHostGetDevicePointer(&host, p->pinned, 0));
         p->time_begin(SPGEMM_K_SCAN);
-        SPG_TRY(launch_row_scan(m, p->nnzc, p->C.row_ptr, p->scan_partial, p->st));
+        SPG_TRY(launch_row_scan(m, p->nnzc, p->C.row_ptr, p->scan_partial, p->st, static_cast<int64_t *>(host), p->d_err));
         p->time_end();
-        p->count(SPGEMM_K_SCAN, 3);
-        int64_t nnzC = 0;
-        {
-            // nnz(C) and the device error word of stage 3, with one synchronisation
-            int64_t both[2] = {0, 0};
-            SPG_TRY(p->d2h2(both, p->C.row_ptr + m, p->d_err));
-            nnzC = both[0];
-            if (both[1] != 0) {
-                status = SPGEMM_ERR_INTERNAL;
-                goto fail;
-            }
+        p->count(SPGEMM_K_SCAN, row_scan_launches(m));
+        // nnz(C) and the device error word of stage 3, with one synchronisation
+        SPG_TRY(cudaStreamSynchronize(p->st));
+        const int64_t nnzC = static_cast<const int64_t *>(p->pinned)[0];
+        if (static_cast<const int64_t *>(p->pinned)[1] != 0) {
+            status = SPGEMM_ERR_INTERNAL;
+            goto fail;
         }
         SPG_TRY(p->alloc_n(&p->C.col_idx, nnzC));
         SPG_TRY(p->alloc_n(&p->C.val, nnzC));
@@ -1258,8 +1274,8 @@ extern "C" spgemm_status spgemm_numeric(spgemm_plan *p, spgemm_csr_out *C_out) {
         p->time_begin(SPGEMM_K_ARRANGE);
         {
             const int64_t s0 = p->bin_start[1], s1 = p->bin_start[BIN_MERGE];
-            SPG_TRY(launch_arrange_short(a, p->bin_rows + s0, s1 - s0, p->bin, p->C.row_ptr, p->C.col_idx,
-                                         p->C.val, p->st));
+            SPG_TRY(launch_arrange_short(a, host_rows(p->bin_rows + s0, s1 - s0), p->bin, p->C.row_ptr, p->C.col_idx,
+                                         p->C.val, m > 0 ? nnzC / m : 0, p->st));
             if (s1 > s0) p->count(SPGEMM_K_ARRANGE);
             const int64_t n37 = p->h_summary.bin_count[BIN_MERGE];
             SPG_TRY(launch_arrange_long(p->items, n37, p->C.row_ptr, p->C.col_idx, p->C.val, p->st));
@@ -1732,8 +1748,8 @@ extern "C" spgemm_status spgemm_numeric_replay(spgemm_plan *p) {
         // bin 1: the single product of each row
         {
             const int64_t s0 = p->bin_start[1], s1 = p->bin_start[2];
-            SPG_TRY(launch_arrange_short(a, p->bin_rows + s0, s1 - s0, p->bin, p->C.row_ptr, p->C.col_idx, p->C.val,
-                                         p->st));
+            SPG_TRY(launch_arrange_short(a, host_rows(p->bin_rows + s0, s1 - s0), p->bin, p->C.row_ptr, p->C.col_idx,
+                                         p->C.val, 1, p->st));
         }
         // bin 37: every leaf fuses its products into its known columns
         int64_t off = 0;
@@ -1915,7 +1931,7 @@ static cudaError_t precise_fill(spgemm_plan *p, bool dev, const int64_t *gate) {
     // bin 1: the single product of each row
     const RowSet r1 = bin_range(p, 1, 1, dev);
     if (!dev) p->time_begin(SPGEMM_K_ARRANGE);
-    e = launch_arrange_short_set(a, r1, p->bin, p->C.row_ptr, p->C.col_idx, p->C.val, p->st);
+    e = launch_arrange_short(a, r1, p->bin, p->C.row_ptr, p->C.col_idx, p->C.val, 1, p->st);
     if (!dev) {
         p->time_end();
         if (r1.n > 0) p->count(SPGEMM_K_ARRANGE);
@@ -1940,17 +1956,18 @@ static spgemm_status run_precise(spgemm_plan *p, spgemm_csr_out *C_out) {
         alloc_dense_keep(p);
         SPG_TRY(precise_count(p, false));
         SPG_TRY(p->alloc_n(&p->C.row_ptr, m + 1));
+        void *host = nullptr;
+        SPG_TRY(cudaHostGetDevicePointer(&host, p->pinned, 0));
         p->time_begin(SPGEMM_K_SCAN);
-        SPG_TRY(launch_row_scan(m, p->nnzc, p->C.row_ptr, p->scan_partial, p->st));
+        SPG_TRY(launch_row_scan(m, p->nnzc, p->C.row_ptr, p->scan_partial, p->st, static_cast<int64_t *>(host), p->d_err));
         p->time_end();
-        p->count(SPGEMM_K_SCAN, 3);
-        int64_t both[2] = {0, 0};
-        SPG_TRY(p->d2h2(both, p->C.row_ptr + m, p->d_err));  // nnz(C), the one size the method reads back
-        if (both[1] != 0) {
+        p->count(SPGEMM_K_SCAN, row_scan_launches(m));
+        SPG_TRY(cudaStreamSynchronize(p->st));  // nnz(C), the one size the method reads back
+        const int64_t nnzC = static_cast<const int64_t *>(p->pinned)[0];
+        if (static_cast<const int64_t *>(p->pinned)[1] != 0) {
             status = SPGEMM_ERR_INTERNAL;
             goto fail;
         }
-        const int64_t nnzC = both[0];
         SPG_TRY(p->alloc_n(&p->C.col_idx, nnzC));
         SPG_TRY(p->alloc_n(&p->C.val, nnzC));
         SPG_TRY(precise_fill(p, false, nullptr));
@@ -1989,8 +2006,8 @@ struct spgemm_dplan {
 static spgemm_status dplan_buffers(spgemm_dplan *d) {
     spgemm_plan *p = d->p;
     spgemm_status status = SPGEMM_OK;
-    const int64_t m = p->A.nrows, nnzA = p->A.nnz;
-    const int64_t nblk = bin_blocks(m);
+    const int64_t m = p->A.nrows;
+    const int64_t nblk = bin_blocks(m, p->A.nnz);
     {
         merge_limits(p);
         if (p->dense_K == 0 && p->B.ncols > 0) return SPGEMM_ERR_SHAPE;
@@ -1998,15 +2015,14 @@ static spgemm_status dplan_buffers(spgemm_dplan *d) {
         SPG_TRY(p->alloc_n(&p->d_err, 1));
         SPG_TRY(p->alloc_n(&d->gate, 1));
         SPG_TRY(p->alloc_n(&p->d_queue, DENSE_QUEUES));
-        SPG_TRY(p->alloc_n(&p->S, nnzA + 1));
-        SPG_TRY(p->alloc_n(&p->scan_partial, std::max(bound_partial_size(nnzA), bin_blocks(m) + 1) + 1));
+        SPG_TRY(p->alloc_n(&p->scan_partial, row_scan_partials(m)));
         SPG_TRY(p->alloc_n(&p->u, m));
         SPG_TRY(p->alloc_n(&p->bin, m));
         SPG_TRY(p->alloc_n(&p->nnzc, m));
         SPG_TRY(p->alloc_n(&p->bin_rows, m));
         SPG_TRY(p->alloc_n(&p->ctil_rp, m + 1));
         SPG_TRY(p->alloc_n(&p->d_hist, (int64_t)NUM_BINS * nblk));
-        SPG_TRY(p->alloc_n(&p->d_capp, nblk));
+        SPG_TRY(p->alloc_n(&p->d_capp, 2 * nblk));
         if (p->dense_K > 0) {
             SPG_TRY(p->alloc_n(&p->dense_flag, m));
             SPG_TRY(p->alloc_n(&p->dense_lo, m));
@@ -2042,30 +2058,25 @@ static cudaError_t dplan_enqueue(spgemm_dplan *d) {
     do {                                     \
         if ((e = (x)) != cudaSuccess) return e; \
     } while (0)
-    DP_TRY(cudaMemsetAsync(p->d_summary, 0, sizeof(BinSummary), p->st));
-    DP_TRY(cudaMemsetAsync(p->d_err, 0, sizeof(int64_t), p->st));
     if (p->npairs > 0) {
         DP_TRY(launch_concat(p->d_pairs, p->npairs, p->d_moff, p->d_koff, p->d_annz_off, p->d_bnnz_off, p->A.nrows,
                              p->B.nrows, p->A.nnz, p->B.nnz, p->cat_a_rp, p->cat_a_col, p->cat_a_val, p->cat_b_rp,
                              p->cat_b_col, p->cat_b_val, false, p->st));
     } else {
-        if (d->a_rp64)
-            DP_TRY(launch_widen_rowptr(static_cast<const int32_t *>(d->A_in.row_ptr), d->a_rp64, m + 1, p->st));
-        if (d->b_rp64 && d->b_rp64 != d->a_rp64)
-            DP_TRY(launch_widen_rowptr(static_cast<const int32_t *>(d->B_in.row_ptr), d->b_rp64, p->B.nrows + 1,
-                                       p->st));
+        const bool widen_b = d->b_rp64 && d->b_rp64 != d->a_rp64;
+        DP_TRY(launch_widen_rowptr(static_cast<const int32_t *>(d->A_in.row_ptr), d->a_rp64, d->a_rp64 ? m + 1 : 0, p->st,
+                                   static_cast<const int32_t *>(d->B_in.row_ptr), d->b_rp64,
+                                   widen_b ? p->B.nrows + 1 : 0));
     }
-    // stage 1 and the column ranges of the bin-37 rows (all of them dense-slice rows)
-    DP_TRY(launch_bound(p->A, p->B, p->S, p->scan_partial, p->st));
-    if (p->dense_K > 0)
-        DP_TRY(launch_dense_mark(p->A, p->B, p->S, p->dense_min_u, 8, p->dense_flag, p->dense_lo, p->dense_hi, p->st));
+    // stage 1, with the column ranges of the bin-37 rows (all of them dense-slice rows), and
     // stage 2: bins (no C~ to size)
     CapPolicy pol{};
     pol.policy = POLICY_PRECISE;
     pol.initial_cap = 1;
     pol.dense = p->dense_flag;
-    DP_TRY(launch_binning(m, p->A.rp, p->S, p->S + p->A.nnz, pol, p->u, p->bin, p->nnzc, p->bin_rows, p->ctil_rp,
-                          p->d_hist, p->d_capp, p->d_summary, p->st));
+    const BoundOut out = bound_out(p);
+    DP_TRY(launch_bound(p->A, p->B, pol, out, p->st));
+    DP_TRY(launch_binning(m, p->A.nnz, pol, out, p->bin_rows, p->ctil_rp, p->d_summary, nullptr, p->st));
     if (p->dense_K > 0) {
         DP_TRY(launch_dense_select(p->bin_rows, m, p->d_summary, p->u, p->dense_flag, p->dense_lo, p->dense_hi,
                                    p->d_select, p->dense_order, p->dense_rows, p->dense_clo, p->dense_chi, p->st));

@@ -1,14 +1,16 @@
 // Stage 1 (upper bound, Algorithm 2) and stage 2 (binning and C~ sizing,
 // Algorithm 3) of the SpGEMM framework, plus input widening and validation.
 //
-// Stage 1 is computed as one exclusive prefix sum S over the nonzeros of A of
-// the lengths of the B rows they select: u_i = S[A.rp[i+1]] - S[A.rp[i]].  Every
-// nonzero costs the same work, so a hub row of A cannot unbalance the kernel the
-// way one-thread-per-row (the paper's launch shape) would.
+// Stage 1 gives a group of lanes to each row of A (as many as the rows' average length
+// asks for) and a whole block to each long row, so a hub row cannot unbalance the kernel the
+// way one-thread-per-row (the paper's launch shape) would.  The same kernel bins the row,
+// counts the bins of its block of rows and finds the column range of the bin-37 rows: u_i
+// never goes through a prefix sum over A's nonzeros, which took 16 bytes of traffic per
+// nonzero and three launches.
 //
 // Stage 2 runs on the GPU instead of a CPU core (the paper's choice, Section 4.1)
-// and without atomics: per-block 38-bin histograms built with warp match/popc,
-// one scan over the (bin, block) counts, and a stable scatter that keeps rows
+// and without device-wide atomics: per-block 38-bin histograms, one block that scans the
+// (bin, block) counts with a warp per bin, and a stable scatter that keeps rows
 // in ascending order inside every bin.
 #include "internal.h"
 #include "scan.cuh"
@@ -38,14 +40,18 @@ int persistent_blocks(const void *kern, int nt, size_t smem, int64_t cap) {
     return (int)(cap > 0 && cap < g ? cap : g);
 }
 
-__global__ void k_widen_rowptr(const int32_t *in, int64_t *out, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_widen_rowptr(const int32_t *in, int64_t *out, int64_t n, const int32_t *in2, int64_t *out2,
+                               int64_t n2) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] = (int64_t)in[i];
+    if (i < n2) out2[i] = (int64_t)in2[i];
 }
 
-cudaError_t launch_widen_rowptr(const int32_t *in, int64_t *out, int64_t n, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    k_widen_rowptr<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, out, n);
+cudaError_t launch_widen_rowptr(const int32_t *in, int64_t *out, int64_t n, cudaStream_t st, const int32_t *in2,
+                                int64_t *out2, int64_t n2) {
+    const int64_t most = n > n2 ? n : n2;
+    if (most <= 0) return cudaSuccess;
+    k_widen_rowptr<<<(unsigned)((most + 255) / 256), 256, 0, st>>>(in, out, n, in2, out2, n2);
     return cudaGetLastError();
 }
 
@@ -78,37 +84,38 @@ cudaError_t launch_validate(const DevCSR &M, int64_t *status, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// ---------------- stage 1 ----------------
-
-struct BRowLen {
-    const int32_t *acol;
-    const int64_t *brp;
-    SPG_DEV int64_t operator()(int64_t j) const {
-        int32_t k = acol[j];
-        return brp[k + 1] - brp[k];
-    }
-};
+// ---------------- stages 1 and 2 ----------------
 
 struct StoreI64 {
     int64_t *out;
     SPG_DEV void operator()(int64_t i, int64_t v) const { out[i] = v; }
 };
 
-int64_t bound_partial_size(int64_t nnzA) { return scan_blocks(nnzA) + 1; }
+constexpr int BIN_NT = 256;
+constexpr int BIN_NW = BIN_NT / 32;
+constexpr int BIN_ROWS_MAX = 2048;  // rows of a block
+constexpr int LONG_STEPS = 16;      // a row longer than this many times its group is taken by the block
 
-cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, int64_t *S, int64_t *partial,
-                         cudaStream_t st) {
-    return device_exclusive_scan(A.nnz, BRowLen{A.col, B.rp}, StoreI64{S}, partial, S + A.nnz, st);
+// Lanes per row: about half the average length of A's rows, so that most rows take a few steps.
+static int bound_group(int64_t m, int64_t nnz) {
+    const int64_t avg = m > 0 ? nnz / m : 0;
+    return avg <= 6 ? 4 : avg <= 24 ? 8 : avg <= 64 ? 16 : 32;
 }
 
-// ---------------- stage 2 ----------------
+// Rows per block: a whole number of passes of 256 / group rows, and about eight blocks per SM
+// (of 152) for large m -- the (bin, block) counts are scanned by one block.
+static int64_t bin_rows_per_block(int64_t m, int64_t nnz) {
+    const int64_t rows = BIN_NT / bound_group(m, nnz);
+    int64_t passes = (m + rows * 1216 - 1) / (rows * 1216);
+    if (passes < 1) passes = 1;
+    if (passes * rows > BIN_ROWS_MAX) passes = BIN_ROWS_MAX / rows;
+    return passes * rows;
+}
 
-constexpr int BIN_NT = 256;
-constexpr int BIN_IPT = 4;
-constexpr int BIN_ROWS = BIN_NT * BIN_IPT;
-constexpr int BIN_NW = BIN_NT / 32;
-
-int64_t bin_blocks(int64_t m) { return (m + BIN_ROWS - 1) / BIN_ROWS; }
+int64_t bin_blocks(int64_t m, int64_t nnz) {
+    const int64_t r = bin_rows_per_block(m, nnz);
+    return (m + r - 1) / r;
+}
 
 // Algorithm 3: bin 0 (u = 0), bin 1 (u = 1), bins 2..32 (u = 2..32, one bin per
 // size), bins 33..36 (33-64, 65-128, 129-256, 257-512), bin 37 (u > 512).
@@ -126,9 +133,9 @@ SPG_DEV int bin_of(int64_t u) {
 // 0..36, the predicted size (never above u_i) for bin 37.  Bin-37 rows computed
 // by the dense-slice kernels take none in every policy, and the precise method
 // has no C~ at all.
-SPG_DEV int64_t cap_of(int64_t u, int b, int64_t i, const CapPolicy &P) {
+SPG_DEV int64_t cap_of(int64_t u, int b, int64_t i, const CapPolicy &P, bool dense) {
     if (P.policy == POLICY_PRECISE) return 0;  // counted first, then computed straight into C
-    if (b == BIN_MERGE && P.dense != nullptr && P.dense[i]) return 0;  // written straight into C
+    if (dense) return 0;  // written straight into C
     if (P.policy == POLICY_UPPER_BOUND) return u;
     if (P.policy == POLICY_LEARNED && P.pred_cap != nullptr && b == BIN_MERGE) {
         int64_t c = P.pred_cap[i];
@@ -139,104 +146,207 @@ SPG_DEV int64_t cap_of(int64_t u, int b, int64_t i, const CapPolicy &P) {
     return u;
 }
 
-__global__ void __launch_bounds__(BIN_NT)
-k_bin_count(int64_t m, const int64_t *arp, const int64_t *S, CapPolicy P, int64_t *u_out,
-            uint8_t *bin_out, int32_t *nnzc, int32_t *hist, int64_t *cap_partial, int64_t nblk) {
-    __shared__ int32_t whist[BIN_NW][NUM_BINS];
-    __shared__ int64_t scratch[BIN_NW + 1];
-    const int lane = lane_id(), wid = warp_id();
-    for (int t = threadIdx.x; t < BIN_NW * NUM_BINS; t += BIN_NT) (&whist[0][0])[t] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * BIN_ROWS;
-    int64_t capsum = 0;
-#pragma unroll
-    for (int k = 0; k < BIN_IPT; ++k) {
-        const int64_t i = base + k * BIN_NT + threadIdx.x;
-        const bool valid = i < m;
-        int b = 255;
-        if (valid) {
-            int64_t u = S[arp[i + 1]] - S[arp[i]];
-            b = bin_of(u);
-            u_out[i] = u;
-            bin_out[i] = (uint8_t)b;
-            nnzc[i] = (b <= 1) ? (int32_t)u : 0;
-            capsum += cap_of(u, b, i, P);
-        }
-        unsigned peers = __match_any_sync(SPG_FULL, b);
-        if (valid && lane == __ffs(peers) - 1) whist[wid][b] += __popc(peers);
-        __syncwarp();
-    }
-    __syncthreads();
-    if (threadIdx.x < NUM_BINS) {
-        int32_t h = 0;
-#pragma unroll
-        for (int w = 0; w < BIN_NW; ++w) h += whist[w][threadIdx.x];
-        hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = h;
-    }
-    capsum = block_reduce_sum<BIN_NT>(capsum, scratch);
-    if (threadIdx.x == 0) cap_partial[blockIdx.x] = capsum;
+SPG_DEV bool dense_row(int b, int64_t i, const CapPolicy &P) {
+    return b == BIN_MERGE && P.dense != nullptr && P.dense[i] != 0;
 }
 
-// One block: exclusive scan of the bin-major (bin, block) histogram and of the
-// per-block C~ sizes; writes the host summary and C~.rp[m].
-__global__ void __launch_bounds__(1024)
-k_bin_scan(int64_t m, int32_t *hist, int64_t nblk, int64_t *cap_partial, int64_t *ctil_rp,
-           const int64_t *sum_u, BinSummary *summary) {
-    __shared__ int64_t scratch[1024 / 32 + 1];
-    __shared__ int64_t bstart[NUM_BINS + 1];
-    const int64_t nh = (int64_t)NUM_BINS * nblk;
-    int64_t carry = 0;
-    for (int64_t base = 0; base < nh; base += 1024) {
-        int64_t i = base + threadIdx.x;
-        int64_t v = (i < nh) ? hist[i] : 0;
-        int64_t tot;
-        int64_t ex = block_exclusive_scan<1024>(v, scratch, tot);
-        if (i < nh) {
-            hist[i] = (int32_t)(carry + ex);
-            if (i % nblk == 0) bstart[i / nblk] = carry + ex;
-        }
-        carry += tot;
+// u_i, bin and row size of every row, the histogram of the block's rows, and the block's sums of
+// C~ entries and of u_i (part[0..nblk), part[nblk..2 nblk)).  Bin-37 rows also get their column
+// range [lo, hi) (first and last column of every B row they select) and the flag that sends them
+// to the dense-slice kernels: u_i >= dmin (dmin > 0), else div u_i >= hi - lo -- their products
+// cover at least a div-th of the columns they can reach, so the accumulator's O(hi - lo) clearing
+// and write-out are small beside them.  Latency-bound (two dependent gathers per nonzero): the
+// 27-point operator on 64^3 (6.9 M nonzeros) takes 65 us here (cold caches) and took 113 us as a
+// prefix sum, a marking pass and a histogram pass.
+template <int G>
+__global__ void __launch_bounds__(BIN_NT)
+k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
+    __shared__ int32_t hist[NUM_BINS];
+    __shared__ int32_t nlong, longs[BIN_ROWS_MAX];
+    __shared__ int64_t scratch[BIN_NW + 1];
+    __shared__ int32_t range[2];
+    constexpr int ROWS = BIN_NT / G;
+    const int gl = threadIdx.x & (G - 1), grp = threadIdx.x / G;
+    const unsigned gm = G == 32 ? SPG_FULL : ((1u << (G & 31)) - 1u) << (lane_id() & ~(G - 1));
+    if (threadIdx.x < NUM_BINS) hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        nlong = 0;
+        if (blockIdx.x == 0) *O.err = 0;
     }
-    carry = 0;
-    for (int64_t base = 0; base < nblk; base += 1024) {
-        int64_t i = base + threadIdx.x;
-        int64_t v = (i < nblk) ? cap_partial[i] : 0;
-        int64_t tot;
-        int64_t ex = block_exclusive_scan<1024>(v, scratch, tot);
-        if (i < nblk) cap_partial[i] = carry + ex;
-        carry += tot;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * R;
+    int64_t capsum = 0, usum = 0;
+    auto sum_of = [&](int64_t p0, int64_t p1, int step) {
+        int64_t u = 0;
+#pragma unroll 4
+        for (int64_t p = p0; p < p1; p += step) {
+            const int32_t k = A.col[p];
+            u += B.rp[k + 1] - B.rp[k];
+        }
+        return u;
+    };
+    auto range_of = [&](int64_t p0, int64_t p1, int step, int32_t &cmin, int32_t &cmax) {
+        cmin = INT32_MAX;
+        cmax = -1;
+        for (int64_t p = p0; p < p1; p += step) {
+            const int32_t k = A.col[p];
+            const int64_t rs = B.rp[k], re = B.rp[k + 1];
+            if (re > rs) {
+                cmin = min(cmin, B.col[rs]);
+                cmax = max(cmax, B.col[re - 1]);
+            }
+        }
+    };
+    // by one thread per row; the range is that of a bin-37 row where flags are wanted
+    auto finish = [&](int64_t i, int64_t u, int b, int32_t cmin, int32_t cmax) {
+        bool dense = false;
+        if (P.dense != nullptr) {
+            if (b == BIN_MERGE) {
+                const int64_t span = (int64_t)cmax - cmin + 1;  // u > 0, so some B row is not empty
+                dense = O.dmin > 0 ? u >= O.dmin : (int64_t)O.div * u >= span;
+                O.lo[i] = cmin;
+                O.hi[i] = cmax + 1;
+            }
+            O.flag[i] = (uint8_t)dense;
+        }
+        O.u[i] = u;
+        O.bin[i] = (uint8_t)b;
+        O.nnzc[i] = (b <= 1) ? (int32_t)u : 0;
+        atomicAdd(&hist[b], 1);
+        capsum += cap_of(u, b, i, P, dense);
+        usum += u;
+    };
+    for (int r0 = 0; r0 < R; r0 += ROWS) {
+        const int64_t i = base + r0 + grp;
+        if (i >= A.nrows) break;  // the whole group
+        const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
+        if (a1 - a0 > LONG_STEPS * G) {
+            if (gl == 0) longs[atomicAdd(&nlong, 1)] = r0 + grp;
+            continue;
+        }
+        int64_t u = sum_of(a0 + gl, a1, G);
+#pragma unroll
+        for (int d = G / 2; d > 0; d >>= 1) u += __shfl_xor_sync(gm, u, d, G);
+        const int b = bin_of(u);
+        int32_t cmin = 0, cmax = 0;
+        if (b == BIN_MERGE && P.dense != nullptr) {
+            range_of(a0 + gl, a1, G, cmin, cmax);
+#pragma unroll
+            for (int d = G / 2; d > 0; d >>= 1) {
+                cmin = min(cmin, __shfl_xor_sync(gm, cmin, d, G));
+                cmax = max(cmax, __shfl_xor_sync(gm, cmax, d, G));
+            }
+        }
+        if (gl == 0) finish(i, u, b, cmin, cmax);
+    }
+    __syncthreads();
+    const int nl = nlong;
+    for (int l = 0; l < nl; ++l) {
+        const int64_t i = base + longs[l];
+        const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
+        if (threadIdx.x < 2) range[threadIdx.x] = threadIdx.x == 0 ? INT32_MAX : -1;
+        const int64_t u = block_reduce_sum<BIN_NT>(sum_of(a0 + threadIdx.x, a1, BIN_NT), scratch);
+        const int b = bin_of(u);
+        if (b == BIN_MERGE && P.dense != nullptr) {
+            int32_t cmin, cmax;
+            range_of(a0 + threadIdx.x, a1, BIN_NT, cmin, cmax);
+            cmin = __reduce_min_sync(SPG_FULL, cmin);
+            cmax = __reduce_max_sync(SPG_FULL, cmax);
+            if (lane_id() == 0) {
+                atomicMin(&range[0], cmin);
+                atomicMax(&range[1], cmax);
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) finish(i, u, b, range[0], range[1]);
+        __syncthreads();
+    }
+    if (threadIdx.x < NUM_BINS) O.hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = hist[threadIdx.x];
+    capsum = block_reduce_sum<BIN_NT>(capsum, scratch);
+    usum = block_reduce_sum<BIN_NT>(usum, scratch);
+    if (threadIdx.x == 0) {
+        O.part[blockIdx.x] = capsum;
+        O.part[nblk + blockIdx.x] = usum;
+    }
+}
+
+// Exclusive scan of v[0..n) in place by one warp; returns the total.
+template <typename T>
+SPG_DEV T warp_scan_array(T *v, int64_t n) {
+    T carry = 0;
+    const int lane = lane_id();
+    for (int64_t i0 = 0; i0 < n; i0 += 128) {
+        T x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = i0 + 32 * q + lane < n ? v[i0 + 32 * q + lane] : T(0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const T inc = warp_inclusive_scan(x[q]);
+            if (i0 + 32 * q + lane < n) v[i0 + 32 * q + lane] = carry + inc - x[q];
+            carry += __shfl_sync(SPG_FULL, inc, 31);
+        }
+    }
+    return carry;
+}
+
+// One block: exclusive scans of every bin's block counts (a warp per bin, offsets inside the
+// bin) and of the per-block C~ sizes; writes the summary, also into host memory the device can
+// write (`host`, when given), and C~.rp[m].
+__global__ void __launch_bounds__(1024)
+k_bin_scan(int64_t m, int32_t *hist, int64_t nblk, int64_t *part, int64_t *ctil_rp, BinSummary *summary,
+           BinSummary *host) {
+    __shared__ int64_t total[NUM_BINS + 2], bstart[NUM_BINS + 1];
+    const int lane = lane_id();
+    for (int b = warp_id(); b < NUM_BINS + 2; b += 32) {
+        const int64_t t = b < NUM_BINS ? (int64_t)warp_scan_array(hist + b * nblk, nblk)
+                                       : warp_scan_array(part + (b - NUM_BINS) * nblk, nblk);
+        if (lane == 0) total[b] = t;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        bstart[NUM_BINS] = m;
-        if (nblk == 0)
-            for (int b = 0; b < NUM_BINS; ++b) bstart[b] = 0;
-        ctil_rp[m] = carry;
-        summary->sum_cap = carry;
-        summary->sum_u = *sum_u;
+        int64_t s = 0;
+        for (int b = 0; b < NUM_BINS; ++b) {
+            bstart[b] = s;
+            s += total[b];
+        }
+        bstart[NUM_BINS] = s;
+        ctil_rp[m] = total[NUM_BINS];
     }
     __syncthreads();
-    if (threadIdx.x < NUM_BINS) summary->bin_count[threadIdx.x] = bstart[threadIdx.x + 1] - bstart[threadIdx.x];
-    if (threadIdx.x <= NUM_BINS) summary->bin_start[threadIdx.x] = bstart[threadIdx.x];
+    BinSummary *dst[2] = {summary, host};
+    for (int k = 0; k < (host != nullptr ? 2 : 1); ++k) {
+        BinSummary *S = dst[k];
+        if (threadIdx.x < NUM_BINS) S->bin_count[threadIdx.x] = total[threadIdx.x];
+        if (threadIdx.x <= NUM_BINS) S->bin_start[threadIdx.x] = bstart[threadIdx.x];
+        if (threadIdx.x < NUM_LAUNCH_CLASSES) S->class_count[threadIdx.x] = 0;
+        if (threadIdx.x == 0) {
+            S->sum_cap = total[NUM_BINS];
+            S->sum_u = total[NUM_BINS + 1];
+            S->dense_count = 0;
+        }
+    }
 }
 
 __global__ void __launch_bounds__(BIN_NT)
-k_bin_scatter(int64_t m, const int64_t *u_in, const uint8_t *bin_in, CapPolicy P,
-              const int32_t *hist_off, const int64_t *cap_off, int64_t nblk, int32_t *bin_rows,
-              int64_t *ctil_rp) {
+k_bin_scatter(int64_t m, int R, const int64_t *u_in, const uint8_t *bin_in, CapPolicy P,
+              const int32_t *hist_off, const int64_t *cap_off, int64_t nblk, const BinSummary *summary,
+              int32_t *bin_rows, int64_t *ctil_rp) {
     __shared__ int32_t wcnt[BIN_NW][NUM_BINS];
     __shared__ int32_t run[NUM_BINS];
     __shared__ int64_t scratch[BIN_NW + 1];
     const int lane = lane_id(), wid = warp_id();
-    if (threadIdx.x < NUM_BINS) run[threadIdx.x] = 0;
-    const int64_t base = (int64_t)blockIdx.x * BIN_ROWS;
+    // the next place of each bin's rows
+    if (threadIdx.x < NUM_BINS)
+        run[threadIdx.x] = (int32_t)summary->bin_start[threadIdx.x] + hist_off[(int64_t)threadIdx.x * nblk + blockIdx.x];
+    const int64_t base = (int64_t)blockIdx.x * R;
+    const int64_t end = min(m, base + R);
     int64_t capcarry = cap_off[blockIdx.x];
     const unsigned lt_mask = (1u << lane) - 1u;
-    for (int k = 0; k < BIN_IPT; ++k) {
+    for (int64_t i0 = base; i0 < end; i0 += BIN_NT) {
         for (int t = threadIdx.x; t < BIN_NW * NUM_BINS; t += BIN_NT) (&wcnt[0][0])[t] = 0;
         __syncthreads();
-        const int64_t i = base + k * BIN_NT + threadIdx.x;
-        const bool valid = i < m;
+        const int64_t i = i0 + threadIdx.x;
+        const bool valid = i < end;
         int b = valid ? (int)bin_in[i] : 255;
         unsigned peers = __match_any_sync(SPG_FULL, b);
         int rank = __popc(peers & lt_mask);
@@ -246,8 +356,8 @@ k_bin_scatter(int64_t m, const int64_t *u_in, const uint8_t *bin_in, CapPolicy P
         if (valid) {
             int pos = run[b] + rank;
             for (int w = 0; w < wid; ++w) pos += wcnt[w][b];
-            bin_rows[(int64_t)hist_off[(int64_t)b * nblk + blockIdx.x] + pos] = (int32_t)i;
-            cap = cap_of(u_in[i], b, i, P);
+            bin_rows[pos] = (int32_t)i;
+            cap = cap_of(u_in[i], b, i, P, dense_row(b, i, P));
         }
         int64_t tot;
         int64_t ex = block_exclusive_scan<BIN_NT>(cap, scratch, tot);
@@ -269,7 +379,7 @@ struct LoadCap {
     const int64_t *u;
     const uint8_t *bin;
     CapPolicy P;
-    SPG_DEV int64_t operator()(int64_t i) const { return cap_of(u[i], (int)bin[i], i, P); }
+    SPG_DEV int64_t operator()(int64_t i) const { return cap_of(u[i], (int)bin[i], i, P, dense_row((int)bin[i], i, P)); }
 };
 
 cudaError_t launch_cap_rescan(int64_t m, const int64_t *u, const uint8_t *bin, CapPolicy P, int64_t *ctil_rp,
@@ -279,20 +389,32 @@ cudaError_t launch_cap_rescan(int64_t m, const int64_t *u, const uint8_t *bin, C
     return cudaMemcpyAsync(ctil_rp + m, total, sizeof(int64_t), cudaMemcpyDeviceToDevice, st);
 }
 
-cudaError_t launch_binning(int64_t m, const int64_t *arp, const int64_t *S,
-                           const int64_t *sum_u_ptr, CapPolicy P, int64_t *u, uint8_t *bin, int32_t *nnzc, int32_t *bin_rows,
-                           int64_t *ctil_rp, int32_t *hist, int64_t *cap_partial,
-                           BinSummary *summary, cudaStream_t st) {
-    const int64_t nblk = bin_blocks(m);
-    if (nblk > 0)
-        k_bin_count<<<(unsigned)nblk, BIN_NT, 0, st>>>(m, arp, S, P, u, bin, nnzc, hist, cap_partial,
-                                                        nblk);
-    k_bin_scan<<<1, 1024, 0, st>>>(m, hist, nblk, cap_partial, ctil_rp, sum_u_ptr, summary);
+cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, const BoundOut &O, cudaStream_t st) {
+    const int64_t nblk = bin_blocks(A.nrows, A.nnz);
+    if (P.dense != nullptr && O.div < 1) return cudaErrorInvalidValue;
+    if (nblk <= 0) return cudaMemsetAsync(O.err, 0, sizeof(int64_t), st);
+    const int R = (int)bin_rows_per_block(A.nrows, A.nnz);
+    auto go = [&](auto kern) {
+        kern<<<(unsigned)nblk, BIN_NT, 0, st>>>(A, B, P, O, R, nblk);
+        return cudaGetLastError();
+    };
+    switch (bound_group(A.nrows, A.nnz)) {
+        case 4: return go(k_bound<4>);
+        case 8: return go(k_bound<8>);
+        case 16: return go(k_bound<16>);
+        default: return go(k_bound<32>);
+    }
+}
+
+cudaError_t launch_binning(int64_t m, int64_t nnzA, const CapPolicy &P, const BoundOut &O, int32_t *bin_rows,
+                           int64_t *ctil_rp, BinSummary *summary, BinSummary *host, cudaStream_t st) {
+    const int64_t nblk = bin_blocks(m, nnzA);
+    k_bin_scan<<<1, 1024, 0, st>>>(m, O.hist, nblk, O.part, ctil_rp, summary, host);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (nblk > 0)
-        k_bin_scatter<<<(unsigned)nblk, BIN_NT, 0, st>>>(m, u, bin, P, hist, cap_partial, nblk,
-                                                          bin_rows, ctil_rp);
+        k_bin_scatter<<<(unsigned)nblk, BIN_NT, 0, st>>>(m, (int)bin_rows_per_block(m, nnzA), O.u, O.bin, P, O.hist,
+                                                          O.part, nblk, summary, bin_rows, ctil_rp);
     return cudaGetLastError();
 }
 
