@@ -54,32 +54,43 @@ cudaError_t launch_dense_bounds(const DevCSR &B, int K, int W, int32_t *bnd, cud
 
 // ---- selection of the dense rows among the bin-37 rows ----
 // Bucket g = 63 - floor(log2 u) (the leading zeros of u) for a dense row, so that
-// larger rows come first; DENSE_BUCKETS for the others.  order[0..nd) lists the
-// dense items, order[nd..n37) the rest.
+// larger rows come first; then the rows that reach few columns (a warp each), in two buckets
+// by width; DENSE_BUCKETS for the others.  order[0..nd) lists the dense items,
+// order[nd..n37) the rest.
 
-constexpr int DENSE_BUCKETS = 64;
+constexpr int DENSE_BUCKETS = 66;
+SPG_DEV int dense_bucket(int64_t u, int32_t width) {
+    return width > DENSE_MID_W ? __clzll((long long)u) : (width > DENSE_NARROW_W ? 64 : 65);
+}
 
 __global__ void k_dense_select_count(const int32_t *bin_rows, int64_t m, const BinSummary *summary, const int64_t *u,
-                                     const uint8_t *flag, int32_t *cls_of, int32_t *count) {
+                                     const uint8_t *flag, const int32_t *lo, const int32_t *hi, int32_t *cls_of,
+                                     int32_t *count) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t n37 = summary->bin_count[BIN_MERGE];
     if (j >= n37) return;
     const int32_t row = bin_rows[m - n37 + j];
     const int64_t uu = u[row];
-    const int g = flag[row] ? __clzll((long long)uu) : DENSE_BUCKETS;
+    const int g = flag[row] ? dense_bucket(uu, hi[row] - lo[row]) : DENSE_BUCKETS;
     cls_of[j] = g;
-    atomicAdd(&count[g], 1);
+    // one add per bucket and warp: most rows fall into few buckets
+    const unsigned peers = __match_any_sync(__activemask(), g);
+    if (lane_id() == __ffs(peers) - 1) atomicAdd(&count[g], __popc(peers));
 }
 
 __global__ void k_dense_select_starts(const int32_t *count, int32_t *start, int32_t *cursor, BinSummary *summary) {
-    if (threadIdx.x == 0) {
+    __shared__ int32_t c[DENSE_BUCKETS + 1];
+    if (threadIdx.x <= DENSE_BUCKETS) {
+        c[threadIdx.x] = count[threadIdx.x];
+        cursor[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x <= DENSE_BUCKETS) {
         int32_t s = 0;
-        for (int g = 0; g <= DENSE_BUCKETS; ++g) {
-            start[g] = s;
-            cursor[g] = 0;
-            if (g == DENSE_BUCKETS) summary->dense_count = s;
-            s += count[g];
-        }
+        for (int g = 0; g < (int)threadIdx.x; ++g) s += c[g];
+        start[threadIdx.x] = s;
+        if (threadIdx.x == DENSE_BUCKETS) summary->dense_count = s;
+        else if (threadIdx.x >= 64) summary->dense_end[threadIdx.x - 64] = s;
     }
 }
 
@@ -91,7 +102,10 @@ __global__ void k_dense_select_scatter(const int32_t *bin_rows, int64_t m, const
     const int64_t n37 = summary->bin_count[BIN_MERGE];
     if (j >= n37) return;
     const int g = cls_of[j];
-    const int32_t pos = start[g] + atomicAdd(&cursor[g], 1);
+    const unsigned peers = __match_any_sync(__activemask(), g);
+    const int leader = __ffs(peers) - 1;
+    int32_t pos = lane_id() == leader ? start[g] + atomicAdd(&cursor[g], __popc(peers)) : 0;
+    pos = __shfl_sync(peers, pos, leader) + __popc(peers & ((1u << lane_id()) - 1u));
     order[pos] = (int32_t)j;
     if (g < DENSE_BUCKETS) {
         const int32_t row = bin_rows[m - n37 + j];
@@ -112,8 +126,8 @@ cudaError_t launch_dense_select(const int32_t *bin_rows, int64_t m, BinSummary *
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int32_t) * (DENSE_BUCKETS + 1), st);
     if (e != cudaSuccess) return e;
     const unsigned g = (unsigned)((m + 255) / 256);
-    k_dense_select_count<<<g, 256, 0, st>>>(bin_rows, m, summary, u, flag, cls_of, count);
-    k_dense_select_starts<<<1, 32, 0, st>>>(count, start, cursor, summary);
+    k_dense_select_count<<<g, 256, 0, st>>>(bin_rows, m, summary, u, flag, lo, hi, cls_of, count);
+    k_dense_select_starts<<<1, 96, 0, st>>>(count, start, cursor, summary);
     k_dense_select_scatter<<<g, 256, 0, st>>>(bin_rows, m, summary, cls_of, start, cursor, lo, hi, order, rows, rlo,
                                               rhi);
     return cudaGetLastError();
@@ -234,7 +248,8 @@ SPG_DEV void prefetch_l2(const void *p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-SPG_DEV int64_t dense_items(const DenseArgs &D) { return (D.dev_n != nullptr ? *D.dev_n : D.n) * (int64_t)D.K; }
+// The (row, slice) items of the wide rows.
+SPG_DEV int64_t dense_items(const DenseArgs &D) { return (D.dev_end != nullptr ? D.dev_end[0] : D.n_wide) * (int64_t)D.K; }
 
 // The columns of slice s that row d of the dense items can reach: [lo, lo + span).
 SPG_DEV int dense_span(const DevCSR &B, const DenseArgs &D, int64_t d, int s, int64_t &lo) {
@@ -308,7 +323,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT, 1536 / NT)
 k_dense_count(DevCSR A, DevCSR B, DenseArgs D, int64_t *err) {
     __shared__ int64_t s_b;
-    unsigned long long *q = D.dev_n != nullptr ? D.queue : nullptr;
+    unsigned long long *q = D.dev_end != nullptr ? D.queue : nullptr;
     const int64_t nb = dense_items(D);
     for (int64_t b = dense_next(q, 0, true, &s_b); b < nb; b = dense_next(q, b, false, &s_b))
         dense_count_item<NT>(A, B, D, b, err);
@@ -552,6 +567,229 @@ k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_co
     }
 }
 
+// ---- rows that reach few columns: a warp per row ----
+// A band, a block or a stencil's neighbourhood: at most W columns, whatever B's width.  One
+// warp holds a sum per column in shared memory and takes the B rows one after another, 32
+// entries at a time: their columns are distinct, so plain fused multiply-adds suffice, and no
+// barrier wider than the warp is needed.  A*A of a band matrix of 50,021 rows and width 40 (80 M
+// products, single precision) takes 73 + 293 us for the count and the sums; a CTA per row
+// took 3.08 ms, and 1.45 ms with the product walk above.  Bound by shared memory and, in double precision, the FP64 pipe.
+// The columns are a bitmap, a word per lane.  A B row whose entries are consecutive columns
+// (last - first + 1 = length, as in a band or a block) sets its bits and finds its columns
+// without reading them.
+constexpr int DN_WARPS = 8;
+constexpr int DN_AHEAD = 4;  // steps of 32 products whose loads are in flight
+
+struct DenseParts {  // per warp: 32 B rows
+    int64_t p0[32];   // first entry in B
+    val_t a[32];      // a_ik
+    int32_t x0[32];   // first column - lo
+    int32_t len[32];  // entries; negative: consecutive columns
+    uint32_t bits[32];
+};
+
+// FILL: sums and C's row (REPLAY: its values only); else the row's count per slice.
+template <int W, bool FILL, bool REPLAY>
+__global__ void __launch_bounds__(DN_WARPS * 32)
+k_dense_narrow(DevCSR A, DevCSR B, DenseArgs D, const int64_t *__restrict__ c_rp, int32_t *__restrict__ c_col,
+               val_t *__restrict__ c_val, int64_t *err, const int64_t *gate) {
+    static_assert(W % 32 == 0 && W <= 1024, "a bitmap word per lane");
+    __shared__ DenseParts parts[DN_WARPS];
+    extern __shared__ __align__(16) unsigned char dn_smem[];
+    if (FILL && gated(gate)) return;
+    const int lane = lane_id();
+    DenseParts &S = parts[warp_id()];
+    val_t *V = reinterpret_cast<val_t *>(dn_smem) + (FILL ? warp_id() * W : 0);
+    const int64_t i0 = D.dev_end ? D.dev_end[0] : (W == DENSE_MID_W ? D.n_wide : D.n_mid);
+    // with the counts on the device, one launch (of the wider kernel) takes all of them
+    const int64_t i1 = D.dev_end ? *D.dev_n : (W == DENSE_MID_W ? D.n_mid : D.n);
+    for (int64_t d = i0 + (int64_t)blockIdx.x * DN_WARPS + warp_id(); d < i1; d += (int64_t)gridDim.x * DN_WARPS) {
+        const int row = D.rows[d];
+        const int32_t lo = D.clo[d];
+        const int span = min(D.chi[d] - lo, W);
+        uint32_t known = 0;       // replay: the columns of C's row
+        bool bad = D.chi[d] - lo > W;  // cannot happen: the items were chosen by their width
+        S.bits[lane] = 0;
+        int64_t o = 0;
+        int n = 0;
+        if (FILL) {
+            o = c_rp[row];
+            n = (int)(c_rp[row + 1] - o);
+            for (int x = lane; x < span; x += 32) V[x] = val_t(0);
+        }
+        __syncwarp();
+        if (REPLAY) {
+            for (int t = lane; t < n; t += 32) {
+                const int x = c_col[o + t] - lo;
+                if ((unsigned)x < (unsigned)span) atomicOr(&S.bits[x >> 5], 1u << (x & 31));
+                else bad = true;  // C's columns were changed since the product
+            }
+            __syncwarp();
+            known = S.bits[lane];
+            __syncwarp();
+            S.bits[lane] = 0;
+            __syncwarp();
+        }
+        uint32_t mine = 0;  // bits of columns [32 lane, 32 lane + 32) set by consecutive parts
+        const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
+        for (int64_t e = a0; e < a1; e += 32) {
+            int len = 0, x0 = 0;
+            bool run = false;
+            int64_t rs = 0;
+            val_t av = val_t(0);
+            if (e + lane < a1) {
+                const int32_t k = A.col[e + lane];
+                if (FILL) av = A.val[e + lane];
+                rs = B.rp[k];
+                len = (int)(B.rp[k + 1] - rs);
+                if (len > 0) {
+                    const int32_t f = B.col[rs], l = B.col[rs + len - 1];
+                    x0 = f - lo;
+                    run = l - f + 1 == len;
+                    // cannot happen: [lo, hi) covers the columns of the row's parts
+                    if (x0 < 0 || l - lo >= span) {
+                        bad = true;
+                        len = 0;
+                    }
+                }
+            }
+            const unsigned nz = __ballot_sync(SPG_FULL, len > 0);
+            const int np = __popc(nz);
+            if (len > 0) {
+                const int q = __popc(nz & ((1u << lane) - 1u));
+                S.p0[q] = rs;
+                if (FILL) S.a[q] = av;
+                S.x0[q] = x0;
+                S.len[q] = run ? -len : len;
+            }
+            __syncwarp();
+            // the columns
+            for (int t = 0; t < np; ++t) {
+                const int ln = S.len[t], f = S.x0[t];
+                if (ln < 0) {
+                    const int b0 = max(f - 32 * lane, 0), b1 = min(f - ln - 32 * lane, 32);
+                    if (b0 < b1) mine |= (b1 - b0 == 32 ? ~0u : ((1u << (b1 - b0)) - 1u) << b0);
+                } else {
+                    const int64_t p = S.p0[t];
+                    for (int i = lane; i < ln; i += 32) {
+                        const int x = __ldg(B.col + p + i) - lo;
+                        if ((unsigned)x < (unsigned)span) atomicOr(&S.bits[x >> 5], 1u << (x & 31));
+                        else bad = true;
+                    }
+                }
+            }
+            if (FILL) {
+                // steps (part t, entries i0..i0+31), their loads DN_AHEAD steps ahead
+                val_t v[DN_AHEAD];
+                int32_t c[DN_AHEAD];
+                int lt = 0, li = 0;  // the next step to load
+                auto load = [&](val_t &vv, int32_t &cc) {
+                    if (lt >= np) return;
+                    const int ln = S.len[lt], m = ln < 0 ? -ln : ln;
+                    const int64_t p = S.p0[lt] + li + lane;
+                    if (li + lane < m) {
+                        vv = __ldg(B.val + p);
+                        cc = ln < 0 ? S.x0[lt] + li + lane : __ldg(B.col + p) - lo;
+                    }
+                    li += 32;
+                    if (li >= m) {
+                        li = 0;
+                        ++lt;
+                    }
+                };
+#pragma unroll
+                for (int u = 0; u < DN_AHEAD; ++u) load(v[u], c[u]);
+                for (int t = 0, i = 0; t < np;) {
+#pragma unroll
+                    for (int u = 0; u < DN_AHEAD; ++u) {
+                        if (t < np) {
+                            const int ln = S.len[t], m = ln < 0 ? -ln : ln;
+                            if (i + lane < m && (unsigned)c[u] < (unsigned)span) V[c[u]] = fma(S.a[t], v[u], V[c[u]]);
+                            i += 32;
+                            if (i >= m) {
+                                i = 0;
+                                ++t;
+                            }
+                            __syncwarp();  // the next B row may add into the same columns
+                            load(v[u], c[u]);
+                        }
+                    }
+                }
+            }
+            __syncwarp();  // the table is reused
+        }
+        const uint32_t bits = mine | S.bits[lane];
+        if (!FILL) {
+            // the columns of every slice the range touches, and zeros elsewhere
+            for (int s = lane; s < D.K; s += 32) D.cnt[d * D.K + s] = 0;
+            __syncwarp();
+            const int s0 = lo / D.W, s1 = (lo + span - 1) / D.W;
+            for (int s = s0; s <= s1 && s < D.K; ++s) {
+                const int64_t b = (int64_t)s * D.W - lo - 32 * lane;  // the slice's first column in this lane's word
+                const int b0 = (int)max(min(b, (int64_t)32), (int64_t)0), b1 = (int)max(min(b + D.W, (int64_t)32), (int64_t)0);
+                const uint32_t m = b1 > b0 ? (b1 - b0 == 32 ? ~0u : ((1u << (b1 - b0)) - 1u) << b0) : 0u;
+                const int c = __reduce_add_sync(SPG_FULL, __popc(bits & m));
+                if (lane == 0) D.cnt[d * D.K + s] = c;
+            }
+            if (__any_sync(SPG_FULL, bad) && lane == 0) atomicExch((unsigned long long *)err, 5ull);
+        } else {
+            const int cw = __popc(bits);
+            const int inc = warp_inclusive_scan(cw);
+            // every product's column is in C, and (but in a replay) C holds nothing else
+            if (REPLAY ? (bits & ~known) != 0u : __shfl_sync(SPG_FULL, inc, 31) != n) bad = true;
+            if (__any_sync(SPG_FULL, bad)) {
+                if (lane == 0) atomicExch((unsigned long long *)err, 6ull);
+                __syncwarp();
+                continue;
+            }
+            const uint32_t out = REPLAY ? known : bits;
+            const int ow = __popc(out);
+            const int before = warp_inclusive_scan(ow) - ow;
+            unsigned words = __ballot_sync(SPG_FULL, out != 0u);
+            while (words) {  // a word's columns are consecutive entries of C
+                const int w = __ffs(words) - 1;
+                words &= words - 1u;
+                const uint32_t wd = __shfl_sync(SPG_FULL, out, w);
+                const int r = __shfl_sync(SPG_FULL, before, w);
+                if ((wd >> lane) & 1u) {
+                    const int q = r + __popc(wd & ((1u << lane) - 1u));
+                    if (!SPG_IN(q < n, 113)) continue;  // the row's entries of C
+                    if (!REPLAY) c_col[o + q] = lo + 32 * w + lane;
+                    c_val[o + q] = V[32 * w + lane];
+                }
+            }
+            __syncwarp();  // the sums are cleared for the next row
+        }
+    }
+}
+
+template <int W, bool FILL, bool REPLAY>
+static cudaError_t launch_narrow(const DevCSR &A, const DevCSR &B, const DenseArgs &D, const int64_t *c_rp,
+                                 int32_t *c_col, val_t *c_val, int64_t *err, const int64_t *gate, cudaStream_t st) {
+    const int64_t n = D.dev_end != nullptr ? D.n : (W == DENSE_MID_W ? D.n_mid - D.n_wide : D.n - D.n_mid);
+    if (n <= 0) return cudaSuccess;
+    auto kern = k_dense_narrow<W, FILL, REPLAY>;
+    const int smem = FILL ? DN_WARPS * W * (int)sizeof(val_t) : 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    const int64_t need = (n + DN_WARPS - 1) / DN_WARPS;
+    const int64_t grid = D.dev_end != nullptr ? persistent_blocks((const void *)kern, DN_WARPS * 32, smem, need) : need;
+    if (grid <= 0 || grid > INT32_MAX) return cudaErrorInvalidValue;
+    kern<<<(unsigned)grid, DN_WARPS * 32, smem, st>>>(A, B, D, c_rp, c_col, c_val, err, gate);
+    return cudaGetLastError();
+}
+
+template <bool FILL, bool REPLAY>
+static cudaError_t launch_narrow_rows(const DevCSR &A, const DevCSR &B, const DenseArgs &D, const int64_t *c_rp,
+                                      int32_t *c_col, val_t *c_val, int64_t *err, const int64_t *gate,
+                                      cudaStream_t st) {
+    cudaError_t e = launch_narrow<DENSE_MID_W, FILL, REPLAY>(A, B, D, c_rp, c_col, c_val, err, gate, st);
+    if (e == cudaSuccess && D.dev_end == nullptr)
+        e = launch_narrow<DENSE_NARROW_W, FILL, REPLAY>(A, B, D, c_rp, c_col, c_val, err, gate, st);
+    return e;
+}
+
 // One thread per dense item (precise method): the slices' offsets inside the row and the
 // row's size nnz(c_i), the sum of its slices' counts.
 __global__ void k_dense_rowsum(DenseArgs D, int32_t *nnzc) {
@@ -579,15 +817,16 @@ static cudaError_t dense_check(const DevCSR &B, const DenseArgs &D) {
 
 cudaError_t launch_dense_count(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t *err, cudaStream_t st) {
     if (D.n <= 0) return cudaSuccess;
-    const int64_t nb = D.n * D.K;
+    const int64_t nb = (D.dev_end != nullptr ? D.n : D.n_wide) * D.K;
     cudaError_t e = dense_check(B, D);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = launch_narrow_rows<false, false>(A, B, D, nullptr, nullptr, nullptr, err, nullptr, st);
+    if (e != cudaSuccess || nb <= 0) return e;
     const int smem = (int)(sizeof(uint32_t) * dense_nw4(D.W));
     auto kern = k_dense_count<DENSE_NT>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     int64_t grid = nb;
-    if (D.dev_n != nullptr) {  // persistent grid over the items counted on the device
+    if (D.dev_end != nullptr) {  // persistent grid over the items counted on the device
         e = cudaMemsetAsync(D.queue, 0, sizeof(unsigned long long), st);
         if (e != cudaSuccess) return e;
         grid = persistent_blocks((const void *)kern, DENSE_NT, smem, nb);
@@ -614,14 +853,18 @@ cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs 
                               const int64_t *gate) {
     if (D.n <= 0) return cudaSuccess;
     cudaError_t e = dense_check(B, D);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess)
+        e = replay ? launch_narrow_rows<true, true>(A, B, D, c_rp, c_col, c_val, err, gate, st)
+                   : launch_narrow_rows<true, false>(A, B, D, c_rp, c_col, c_val, err, gate, st);
+    const int64_t nb = (D.dev_end != nullptr ? D.n : D.n_wide) * D.K;
+    if (e != cudaSuccess || nb <= 0) return e;
     // a persistent grid of nt threads per CTA over the items with counts in (cmin, cmax]
     auto go = [&](auto kern, int nt, int smem, int vcap, unsigned long long *q, int cmin, int cmax) -> cudaError_t {
         cudaError_t x = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (x == cudaSuccess) x = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         if (x == cudaSuccess) x = cudaMemsetAsync(q, 0, sizeof(unsigned long long), st);
         if (x != cudaSuccess) return x;
-        const int grid = persistent_blocks((const void *)kern, nt, smem, D.n * D.K);
+        const int grid = persistent_blocks((const void *)kern, nt, smem, nb);
         if (grid <= 0) return cudaErrorInvalidValue;
         kern<<<(unsigned)grid, nt, smem, st>>>(A, B, D, c_rp, c_col, c_val, err, gate, vcap, q, cmin, cmax);
         return cudaGetLastError();

@@ -32,6 +32,8 @@ struct DevCSR {
 };
 
 // Host-visible summary written by stage 2 (copied back in one transfer).
+// Rows of the dense-slice kernels that reach at most so many columns take a warp each.
+constexpr int DENSE_MID_W = 1024, DENSE_NARROW_W = 256;
 constexpr int NUM_LAUNCH_CLASSES = 8;  // learned: shared-memory classes of bin-37 rows
 
 struct BinSummary {
@@ -42,6 +44,8 @@ struct BinSummary {
     int64_t pad;
     int64_t class_count[NUM_LAUNCH_CLASSES];  // learned: bin-37 rows per launch class
     int64_t dense_count;                      // bin-37 rows computed by the dense-slice kernels
+    int64_t dense_end[2];                     // of these, the first [0] reach more than DENSE_MID_W columns,
+                                              // the next up to [1] more than DENSE_NARROW_W
     int64_t bin_start[NUM_BINS + 1];          // offsets of the bins in bin_rows (for launches sized on the device)
 };
 
@@ -219,14 +223,16 @@ struct DenseArgs {
     const int32_t *rows;   // their rows of A
     const int32_t *clo;    // and the column range [clo, chi) that each row's products can reach
     const int32_t *chi;
-    int64_t n;             // number of dense items
+    int64_t n;             // number of dense items: the first n_wide reach more than DENSE_MID_W
+    int64_t n_wide, n_mid; // columns, those up to n_mid more than DENSE_NARROW_W
     int K;                 // column slices of B
     int W;                 // slice width (a multiple of 32); slice s holds columns [s W, (s + 1) W)
     const int32_t *bnd;    // K > 1: per B row, K + 1 offsets of the slices' first entries in the row
     int32_t *cnt;          // n K columns per (row, slice)
     int32_t *soff;         // n K offsets of the slices inside their row of C
-    const int64_t *dev_n = nullptr;  // when set: the number of dense items is *dev_n (<= n), read on
-                                     // the device; the kernels run persistent grids over (item, slice)
+    const int64_t *dev_n = nullptr;  // when set: the number of dense items is *dev_n (<= n), and n_wide
+    const int64_t *dev_end = nullptr;  // and n_mid are dev_end[0..1], read on the device; the kernels run
+                                     // persistent grids over (item, slice)
     unsigned long long *queue = nullptr;  // DENSE_QUEUES work counters (count, fills by size), zeroed
                                           // by the launchers
     uint32_t *keep = nullptr;  // when set: keep_words words per (row, slice), where the count leaves
@@ -235,8 +241,9 @@ struct DenseArgs {
 };
 cudaError_t launch_dense_bounds(const DevCSR &B, int K, int W, int32_t *bnd, cudaStream_t st);
 int64_t dense_select_scratch(int64_t m);
-// order[0..nd) = items of the flagged bin-37 rows (larger u first), order[nd..n37) = the rest;
-// rows, rlo, rhi [0..nd) = their rows and column ranges; nd goes to summary->dense_count
+// order[0..nd) = items of the flagged bin-37 rows (the wide ones, larger u first, then the
+// narrow ones), order[nd..n37) = the rest; rows, rlo, rhi [0..nd) = their rows and column
+// ranges; nd and the ends of the wide ones go to the summary
 cudaError_t launch_dense_select(const int32_t *bin_rows, int64_t m, BinSummary *summary, const int64_t *u,
                                 const uint8_t *flag, const int32_t *lo, const int32_t *hi, int32_t *scratch,
                                 int32_t *order, int32_t *rows, int32_t *rlo, int32_t *rhi, cudaStream_t st);

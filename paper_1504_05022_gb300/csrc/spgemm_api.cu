@@ -204,7 +204,8 @@ struct spgemm_plan {
     // dense column slices for the longest bin-37 rows (off when dense_K == 0)
     int dense_K = 0, dense_W = 0;
     int64_t dense_min_u = 0;              // > 0: absolute threshold on u_i; 0: the row's column range
-    int64_t dense_n = 0;                  // dense bin-37 rows
+    int64_t dense_n = 0;                  // dense bin-37 rows: the first dense_wide of them take a CTA per
+    int64_t dense_wide = 0, dense_mid = 0;  // slice, the others (up to dense_mid: the wider) a warp per row
     uint8_t *dense_flag = nullptr;        // per row: 1 = dense-slice row (symbolic only)
     int32_t *dense_lo = nullptr, *dense_hi = nullptr;  // per row: column range (symbolic only)
     int32_t *dense_order = nullptr;       // bin-37 items: the dense ones (larger first), then the rest
@@ -216,8 +217,8 @@ struct spgemm_plan {
     int dense_keep_words = 0;        // words per (row, slice) of dense_keep
     cudaEvent_t dense_count_done = nullptr;  // the counts' stream reached the end of the counting pass
     DenseArgs dense_args() const {
-        DenseArgs D{dense_order, dense_rows, dense_clo, dense_chi, dense_n, dense_K, dense_W, dense_bnd,
-                    dense_cnt, dense_soff};
+        DenseArgs D{dense_order, dense_rows, dense_clo, dense_chi, dense_n, dense_wide, dense_mid, dense_K, dense_W,
+                    dense_bnd, dense_cnt, dense_soff};
         D.queue = d_queue;
         D.keep = dense_keep;
         D.keep_words = dense_keep_words;
@@ -697,11 +698,13 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
         p->stats.sum_u = p->h_summary.sum_u;
         p->stats.nnz_ctilde = p->h_summary.sum_cap;
         p->dense_n = p->dense_K > 0 ? p->h_summary.dense_count : 0;
+        p->dense_wide = p->dense_K > 0 ? p->h_summary.dense_end[0] : 0;
+        p->dense_mid = p->dense_K > 0 ? p->h_summary.dense_end[1] : 0;
         p->stats.rows_dense = p->dense_n;
         p->stats.dense_slices = p->dense_n > 0 ? p->dense_K : 0;
         if (p->dense_n > 0) {
             // kept for values-only replay: the slice boundaries, counts and offsets
-            if (p->dense_K > 1) {
+            if (p->dense_K > 1 && p->dense_wide > 0) {
                 SPG_TRY(p->alloc_n(&p->dense_bnd, p->B.nrows * (p->dense_K + 1)));
                 SPG_TRY(launch_dense_bounds(p->B, p->dense_K, p->dense_W, p->dense_bnd, p->st));
                 p->count(SPGEMM_K_OTHER);
@@ -980,9 +983,9 @@ static void alloc_dense_keep(spgemm_plan *p) {
     p->dense_keep_words = 0;
     const int want = p->opts.dense_keep;
     const int kw = p->dense_K > 0 ? dense_keep_words(p->dense_W) : 0;
-    if (p->dense_n == 0 || want < 0 || (want == 0 && p->opts.alloc_policy == SPGEMM_ALLOC_PRECISE))
+    if (p->dense_wide == 0 || want < 0 || (want == 0 && p->opts.alloc_policy == SPGEMM_ALLOC_PRECISE))
         return;
-    const int64_t words = p->dense_n * p->dense_K * (int64_t)kw;
+    const int64_t words = p->dense_wide * p->dense_K * (int64_t)kw;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
@@ -1882,6 +1885,7 @@ static DenseArgs dense_args_of(const spgemm_plan *p, bool dev) {
     if (dev) {
         D.n = p->A.nrows;  // every row may be in bin 37: the arrays hold n K entries
         D.dev_n = &p->d_summary->dense_count;
+        D.dev_end = p->d_summary->dense_end;
         D.queue = p->d_queue;
         D.keep = nullptr;  // tables sized for every row: no room kept for bitmaps
         D.keep_words = 0;

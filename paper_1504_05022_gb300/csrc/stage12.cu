@@ -91,22 +91,26 @@ struct StoreI64 {
     SPG_DEV void operator()(int64_t i, int64_t v) const { out[i] = v; }
 };
 
-constexpr int BIN_NT = 256;
+constexpr int BOUND_NT = 512;
+constexpr int BIN_NT = 256;  // of the scatter
 constexpr int BIN_NW = BIN_NT / 32;
-constexpr int BIN_ROWS_MAX = 2048;  // rows of a block
+constexpr int BIN_ROWS_MAX = 4096;  // rows of a block
 constexpr int LONG_STEPS = 16;      // a row longer than this many times its group is taken by the block
 
-// Lanes per row: about half the average length of A's rows, so that most rows take a few steps.
+// Lanes per row: a quarter of the average length of A's rows or more, so that a lane has about
+// four entries' gathers in flight; more lanes while that leaves SMs without a block.
 static int bound_group(int64_t m, int64_t nnz) {
     const int64_t avg = m > 0 ? nnz / m : 0;
-    return avg <= 6 ? 4 : avg <= 24 ? 8 : avg <= 64 ? 16 : 32;
+    int g = avg <= 16 ? 4 : avg <= 32 ? 8 : avg <= 64 ? 16 : 32;
+    while (g < 32 && g < avg && m * g < (int64_t)152 * BOUND_NT) g *= 2;
+    return g;
 }
 
-// Rows per block: a whole number of passes of 256 / group rows, and about eight blocks per SM
+// Rows per block: a whole number of passes of BOUND_NT / group rows, and about four blocks per SM
 // (of 152) for large m -- the (bin, block) counts are scanned by one block.
 static int64_t bin_rows_per_block(int64_t m, int64_t nnz) {
-    const int64_t rows = BIN_NT / bound_group(m, nnz);
-    int64_t passes = (m + rows * 1216 - 1) / (rows * 1216);
+    const int64_t rows = BOUND_NT / bound_group(m, nnz);
+    int64_t passes = (m + rows * 608 - 1) / (rows * 608);
     if (passes < 1) passes = 1;
     if (passes * rows > BIN_ROWS_MAX) passes = BIN_ROWS_MAX / rows;
     return passes * rows;
@@ -156,16 +160,16 @@ SPG_DEV bool dense_row(int b, int64_t i, const CapPolicy &P) {
 // to the dense-slice kernels: u_i >= dmin (dmin > 0), else div u_i >= hi - lo -- their products
 // cover at least a div-th of the columns they can reach, so the accumulator's O(hi - lo) clearing
 // and write-out are small beside them.  Latency-bound (two dependent gathers per nonzero): the
-// 27-point operator on 64^3 (6.9 M nonzeros) takes 65 us here (cold caches) and took 113 us as a
+// 27-point operator on 64^3 (6.9 M nonzeros) takes 37 us here (cold caches) and took 113 us as a
 // prefix sum, a marking pass and a histogram pass.
 template <int G>
-__global__ void __launch_bounds__(BIN_NT)
+__global__ void __launch_bounds__(BOUND_NT, 4)
 k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
     __shared__ int32_t hist[NUM_BINS];
     __shared__ int32_t nlong, longs[BIN_ROWS_MAX];
-    __shared__ int64_t scratch[BIN_NW + 1];
+    __shared__ int64_t scratch[BOUND_NT / 32 + 1];
     __shared__ int32_t range[2];
-    constexpr int ROWS = BIN_NT / G;
+    constexpr int ROWS = BOUND_NT / G;
     const int gl = threadIdx.x & (G - 1), grp = threadIdx.x / G;
     const unsigned gm = G == 32 ? SPG_FULL : ((1u << (G & 31)) - 1u) << (lane_id() & ~(G - 1));
     if (threadIdx.x < NUM_BINS) hist[threadIdx.x] = 0;
@@ -245,11 +249,11 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
         const int64_t i = base + longs[l];
         const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
         if (threadIdx.x < 2) range[threadIdx.x] = threadIdx.x == 0 ? INT32_MAX : -1;
-        const int64_t u = block_reduce_sum<BIN_NT>(sum_of(a0 + threadIdx.x, a1, BIN_NT), scratch);
+        const int64_t u = block_reduce_sum<BOUND_NT>(sum_of(a0 + threadIdx.x, a1, BOUND_NT), scratch);
         const int b = bin_of(u);
         if (b == BIN_MERGE && P.dense != nullptr) {
             int32_t cmin, cmax;
-            range_of(a0 + threadIdx.x, a1, BIN_NT, cmin, cmax);
+            range_of(a0 + threadIdx.x, a1, BOUND_NT, cmin, cmax);
             cmin = __reduce_min_sync(SPG_FULL, cmin);
             cmax = __reduce_max_sync(SPG_FULL, cmax);
             if (lane_id() == 0) {
@@ -262,8 +266,8 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
         __syncthreads();
     }
     if (threadIdx.x < NUM_BINS) O.hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = hist[threadIdx.x];
-    capsum = block_reduce_sum<BIN_NT>(capsum, scratch);
-    usum = block_reduce_sum<BIN_NT>(usum, scratch);
+    capsum = block_reduce_sum<BOUND_NT>(capsum, scratch);
+    usum = block_reduce_sum<BOUND_NT>(usum, scratch);
     if (threadIdx.x == 0) {
         O.part[blockIdx.x] = capsum;
         O.part[nblk + blockIdx.x] = usum;
@@ -275,12 +279,13 @@ template <typename T>
 SPG_DEV T warp_scan_array(T *v, int64_t n) {
     T carry = 0;
     const int lane = lane_id();
-    for (int64_t i0 = 0; i0 < n; i0 += 128) {
-        T x[4];
+    constexpr int UN = 8;
+    for (int64_t i0 = 0; i0 < n; i0 += 32 * UN) {
+        T x[UN];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = i0 + 32 * q + lane < n ? v[i0 + 32 * q + lane] : T(0);
+        for (int q = 0; q < UN; ++q) x[q] = i0 + 32 * q + lane < n ? v[i0 + 32 * q + lane] : T(0);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < UN; ++q) {
             const T inc = warp_inclusive_scan(x[q]);
             if (i0 + 32 * q + lane < n) v[i0 + 32 * q + lane] = carry + inc - x[q];
             carry += __shfl_sync(SPG_FULL, inc, 31);
@@ -323,6 +328,7 @@ k_bin_scan(int64_t m, int32_t *hist, int64_t nblk, int64_t *part, int64_t *ctil_
             S->sum_cap = total[NUM_BINS];
             S->sum_u = total[NUM_BINS + 1];
             S->dense_count = 0;
+            S->dense_end[0] = S->dense_end[1] = 0;
         }
     }
 }
@@ -395,7 +401,7 @@ cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, c
     if (nblk <= 0) return cudaMemsetAsync(O.err, 0, sizeof(int64_t), st);
     const int R = (int)bin_rows_per_block(A.nrows, A.nnz);
     auto go = [&](auto kern) {
-        kern<<<(unsigned)nblk, BIN_NT, 0, st>>>(A, B, P, O, R, nblk);
+        kern<<<(unsigned)nblk, BOUND_NT, 0, st>>>(A, B, P, O, R, nblk);
         return cudaGetLastError();
     };
     switch (bound_group(A.nrows, A.nnz)) {
