@@ -29,10 +29,7 @@ constexpr int OFF_MU = OFF_B3 + MLP_OUT;
 constexpr int OFF_SG = OFF_MU + MLP_IN;
 static_assert(OFF_MU == SPGEMM_MLP_NUM_PARAMS, "parameter layout");
 static_assert(OFF_SG + MLP_IN == SPGEMM_MLP_NUM_TOTAL, "parameter layout");
-// per-sample record kept between the forward/backward pass and the reduction
-constexpr int REC = MLP_IN + 2 * MLP_HID + MLP_HID + MLP_HID + MLP_OUT;  // xh, h1, h2, dz1, dz2, dout
-constexpr int R_XH = 0, R_H1 = MLP_IN, R_H2 = R_H1 + MLP_HID, R_DZ1 = R_H2 + MLP_HID,
-              R_DZ2 = R_DZ1 + MLP_HID, R_DOUT = R_DZ2 + MLP_HID;
+constexpr int MLP_WORK = 153;  // floats of scratch per sample (spgemm_mlp_work_floats)
 
 // ---------------- features ----------------
 
@@ -144,110 +141,243 @@ __global__ void k_mlp_forward(const float *__restrict__ params, const float *__r
     for (int k = 0; k < MLP_OUT; ++k) out[s * MLP_OUT + k] = o[k];
 }
 
-// Forward and backward of one sample per thread; records activations and deltas
-// for the reduction kernel and accumulates the summed loss.
-__global__ void k_mlp_fwd_bwd(const float *__restrict__ params, const float *__restrict__ X,
-                              const int32_t *__restrict__ cls, const float *__restrict__ y, int64_t n,
-                              float *__restrict__ rec, double *__restrict__ loss) {
-    __shared__ float P[SPGEMM_MLP_NUM_TOTAL];
-    __shared__ double lsum[8];
-    for (int t = threadIdx.x; t < SPGEMM_MLP_NUM_TOTAL; t += blockDim.x) P[t] = params[t];
-    __syncthreads();
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (s < n) {
-        float xh[MLP_IN], h1[MLP_HID], h2[MLP_HID], o[MLP_OUT];
-        mlp_forward_one(P, X + s * MLP_IN, xh, h1, h2, o);
-        float mx = o[0];
-#pragma unroll
-        for (int k = 1; k < MLP_CLS; ++k) mx = fmaxf(mx, o[k]);
-        float se = 0.f;
-#pragma unroll
-        for (int k = 0; k < MLP_CLS; ++k) se += expf(o[k] - mx);
-        const int c = cls[s];
-        const float r = o[MLP_CLS] - y[s];
-        l = (double)(logf(se) + mx - o[c]) + 0.5 * (double)r * (double)r;
-        float *R = rec + s * REC;
-        float dout[MLP_OUT];
-#pragma unroll
-        for (int k = 0; k < MLP_CLS; ++k) dout[k] = expf(o[k] - mx) / se - (k == c ? 1.f : 0.f);
-        dout[MLP_CLS] = r;
-        float dz2[MLP_HID];
-#pragma unroll 4
-        for (int i = 0; i < MLP_HID; ++i) {
-            float d = 0.f;
-            for (int k = 0; k < MLP_OUT; ++k) d = fmaf(dout[k], P[OFF_W3 + k * MLP_HID + i], d);
-            dz2[i] = h2[i] > 0.f ? d : 0.f;
-        }
-#pragma unroll 4
-        for (int i = 0; i < MLP_HID; ++i) {
-            float d = 0.f;
-#pragma unroll 8
-            for (int k = 0; k < MLP_HID; ++k) d = fmaf(dz2[k], P[OFF_W2 + k * MLP_HID + i], d);
-            R[R_DZ1 + i] = h1[i] > 0.f ? d : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < MLP_IN; ++i) R[R_XH + i] = xh[i];
-#pragma unroll
-        for (int i = 0; i < MLP_HID; ++i) {
-            R[R_H1 + i] = h1[i];
-            R[R_H2 + i] = h2[i];
-            R[R_DZ2 + i] = dz2[i];
-        }
-#pragma unroll
-        for (int k = 0; k < MLP_OUT; ++k) R[R_DOUT + k] = dout[k];
-    }
-    // block sum of the loss, one atomic per block
-    for (int d = 16; d > 0; d >>= 1) l += __shfl_xor_sync(SPG_FULL, l, d);
-    if ((threadIdx.x & 31) == 0) lsum[threadIdx.x >> 5] = l;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += lsum[w];
-        atomicAdd(loss, t);
-    }
+// Loss and gradients of a batch in two launches.
+//
+// k_mlp_loss_grad: a CTA takes tiles of MLP_TILE samples.  Four threads share a sample, each with
+// a quarter of every layer's neurons; activations and deltas lie in shared memory, a row per
+// neuron, so that the weight gradients are products of those rows over the tile's samples,
+// accumulated in registers over the CTA's tiles.  Every CTA leaves one partial gradient (and
+// loss), which k_mlp_grad_sum adds in a fixed order: the result does not depend on timing.
+// Each neuron's sum runs over its inputs in ascending order from the bias, as in
+// mlp_forward_one.  Bound by shared-memory reads and latency (two CTAs per SM at 8,192 samples).
+// A step of 8,192 samples with its Adam update takes 23 us; it took 118 us when one thread ran a
+// whole sample and wrote a 612-byte record of it, which the reduction read with a stride.
+constexpr int MLP_TILE = 64;
+constexpr int MLP_NT = 4 * MLP_TILE;
+constexpr int MLP_LD = MLP_TILE + 4;   // floats per row: 16-byte aligned, rows 4 banks apart
+constexpr int MLP_MAX_CTAS = 304;      // partial gradients (two CTAs on each of 152 SMs)
+constexpr int MLP_Q = MLP_HID / 4;     // a thread's neurons of a hidden layer
+constexpr int MLP_PART = SPGEMM_MLP_NUM_PARAMS + 3;  // floats of a partial, with its loss as a double
+static_assert(MLP_PART % 2 == 0 && MLP_Q == 8, "");
+
+struct MlpShared {
+    float w1t[MLP_IN][MLP_HID], w2t[MLP_HID][MLP_HID], w2[MLP_HID][MLP_HID];
+    float w3t[MLP_HID][20], w3[MLP_OUT][MLP_HID];  // *t: by input, then neuron
+    float b1[MLP_HID], b2[MLP_HID], b3[20], mu[MLP_IN], sg[MLP_IN];
+    float xh[MLP_IN][MLP_LD], h1[MLP_HID][MLP_LD], h2[MLP_HID][MLP_LD];
+    float dz1[MLP_HID][MLP_LD], dz2[MLP_HID][MLP_LD], out[MLP_OUT][MLP_LD], dout[MLP_OUT][MLP_LD];
+    double loss[MLP_TILE];
+};
+
+// z[0..8) += w[0..8) * x (w 16-byte aligned, the same for the whole warp)
+SPG_DEV void mlp_fma8(float (&z)[MLP_Q], const float *w, float x) {
+    const float4 a = *reinterpret_cast<const float4 *>(w), b = *reinterpret_cast<const float4 *>(w + 4);
+    z[0] = fmaf(a.x, x, z[0]);
+    z[1] = fmaf(a.y, x, z[1]);
+    z[2] = fmaf(a.z, x, z[2]);
+    z[3] = fmaf(a.w, x, z[3]);
+    z[4] = fmaf(b.x, x, z[4]);
+    z[5] = fmaf(b.y, x, z[5]);
+    z[6] = fmaf(b.z, x, z[6]);
+    z[7] = fmaf(b.w, x, z[7]);
 }
 
-// One block per output neuron of a layer: gradient row (weights and bias) summed
-// over all samples.  Blocks 0..31: layer 1, 32..63: layer 2, 64..80: layer 3.
-__global__ void k_mlp_grad_reduce(const float *__restrict__ rec, int64_t n, float *__restrict__ grad) {
-    const int b = blockIdx.x;
-    int o, nin, din, ain, gw, gb;
-    if (b < MLP_HID) {  // layer 1
-        o = b; nin = MLP_IN; din = R_DZ1; ain = R_XH; gw = OFF_W1; gb = OFF_B1;
-    } else if (b < 2 * MLP_HID) {  // layer 2
-        o = b - MLP_HID; nin = MLP_HID; din = R_DZ2; ain = R_H1; gw = OFF_W2; gb = OFF_B2;
-    } else {  // layer 3
-        o = b - 2 * MLP_HID; nin = MLP_HID; din = R_DOUT; ain = R_H2; gw = OFF_W3; gb = OFF_B3;
+// acc += the product of rows x and y over four samples, in pairs (a quarter of the roundings
+// that reach the long sum)
+SPG_DEV float mlp_dot4(float acc, const float4 &x, const float4 &y) {
+    return acc + (fmaf(x.w, y.w, x.z * y.z) + fmaf(x.y, y.y, x.x * y.x));
+}
+
+__global__ void __launch_bounds__(MLP_NT)
+k_mlp_loss_grad(const float *__restrict__ params, const float *__restrict__ X, const int32_t *__restrict__ cls,
+                const float *__restrict__ y, int64_t n, float *__restrict__ part, float *__restrict__ grad,
+                double *__restrict__ loss) {
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    MlpShared &S = *reinterpret_cast<MlpShared *>(mlp_smem);
+    const int tid = threadIdx.x;
+    for (int t = tid; t < MLP_HID * MLP_IN; t += MLP_NT) S.w1t[t % MLP_IN][t / MLP_IN] = params[OFF_W1 + t];
+    for (int t = tid; t < MLP_HID * MLP_HID; t += MLP_NT) {
+        const float w = params[OFF_W2 + t];
+        S.w2t[t % MLP_HID][t / MLP_HID] = w;
+        S.w2[t / MLP_HID][t % MLP_HID] = w;
     }
-    float acc[MLP_HID + 1];
+    for (int t = tid; t < MLP_OUT * MLP_HID; t += MLP_NT) {
+        const float w = params[OFF_W3 + t];
+        S.w3t[t % MLP_HID][t / MLP_HID] = w;
+        S.w3[t / MLP_HID][t % MLP_HID] = w;
+    }
+    if (tid < MLP_HID) {
+        S.b1[tid] = params[OFF_B1 + tid];
+        S.b2[tid] = params[OFF_B2 + tid];
+    }
+    if (tid < MLP_OUT) S.b3[tid] = params[OFF_B3 + tid];
+    if (tid < MLP_IN) {
+        S.mu[tid] = params[OFF_MU + tid];
+        S.sg[tid] = params[OFF_SG + tid];
+    }
+    const int s = tid & (MLP_TILE - 1), q = tid / MLP_TILE;  // sample of the tile, quarter (the same for a warp)
+    const int o0 = q * MLP_Q;                                // the thread's hidden neurons
+    // the thread's gradients: W2 rows {ta, ta + 16} x columns {tb, tb + 16}; W1 (tid / 8, tid % 8);
+    // W3 rows {tid / 32, tid / 32 + 8} and, in the first warp, row 16, column tid % 32; a bias
+    const int ta = tid >> 4, tb = tid & 15, ra = tid >> 5, rb = tid & 31;
+    float g2[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, g1 = 0.f, g3[3] = {0.f, 0.f, 0.f}, gb = 0.f;
+    double lsum = 0.0;
+    for (int64_t base = (int64_t)blockIdx.x * MLP_TILE; base < n; base += (int64_t)gridDim.x * MLP_TILE) {
+        const int64_t i = base + s;
+        const bool ok = i < n;  // past the end: zero deltas
+        __syncthreads();  // the weights are in place; the last tile's rows are free
+        // a quarter's two inputs
 #pragma unroll
-    for (int i = 0; i <= MLP_HID; ++i) acc[i] = 0.f;
-    for (int64_t s = threadIdx.x; s < n; s += blockDim.x) {
-        const float *R = rec + s * REC;
-        const float d = R[din + o];
-        if (d != 0.f) {
+        for (int k = 0; k < MLP_IN / 4; ++k) {
+            const int f = q * (MLP_IN / 4) + k;
+            S.xh[f][s] = ok ? (X[i * MLP_IN + f] - S.mu[f]) / S.sg[f] : 0.f;
+        }
+        __syncthreads();
+        float h[MLP_Q];
 #pragma unroll
-            for (int i = 0; i < MLP_HID; ++i)
-                if (i < nin) acc[i] = fmaf(d, R[ain + i], acc[i]);
-            acc[MLP_HID] += d;
+        for (int k = 0; k < MLP_Q; ++k) h[k] = S.b1[o0 + k];
+#pragma unroll
+        for (int k = 0; k < MLP_IN; ++k) mlp_fma8(h, &S.w1t[k][o0], S.xh[k][s]);
+#pragma unroll
+        for (int k = 0; k < MLP_Q; ++k) S.h1[o0 + k][s] = h[k] > 0.f ? h[k] : 0.f;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < MLP_Q; ++k) h[k] = S.b2[o0 + k];
+#pragma unroll 8
+        for (int k = 0; k < MLP_HID; ++k) mlp_fma8(h, &S.w2t[k][o0], S.h1[k][s]);
+#pragma unroll
+        for (int k = 0; k < MLP_Q; ++k) {
+            h[k] = h[k] > 0.f ? h[k] : 0.f;
+            S.h2[o0 + k][s] = h[k];
+        }
+        __syncthreads();
+        // outputs 4q..4q+3, and 16 by the first quarter
+        {
+            float o[4] = {S.b3[4 * q], S.b3[4 * q + 1], S.b3[4 * q + 2], S.b3[4 * q + 3]}, o16 = S.b3[16];
+#pragma unroll 8
+            for (int k = 0; k < MLP_HID; ++k) {
+                const float x = S.h2[k][s];
+                const float4 w = *reinterpret_cast<const float4 *>(&S.w3t[k][4 * q]);
+                o[0] = fmaf(w.x, x, o[0]);
+                o[1] = fmaf(w.y, x, o[1]);
+                o[2] = fmaf(w.z, x, o[2]);
+                o[3] = fmaf(w.w, x, o[3]);
+                if (q == 0) o16 = fmaf(S.w3t[k][16], x, o16);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) S.out[4 * q + k][s] = o[k];
+            if (q == 0) S.out[16][s] = o16;
+        }
+        __syncthreads();
+        {
+            float o[MLP_CLS];
+#pragma unroll
+            for (int k = 0; k < MLP_CLS; ++k) o[k] = S.out[k][s];
+            float mx = o[0];
+#pragma unroll
+            for (int k = 1; k < MLP_CLS; ++k) mx = fmaxf(mx, o[k]);
+            float ex[MLP_CLS], se = 0.f;
+#pragma unroll
+            for (int k = 0; k < MLP_CLS; ++k) {
+                ex[k] = expf(o[k] - mx);
+                se += ex[k];
+            }
+            const int c = ok ? cls[i] : 0;
+#pragma unroll
+            for (int k = 0; k < MLP_CLS; ++k)
+                if (k / 4 == q) S.dout[k][s] = ok ? ex[k] / se - (k == c ? 1.f : 0.f) : 0.f;
+            if (q == 0) {
+                const float r = ok ? S.out[MLP_CLS][s] - y[i] : 0.f;
+                S.dout[MLP_CLS][s] = r;
+                if (ok) lsum += (double)(logf(se) + mx - S.out[c][s]) + 0.5 * (double)r * (double)r;
+            }
+        }
+        __syncthreads();
+        float dz[MLP_Q];
+#pragma unroll
+        for (int k = 0; k < MLP_Q; ++k) dz[k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < MLP_OUT; ++k) mlp_fma8(dz, &S.w3[k][o0], S.dout[k][s]);
+#pragma unroll
+        for (int k = 0; k < MLP_Q; ++k) S.dz2[o0 + k][s] = h[k] > 0.f ? dz[k] : 0.f;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < MLP_Q; ++k) dz[k] = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < MLP_HID; ++k) mlp_fma8(dz, &S.w2[k][o0], S.dz2[k][s]);
+#pragma unroll
+        for (int k = 0; k < MLP_Q; ++k) S.dz1[o0 + k][s] = S.h1[o0 + k][s] > 0.f ? dz[k] : 0.f;
+        __syncthreads();
+        // the gradients, four samples at a time
+#pragma unroll 4
+        for (int t = 0; t < MLP_TILE; t += 4) {
+            auto row = [&](const float (*m)[MLP_LD], int r) { return *reinterpret_cast<const float4 *>(&m[r][t]); };
+            const float4 a0 = row(S.dz2, ta), a1 = row(S.dz2, ta + 16), c0 = row(S.h1, tb), c1 = row(S.h1, tb + 16);
+            g2[0][0] = mlp_dot4(g2[0][0], a0, c0);
+            g2[0][1] = mlp_dot4(g2[0][1], a0, c1);
+            g2[1][0] = mlp_dot4(g2[1][0], a1, c0);
+            g2[1][1] = mlp_dot4(g2[1][1], a1, c1);
+            g1 = mlp_dot4(g1, row(S.dz1, tid >> 3), row(S.xh, tid & 7));
+            const float4 d = row(S.h2, rb);
+            g3[0] = mlp_dot4(g3[0], row(S.dout, ra), d);
+            g3[1] = mlp_dot4(g3[1], row(S.dout, ra + 8), d);
+            if (ra == 0) g3[2] = mlp_dot4(g3[2], row(S.dout, 16), d);
+            if (tid < 2 * MLP_HID + MLP_OUT) {
+                const float4 v = tid < MLP_HID ? row(S.dz1, tid)
+                                 : tid < 2 * MLP_HID ? row(S.dz2, tid - MLP_HID) : row(S.dout, tid - 2 * MLP_HID);
+                gb += (v.x + v.y) + (v.z + v.w);
+            }
         }
     }
-    __shared__ float red[MLP_HID + 1][8];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i <= MLP_HID; ++i) {
-        float v = acc[i];
-        for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(SPG_FULL, v, d);
-        if (lane == 0) red[i][w] = v;
-    }
+    // the loss of the CTA's samples, in the order of the tile's slots
     __syncthreads();
-    if (threadIdx.x <= MLP_HID) {
-        const int i = threadIdx.x;
-        float v = 0.f;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) v += red[i][k];
-        if (i < nin) grad[gw + o * nin + i] = v;
-        else if (i == MLP_HID) grad[gb + o] = v;
+    if (q == 0) S.loss[s] = lsum;
+    __syncthreads();
+    // one CTA: the result itself; else a partial of MLP_PART floats, the loss first
+    float *g = gridDim.x == 1 ? grad : part + (int64_t)blockIdx.x * MLP_PART + 2;
+    if (tid == 0) {
+        double t = 0.0;
+        for (int k = 0; k < MLP_TILE; ++k) t += S.loss[k];
+        *(gridDim.x == 1 ? loss : reinterpret_cast<double *>(part + (int64_t)blockIdx.x * MLP_PART)) = t;
+    }
+    g[OFF_W1 + tid] = g1;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) g[OFF_W2 + (ta + 16 * a) * MLP_HID + tb + 16 * b] = g2[a][b];
+    g[OFF_W3 + ra * MLP_HID + rb] = g3[0];
+    g[OFF_W3 + (ra + 8) * MLP_HID + rb] = g3[1];
+    if (ra == 0) g[OFF_W3 + 16 * MLP_HID + rb] = g3[2];
+    if (tid < MLP_HID) g[OFF_B1 + tid] = gb;
+    else if (tid < 2 * MLP_HID) g[OFF_B2 + tid - MLP_HID] = gb;
+    else if (tid < 2 * MLP_HID + MLP_OUT) g[OFF_B3 + tid - 2 * MLP_HID] = gb;
+}
+
+// Sums the partial gradients: 64 parameters per CTA, eight threads a parameter, each over every
+// eighth partial in ascending order, in four interleaved sums added pairwise.  The last CTA sums
+// the losses.
+__global__ void __launch_bounds__(512)
+k_mlp_grad_sum(const float *__restrict__ part, int np, float *__restrict__ grad, double *__restrict__ loss) {
+    __shared__ float acc[8][64];
+    const int c = threadIdx.x & 63, r = threadIdx.x >> 6;
+    const int k = blockIdx.x * 64 + c;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (k < SPGEMM_MLP_NUM_PARAMS) {
+        for (int p0 = r; p0 < np; p0 += 32) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (p0 + 8 * j < np) v[j] += part[(int64_t)(p0 + 8 * j) * MLP_PART + 2 + k];
+        }
+    }
+    acc[r][c] = (v[0] + v[1]) + (v[2] + v[3]);
+    __syncthreads();
+    if (r == 0 && k < SPGEMM_MLP_NUM_PARAMS)
+        grad[k] = ((acc[0][c] + acc[1][c]) + (acc[2][c] + acc[3][c])) + ((acc[4][c] + acc[5][c]) + (acc[6][c] + acc[7][c]));
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) {
+        double t = 0.0;
+        for (int p = threadIdx.x; p < np; p += 32) t += *reinterpret_cast<const double *>(part + (int64_t)p * MLP_PART);
+        t = warp_reduce_sum(t);
+        if (threadIdx.x == 0) *loss = t;
     }
 }
 
@@ -472,18 +602,27 @@ extern "C" spgemm_status spgemm_mlp_loss_grad(const float *params, const float *
     if (n < 0 || !params || !grad || !loss || (n > 0 && (!X || !cls || !y || !work)))
         return SPGEMM_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(loss, 0, sizeof(double), st) != cudaSuccess) return SPGEMM_ERR_CUDA;
     if (n == 0) {
+        if (cudaMemsetAsync(loss, 0, sizeof(double), st) != cudaSuccess) return SPGEMM_ERR_CUDA;
         if (cudaMemsetAsync(grad, 0, sizeof(float) * SPGEMM_MLP_NUM_PARAMS, st) != cudaSuccess)
             return SPGEMM_ERR_CUDA;
         return SPGEMM_OK;
     }
-    k_mlp_fwd_bwd<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(params, X, cls, y, n, work, loss);
-    k_mlp_grad_reduce<<<2 * MLP_HID + MLP_OUT, 256, 0, st>>>(work, n, grad);
+    // at most n / MLP_TILE + 1 partials (none for one CTA), which n * MLP_WORK floats hold; their
+    // losses are doubles
+    const int64_t tiles = (n + MLP_TILE - 1) / MLP_TILE;
+    const int ctas = (int)(tiles < MLP_MAX_CTAS ? tiles : MLP_MAX_CTAS);
+    static_assert((int64_t)MLP_TILE * MLP_WORK >= 2 * MLP_PART, "the partials of n > MLP_TILE samples fit");
+    if (ctas > 1 && reinterpret_cast<uintptr_t>(work) % 8 != 0) work += 1;  // 4-byte aligned: one float is spare
+    if (cudaFuncSetAttribute(k_mlp_loss_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(MlpShared)) !=
+        cudaSuccess)
+        return SPGEMM_ERR_CUDA;
+    k_mlp_loss_grad<<<ctas, MLP_NT, sizeof(MlpShared), st>>>(params, X, cls, y, n, work, grad, loss);
+    if (ctas > 1) k_mlp_grad_sum<<<(SPGEMM_MLP_NUM_PARAMS + 63) / 64, 512, 0, st>>>(work, ctas, grad, loss);
     return cudaGetLastError() == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;
 }
 
-extern "C" int64_t spgemm_mlp_work_floats(int64_t n) { return n * (int64_t)REC; }
+extern "C" int64_t spgemm_mlp_work_floats(int64_t n) { return n * (int64_t)MLP_WORK; }
 
 extern "C" spgemm_status spgemm_mlp_adam(float *params, const float *grad, float *m, float *v, int64_t step,
                                          float lr, float grad_scale, spgemm_stream_t stream) {
