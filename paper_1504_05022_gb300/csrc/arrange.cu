@@ -161,9 +161,22 @@ k_arrange_long(MergeItems it, const int64_t *__restrict__ c_rp, int32_t *__restr
             const int32_t *sc = it.home_col[x];
             const val_t *sv = it.home_val[x];
             if (!SPG_IN(o + n <= c_rp[it.row[j] + 1], 105)) break;  // the leaves fill the row of C exactly
-            for (int64_t t = threadIdx.x; t < n; t += ARR_NT) {
-                c_col[o + t] = sc[t];
-                c_val[o + t] = sv[t];
+            constexpr int UN = 4;  // loads in flight per thread
+            for (int64_t t = threadIdx.x; t < n; t += UN * ARR_NT) {
+                int32_t c[UN];
+                val_t v[UN];
+#pragma unroll
+                for (int u = 0; u < UN; ++u)
+                    if (t + u * ARR_NT < n) c[u] = __ldcs(sc + t + u * ARR_NT);
+#pragma unroll
+                for (int u = 0; u < UN; ++u)
+                    if (t + u * ARR_NT < n) v[u] = __ldcs(sv + t + u * ARR_NT);
+#pragma unroll
+                for (int u = 0; u < UN; ++u)
+                    if (t + u * ARR_NT < n) {
+                        c_col[o + t + u * ARR_NT] = c[u];
+                        c_val[o + t + u * ARR_NT] = v[u];
+                    }
             }
             o += n;
         }

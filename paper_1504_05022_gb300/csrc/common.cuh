@@ -71,6 +71,20 @@ SPG_DEV int split_next_leaf(const MergeItems &it, int root, int x) {
     return -1;
 }
 
+// Threads of the CTA that takes a bin-37 row of u products and nA entries of A in registers
+// (k_merge_small), 0 when the row goes to the batched kernel.  small_u: the most products of such
+// a row (0: none).
+SPG_DEV int merge_small_threads(int64_t u, int nA, int small_u) {
+    if (u > small_u) return 0;
+    if (u <= 128 * 16 && nA <= 256) return 128;
+    if (u <= 256 * 16 && nA <= 512) return 256;
+    return u <= 512 * 16 && nA <= 1024 ? 512 : 0;
+}
+// A whole row that no launch of the batched kernel has begun.
+SPG_DEV bool merge_fresh(const MergeItems &it, int j) {
+    return it.src_len[j] == 0 && it.ck_entry[j] == 0 && it.ck_off[j] == 0 && it.clo[j] == 0 && it.chi[j] == INT32_MAX;
+}
+
 // True when a gate word is set: the launch must write nothing.
 SPG_DEV bool gated(const int64_t *gate) { return gate != nullptr && *gate != 0; }
 SPG_DEV int warp_id() { return threadIdx.x >> 5; }

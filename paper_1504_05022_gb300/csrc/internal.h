@@ -187,7 +187,13 @@ struct MergeLaunch {
     int bm_words;            // > 0: bitmap kernel; flat: bitmap words, two-level: level-1 words
     int bm_two;              // 1: two-level index
     int bm_miss;             // bitmap kernel: miss-buffer entries
+    const int64_t *u;        // bound of every row of C
+    int small_u;             // bitmap kernel: fresh rows of at most this many products (and few enough
+                             // entries of A) are taken whole by k_merge_small; 0: none.  At most the
+                             // largest capacity, so that such a row never has to be split
 };
+constexpr int MERGE_SMALL_U = 8192;  // the most small_u can be
+cudaError_t launch_merge_small(const StageArgs &a, const MergeItems &it, const MergeLaunch &L, cudaStream_t st);
 
 int merge_smem_bytes(int cap, int batch, int wide_above);
 // Bitmap form of the bin-37 kernel (merge_bm.cu): a flat bitmap index for B with at
@@ -299,8 +305,8 @@ cudaError_t launch_concat(const PairDesc *d, int64_t npairs, const int64_t *moff
                           val_t *b_val, bool values_only, cudaStream_t st);
 cudaError_t launch_gather_first(const PairDesc *d, int64_t npairs, const int64_t *c_rp, int64_t M, int64_t *out,
                                 cudaStream_t st);
-cudaError_t launch_pair_products(const PairDesc *d, int64_t npairs, int64_t *prod, int64_t *clow,
-                                 cudaStream_t st);
+cudaError_t launch_pair_products(const PairDesc *d, int64_t npairs, const int64_t *moff, int64_t M, int64_t *prod,
+                                 int64_t *clow, cudaStream_t st);
 cudaError_t launch_split_out(const PairDesc *d, int64_t npairs, const int64_t *c_rp, int64_t M, int64_t *rp_out,
                              cudaStream_t st);
 

@@ -289,13 +289,11 @@ SPG_DEV int bm_merge_misses(const BmSmem &s, Index &ix, int rlen, int nm, int32_
     return fnew;
 }
 
-template <int NT, int MINB, bool TWO>
-__global__ void __launch_bounds__(NT, MINB)
-k_merge_bm(StageArgs a, MergeItems it, MergeLaunch L) {
-    extern __shared__ __align__(16) unsigned char bm_smem[];
-    __shared__ int64_t scan64[NT / 32 + 1];
-    __shared__ int32_t scan32[NT / 32 + 1];
-    __shared__ int32_t s_nmiss;
+// One work item, by the whole CTA.
+template <int NT, bool TWO>
+SPG_DEV void merge_bm_item(const StageArgs &a, const MergeItems &it, const MergeLaunch &L, int64_t w, int j,
+                           unsigned char *bm_smem, int64_t *scan64, int32_t *scan32, int32_t *nmiss_shared) {
+    int32_t &s_nmiss = *nmiss_shared;
     constexpr int W = NT;
     using Index = typename std::conditional<TWO, TwoIndex, FlatIndex>::type;
     BmSmem s;
@@ -305,8 +303,6 @@ k_merge_bm(StageArgs a, MergeItems it, MergeLaunch L) {
     const int mcap = L.bm_miss;
     bm_layout(L.cap, L.bm_words, mcap, W, TWO, bm_smem, &s, &fi, &ti);
 
-    const int64_t w = blockIdx.x;
-    const int j = L.work ? L.work[w] : (int)(L.work_base + w);
     const int row = it.row[j];
     const int32_t clo = it.clo[j], chi = it.chi[j];
     const bool filtered = (clo > 0) || (chi < INT32_MAX);
@@ -551,6 +547,36 @@ k_merge_bm(StageArgs a, MergeItems it, MergeLaunch L) {
     }
 }
 
+// A CTA looks at `per` items and takes those that k_merge_small does not.
+template <int NT, int MINB, bool TWO>
+__global__ void __launch_bounds__(NT, MINB)
+k_merge_bm(StageArgs a, MergeItems it, MergeLaunch L, int per) {
+    extern __shared__ __align__(16) unsigned char bm_smem[];
+    __shared__ int64_t scan64[NT / 32 + 1];
+    __shared__ int32_t scan32[NT / 32 + 1];
+    __shared__ int32_t s_nmiss;
+    __shared__ unsigned s_take;
+    const int64_t w0 = (int64_t)blockIdx.x * per;
+    if (threadIdx.x < 32) {
+        bool take = false;
+        if ((int)threadIdx.x < per && w0 + threadIdx.x < L.nwork) {
+            const int j = L.work ? L.work[w0 + threadIdx.x] : (int)(L.work_base + w0 + threadIdx.x);
+            const int row = it.row[j];
+            const int nA = (int)min(a.A.rp[row + 1] - a.A.rp[row], (int64_t)INT_MAX);
+            take = L.small_u <= 0 || merge_small_threads(L.u[row], nA, L.small_u) == 0 || !merge_fresh(it, j);
+        }
+        const unsigned m = __ballot_sync(SPG_FULL, take);
+        if (threadIdx.x == 0) s_take = m;
+    }
+    __syncthreads();
+    for (unsigned m = s_take; m != 0u; m &= m - 1u) {
+        const int64_t w = w0 + __ffs(m) - 1;
+        const int j = L.work ? L.work[w] : (int)(L.work_base + w);
+        merge_bm_item<NT, TWO>(a, it, L, w, j, bm_smem, scan64, scan32, &s_nmiss);
+        __syncthreads();  // the item's shared memory is free
+    }
+}
+
 // Threads per CTA (same rule as k_merge).
 static int bm_threads(int cap, int wide_above) {
     if (wide_above <= 0) wide_above = 2048;
@@ -575,7 +601,11 @@ static cudaError_t launch_bm_nt(const StageArgs &a, const MergeItems &s, const M
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)L.nwork, NT, smem, st>>>(a, s, L);
+    // without rows for k_merge_small a CTA per item; else most items are not this kernel's, and a
+    // CTA looks at up to 32 (fewer while that leaves SMs idle)
+    int64_t per = 1;
+    if (L.small_u > 0) per = std::max<int64_t>(1, std::min<int64_t>(32, L.nwork / (152 * 16)));
+    kern<<<(unsigned)((L.nwork + per - 1) / per), NT, smem, st>>>(a, s, L, (int)per);
     return cudaGetLastError();
 }
 
@@ -595,6 +625,8 @@ cudaError_t launch_merge_bm(const StageArgs &a, const MergeItems &s, const Merge
     if (L.level1 || L.bm_words <= 0 || L.batch > nt * BM_IPT || L.batch < 32 || L.bm_miss < L.batch ||
         span < a.B.ncols)
         return cudaErrorInvalidValue;
+    const cudaError_t e = launch_merge_small(a, s, L, st);
+    if (e != cudaSuccess) return e;
     const int smem = merge_bm_smem_bytes(L.cap, L.bm_words, L.bm_miss, L.wide_above, L.bm_two != 0);
     return L.bm_two ? launch_bm<true>(a, s, L, nt, smem, st) : launch_bm<false>(a, s, L, nt, smem, st);
 }

@@ -878,6 +878,8 @@ spgemm_status run_progressive(spgemm_plan *p, const int32_t *work_in, int64_t wo
                 L.bm_words = p->bm_words;
                 L.bm_miss = p->bm_miss;
                 L.bm_two = p->bm_two;
+                L.u = p->u;
+                L.small_u = std::min(MERGE_SMALL_U, p->capmax);
                 L.work = work;
                 L.work_base = work_base;
                 L.nwork = nwork;
@@ -1117,6 +1119,8 @@ spgemm_status run_bin37(spgemm_plan *p) {
                 L.bm_words = p->bm_words;
                 L.bm_miss = p->bm_miss;
                 L.bm_two = p->bm_two;
+                L.u = p->u;
+                L.small_u = std::min(MERGE_SMALL_U, p->capmax);
                 L.work = p->class_order + off;
                 L.nwork = cnt;
                 L.cap = ccap;
@@ -1159,6 +1163,8 @@ spgemm_status run_bin37(spgemm_plan *p) {
                 L.bm_words = p->bm_words;
                 L.bm_miss = p->bm_miss;
                 L.bm_two = p->bm_two;
+                L.u = p->u;
+                L.small_u = std::min(MERGE_SMALL_U, p->capmax);
                 L.work = lists[k];
                 L.nwork = nk;
                 L.cap = lv[k];
@@ -1519,7 +1525,7 @@ extern "C" spgemm_status spgemm_batched_symbolic(int64_t npairs, const spgemm_cs
             int64_t *d_prod = nullptr, *d_clow = nullptr;
             SPG_TRY(p->alloc_n(&d_prod, npairs, LIFE_SYMBOLIC));
             SPG_TRY(p->alloc_n(&d_clow, npairs, LIFE_SYMBOLIC));
-            SPG_TRY(launch_pair_products(p->d_pairs, npairs, d_prod, d_clow, p->st));
+            SPG_TRY(launch_pair_products(p->d_pairs, npairs, p->d_moff, M, d_prod, d_clow, p->st));
             p->count(SPGEMM_K_OTHER);
             std::vector<int64_t> prod(npairs), clow(npairs);
             SPG_TRY(cudaStreamSynchronize(p->st));

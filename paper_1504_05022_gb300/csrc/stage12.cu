@@ -2,8 +2,8 @@
 // Algorithm 3) of the SpGEMM framework, plus input widening and validation.
 //
 // Stage 1 gives a group of lanes to each row of A (as many as the rows' average length
-// asks for) and a whole block to each long row, so a hub row cannot unbalance the kernel the
-// way one-thread-per-row (the paper's launch shape) would.  The same kernel bins the row,
+// asks for), a warp to each long row and a whole block to a hub row, so that none unbalances the
+// kernel the way one-thread-per-row (the paper's launch shape) would.  The same kernel bins the row,
 // counts the bins of its block of rows and finds the column range of the bin-37 rows: u_i
 // never goes through a prefix sum over A's nonzeros, which took 16 bytes of traffic per
 // nonzero and three launches.
@@ -94,8 +94,8 @@ struct StoreI64 {
 constexpr int BOUND_NT = 512;
 constexpr int BIN_NT = 256;  // of the scatter
 constexpr int BIN_NW = BIN_NT / 32;
-constexpr int BIN_ROWS_MAX = 4096;  // rows of a block
-constexpr int LONG_STEPS = 16;      // a row longer than this many times its group is taken by the block
+constexpr int LONG_STEPS = 16;      // a row longer than this many times its group is taken by a warp,
+constexpr int HUB_ENTRIES = 1024;   // one of more entries than this by the block
 
 // Lanes per row: a quarter of the average length of A's rows or more, so that a lane has about
 // four entries' gathers in flight; more lanes while that leaves SMs without a block.
@@ -106,14 +106,13 @@ static int bound_group(int64_t m, int64_t nnz) {
     return g;
 }
 
-// Rows per block: a whole number of passes of BOUND_NT / group rows, and about four blocks per SM
-// (of 152) for large m -- the (bin, block) counts are scanned by one block.
+// Stage 1 runs a block per BOUND_NT / group rows, so that a run of hub rows (the low rows of an
+// R-MAT matrix) spreads over the SMs; stage 2 bins blocks of that many rows times a factor that
+// leaves about four per SM (of 152), since one block scans the (bin, block) counts.
 static int64_t bin_rows_per_block(int64_t m, int64_t nnz) {
     const int64_t rows = BOUND_NT / bound_group(m, nnz);
-    int64_t passes = (m + rows * 608 - 1) / (rows * 608);
-    if (passes < 1) passes = 1;
-    if (passes * rows > BIN_ROWS_MAX) passes = BIN_ROWS_MAX / rows;
-    return passes * rows;
+    const int64_t factor = (m + rows * 608 - 1) / (rows * 608);
+    return rows * (factor < 1 ? 1 : factor);
 }
 
 int64_t bin_blocks(int64_t m, int64_t nnz) {
@@ -154,22 +153,22 @@ SPG_DEV bool dense_row(int b, int64_t i, const CapPolicy &P) {
     return b == BIN_MERGE && P.dense != nullptr && P.dense[i] != 0;
 }
 
-// u_i, bin and row size of every row, the histogram of the block's rows, and the block's sums of
-// C~ entries and of u_i (part[0..nblk), part[nblk..2 nblk)).  Bin-37 rows also get their column
+// u_i, bin and row size of every row, and per `factor` blocks the histogram of the rows and the
+// sums of C~ entries and of u_i (part[0..nblk), part[nblk..2 nblk)), zeroed before when factor > 1.  Bin-37 rows also get their column
 // range [lo, hi) (first and last column of every B row they select) and the flag that sends them
 // to the dense-slice kernels: u_i >= dmin (dmin > 0), else div u_i >= hi - lo -- their products
 // cover at least a div-th of the columns they can reach, so the accumulator's O(hi - lo) clearing
 // and write-out are small beside them.  Latency-bound (two dependent gathers per nonzero): the
-// 27-point operator on 64^3 (6.9 M nonzeros) takes 37 us here (cold caches) and took 113 us as a
+// 27-point operator on 64^3 (6.9 M nonzeros) takes 45 us here (cold caches) and took 113 us as a
 // prefix sum, a marking pass and a histogram pass.
 template <int G>
-__global__ void __launch_bounds__(BOUND_NT, 4)
-k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
+__global__ void __launch_bounds__(BOUND_NT, 3)
+k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
     __shared__ int32_t hist[NUM_BINS];
-    __shared__ int32_t nlong, longs[BIN_ROWS_MAX];
+    constexpr int ROWS = BOUND_NT / G;
+    __shared__ int32_t nlong, longs[ROWS];
     __shared__ int64_t scratch[BOUND_NT / 32 + 1];
     __shared__ int32_t range[2];
-    constexpr int ROWS = BOUND_NT / G;
     const int gl = threadIdx.x & (G - 1), grp = threadIdx.x / G;
     const unsigned gm = G == 32 ? SPG_FULL : ((1u << (G & 31)) - 1u) << (lane_id() & ~(G - 1));
     if (threadIdx.x < NUM_BINS) hist[threadIdx.x] = 0;
@@ -178,7 +177,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
         if (blockIdx.x == 0) *O.err = 0;
     }
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * R;
+    const int64_t base = (int64_t)blockIdx.x * ROWS;
     int64_t capsum = 0, usum = 0;
     auto sum_of = [&](int64_t p0, int64_t p1, int step) {
         int64_t u = 0;
@@ -192,12 +191,24 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
     auto range_of = [&](int64_t p0, int64_t p1, int step, int32_t &cmin, int32_t &cmax) {
         cmin = INT32_MAX;
         cmax = -1;
-        for (int64_t p = p0; p < p1; p += step) {
-            const int32_t k = A.col[p];
-            const int64_t rs = B.rp[k], re = B.rp[k + 1];
-            if (re > rs) {
-                cmin = min(cmin, B.col[rs]);
-                cmax = max(cmax, B.col[re - 1]);
+        constexpr int UN = 4;  // entries whose dependent gathers are in flight together
+        for (int64_t p = p0; p < p1; p += UN * step) {
+            int64_t rs[UN], re[UN];
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                rs[u] = re[u] = 0;
+                if (p + u * step < p1) {
+                    const int32_t k = A.col[p + u * step];
+                    rs[u] = B.rp[k];
+                    re[u] = B.rp[k + 1];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UN; ++u) {
+                if (re[u] > rs[u]) {
+                    cmin = min(cmin, B.col[rs[u]]);
+                    cmax = max(cmax, B.col[re[u] - 1]);
+                }
             }
         }
     };
@@ -220,34 +231,49 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
         capsum += cap_of(u, b, i, P, dense);
         usum += u;
     };
-    for (int r0 = 0; r0 < R; r0 += ROWS) {
-        const int64_t i = base + r0 + grp;
-        if (i >= A.nrows) break;  // the whole group
-        const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
+    const int64_t mine = base + grp;
+    if (mine < A.nrows) {  // the whole group
+        const int64_t a0 = A.rp[mine], a1 = A.rp[mine + 1];
         if (a1 - a0 > LONG_STEPS * G) {
-            if (gl == 0) longs[atomicAdd(&nlong, 1)] = r0 + grp;
-            continue;
-        }
-        int64_t u = sum_of(a0 + gl, a1, G);
+            if (gl == 0) longs[atomicAdd(&nlong, 1)] = grp;
+        } else {
+            int64_t u = sum_of(a0 + gl, a1, G);
 #pragma unroll
-        for (int d = G / 2; d > 0; d >>= 1) u += __shfl_xor_sync(gm, u, d, G);
-        const int b = bin_of(u);
-        int32_t cmin = 0, cmax = 0;
-        if (b == BIN_MERGE && P.dense != nullptr) {
-            range_of(a0 + gl, a1, G, cmin, cmax);
+            for (int d = G / 2; d > 0; d >>= 1) u += __shfl_xor_sync(gm, u, d, G);
+            const int b = bin_of(u);
+            int32_t cmin = 0, cmax = 0;
+            if (b == BIN_MERGE && P.dense != nullptr) {
+                range_of(a0 + gl, a1, G, cmin, cmax);
 #pragma unroll
-            for (int d = G / 2; d > 0; d >>= 1) {
-                cmin = min(cmin, __shfl_xor_sync(gm, cmin, d, G));
-                cmax = max(cmax, __shfl_xor_sync(gm, cmax, d, G));
+                for (int d = G / 2; d > 0; d >>= 1) {
+                    cmin = min(cmin, __shfl_xor_sync(gm, cmin, d, G));
+                    cmax = max(cmax, __shfl_xor_sync(gm, cmax, d, G));
+                }
             }
+            if (gl == 0) finish(mine, u, b, cmin, cmax);
         }
-        if (gl == 0) finish(i, u, b, cmin, cmax);
     }
     __syncthreads();
     const int nl = nlong;
+    for (int l = warp_id(); l < nl; l += BOUND_NT / 32) {
+        const int64_t i = base + longs[l];
+        const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
+        if (a1 - a0 > HUB_ENTRIES) continue;
+        const int64_t u = warp_reduce_sum(sum_of(a0 + lane_id(), a1, 32));
+        const int b = bin_of(u);
+        int32_t cmin = 0, cmax = 0;
+        if (b == BIN_MERGE && P.dense != nullptr) {
+            range_of(a0 + lane_id(), a1, 32, cmin, cmax);
+            cmin = __reduce_min_sync(SPG_FULL, cmin);
+            cmax = __reduce_max_sync(SPG_FULL, cmax);
+        }
+        if (lane_id() == 0) finish(i, u, b, cmin, cmax);
+    }
     for (int l = 0; l < nl; ++l) {
         const int64_t i = base + longs[l];
         const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
+        if (a1 - a0 <= HUB_ENTRIES) continue;
+        __syncthreads();
         if (threadIdx.x < 2) range[threadIdx.x] = threadIdx.x == 0 ? INT32_MAX : -1;
         const int64_t u = block_reduce_sum<BOUND_NT>(sum_of(a0 + threadIdx.x, a1, BOUND_NT), scratch);
         const int b = bin_of(u);
@@ -263,14 +289,24 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int64_t nblk) {
             __syncthreads();
         }
         if (threadIdx.x == 0) finish(i, u, b, range[0], range[1]);
-        __syncthreads();
     }
-    if (threadIdx.x < NUM_BINS) O.hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = hist[threadIdx.x];
+    __syncthreads();
     capsum = block_reduce_sum<BOUND_NT>(capsum, scratch);
     usum = block_reduce_sum<BOUND_NT>(usum, scratch);
-    if (threadIdx.x == 0) {
-        O.part[blockIdx.x] = capsum;
-        O.part[nblk + blockIdx.x] = usum;
+    const int64_t blk = blockIdx.x / factor;
+    if (factor == 1) {
+        if (threadIdx.x < NUM_BINS) O.hist[(int64_t)threadIdx.x * nblk + blk] = hist[threadIdx.x];
+        if (threadIdx.x == 0) {
+            O.part[blk] = capsum;
+            O.part[nblk + blk] = usum;
+        }
+    } else {
+        if (threadIdx.x < NUM_BINS && hist[threadIdx.x] != 0)
+            atomicAdd(&O.hist[(int64_t)threadIdx.x * nblk + blk], hist[threadIdx.x]);
+        if (threadIdx.x == 0) {
+            atomicAdd((unsigned long long *)&O.part[blk], (unsigned long long)capsum);
+            atomicAdd((unsigned long long *)&O.part[nblk + blk], (unsigned long long)usum);
+        }
     }
 }
 
@@ -399,9 +435,15 @@ cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, c
     const int64_t nblk = bin_blocks(A.nrows, A.nnz);
     if (P.dense != nullptr && O.div < 1) return cudaErrorInvalidValue;
     if (nblk <= 0) return cudaMemsetAsync(O.err, 0, sizeof(int64_t), st);
-    const int R = (int)bin_rows_per_block(A.nrows, A.nnz);
+    const int64_t rows = BOUND_NT / bound_group(A.nrows, A.nnz);
+    const int factor = (int)(bin_rows_per_block(A.nrows, A.nnz) / rows);
+    if (factor > 1) {
+        cudaError_t e = cudaMemsetAsync(O.hist, 0, sizeof(int32_t) * NUM_BINS * nblk, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(O.part, 0, sizeof(int64_t) * 2 * nblk, st);
+        if (e != cudaSuccess) return e;
+    }
     auto go = [&](auto kern) {
-        kern<<<(unsigned)nblk, BOUND_NT, 0, st>>>(A, B, P, O, R, nblk);
+        kern<<<(unsigned)((A.nrows + rows - 1) / rows), BOUND_NT, 0, st>>>(A, B, P, O, factor, nblk);
         return cudaGetLastError();
     };
     switch (bound_group(A.nrows, A.nnz)) {
