@@ -26,6 +26,7 @@
 #include "common.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace spg {
 
@@ -145,6 +146,7 @@ cudaError_t launch_dense_select(const int32_t *bin_rows, int64_t m, BinSummary *
 // passes with a barrier per part for the long parts, held the 2^16-row R-MAT to a quarter of
 // the rate of the shared-memory atomics.)
 constexpr int DENSE_UN = 4;  // groups of 32 products in flight per warp
+constexpr int DENSE_STAGE = 256;  // columns of 32 words (of 1,024) that a warp stages before it writes them to C
 
 template <int NT>
 struct DenseWin {
@@ -194,9 +196,10 @@ SPG_DEV int dense_window(const DevCSR &A, const DevCSR &B, const DenseArgs &D, i
     return (int)(tot & 0xffffffff);
 }
 
-// f(p, a, ok): DENSE_UN entry positions p[] of B, the a_ik that multiply them (VALS) and which
-// are valid, called by whole warps.  Each access of a warp reads consecutive entries of few
-// B rows.
+// f(p, a, ok, full): DENSE_UN entry positions p[] of B, the a_ik that multiply them (VALS) and
+// which are valid, called by whole warps.  Each access of a warp reads consecutive entries of few
+// B rows.  Where the DENSE_UN groups lie inside one part (full = true_type: consecutive entries,
+// all valid, one a_ik), nothing is looked up at all: 4 instructions a group instead of 16.
 template <int NT, bool VALS, typename F>
 SPG_DEV void dense_walk(const DenseWin<NT> &w, int T, F f) {
     constexpr int NW = NT / 32, ST = NT / 32;
@@ -204,18 +207,31 @@ SPG_DEV void dense_walk(const DenseWin<NT> &w, int T, F f) {
     const int64_t G = (T + 31) >> 5;
     const int g0 = (int)(G * wid / NW), g1 = (int)(G * (wid + 1) / NW);
     if (g0 >= g1) return;
+    const int end = min(T, g1 << 5);
     // the part of product 32 g0: among every ST-th start, then among the ST after it
     const int c = __popc(__ballot_sync(SPG_FULL, w.start[lane * ST] <= (g0 << 5))) - 1;
     int t = c * ST - 1 + __popc(__ballot_sync(SPG_FULL, lane < ST && w.start[c * ST + (lane < ST ? lane : 0)] <= (g0 << 5)));
     const unsigned le = (2u << lane) - 1u;  // the lanes up to this one
-    for (int g = g0; g < g1; g += DENSE_UN) {
+    for (int q0 = g0 << 5; q0 < end; q0 += 32 * DENSE_UN) {
         int64_t p[DENSE_UN];
         val_t a[DENSE_UN];
         bool ok[DENSE_UN];
+        if (min(w.start[t + 1], end) - q0 >= 32 * DENSE_UN) {
+#pragma unroll
+            for (int u = 0; u < DENSE_UN; ++u) {
+                p[u] = w.base[t] + (q0 + lane) + 32 * u;
+                if (VALS) a[u] = w.av[t];
+                ok[u] = true;
+            }
+            f(p, a, ok, std::true_type());
+            // the next products may begin a part
+            if (w.start[t + 1] == q0 + 32 * DENSE_UN) ++t;
+            continue;
+        }
 #pragma unroll
         for (int u = 0; u < DENSE_UN; ++u) {
-            const int q = (g + u) << 5;
-            const bool on = g + u < g1;
+            const int q = q0 + 32 * u;
+            const bool on = q < end;
             const unsigned d = (unsigned)(w.start[t + 1 + lane] - q);
             const unsigned m = __reduce_or_sync(SPG_FULL, (on && d < 32u) ? 1u << d : 0u);
             const int pt = t + __popc(m & le);
@@ -224,7 +240,7 @@ SPG_DEV void dense_walk(const DenseWin<NT> &w, int T, F f) {
             if (VALS) a[u] = w.av[pt];
             t += __popc(m);
         }
-        f(p, a, ok);
+        f(p, a, ok, std::false_type());
     }
 }
 
@@ -267,14 +283,14 @@ SPG_DEV bool dense_mark_columns(const DevCSR &A, const DevCSR &B, const DenseArg
     const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
     for (int64_t e = a0; e < a1; e += NT) {
         const int T = dense_window<NT, false>(A, B, D, s, e, a1, win);
-        dense_walk<NT, false>(win, T, [&](const int64_t *p, const val_t *, const bool *ok) {
+        dense_walk<NT, false>(win, T, [&](const int64_t *p, const val_t *, const bool *ok, auto full) {
             int32_t c[DENSE_UN];
 #pragma unroll
             for (int u = 0; u < DENSE_UN; ++u)
-                if (ok[u]) c[u] = __ldg(B.col + p[u]);
+                if (full || ok[u]) c[u] = __ldg(B.col + p[u]);
 #pragma unroll
             for (int u = 0; u < DENSE_UN; ++u) {
-                if (!ok[u]) continue;
+                if (!full && !ok[u]) continue;
                 const int x = (int)(c[u] - lo);
                 if ((unsigned)x < (unsigned)span) mark(x);
                 else bad = true;
@@ -353,8 +369,8 @@ __global__ void k_dense_rows(MergeItems it, DenseArgs D) {
 // columns, i.e. its place in the row of C, so one 8-byte shared load leads from a column to
 // its sum.  The columns are written and the sums cleared first, straight in C; in double
 // precision every product is then added in C itself (an atomic add performed in L2, which
-// holds the slice just cleared): no buffer of sums, so a CTA needs 32 KB for the widest slice,
-// five CTAs share an SM and any number of entries takes one pass.  Measured over the chip
+// holds the slice just cleared): no buffer of sums, so a CTA needs 42 KB for the widest slice,
+// four CTAs of 256 threads share an SM and any number of entries takes one pass.  Measured over the chip
 // with random addresses: 214-280 G adds/s in L2 against 288-372 G/s for fp64 atomics in shared
 // memory, which would leave one or two CTAs per SM.  In single precision the sums are kept in
 // shared memory (SHV: 786-1,171 G adds/s, and global float atomics flush denormals), one per
@@ -363,9 +379,9 @@ __global__ void k_dense_rows(MergeItems it, DenseArgs D) {
 __host__ __device__ inline int dense_nw4(int W) { return ((W + 31) / 32 + 4) & ~3; }
 
 // Turns the words of a slice's bitmap into the index: the groups of four words from src(g)
-// are counted, ranked and written as pairs.  Returns the number of set bits; put(g, bits,
-// rank) is called for every group by the thread that ranked it, after `enter(total)` was
-// true (else the caller must return).  The index is complete after the caller's next barrier.
+// are counted, ranked and written as pairs.  Unless enter(number of set bits) is false (the
+// caller must then return), put(w) is called by whole warps for every 32 words from w on, once
+// their pairs are written.  The index is complete after the caller's next barrier.
 template <int NT, typename S, typename E, typename P>
 SPG_DEV bool dense_index(uint2 *idx, int nwords, int32_t *scan32, S src, E enter, P put) {
     constexpr int NW = NT / 32, RG = (DENSE_W_MAX / 128 + NT - 1) / NT;
@@ -403,8 +419,9 @@ SPG_DEV bool dense_index(uint2 *idx, int nwords, int32_t *scan32, S src, E enter
             uint4 *o4 = reinterpret_cast<uint4 *>(idx + 4 * g);
             o4[0] = make_uint4(b[i].x, (unsigned)ex, b[i].y, (unsigned)(ex + c0));
             o4[1] = make_uint4(b[i].z, (unsigned)(ex + c1), b[i].w, (unsigned)(ex + c2));
-            put(g, b[i], ex);
         }
+        __syncwarp();
+        for (int w = 4 * (g - lane); w < nwords && w < 4 * (g - lane) + 128; w += 32) put(w);
     }
     return true;
 }
@@ -413,12 +430,12 @@ SPG_DEV bool dense_index(uint2 *idx, int nwords, int32_t *scan32, S src, E enter
 // from the slice's known entries of C and only the values are written.
 template <int NT, bool REPLAY, bool SHV>
 SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t b, const int64_t *c_rp,
-                             int32_t *c_col, val_t *c_val, int64_t *err, int vcap, int cmin, int cmax) {
+                             int32_t *c_col, val_t *c_val, int64_t *err, int vcap) {
     extern __shared__ __align__(16) unsigned char df_smem[];
     __shared__ DenseWin<NT> win;
     __shared__ int32_t scan32[NT / 32 + 1];
-    const int expected = D.cnt[b];
-    if (expected <= cmin || expected > cmax) return;  // empty, or another launch's item
+    __shared__ uint16_t stage[NT / 32][DENSE_STAGE];
+    const int expected = D.cnt[b];  // > 0
     const int64_t d = b / D.K;
     const int s = (int)(b - d * D.K);
     const int row = D.rows[d];
@@ -458,20 +475,30 @@ SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &
             return make_uint4(p.x, p.z, q.x, q.z);
         },
         [&](int tot) { return tot == expected; },
-        [&](int g, const uint4 &w, int r) {
+        [&](int w) {
+            // C's columns of 32 words, a word per lane
             if (REPLAY) return;
-            const uint32_t wd[4] = {w.x, w.y, w.z, w.w};
-            int64_t q = o + r;
-            int32_t base = (int32_t)(lo + ((int64_t)g << 7));
-#pragma unroll
-            for (int k = 0; k < 4; ++k, base += 32) {
-                uint32_t bits = wd[k];
-                if (!SPG_IN(q + __popc(bits) <= o + expected, 110)) return;  // the slice's entries of C
-                while (bits) {
-                    const int t = __ffs(bits) - 1;
-                    bits &= bits - 1u;
-                    c_col[q++] = base + t;
-                }
+            const int lane = lane_id();
+            const uint2 wd = w + lane < nwords ? idx[w + lane] : make_uint2(0u, 0u);
+            uint32_t bits = wd.x;
+            const unsigned some = __ballot_sync(SPG_FULL, bits != 0u);
+            if (some == 0u) return;
+            const int last = 31 - __clz(some);
+            const int r0 = __shfl_sync(SPG_FULL, (int)wd.y, __ffs(some) - 1);
+            const int n = __shfl_sync(SPG_FULL, (int)wd.y + __popc(bits), last) - r0;
+            if (!SPG_IN(r0 + n <= expected, 110)) return;  // the slice's entries of C
+            const int32_t base = (int32_t)(lo + ((int64_t)w << 5));
+            if (n <= DENSE_STAGE) {
+                // few columns per word: staged, so that the warp's stores are contiguous (lane by
+                // lane every store would touch a sector of its own)
+                uint16_t *sg = stage[warp_id()];
+                for (int q = (int)wd.y - r0; bits; bits &= bits - 1u) sg[q++] = (uint16_t)((lane << 5) + __ffs(bits) - 1);
+                __syncwarp();
+                for (int t = lane; t < n; t += 32) c_col[o + r0 + t] = base + sg[t];
+                __syncwarp();
+            } else {
+                int64_t q = o + (int)wd.y;
+                for (; bits; bits &= bits - 1u) c_col[q++] = base + (lane << 5) + __ffs(bits) - 1;
             }
         });
     if (!match) {  // the counting pass saw other columns: cannot happen
@@ -503,18 +530,18 @@ SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &
         const int x0 = w0 << 5, x1 = min(span, w1 << 5);
         for (int64_t e = a0; e < a1; e += NT) {
             const int T = dense_window<NT, true>(A, B, D, s, e, a1, win);
-            dense_walk<NT, true>(win, T, [&](const int64_t *p, const val_t *a, const bool *ok) {
+            dense_walk<NT, true>(win, T, [&](const int64_t *p, const val_t *a, const bool *ok, auto full) {
                 int32_t c[DENSE_UN];
                 val_t v[DENSE_UN];
 #pragma unroll
                 for (int u = 0; u < DENSE_UN; ++u)
-                    if (ok[u]) c[u] = __ldg(B.col + p[u]);
+                    if (full || ok[u]) c[u] = __ldg(B.col + p[u]);
 #pragma unroll
                 for (int u = 0; u < DENSE_UN; ++u)
-                    if (ok[u]) v[u] = __ldg(B.val + p[u]);
+                    if (full || ok[u]) v[u] = __ldg(B.val + p[u]);
 #pragma unroll
                 for (int u = 0; u < DENSE_UN; ++u) {
-                    if (!ok[u]) continue;
+                    if (!full && !ok[u]) continue;
                     const int x = (int)(c[u] - lo);
                     if (SHV && (x < x0 || x >= x1)) continue;  // another piece's
                     const bool in = (unsigned)x < (unsigned)span;
@@ -540,30 +567,56 @@ SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicExch((unsigned long long *)err, 6ull);
 }
 
-// A persistent grid that takes the items whose count lies in (cmin, cmax] from a work counter.
+// Ticket t of a grid of `ctas`: the first item of its run and the run's length.  The first four
+// tickets per CTA are single items (the list begins with the heaviest rows), the next four are
+// pairs, and so on up to runs of 32.
+SPG_DEV int64_t dense_run(int64_t t, int64_t ctas, int &len) {
+    const int64_t c = 4 * ctas;
+    const int64_t l = min(t / c, (int64_t)5);
+    len = 1 << l;
+    return c * (len - 1) + (t - l * c) * len;
+}
+
+// A persistent grid over the items whose count lies in (cmin, cmax].  A CTA takes a run of
+// consecutive items from the work counter, looks at all their counts at once and fills the
+// ones that are its own.
 template <int NT, int MINB, bool REPLAY, bool SHV>
 __global__ void __launch_bounds__(NT, MINB)
 k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_col, val_t *c_val, int64_t *err,
              const int64_t *gate, int vcap, unsigned long long *counter, int cmin, int cmax) {
-    __shared__ int64_t s_b, s_nx;
+    __shared__ int64_t s_base;
+    __shared__ unsigned s_mask;
     if (gated(gate)) return;
     const int64_t nb = dense_items(D);
-    int64_t b = dense_next(counter, 0, true, &s_b);
-    while (b < nb) {
-        // the CTA's next item is taken one item ahead, so that its kept bitmap (written by the
-        // counting pass, long out of L2) is on its way into L2 while this item is filled
-        if (threadIdx.x == 0) {
-            const int64_t nx = (int64_t)atomicAdd(counter, 1ull);
-            s_nx = nx;
-            if (!REPLAY && D.keep != nullptr && nx < nb) {
-                const int c = D.cnt[nx];
-                if (c > cmin && c <= cmax) prefetch_l2(D.keep + nx * (int64_t)D.keep_words, 4u * (uint32_t)D.keep_words);
+    while (true) {
+        if (threadIdx.x < 32) {
+            int64_t t = 0;
+            if (threadIdx.x == 0) t = (int64_t)atomicAdd(counter, 1ull);
+            int run;
+            const int64_t base = dense_run(__shfl_sync(SPG_FULL, t, 0), gridDim.x, run);
+            const int64_t i = base + threadIdx.x;
+            const int c = ((int)threadIdx.x < run && i < nb) ? D.cnt[i] : 0;
+            const unsigned m = __ballot_sync(SPG_FULL, c > cmin && c <= cmax);
+            if (threadIdx.x == 0) {
+                s_base = base;
+                s_mask = m;
             }
         }
-        dense_fill_item<NT, REPLAY, SHV>(A, B, D, b, c_rp, c_col, c_val, err, vcap, cmin, cmax);
-        __syncthreads();  // s_nx is visible and the item's shared memory is free
-        b = s_nx;
-        __syncthreads();  // every thread has read s_nx before thread 0 overwrites it
+        __syncthreads();
+        const int64_t base = s_base;
+        unsigned mask = s_mask;
+        if (base >= nb) return;
+        while (mask) {
+            const int64_t b = base + __ffs(mask) - 1;
+            mask &= mask - 1u;
+            // the next item's kept bitmap (written by the counting pass, long out of L2) is on its
+            // way into L2 while this item is filled
+            if (threadIdx.x == 0 && !REPLAY && D.keep != nullptr && mask)
+                prefetch_l2(D.keep + (base + __ffs(mask) - 1) * (int64_t)D.keep_words, 4u * (uint32_t)D.keep_words);
+            dense_fill_item<NT, REPLAY, SHV>(A, B, D, b, c_rp, c_col, c_val, err, vcap);
+            __syncthreads();  // the item's shared memory is free
+        }
+        __syncthreads();  // every thread has read the run before the next one
     }
 }
 
@@ -805,6 +858,7 @@ __global__ void k_dense_rowsum(DenseArgs D, int32_t *nnzc) {
 }
 
 constexpr int DENSE_NT = 256;
+constexpr int DENSE_FEW = 4096;  // entries of a (row, slice) filled by the smaller CTAs in double
 
 int dense_keep_words(int W) { return dense_nw4(W); }  // a multiple of 4: every item's bitmap starts on a 16-byte boundary
 
@@ -871,13 +925,21 @@ cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs 
     };
     const int index = (int)(sizeof(uint2) * (size_t)dense_nw4(D.W));
     if constexpr (sizeof(val_t) == 8) {
-        return replay ? go(k_dense_fill<DENSE_NT, 5, true, false>, DENSE_NT, index, 0, D.queue + 1, 0, INT32_MAX)
-                      : go(k_dense_fill<DENSE_NT, 5, false, false>, DENSE_NT, index, 0, D.queue + 1, 0, INT32_MAX);
+        // few entries: four CTAs of 256 threads per SM.  Many: two of 512, half as many rows of C
+        // in flight, since their sums must stay in L2 while they are added to (16 k entries per
+        // row, R-MAT 2^16 x 16: 1.62 ms at 304 CTAs, 2.34 at 608, 2.90 at 760; 3.2 k entries, 2^18 x
+        // 8: 10.2 ms at 304, 8.8 at 608)
+        e = replay ? go(k_dense_fill<256, 4, true, false>, 256, index, 0, D.queue + 1, 0, DENSE_FEW)
+                   : go(k_dense_fill<256, 4, false, false>, 256, index, 0, D.queue + 1, 0, DENSE_FEW);
+        if (e != cudaSuccess || D.W <= DENSE_FEW) return e;  // a slice has at most W entries
+        return replay ? go(k_dense_fill<512, 2, true, false>, 512, index, 0, D.queue + 2, DENSE_FEW, INT32_MAX)
+                      : go(k_dense_fill<512, 2, false, false>, 512, index, 0, D.queue + 2, DENSE_FEW, INT32_MAX);
     } else {
         // sums in shared memory: the items whose entries fit a quarter of an SM's shared memory at
         // four CTAs of 256 threads per SM, those that fit a half at two of 512, the rest at one of 1,024
         auto room = [&](int per_sm, int nt) {  // sums that fit beside the index
-            const int fixed = 1024 + 512 + nt * (int)(sizeof(int64_t) + sizeof(val_t) + sizeof(int32_t)) + nt / 4;
+            const int fixed = 1024 + 512 + nt * (int)(sizeof(int64_t) + sizeof(val_t) + sizeof(int32_t)) + nt / 4 +
+                          nt / 32 * DENSE_STAGE * (int)sizeof(uint16_t);
             return (std::min(227 * 1024, 228 * 1024 / per_sm) - fixed - index) / (int)sizeof(val_t) & ~31;
         };
         const int v4 = room(4, 256), v2 = room(2, 512), v1 = room(1, 1024);
