@@ -20,35 +20,51 @@ using namespace spg;
 
 namespace {
 
+// Two pools per device: what a plan keeps (results and the O(rows) tables) and its temporaries.
+// A large block carved out of freed memory of other sizes makes the pool map it anew, which
+// holds up the host for 0.7 ms per GB: in one pool, C of R-MAT 2^20 x 8 (43 GB) was placed over the
+// slice bitmaps and temporary rows of the call before it (21 GB) and the other way round, 30 ms a
+// product.  Apart, a repeated product finds its own blocks again.
 struct DevicePool {
     int device;
-    cudaMemPool_t pool;
+    cudaMemPool_t kept, temp;
 };
 
 std::mutex g_pool_mu;
 std::vector<DevicePool> g_pools;
 
-cudaError_t get_pool(int device, cudaMemPool_t *out) {
-    std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (auto &p : g_pools)
-        if (p.device == device) {
-            *out = p.pool;
-            return cudaSuccess;
-        }
+cudaError_t make_pool(int device, cudaMemPool_t *out) {
     cudaMemPoolProps props;
     std::memset(&props, 0, sizeof(props));
     props.allocType = cudaMemAllocationTypePinned;
     props.handleTypes = cudaMemHandleTypeNone;
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = device;
-    cudaMemPool_t pool;
-    cudaError_t e = cudaMemPoolCreate(&pool, &props);
+    cudaError_t e = cudaMemPoolCreate(out, &props);
     if (e != cudaSuccess) return e;
     uint64_t thr = UINT64_MAX;  // keep freed blocks for reuse by later calls
-    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+    e = cudaMemPoolSetAttribute(*out, cudaMemPoolAttrReleaseThreshold, &thr);
+    if (e != cudaSuccess) cudaMemPoolDestroy(*out);
+    return e;
+}
+
+cudaError_t get_pools(int device, DevicePool *out) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (auto &p : g_pools)
+        if (p.device == device) {
+            *out = p;
+            return cudaSuccess;
+        }
+    DevicePool p{device, nullptr, nullptr};
+    cudaError_t e = make_pool(device, &p.kept);
     if (e != cudaSuccess) return e;
-    g_pools.push_back({device, pool});
-    *out = pool;
+    e = make_pool(device, &p.temp);
+    if (e != cudaSuccess) {
+        cudaMemPoolDestroy(p.kept);
+        return e;
+    }
+    g_pools.push_back(p);
+    *out = p;
     return cudaSuccess;
 }
 
@@ -164,17 +180,19 @@ struct spgemm_plan {
     int device = 0;
     cudaStream_t st = nullptr;
     spgemm_opts opts{};
-    cudaMemPool_t pool = nullptr;
+    DevicePool pools{};
     DevCSR A{}, B{};
-    std::vector<void *> allocs;
-    // temporaries: freed when the stage that needs them is over (symbolic: stage-1
-    // prefix and binning scratch; numeric: C~, merge pools and lists)
-    struct Temp {
-        void *ptr;
-        int64_t bytes;
-        int life;
+    // Device memory by lifetime (symbolic: stage-1 and binning scratch; numeric: C~, merge pools
+    // and lists; plan: the rest).  Small arrays share blocks of CHUNK bytes: a product on a few
+    // thousand rows makes 5 allocations instead of 21, which had taken a sixth of its time.
+    struct Memory {
+        std::vector<void *> blocks;
+        int64_t bytes = 0;        // requested
+        char *open = nullptr;     // rest of the last shared block
+        size_t room = 0;
     };
-    std::vector<Temp> temps;
+    Memory mem[3];
+    static constexpr size_t CHUNK = 512 * 1024, SMALL = 64 * 1024;
     int64_t bytes_ctilde = 0;
     int64_t bytes_held = 0;  // device bytes the plan holds now
     int64_t bytes_peak = 0;  // largest bytes_held so far
@@ -261,8 +279,48 @@ struct spgemm_plan {
             *p = nullptr;
             return cudaErrorMemoryAllocation;
         }
+        Memory &m = mem[life];
+        const size_t need = (bytes + 255) & ~size_t(255);
+        cudaError_t e = cudaSuccess;
+        if (need > SMALL) {
+            e = alloc_block(p, bytes, life);
+        } else {
+            if (m.room < need) {
+                void *q = nullptr;
+                e = alloc_block(&q, CHUNK, life);
+                if (e == cudaSuccess) {
+                    m.open = static_cast<char *>(q);
+                    m.room = CHUNK;
+                }
+            }
+            if (e == cudaSuccess) {
+                *p = m.open;
+                m.open += need;
+                m.room -= need;
+            }
+        }
+        if (e != cudaSuccess) {
+            *p = nullptr;
+            return e;
+        }
+        m.bytes += (int64_t)bytes;
+        bytes_held += (int64_t)bytes;
+        bytes_peak = std::max(bytes_peak, bytes_held);
+        return cudaSuccess;
+    }
+    cudaError_t alloc_block(void **p, size_t bytes, int life) {
         const auto t0 = std::chrono::steady_clock::now();
+        const cudaMemPool_t pool = life == LIFE_PLAN ? pools.kept : pools.temp;
         cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+        if (e == cudaErrorMemoryAllocation) {
+            // the other pool may hold unused memory: give both pools' back and try once more
+            cudaGetLastError();
+            if (cudaStreamSynchronize(st) == cudaSuccess) {
+                cudaMemPoolTrimTo(pools.kept, 0);
+                cudaMemPoolTrimTo(pools.temp, 0);
+                e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+            }
+        }
         stats.alloc_host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         stats.allocs += 1;
         if (e != cudaSuccess) {
@@ -270,28 +328,31 @@ struct spgemm_plan {
             cudaGetLastError();
             return e;
         }
-        if (life == LIFE_PLAN) allocs.push_back(*p);
-        else temps.push_back(Temp{*p, (int64_t)bytes, life});
-        bytes_held += (int64_t)bytes;
-        bytes_peak = std::max(bytes_peak, bytes_held);
+        mem[life].blocks.push_back(*p);
         return cudaSuccess;
     }
     template <typename T>
     cudaError_t alloc_n(T **p, int64_t n, int life = LIFE_PLAN) {
         return alloc(reinterpret_cast<void **>(p), sizeof(T) * (size_t)std::max<int64_t>(n, 1), life);
     }
+    // columns and values of n entries in one block: results of the same size find each other's
+    // memory again
+    cudaError_t alloc_entries(int32_t **col, val_t **val, int64_t n, int life) {
+        const int64_t vb = (sizeof(val_t) * std::max<int64_t>(n, 1) + 255) & ~int64_t(255);
+        void *q = nullptr;
+        cudaError_t e = alloc(&q, (size_t)vb + sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1), life);
+        *val = static_cast<val_t *>(q);
+        *col = q ? reinterpret_cast<int32_t *>(static_cast<char *>(q) + vb) : nullptr;
+        return e;
+    }
+    void free_memory(Memory &m) {
+        for (void *q : m.blocks) cudaFreeAsync(q, st);
+        bytes_held -= m.bytes;
+        m = Memory{};
+    }
     // Frees (stream-ordered) every temporary whose life ends at or before `life`.
     void release_temps(int life) {
-        size_t k = 0;
-        for (auto &t : temps) {
-            if (t.life <= life) {
-                cudaFreeAsync(t.ptr, st);
-                bytes_held -= t.bytes;
-            } else {
-                temps[k++] = t;
-            }
-        }
-        temps.resize(k);
+        for (int l = 0; l <= life && l < LIFE_PLAN; ++l) free_memory(mem[l]);
     }
     void time_begin(int kind) {
         if (!opts.record_timing) return;
@@ -357,10 +418,7 @@ struct spgemm_plan {
             if (t.b) cudaEventDestroy(t.b);
         }
         timers.clear();
-        for (void *p : allocs) cudaFreeAsync(p, st);
-        allocs.clear();
-        for (auto &t : temps) cudaFreeAsync(t.ptr, st);
-        temps.clear();
+        for (Memory &m : mem) free_memory(m);
         bytes_held = 0;
         put_pinned(pinned);
         pinned = nullptr;
@@ -539,7 +597,7 @@ static spgemm_status plan_begin(const spgemm_opts *opts, spgemm_stream_t stream,
     spgemm_status status = SPGEMM_OK;
     {
         SPG_TRY(cudaGetDevice(&p->device));
-        SPG_TRY(get_pool(p->device, &p->pool));
+        SPG_TRY(get_pools(p->device, &p->pools));
         SPG_TRY(cudaDeviceGetAttribute(&p->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
         p->pinned = get_pinned();
         if (!p->pinned) {
@@ -714,8 +772,7 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
             SPG_TRY(p->alloc_n(&p->d_queue, DENSE_QUEUES));  // work counters of the fill launches
         }
         // C~ (hybrid: u_i for bins 0..36, 256 for bin 37)
-        SPG_TRY(p->alloc_n(&p->ctil_col, p->h_summary.sum_cap, LIFE_NUMERIC));
-        SPG_TRY(p->alloc_n(&p->ctil_val, p->h_summary.sum_cap, LIFE_NUMERIC));
+        SPG_TRY(p->alloc_entries(&p->ctil_col, &p->ctil_val, p->h_summary.sum_cap, LIFE_NUMERIC));
         p->bytes_ctilde += p->h_summary.sum_cap * ENTRY_BYTES;
         p->release_temps(LIFE_SYMBOLIC);
         p->dense_flag = nullptr;
@@ -989,10 +1046,14 @@ static void alloc_dense_keep(spgemm_plan *p) {
         return;
     const int64_t words = p->dense_wide * p->dense_K * (int64_t)kw;
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    uint64_t reserved = 0, used = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+        cudaMemPoolGetAttribute(p->pools.temp, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+        cudaMemPoolGetAttribute(p->pools.temp, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
+    free_b += (size_t)(reserved - std::min(used, reserved));  // the pool's unused memory is free to the plan
     if ((uint64_t)words * sizeof(uint32_t) > free_b / 4) return;
     if (p->alloc_n(&p->dense_keep, words, LIFE_NUMERIC) != cudaSuccess) {
         p->dense_keep = nullptr;
@@ -1247,8 +1308,7 @@ extern "C" spgemm_status spgemm_numeric(spgemm_plan *p, spgemm_csr_out *C_out) {
             status = SPGEMM_ERR_INTERNAL;
             goto fail;
         }
-        SPG_TRY(p->alloc_n(&p->C.col_idx, nnzC));
-        SPG_TRY(p->alloc_n(&p->C.val, nnzC));
+        SPG_TRY(p->alloc_entries(&p->C.col_idx, &p->C.val, nnzC, LIFE_PLAN));
         cudaEvent_t fill_done = nullptr;
         if (p->dense_n > 0) {
             // the dense-slice rows write their values straight into C, beside the copy of
@@ -1362,14 +1422,15 @@ extern "C" spgemm_status spgemm_check_status(int64_t *code_out, int32_t reset) {
 
 extern "C" spgemm_status spgemm_pool_trim(int32_t device, int64_t keep_bytes) {
     if (device < 0 || keep_bytes < 0) return SPGEMM_ERR_INVALID_ARG;
-    cudaMemPool_t pool = nullptr;
+    DevicePool pools{};
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
         for (auto &q : g_pools)
-            if (q.device == device) pool = q.pool;
+            if (q.device == device) pools = q;
     }
-    if (pool == nullptr) return SPGEMM_OK;
-    return from_cuda(cudaMemPoolTrimTo(pool, (size_t)keep_bytes));
+    if (pools.kept == nullptr) return SPGEMM_OK;
+    const cudaError_t e = cudaMemPoolTrimTo(pools.temp, 0);
+    return from_cuda(e != cudaSuccess ? e : cudaMemPoolTrimTo(pools.kept, (size_t)keep_bytes));
 }
 
 extern "C" spgemm_status spgemm_free(spgemm_plan *p) {
@@ -1978,8 +2039,7 @@ static spgemm_status run_precise(spgemm_plan *p, spgemm_csr_out *C_out) {
             status = SPGEMM_ERR_INTERNAL;
             goto fail;
         }
-        SPG_TRY(p->alloc_n(&p->C.col_idx, nnzC));
-        SPG_TRY(p->alloc_n(&p->C.val, nnzC));
+        SPG_TRY(p->alloc_entries(&p->C.col_idx, &p->C.val, nnzC, LIFE_PLAN));
         SPG_TRY(precise_fill(p, false, nullptr));
         p->C.nrows = m;
         p->C.ncols = p->B.ncols;
