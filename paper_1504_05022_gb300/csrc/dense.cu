@@ -912,11 +912,12 @@ cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs 
                    : launch_narrow_rows<true, false>(A, B, D, c_rp, c_col, c_val, err, gate, st);
     const int64_t nb = (D.dev_end != nullptr ? D.n : D.n_wide) * D.K;
     if (e != cudaSuccess || nb <= 0) return e;
+    e = cudaMemsetAsync(D.queue + 1, 0, sizeof(unsigned long long) * (DENSE_QUEUES - 1), st);
+    if (e != cudaSuccess) return e;
     // a persistent grid of nt threads per CTA over the items with counts in (cmin, cmax]
     auto go = [&](auto kern, int nt, int smem, int vcap, unsigned long long *q, int cmin, int cmax) -> cudaError_t {
         cudaError_t x = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (x == cudaSuccess) x = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (x == cudaSuccess) x = cudaMemsetAsync(q, 0, sizeof(unsigned long long), st);
         if (x != cudaSuccess) return x;
         const int grid = persistent_blocks((const void *)kern, nt, smem, nb);
         if (grid <= 0) return cudaErrorInvalidValue;

@@ -59,6 +59,15 @@ struct EscSmem {
     int32_t start[2 * G];   // first product of the part; INT_MAX past the last part
 };
 
+// The groups of a warp lie 4 G bytes apart modulo the 128 bytes of the banks, so that their
+// accesses do not meet in the same banks.
+template <int G, int E, typename K, bool COUNT>
+struct EscGroup : EscSmem<G, E, K, COUNT> {
+    static constexpr int RAW = (int)sizeof(EscSmem<G, E, K, COUNT>);
+    static constexpr int GAP = ((4 * G - RAW) % 128 + 128) % 128;
+    unsigned char gap[GAP == 0 ? 128 : GAP];
+};
+
 // COUNT: the counting pass of the precise method (Section 3.1): the same expansion and sort
 // on the columns alone, and nnz(c_i) = the number of distinct columns, written to a.nnzc.
 // The groups stride over the rows (one pass when the grid covers them).
@@ -71,7 +80,7 @@ k_esc(StageArgs a, RowSet R) {
     static_assert(N <= 512 && (COUNT || sizeof(K) == 8 || (1 << LB) == N), "N is a power of two");
     constexpr K PAD = ~K(0);
     constexpr int U = E < 4 ? E : 4;  // groups of G products in flight
-    using Smem = EscSmem<G, E, K, COUNT>;
+    using Smem = EscGroup<G, E, K, COUNT>;
     __shared__ Smem smem[GROUPS];
     if (!COUNT && gated(a.gate)) return;
     const int32_t *rows;

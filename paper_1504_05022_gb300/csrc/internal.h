@@ -41,7 +41,7 @@ struct BinSummary {
     int64_t sum_cap;   // nnz(C~) of the initial allocation
     int64_t sum_u;     // sum u_i
     int64_t status;    // validation result (0 = ok)
-    int64_t pad;
+    int64_t merge_batched;  // bin-37 rows, not flagged dense by stage 1, that k_merge_small cannot take
     int64_t class_count[NUM_LAUNCH_CLASSES];  // learned: bin-37 rows per launch class
     int64_t dense_count;                      // bin-37 rows computed by the dense-slice kernels
     int64_t dense_end[2];                     // of these, the first [0] reach more than DENSE_MID_W columns,
@@ -81,7 +81,8 @@ cudaError_t launch_validate(const DevCSR &M, int64_t *status, cudaStream_t st);
 // What stage 1 writes: per row u_i (Algorithm 2), its bin, nnz(c_i) where the bound is exact
 // (bins 0 and 1), and with CapPolicy::dense set the dense-slice flag (the same array) and the
 // column range of the bin-37 rows; per block of rows (bin_blocks(m, nnzA) of them) the bin
-// histogram (NUM_BINS x blocks) and the sums of C~ entries and of u_i (2 x blocks).  *err = 0.
+// histogram (NUM_BINS x blocks) and the sums of C~ entries, of u_i and of the bin-37 rows for the
+// batched merge kernel (3 x blocks).  *err = 0.
 struct BoundOut {
     int64_t *u;
     uint8_t *bin;
@@ -90,6 +91,7 @@ struct BoundOut {
     int32_t *lo, *hi;
     int64_t dmin;  // a bin-37 row is dense when u_i >= dmin (dmin > 0),
     int div;       // else when div u_i >= the width of its column range
+    int small_u;   // as MergeLaunch::small_u
     int32_t *hist;
     int64_t *part;
     int64_t *err;
@@ -191,6 +193,7 @@ struct MergeLaunch {
     int small_u;             // bitmap kernel: fresh rows of at most this many products (and few enough
                              // entries of A) are taken whole by k_merge_small; 0: none.  At most the
                              // largest capacity, so that such a row never has to be split
+    int only_small;          // every item is such a row: the batched kernel is not launched
 };
 constexpr int MERGE_SMALL_U = 8192;  // the most small_u can be
 cudaError_t launch_merge_small(const StageArgs &a, const MergeItems &it, const MergeLaunch &L, cudaStream_t st);

@@ -626,7 +626,7 @@ cudaError_t launch_merge_bm(const StageArgs &a, const MergeItems &s, const Merge
         span < a.B.ncols)
         return cudaErrorInvalidValue;
     const cudaError_t e = launch_merge_small(a, s, L, st);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || L.only_small) return e;
     const int smem = merge_bm_smem_bytes(L.cap, L.bm_words, L.bm_miss, L.wide_above, L.bm_two != 0);
     return L.bm_two ? launch_bm<true>(a, s, L, nt, smem, st) : launch_bm<false>(a, s, L, nt, smem, st);
 }

@@ -209,6 +209,12 @@ struct spgemm_plan {
     int32_t *d_hist = nullptr, *d_select = nullptr;
     int64_t *d_capp = nullptr;
     unsigned long long *d_queue = nullptr;
+    // products sized on the device: streams of the plan's own on which the launches of a phase that
+    // do not depend on each other run side by side (fork / join around them)
+    static constexpr int NUM_BRANCHES = 4;
+    cudaStream_t branch[NUM_BRANCHES] = {nullptr};
+    cudaEvent_t branch_event[NUM_BRANCHES + 1] = {nullptr};
+    int next_branch = -1;  // < 0: everything on st
     BinSummary h_summary{};
     int64_t bin_start[NUM_BINS + 1] = {0};
     // bin 37 work items
@@ -219,6 +225,7 @@ struct spgemm_plan {
     int32_t *class_order = nullptr;   // bin-37 item indices grouped by launch class
     int32_t class_caps[NUM_LAUNCH_CLASSES] = {0};
     int capmax = 0, batch = 0, wide_above = 2048, bm_words = 0, bm_miss = 0, bm_two = 0;
+    int small_u = 0;                  // rows of bin 37 for k_merge_small (MergeLaunch)
     // dense column slices for the longest bin-37 rows (off when dense_K == 0)
     int dense_K = 0, dense_W = 0;
     int64_t dense_min_u = 0;              // > 0: absolute threshold on u_i; 0: the row's column range
@@ -354,6 +361,44 @@ struct spgemm_plan {
     void release_temps(int life) {
         for (int l = 0; l <= life && l < LIFE_PLAN; ++l) free_memory(mem[l]);
     }
+    cudaError_t make_branches() {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < NUM_BRANCHES && e == cudaSuccess; ++i)
+            e = cudaStreamCreateWithFlags(&branch[i], cudaStreamNonBlocking);
+        for (int i = 0; i <= NUM_BRANCHES && e == cudaSuccess; ++i)
+            e = cudaEventCreateWithFlags(&branch_event[i], cudaEventDisableTiming);
+        return e;
+    }
+    void drop_branches() {
+        for (cudaStream_t &b : branch) {
+            if (b) cudaStreamDestroy(b);  // its work is joined to st
+            b = nullptr;
+        }
+        for (cudaEvent_t &e : branch_event) {
+            if (e) cudaEventDestroy(e);
+            e = nullptr;
+        }
+    }
+    // From here on stream() deals the branches out in turn, until join() waits for them on st.
+    cudaError_t fork() {
+        if (branch[0] == nullptr) return cudaSuccess;
+        cudaError_t e = cudaEventRecord(branch_event[NUM_BRANCHES], st);
+        for (int i = 0; i < NUM_BRANCHES && e == cudaSuccess; ++i)
+            e = cudaStreamWaitEvent(branch[i], branch_event[NUM_BRANCHES], 0);
+        next_branch = 0;
+        return e;
+    }
+    cudaStream_t stream() { return next_branch < 0 ? st : branch[next_branch++ % NUM_BRANCHES]; }
+    cudaError_t join() {
+        if (branch[0] == nullptr) return cudaSuccess;
+        next_branch = -1;
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < NUM_BRANCHES && e == cudaSuccess; ++i) {
+            e = cudaEventRecord(branch_event[i], branch[i]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, branch_event[i], 0);
+        }
+        return e;
+    }
     void time_begin(int kind) {
         if (!opts.record_timing) return;
         Timer t{kind, nullptr, nullptr};
@@ -418,6 +463,7 @@ struct spgemm_plan {
             if (t.b) cudaEventDestroy(t.b);
         }
         timers.clear();
+        drop_branches();
         for (Memory &m : mem) free_memory(m);
         bytes_held = 0;
         put_pinned(pinned);
@@ -452,6 +498,7 @@ static void merge_limits(spgemm_plan *p) {
     if (p->opts.smem_cap_max > 0) capmax = std::min(capmax, std::max(256, p->opts.smem_cap_max));
     p->batch = batch;
     p->capmax = capmax;
+    p->small_u = p->bm_words > 0 ? std::min(MERGE_SMALL_U, capmax) : 0;
     // dense column slices: B's columns cut into equal slices of at most DENSE_W_MAX columns
     // (a multiple of 32); a fill CTA holds the slice's bitmap and rank directory and a
     // compact buffer of sums, one per column of the result; dense_span narrows the slices
@@ -568,14 +615,14 @@ cudaError_t launch_short_bins(spgemm_plan *p, const StageArgs &a, bool account, 
         const int lo = r[0], hi = std::min(r[1], hmax);
         if (lo > hi) continue;
         const RowSet R = bin_range(p, lo, hi, dev);
-        if (R.n > 0 && run(SPGEMM_K_HEAP, [&] { return launch_heap_set(a, R, hi, heap_nt, p->st); }) != cudaSuccess)
+        if (R.n > 0 && run(SPGEMM_K_HEAP, [&] { return launch_heap_set(a, R, hi, heap_nt, p->stream()); }) != cudaSuccess)
             return e;
     }
     for (auto &r : kEscRanges) {
         const int lo = std::max(r.lo, hmax + 1), hi = r.hi;
         if (lo > hi) continue;
         const RowSet R = bin_range(p, lo, hi, dev);
-        if (R.n > 0 && run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, r.max_u, false, p->st); }) != cudaSuccess)
+        if (R.n > 0 && run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, r.max_u, false, p->stream()); }) != cudaSuccess)
             return e;
     }
     return cudaSuccess;
@@ -630,6 +677,7 @@ static BoundOut bound_out(const spgemm_plan *p) {
     o.hi = p->dense_hi;
     o.dmin = p->dense_min_u;
     o.div = p->opts.dense_span_div > 0 ? p->opts.dense_span_div : 8;
+    o.small_u = p->small_u;
     o.hist = p->d_hist;
     o.part = p->d_capp;
     o.err = p->d_err;
@@ -681,7 +729,7 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
         SPG_TRY(p->alloc_n(&p->ctil_rp, m + 1));
         {
             SPG_TRY(p->alloc_n(&p->d_hist, (int64_t)NUM_BINS * nblk, LIFE_SYMBOLIC));
-            SPG_TRY(p->alloc_n(&p->d_capp, 2 * nblk, LIFE_SYMBOLIC));
+            SPG_TRY(p->alloc_n(&p->d_capp, 3 * nblk, LIFE_SYMBOLIC));
             pol.policy = o.alloc_policy;
             pol.initial_cap = o.initial_cap;
             pol.pred_cap = nullptr;  // learned: bin-37 sizes are set after the prediction below
@@ -936,7 +984,8 @@ spgemm_status run_progressive(spgemm_plan *p, const int32_t *work_in, int64_t wo
                 L.bm_miss = p->bm_miss;
                 L.bm_two = p->bm_two;
                 L.u = p->u;
-                L.small_u = std::min(MERGE_SMALL_U, p->capmax);
+                L.small_u = p->small_u;
+                L.only_small = p->h_summary.merge_batched == 0;
                 L.work = work;
                 L.work_base = work_base;
                 L.nwork = nwork;
@@ -1110,6 +1159,16 @@ spgemm_status run_bin37(spgemm_plan *p) {
     cudaEvent_t dense_done = p->dense_count_done;
     p->dense_count_done = nullptr;
     {
+        if (p->dense_n == n37) {  // every row by the slice kernels: no work items
+            if (dense_done) {
+                SPG_TRY(cudaStreamWaitEvent(p->st, dense_done, 0));
+                cudaEventDestroy(dense_done);
+                dense_done = nullptr;
+            }
+            SPG_TRY(launch_dense_rowsum(p->dense_args(), p->nnzc, p->st));
+            p->count(SPGEMM_K_MERGE);
+            return SPGEMM_OK;
+        }
         SPG_TRY(reserve_items(p, n37));
         p->n_items = n37;
         SPG_TRY(p->alloc_n(&ovf_count, 1, LIFE_NUMERIC));
@@ -1181,7 +1240,8 @@ spgemm_status run_bin37(spgemm_plan *p) {
                 L.bm_miss = p->bm_miss;
                 L.bm_two = p->bm_two;
                 L.u = p->u;
-                L.small_u = std::min(MERGE_SMALL_U, p->capmax);
+                L.small_u = p->small_u;
+                L.only_small = p->h_summary.merge_batched == 0;
                 L.work = p->class_order + off;
                 L.nwork = cnt;
                 L.cap = ccap;
@@ -1225,7 +1285,8 @@ spgemm_status run_bin37(spgemm_plan *p) {
                 L.bm_miss = p->bm_miss;
                 L.bm_two = p->bm_two;
                 L.u = p->u;
-                L.small_u = std::min(MERGE_SMALL_U, p->capmax);
+                L.small_u = p->small_u;
+                L.only_small = p->h_summary.merge_batched == 0;
                 L.work = lists[k];
                 L.nwork = nk;
                 L.cap = lv[k];
@@ -1347,8 +1408,10 @@ extern "C" spgemm_status spgemm_numeric(spgemm_plan *p, spgemm_csr_out *C_out) {
                                          p->C.val, m > 0 ? nnzC / m : 0, p->st));
             if (s1 > s0) p->count(SPGEMM_K_ARRANGE);
             const int64_t n37 = p->h_summary.bin_count[BIN_MERGE];
-            SPG_TRY(launch_arrange_long(p->items, n37, p->C.row_ptr, p->C.col_idx, p->C.val, p->st));
-            if (n37 > 0) p->count(SPGEMM_K_ARRANGE);
+            if (n37 > p->dense_n) {
+                SPG_TRY(launch_arrange_long(p->items, n37, p->C.row_ptr, p->C.col_idx, p->C.val, p->st));
+                p->count(SPGEMM_K_ARRANGE);
+            }
         }
         p->time_end();
         if (fill_done) {
@@ -1741,7 +1804,7 @@ fail:
 static spgemm_status prepare_replay(spgemm_plan *p) {
     spgemm_status status = SPGEMM_OK;
     const int64_t n37 = p->h_summary.bin_count[BIN_MERGE];
-    if (p->opts.alloc_policy == SPGEMM_ALLOC_PRECISE) {
+    if (p->opts.alloc_policy == SPGEMM_ALLOC_PRECISE || p->dense_n == n37) {
         // every bin-37 row is a dense-slice row, replayed by the fill kernel
         p->replay_ready = true;
         return SPGEMM_OK;
@@ -1977,14 +2040,25 @@ static cudaError_t precise_count(spgemm_plan *p, bool dev) {
     cudaError_t e;
     for (auto &r : kEscRanges) {
         const RowSet R = bin_range(p, r.lo, r.hi, dev);
-        if (R.n > 0 && (e = run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, r.max_u, true, p->st); })) != cudaSuccess)
+        if (R.n > 0 && (e = run(SPGEMM_K_ESC, [&] { return launch_esc_set(a, R, r.max_u, true, p->stream()); })) != cudaSuccess)
             return e;
     }
     if (p->dense_K > 0 && (dev || p->dense_n > 0)) {
         const DenseArgs D = dense_args_of(p, dev);
-        if ((e = run(SPGEMM_K_MERGE, [&] { return launch_dense_count(p->A, p->B, D, p->d_err, p->st); })) != cudaSuccess)
+        const cudaStream_t ds = p->stream();
+        if (dev) {
+            // the slice rows of this run, and B's slice boundaries
+            if ((e = launch_dense_select(p->bin_rows, p->A.nrows, p->d_summary, p->u, p->dense_flag, p->dense_lo,
+                                         p->dense_hi, p->d_select, p->dense_order, p->dense_rows, p->dense_clo,
+                                         p->dense_chi, ds)) != cudaSuccess)
+                return e;
+            if (p->dense_K > 1 &&
+                (e = launch_dense_bounds(p->B, p->dense_K, p->dense_W, p->dense_bnd, ds)) != cudaSuccess)
+                return e;
+        }
+        if ((e = run(SPGEMM_K_MERGE, [&] { return launch_dense_count(p->A, p->B, D, p->d_err, ds); })) != cudaSuccess)
             return e;
-        if ((e = run(SPGEMM_K_OTHER, [&] { return launch_dense_rowsum(D, p->nnzc, p->st); })) != cudaSuccess) return e;
+        if ((e = run(SPGEMM_K_OTHER, [&] { return launch_dense_rowsum(D, p->nnzc, ds); })) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -2002,7 +2076,7 @@ static cudaError_t precise_fill(spgemm_plan *p, bool dev, const int64_t *gate) {
     // bin 1: the single product of each row
     const RowSet r1 = bin_range(p, 1, 1, dev);
     if (!dev) p->time_begin(SPGEMM_K_ARRANGE);
-    e = launch_arrange_short(a, r1, p->bin, p->C.row_ptr, p->C.col_idx, p->C.val, 1, p->st);
+    e = launch_arrange_short(a, r1, p->bin, p->C.row_ptr, p->C.col_idx, p->C.val, 1, p->stream());
     if (!dev) {
         p->time_end();
         if (r1.n > 0) p->count(SPGEMM_K_ARRANGE);
@@ -2010,8 +2084,8 @@ static cudaError_t precise_fill(spgemm_plan *p, bool dev, const int64_t *gate) {
     if (e != cudaSuccess) return e;
     if (p->dense_K > 0 && (dev || p->dense_n > 0)) {
         if (!dev) p->time_begin(SPGEMM_K_MERGE);
-        e = launch_dense_fill(p->A, p->B, dense_args_of(p, dev), p->C.row_ptr, p->C.col_idx, p->C.val, p->d_err, p->st,
-                              false, gate);
+        e = launch_dense_fill(p->A, p->B, dense_args_of(p, dev), p->C.row_ptr, p->C.col_idx, p->C.val, p->d_err,
+                              p->stream(), false, gate);
         if (!dev) {
             p->time_end();
             p->count(SPGEMM_K_MERGE);
@@ -2092,7 +2166,7 @@ static spgemm_status dplan_buffers(spgemm_dplan *d) {
         SPG_TRY(p->alloc_n(&p->bin_rows, m));
         SPG_TRY(p->alloc_n(&p->ctil_rp, m + 1));
         SPG_TRY(p->alloc_n(&p->d_hist, (int64_t)NUM_BINS * nblk));
-        SPG_TRY(p->alloc_n(&p->d_capp, 2 * nblk));
+        SPG_TRY(p->alloc_n(&p->d_capp, 3 * nblk));
         if (p->dense_K > 0) {
             SPG_TRY(p->alloc_n(&p->dense_flag, m));
             SPG_TRY(p->alloc_n(&p->dense_lo, m));
@@ -2109,6 +2183,7 @@ static spgemm_status dplan_buffers(spgemm_dplan *d) {
         SPG_TRY(p->alloc_n(&p->C.row_ptr, m + 1));
         SPG_TRY(p->alloc_n(&p->C.col_idx, d->c_cap));
         SPG_TRY(p->alloc_n(&p->C.val, d->c_cap));
+        SPG_TRY(p->make_branches());
         SPG_TRY(cudaStreamSynchronize(p->st));  // the buffers exist before any capture
         p->C.nrows = m;
         p->C.ncols = p->B.ncols;
@@ -2147,16 +2222,21 @@ static cudaError_t dplan_enqueue(spgemm_dplan *d) {
     const BoundOut out = bound_out(p);
     DP_TRY(launch_bound(p->A, p->B, pol, out, p->st));
     DP_TRY(launch_binning(m, p->A.nnz, pol, out, p->bin_rows, p->ctil_rp, p->d_summary, nullptr, p->st));
-    if (p->dense_K > 0) {
-        DP_TRY(launch_dense_select(p->bin_rows, m, p->d_summary, p->u, p->dense_flag, p->dense_lo, p->dense_hi,
-                                   p->d_select, p->dense_order, p->dense_rows, p->dense_clo, p->dense_chi, p->st));
-        if (p->dense_K > 1) DP_TRY(launch_dense_bounds(p->B, p->dense_K, p->dense_W, p->dense_bnd, p->st));
-    }
-    // stage 3, counting pass; stage 4, row pointers; then the fill pass straight into C
-    DP_TRY(precise_count(p, true));
+    // stage 3, counting pass; stage 4, row pointers; then the fill pass straight into C.  The
+    // launches of a pass write different rows: they run side by side, so that the ones whose bins
+    // are empty (most, for a stencil) cost no time of their own
+    DP_TRY(p->fork());
+    e = precise_count(p, true);
+    cudaError_t j = p->join();
+    DP_TRY(e);
+    DP_TRY(j);
     DP_TRY(launch_row_scan(m, p->nnzc, p->C.row_ptr, p->scan_partial, p->st));
     DP_TRY(launch_gate(p->C.row_ptr, m, d->c_cap, d->gate, p->d_err, p->st));
-    DP_TRY(precise_fill(p, true, d->gate));
+    DP_TRY(p->fork());
+    e = precise_fill(p, true, d->gate);
+    j = p->join();
+    DP_TRY(e);
+    DP_TRY(j);
     if (p->npairs > 0) {
         DP_TRY(launch_split_out(p->d_pairs, p->npairs, p->C.row_ptr, m, p->split_rp, p->st));
         DP_TRY(launch_gather_first(p->d_pairs, p->npairs, p->C.row_ptr, m, d->d_first, p->st));

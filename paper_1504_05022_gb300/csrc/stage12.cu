@@ -154,7 +154,8 @@ SPG_DEV bool dense_row(int b, int64_t i, const CapPolicy &P) {
 }
 
 // u_i, bin and row size of every row, and per `factor` blocks the histogram of the rows and the
-// sums of C~ entries and of u_i (part[0..nblk), part[nblk..2 nblk)), zeroed before when factor > 1.  Bin-37 rows also get their column
+// sums of C~ entries and of u_i and the rows that only the batched merge kernel can take
+// (part[0..nblk), part[nblk..2 nblk), part[2 nblk..3 nblk)), zeroed before when factor > 1.  Bin-37 rows also get their column
 // range [lo, hi) (first and last column of every B row they select) and the flag that sends them
 // to the dense-slice kernels: u_i >= dmin (dmin > 0), else div u_i >= hi - lo -- their products
 // cover at least a div-th of the columns they can reach, so the accumulator's O(hi - lo) clearing
@@ -178,7 +179,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
     }
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * ROWS;
-    int64_t capsum = 0, usum = 0;
+    int64_t capsum = 0, usum = 0, batched = 0;
     auto sum_of = [&](int64_t p0, int64_t p1, int step) {
         int64_t u = 0;
 #pragma unroll 4
@@ -213,7 +214,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
         }
     };
     // by one thread per row; the range is that of a bin-37 row where flags are wanted
-    auto finish = [&](int64_t i, int64_t u, int b, int32_t cmin, int32_t cmax) {
+    auto finish = [&](int64_t i, int64_t u, int b, int64_t nA, int32_t cmin, int32_t cmax) {
         bool dense = false;
         if (P.dense != nullptr) {
             if (b == BIN_MERGE) {
@@ -230,6 +231,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
         atomicAdd(&hist[b], 1);
         capsum += cap_of(u, b, i, P, dense);
         usum += u;
+        if (b == BIN_MERGE && !dense && merge_small_threads(u, (int)min(nA, (int64_t)INT32_MAX), O.small_u) == 0) ++batched;
     };
     const int64_t mine = base + grp;
     if (mine < A.nrows) {  // the whole group
@@ -250,7 +252,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
                     cmax = max(cmax, __shfl_xor_sync(gm, cmax, d, G));
                 }
             }
-            if (gl == 0) finish(mine, u, b, cmin, cmax);
+            if (gl == 0) finish(mine, u, b, a1 - a0, cmin, cmax);
         }
     }
     __syncthreads();
@@ -267,7 +269,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
             cmin = __reduce_min_sync(SPG_FULL, cmin);
             cmax = __reduce_max_sync(SPG_FULL, cmax);
         }
-        if (lane_id() == 0) finish(i, u, b, cmin, cmax);
+        if (lane_id() == 0) finish(i, u, b, a1 - a0, cmin, cmax);
     }
     for (int l = 0; l < nl; ++l) {
         const int64_t i = base + longs[l];
@@ -288,17 +290,19 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
             }
             __syncthreads();
         }
-        if (threadIdx.x == 0) finish(i, u, b, range[0], range[1]);
+        if (threadIdx.x == 0) finish(i, u, b, a1 - a0, range[0], range[1]);
     }
     __syncthreads();
     capsum = block_reduce_sum<BOUND_NT>(capsum, scratch);
     usum = block_reduce_sum<BOUND_NT>(usum, scratch);
+    batched = block_reduce_sum<BOUND_NT>(batched, scratch);
     const int64_t blk = blockIdx.x / factor;
     if (factor == 1) {
         if (threadIdx.x < NUM_BINS) O.hist[(int64_t)threadIdx.x * nblk + blk] = hist[threadIdx.x];
         if (threadIdx.x == 0) {
             O.part[blk] = capsum;
             O.part[nblk + blk] = usum;
+            O.part[2 * nblk + blk] = batched;
         }
     } else {
         if (threadIdx.x < NUM_BINS && hist[threadIdx.x] != 0)
@@ -306,6 +310,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
         if (threadIdx.x == 0) {
             atomicAdd((unsigned long long *)&O.part[blk], (unsigned long long)capsum);
             atomicAdd((unsigned long long *)&O.part[nblk + blk], (unsigned long long)usum);
+            if (batched) atomicAdd((unsigned long long *)&O.part[2 * nblk + blk], (unsigned long long)batched);
         }
     }
 }
@@ -336,9 +341,9 @@ SPG_DEV T warp_scan_array(T *v, int64_t n) {
 __global__ void __launch_bounds__(1024)
 k_bin_scan(int64_t m, int32_t *hist, int64_t nblk, int64_t *part, int64_t *ctil_rp, BinSummary *summary,
            BinSummary *host) {
-    __shared__ int64_t total[NUM_BINS + 2], bstart[NUM_BINS + 1];
+    __shared__ int64_t total[NUM_BINS + 3], bstart[NUM_BINS + 1];
     const int lane = lane_id();
-    for (int b = warp_id(); b < NUM_BINS + 2; b += 32) {
+    for (int b = warp_id(); b < NUM_BINS + 3; b += 32) {
         const int64_t t = b < NUM_BINS ? (int64_t)warp_scan_array(hist + b * nblk, nblk)
                                        : warp_scan_array(part + (b - NUM_BINS) * nblk, nblk);
         if (lane == 0) total[b] = t;
@@ -363,6 +368,7 @@ k_bin_scan(int64_t m, int32_t *hist, int64_t nblk, int64_t *part, int64_t *ctil_
         if (threadIdx.x == 0) {
             S->sum_cap = total[NUM_BINS];
             S->sum_u = total[NUM_BINS + 1];
+            S->merge_batched = total[NUM_BINS + 2];
             S->dense_count = 0;
             S->dense_end[0] = S->dense_end[1] = 0;
         }
@@ -439,7 +445,7 @@ cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, c
     const int factor = (int)(bin_rows_per_block(A.nrows, A.nnz) / rows);
     if (factor > 1) {
         cudaError_t e = cudaMemsetAsync(O.hist, 0, sizeof(int32_t) * NUM_BINS * nblk, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(O.part, 0, sizeof(int64_t) * 2 * nblk, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(O.part, 0, sizeof(int64_t) * 3 * nblk, st);
         if (e != cudaSuccess) return e;
     }
     auto go = [&](auto kern) {
