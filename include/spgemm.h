@@ -227,9 +227,10 @@ spgemm_status spgemm_numeric(spgemm_plan *plan, spgemm_csr_out *C_out);
    the plan itself.  NULL is accepted. */
 spgemm_status spgemm_free(spgemm_plan *plan);
 
-/* Every plan allocates from one stream-ordered memory pool per device, which keeps the
-   blocks freed by earlier plans for reuse (no release threshold), so a process that ran a
-   large product keeps holding that device memory.  This returns the pool's unused memory
+/* Every plan allocates from two stream-ordered memory pools per device (results, temporaries).
+   Blocks freed by earlier plans are kept for reuse: up to half of the device's memory by size,
+   the rest in the pools (no release threshold), so a process that ran a large product keeps
+   holding that device memory.  This returns the unused memory
    on `device` to the system, keeping at most keep_bytes (cudaMemPoolTrimTo).  Synchronise
    the streams of the plans freed on that device first: blocks whose stream-ordered free has
    not run yet are still in use.  SPGEMM_ERR_INVALID_ARG for a negative device or

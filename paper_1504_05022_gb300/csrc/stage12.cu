@@ -106,11 +106,17 @@ static int bound_group(int64_t m, int64_t nnz) {
     return g;
 }
 
-// Stage 1 runs a block per BOUND_NT / group rows, so that a run of hub rows (the low rows of an
-// R-MAT matrix) spreads over the SMs; stage 2 bins blocks of that many rows times a factor that
-// leaves about four per SM (of 152), since one block scans the (bin, block) counts.
-static int64_t bin_rows_per_block(int64_t m, int64_t nnz) {
+// Stage 1 runs a block per BOUND_NT / group rows, or twice as many where that leaves blocks
+// enough (more would let a run of hub rows, the low rows of an R-MAT matrix, hold up an SM: 13
+// times as many took 1.7 ms at 2^20 rows, once 0.42); stage 2 bins blocks of that many rows
+// times a factor that leaves about four per SM (of 152), since one block scans the counts.
+static int64_t bound_rows(int64_t m, int64_t nnz) {
     const int64_t rows = BOUND_NT / bound_group(m, nnz);
+    const int64_t fold = m / (rows * 608);
+    return rows * (fold < 1 ? 1 : fold > 2 ? 2 : fold);
+}
+static int64_t bin_rows_per_block(int64_t m, int64_t nnz) {
+    const int64_t rows = bound_rows(m, nnz);
     const int64_t factor = (m + rows * 608 - 1) / (rows * 608);
     return rows * (factor < 1 ? 1 : factor);
 }
@@ -164,10 +170,10 @@ SPG_DEV bool dense_row(int b, int64_t i, const CapPolicy &P) {
 // prefix sum, a marking pass and a histogram pass.
 template <int G>
 __global__ void __launch_bounds__(BOUND_NT, 3)
-k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
+k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int factor, int64_t nblk) {
     __shared__ int32_t hist[NUM_BINS];
     constexpr int ROWS = BOUND_NT / G;
-    __shared__ int32_t nlong, longs[ROWS];
+    __shared__ int32_t nlong, longs[2 * ROWS];
     __shared__ int64_t scratch[BOUND_NT / 32 + 1];
     __shared__ int32_t range[2];
     const int gl = threadIdx.x & (G - 1), grp = threadIdx.x / G;
@@ -178,7 +184,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
         if (blockIdx.x == 0) *O.err = 0;
     }
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * ROWS;
+    const int64_t base = (int64_t)blockIdx.x * R;
     int64_t capsum = 0, usum = 0, batched = 0;
     auto sum_of = [&](int64_t p0, int64_t p1, int step) {
         int64_t u = 0;
@@ -192,6 +198,7 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
     auto range_of = [&](int64_t p0, int64_t p1, int step, int32_t &cmin, int32_t &cmax) {
         cmin = INT32_MAX;
         cmax = -1;
+        int64_t sum = 0;
         constexpr int UN = 4;  // entries whose dependent gathers are in flight together
         for (int64_t p = p0; p < p1; p += UN * step) {
             int64_t rs[UN], re[UN];
@@ -210,8 +217,10 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
                     cmin = min(cmin, B.col[rs[u]]);
                     cmax = max(cmax, B.col[re[u] - 1]);
                 }
+                sum += re[u] - rs[u];
             }
         }
+        return sum;
     };
     // by one thread per row; the range is that of a bin-37 row where flags are wanted
     auto finish = [&](int64_t i, int64_t u, int b, int64_t nA, int32_t cmin, int32_t cmax) {
@@ -233,27 +242,28 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
         usum += u;
         if (b == BIN_MERGE && !dense && merge_small_threads(u, (int)min(nA, (int64_t)INT32_MAX), O.small_u) == 0) ++batched;
     };
-    const int64_t mine = base + grp;
-    if (mine < A.nrows) {  // the whole group
-        const int64_t a0 = A.rp[mine], a1 = A.rp[mine + 1];
+    for (int r0 = 0; r0 < R; r0 += ROWS) {
+        const int64_t i = base + r0 + grp;
+        if (i >= A.nrows) break;  // the whole group
+        const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
         if (a1 - a0 > LONG_STEPS * G) {
-            if (gl == 0) longs[atomicAdd(&nlong, 1)] = grp;
-        } else {
-            int64_t u = sum_of(a0 + gl, a1, G);
-#pragma unroll
-            for (int d = G / 2; d > 0; d >>= 1) u += __shfl_xor_sync(gm, u, d, G);
-            const int b = bin_of(u);
-            int32_t cmin = 0, cmax = 0;
-            if (b == BIN_MERGE && P.dense != nullptr) {
-                range_of(a0 + gl, a1, G, cmin, cmax);
-#pragma unroll
-                for (int d = G / 2; d > 0; d >>= 1) {
-                    cmin = min(cmin, __shfl_xor_sync(gm, cmin, d, G));
-                    cmax = max(cmax, __shfl_xor_sync(gm, cmax, d, G));
-                }
-            }
-            if (gl == 0) finish(mine, u, b, a1 - a0, cmin, cmax);
+            if (gl == 0) longs[atomicAdd(&nlong, 1)] = r0 + grp;
+            continue;
         }
+        int64_t u = sum_of(a0 + gl, a1, G);
+#pragma unroll
+        for (int d = G / 2; d > 0; d >>= 1) u += __shfl_xor_sync(gm, u, d, G);
+        const int b = bin_of(u);
+        int32_t cmin = 0, cmax = 0;
+        if (b == BIN_MERGE && P.dense != nullptr) {
+            range_of(a0 + gl, a1, G, cmin, cmax);
+#pragma unroll
+            for (int d = G / 2; d > 0; d >>= 1) {
+                cmin = min(cmin, __shfl_xor_sync(gm, cmin, d, G));
+                cmax = max(cmax, __shfl_xor_sync(gm, cmax, d, G));
+            }
+        }
+        if (gl == 0) finish(i, u, b, a1 - a0, cmin, cmax);
     }
     __syncthreads();
     const int nl = nlong;
@@ -261,14 +271,16 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
         const int64_t i = base + longs[l];
         const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
         if (a1 - a0 > HUB_ENTRIES) continue;
-        const int64_t u = warp_reduce_sum(sum_of(a0 + lane_id(), a1, 32));
-        const int b = bin_of(u);
         int32_t cmin = 0, cmax = 0;
-        if (b == BIN_MERGE && P.dense != nullptr) {
-            range_of(a0 + lane_id(), a1, 32, cmin, cmax);
+        int64_t u;
+        if (P.dense != nullptr) {  // most long rows are in bin 37: one pass for both
+            u = warp_reduce_sum(range_of(a0 + lane_id(), a1, 32, cmin, cmax));
             cmin = __reduce_min_sync(SPG_FULL, cmin);
             cmax = __reduce_max_sync(SPG_FULL, cmax);
+        } else {
+            u = warp_reduce_sum(sum_of(a0 + lane_id(), a1, 32));
         }
+        const int b = bin_of(u);
         if (lane_id() == 0) finish(i, u, b, a1 - a0, cmin, cmax);
     }
     for (int l = 0; l < nl; ++l) {
@@ -293,25 +305,29 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int factor, int64_t nblk) {
         if (threadIdx.x == 0) finish(i, u, b, a1 - a0, range[0], range[1]);
     }
     __syncthreads();
-    capsum = block_reduce_sum<BOUND_NT>(capsum, scratch);
-    usum = block_reduce_sum<BOUND_NT>(usum, scratch);
-    batched = block_reduce_sum<BOUND_NT>(batched, scratch);
+    // the block's three sums, a warp's at a time
+    __shared__ int64_t sums[3][BOUND_NT / 32];
+    capsum = warp_reduce_sum(capsum);
+    usum = warp_reduce_sum(usum);
+    batched = warp_reduce_sum(batched);
+    if (lane_id() == 0) {
+        sums[0][warp_id()] = capsum;
+        sums[1][warp_id()] = usum;
+        sums[2][warp_id()] = batched;
+    }
+    __syncthreads();
     const int64_t blk = blockIdx.x / factor;
-    if (factor == 1) {
-        if (threadIdx.x < NUM_BINS) O.hist[(int64_t)threadIdx.x * nblk + blk] = hist[threadIdx.x];
-        if (threadIdx.x == 0) {
-            O.part[blk] = capsum;
-            O.part[nblk + blk] = usum;
-            O.part[2 * nblk + blk] = batched;
-        }
-    } else {
-        if (threadIdx.x < NUM_BINS && hist[threadIdx.x] != 0)
-            atomicAdd(&O.hist[(int64_t)threadIdx.x * nblk + blk], hist[threadIdx.x]);
-        if (threadIdx.x == 0) {
-            atomicAdd((unsigned long long *)&O.part[blk], (unsigned long long)capsum);
-            atomicAdd((unsigned long long *)&O.part[nblk + blk], (unsigned long long)usum);
-            if (batched) atomicAdd((unsigned long long *)&O.part[2 * nblk + blk], (unsigned long long)batched);
-        }
+    if (threadIdx.x < NUM_BINS) {
+        int32_t *h = &O.hist[(int64_t)threadIdx.x * nblk + blk];
+        if (factor == 1) *h = hist[threadIdx.x];
+        else if (hist[threadIdx.x] != 0) atomicAdd(h, hist[threadIdx.x]);
+    } else if (threadIdx.x >= 64 && threadIdx.x < 67) {
+        const int k = threadIdx.x - 64;
+        int64_t t = 0;
+        for (int w = 0; w < BOUND_NT / 32; ++w) t += sums[k][w];
+        int64_t *o = &O.part[k * nblk + blk];
+        if (factor == 1) *o = t;
+        else if (t != 0) atomicAdd((unsigned long long *)o, (unsigned long long)t);
     }
 }
 
@@ -441,7 +457,7 @@ cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, c
     const int64_t nblk = bin_blocks(A.nrows, A.nnz);
     if (P.dense != nullptr && O.div < 1) return cudaErrorInvalidValue;
     if (nblk <= 0) return cudaMemsetAsync(O.err, 0, sizeof(int64_t), st);
-    const int64_t rows = BOUND_NT / bound_group(A.nrows, A.nnz);
+    const int64_t rows = bound_rows(A.nrows, A.nnz);
     const int factor = (int)(bin_rows_per_block(A.nrows, A.nnz) / rows);
     if (factor > 1) {
         cudaError_t e = cudaMemsetAsync(O.hist, 0, sizeof(int32_t) * NUM_BINS * nblk, st);
@@ -449,7 +465,7 @@ cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, c
         if (e != cudaSuccess) return e;
     }
     auto go = [&](auto kern) {
-        kern<<<(unsigned)((A.nrows + rows - 1) / rows), BOUND_NT, 0, st>>>(A, B, P, O, factor, nblk);
+        kern<<<(unsigned)((A.nrows + rows - 1) / rows), BOUND_NT, 0, st>>>(A, B, P, O, (int)rows, factor, nblk);
         return cudaGetLastError();
     };
     switch (bound_group(A.nrows, A.nnz)) {
