@@ -104,10 +104,11 @@ def src_digest(files):
 
 
 KERNEL_SOURCES = {
-    "merge": ["paper_1504_05022_gb300/csrc/merge.cu", "paper_1504_05022_gb300/csrc/merge_bm.cu", "paper_1504_05022_gb300/csrc/merge_small.cu",
+    "merge": ["paper_1504_05022_gb300/csrc/merge.cu", "paper_1504_05022_gb300/csrc/merge_bm.cu",
+              "paper_1504_05022_gb300/csrc/merge_small.cu",
               "paper_1504_05022_gb300/csrc/dense.cu", "paper_1504_05022_gb300/csrc/common.cuh"],
     "arrange": ["paper_1504_05022_gb300/csrc/arrange.cu", "paper_1504_05022_gb300/csrc/scan.cuh"],
-    "esc": ["paper_1504_05022_gb300/csrc/esc.cu"],
+    "esc": ["paper_1504_05022_gb300/csrc/esc.cu", "paper_1504_05022_gb300/csrc/net.cu"],
     "heap": ["paper_1504_05022_gb300/csrc/heap.cu"],
     "bound": ["paper_1504_05022_gb300/csrc/stage12.cu", "paper_1504_05022_gb300/csrc/scan.cuh"],
     "bin": ["paper_1504_05022_gb300/csrc/stage12.cu"],

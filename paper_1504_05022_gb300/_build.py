@@ -26,7 +26,7 @@ LIB_CHECK = os.path.join(BUILD, "check", "libspgemm_check.so")
 VARIANTS = {"f64": (LIB, BUILD, []), "f32": (LIB_F32, os.path.join(BUILD, "f32"), ["-DSPGEMM_FLOAT"]),
             "check": (LIB_CHECK, os.path.join(BUILD, "check"), ["-DSPGEMM_CHECK"])}
 
-SOURCES = ["stage12.cu", "heap.cu", "esc.cu", "merge.cu", "merge_bm.cu", "merge_small.cu", "dense.cu", "merge_micro.cu", "arrange.cu", "predictor.cu", "replay.cu", "batched.cu",
+SOURCES = ["stage12.cu", "heap.cu", "esc.cu", "net.cu", "merge.cu", "merge_bm.cu", "merge_small.cu", "dense.cu", "merge_micro.cu", "arrange.cu", "predictor.cu", "replay.cu", "batched.cu",
            "spgemm_api.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -145,6 +145,8 @@ cudaError_t launch_heap_set(const StageArgs &a, const RowSet &R, int slots, int 
 // rows of at most max_u (<= 512) products.  count_only: nnz(c_i) of every row into a.nnzc and
 // nothing else (the counting pass of the precise method, Section 3.1)
 cudaError_t launch_esc_set(const StageArgs &a, const RowSet &R, int max_u, bool count_only, cudaStream_t st);
+// the same for max_u <= 32, a thread per row (net.cu)
+cudaError_t launch_net_set(const StageArgs &a, const RowSet &R, int max_u, bool count_only, cudaStream_t st);
 
 // Bin-37 work items.  Item j < n37 is the j-th row of bin 37 with the full
 // column range.  An item whose sequence outgrows the largest shared-memory

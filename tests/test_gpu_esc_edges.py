@@ -60,3 +60,40 @@ def test_esc_exact(dtype, ncols, longest):
             C.val.zero_()
             plan.replay()
             plan.check()
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("ncols", [900, (1 << 27) - 1, 1 << 29])
+@pytest.mark.parametrize("longest", [1, 3, 12])
+def test_many_short_rows_exact(dtype, ncols, longest):
+    """Enough rows of u_i = 2..32 for the kernels with a thread per row (every network width), with
+    empty B rows, many and no equal columns, and 32- and 64-bit keys."""
+    import oracle
+    import paper_1504_05022_gb300 as spg
+    rng = np.random.default_rng(longest + ncols % 97)
+    m, nb = 60000, 5000
+    n = rng.integers(0, longest + 1, nb)
+    n[0] = 0
+    b_r = np.repeat(np.arange(nb), n)
+    pool = np.unique(rng.integers(0, ncols, 40 if ncols == 900 else 20000))
+    b_c = np.concatenate([np.sort(rng.choice(pool, size=x, replace=False)) for x in n])
+    B = gen.from_coo(nb, ncols, b_r, b_c, rng.integers(-4, 5, b_r.size).astype(np.float64))
+    k = rng.integers(1, max(2, 64 // (longest + 1)), m)
+    a_r = np.repeat(np.arange(m), k)
+    A = gen.from_coo(m, nb, a_r, rng.integers(0, nb, a_r.size), None)
+    A.val = rng.integers(-4, 5, A.nnz).astype(np.float64)
+    used = np.unique(B.col)
+    ref = oracle.spgemm(A, gen.HostCSR(nb, used.size, B.row_ptr, np.searchsorted(used, B.col).astype(np.int32), B.val))
+    Ad, Bd = (spg.CSR.from_host(M, dtype=dtype) for M in (A, B))
+    plans = [spg.Plan(Ad, Bd, alloc_policy=p) for p in ["hybrid"] + (["precise"] if ncols == 900 else [])]
+    bins = plans[0].stats()["bin_count"]
+    assert max(sum(bins[2:9]), sum(bins[9:17]), sum(bins[17:33])) >= 16384
+    for plan in plans:
+        C = plan.numeric()
+        for _ in range(2):  # the product, then a values-only replay
+            rp, col, val = C.to_host()
+            assert np.array_equal(rp, ref.row_ptr) and np.array_equal(col, used[ref.col])
+            assert np.array_equal(val.astype(np.float64), ref.val)
+            C.val.zero_()
+            plan.replay()
+            plan.check()
