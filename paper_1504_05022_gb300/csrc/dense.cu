@@ -629,15 +629,25 @@ k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_co
 // took 3.08 ms, and 1.45 ms with the product walk above.  Bound by shared memory and, in double precision, the FP64 pipe.
 // The columns are a bitmap, a word per lane.  A B row whose entries are consecutive columns
 // (last - first + 1 = length, as in a band or a block) sets its bits and finds its columns
-// without reading them.
+// without reading them, and 32 such rows (a window of A) are summed in registers: lane l holds
+// the sums of columns l, l + 32, ..., and no sum passes through shared memory.
 constexpr int DN_WARPS = 8;
 constexpr int DN_AHEAD = 4;  // steps of 32 products whose loads are in flight
+// Register steps (a word of the range for one part) taken for one shared-memory step of 32
+// products.  Float: bands of 24 to 100 entries 334-1619 -> 312-1239 us for the product, a band
+// of 201 times one of 3 is better left in shared memory (1364 against 1974 us).  Double: FMAs of
+// lanes outside a part cost as much as the others (a band of 64: 893 us in shared memory, 1090
+// in registers), so only where the parts fill their words (blocks of 64: 905 -> 755 us).
+constexpr int DN_REG_PER_STEP = sizeof(val_t) == 4 ? 4 : 1;
 
+struct __align__(16) DensePart {
+    int64_t p0;  // first entry in B
+    int32_t x0;  // first column - lo
+    int32_t len; // entries; negative: consecutive columns
+};
 struct DenseParts {  // per warp: 32 B rows
-    int64_t p0[32];   // first entry in B
-    val_t a[32];      // a_ik
-    int32_t x0[32];   // first column - lo
-    int32_t len[32];  // entries; negative: consecutive columns
+    DensePart part[32];
+    val_t a[32];     // a_ik
     uint32_t bits[32];
 };
 
@@ -684,6 +694,10 @@ k_dense_narrow(DevCSR A, DevCSR B, DenseArgs D, const int64_t *__restrict__ c_rp
             __syncwarp();
         }
         uint32_t mine = 0;  // bits of columns [32 lane, 32 lane + 32) set by consecutive parts
+        constexpr int REGS = FILL && W <= 256 ? W / 32 : 0;
+        val_t acc[REGS > 0 ? REGS : 1];
+#pragma unroll
+        for (int r = 0; r < REGS; ++r) acc[r] = val_t(0);
         const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
         for (int64_t e = a0; e < a1; e += 32) {
             int len = 0, x0 = 0;
@@ -710,20 +724,21 @@ k_dense_narrow(DevCSR A, DevCSR B, DenseArgs D, const int64_t *__restrict__ c_rp
             const int np = __popc(nz);
             if (len > 0) {
                 const int q = __popc(nz & ((1u << lane) - 1u));
-                S.p0[q] = rs;
+                S.part[q] = DensePart{rs, x0, run ? -len : len};
                 if (FILL) S.a[q] = av;
-                S.x0[q] = x0;
-                S.len[q] = run ? -len : len;
             }
+            // every column of the range is asked for every part: not for parts much shorter
+            const bool runs = FILL && REGS > 0 && !__any_sync(SPG_FULL, len > 0 && !run) &&
+                              DN_REG_PER_STEP * (int)__reduce_add_sync(SPG_FULL, (unsigned)(len + 31) >> 5) >= np * ((span + 31) >> 5);
             __syncwarp();
             // the columns
             for (int t = 0; t < np; ++t) {
-                const int ln = S.len[t], f = S.x0[t];
+                const int ln = S.part[t].len, f = S.part[t].x0;
                 if (ln < 0) {
                     const int b0 = max(f - 32 * lane, 0), b1 = min(f - ln - 32 * lane, 32);
                     if (b0 < b1) mine |= (b1 - b0 == 32 ? ~0u : ((1u << (b1 - b0)) - 1u) << b0);
                 } else {
-                    const int64_t p = S.p0[t];
+                    const int64_t p = S.part[t].p0;
                     for (int i = lane; i < ln; i += 32) {
                         const int x = __ldg(B.col + p + i) - lo;
                         if ((unsigned)x < (unsigned)span) atomicOr(&S.bits[x >> 5], 1u << (x & 31));
@@ -731,18 +746,41 @@ k_dense_narrow(DevCSR A, DevCSR B, DenseArgs D, const int64_t *__restrict__ c_rp
                     }
                 }
             }
-            if (FILL) {
+            if (runs) {
+#pragma unroll
+                for (int r = 0; r < REGS; ++r) {
+                    if (32 * r >= span) break;
+                    const int x = 32 * r + lane;
+                    for (int t = 0; t < np; t += DN_AHEAD) {
+                        val_t v[DN_AHEAD];
+                        bool ok[DN_AHEAD];
+#pragma unroll
+                        for (int u = 0; u < DN_AHEAD; ++u) {
+                            ok[u] = false;
+                            if (t + u < np) {
+                                const DensePart q = S.part[t + u];
+                                ok[u] = (unsigned)(x - q.x0) < (unsigned)-q.len;
+                                if (ok[u]) v[u] = __ldg(B.val + q.p0 + (x - q.x0));
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < DN_AHEAD; ++u)
+                            if (ok[u]) acc[r] = fma(S.a[t + u], v[u], acc[r]);
+                    }
+                }
+            } else if (FILL) {
                 // steps (part t, entries i0..i0+31), their loads DN_AHEAD steps ahead
                 val_t v[DN_AHEAD];
                 int32_t c[DN_AHEAD];
                 int lt = 0, li = 0;  // the next step to load
                 auto load = [&](val_t &vv, int32_t &cc) {
                     if (lt >= np) return;
-                    const int ln = S.len[lt], m = ln < 0 ? -ln : ln;
-                    const int64_t p = S.p0[lt] + li + lane;
+                    const DensePart q = S.part[lt];
+                    const int ln = q.len, m = ln < 0 ? -ln : ln;
+                    const int64_t p = q.p0 + li + lane;
                     if (li + lane < m) {
                         vv = __ldg(B.val + p);
-                        cc = ln < 0 ? S.x0[lt] + li + lane : __ldg(B.col + p) - lo;
+                        cc = ln < 0 ? q.x0 + li + lane : __ldg(B.col + p) - lo;
                     }
                     li += 32;
                     if (li >= m) {
@@ -756,7 +794,7 @@ k_dense_narrow(DevCSR A, DevCSR B, DenseArgs D, const int64_t *__restrict__ c_rp
 #pragma unroll
                     for (int u = 0; u < DN_AHEAD; ++u) {
                         if (t < np) {
-                            const int ln = S.len[t], m = ln < 0 ? -ln : ln;
+                            const int ln = S.part[t].len, m = ln < 0 ? -ln : ln;
                             if (i + lane < m && (unsigned)c[u] < (unsigned)span) V[c[u]] = fma(S.a[t], v[u], V[c[u]]);
                             i += 32;
                             if (i >= m) {
@@ -795,6 +833,10 @@ k_dense_narrow(DevCSR A, DevCSR B, DenseArgs D, const int64_t *__restrict__ c_rp
                 __syncwarp();
                 continue;
             }
+#pragma unroll
+            for (int r = 0; r < REGS; ++r)
+                if (32 * r + lane < span) V[32 * r + lane] += acc[r];
+            __syncwarp();
             const uint32_t out = REPLAY ? known : bits;
             const int ow = __popc(out);
             const int before = warp_inclusive_scan(ow) - ow;

@@ -76,6 +76,44 @@ def test_narrow_rows_exact(oracle_mod, dtype, ncols, span, policy):
         assert np.array_equal(val.astype(np.float64), scale * ref.val)
 
 
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("long", [True, False])
+@pytest.mark.parametrize("scattered", [0, 1, 33])
+def test_consecutive_parts_exact(oracle_mod, dtype, long, scattered):
+    """Rows whose B rows are runs of consecutive columns, long or short beside the range, with
+    `scattered` others (whole windows of 32 runs, mixed windows); small integers are exact."""
+    import paper_1504_05022_gb300 as spg
+    rng = np.random.default_rng(40 + scattered + long)
+    ar, ac, br, bc, nb = [], [], [], [], 0
+    for i, w in enumerate((31, 32, 33, 63, 64, 65, 200, 255, 256, 257)):
+        lo = int(rng.integers(0, 3000))
+        for q in range(700 if not long else 96):
+            n = max(1, w - q % 3) if long else 1 + q % 2
+            f = lo + (0 if q == 0 else w - n if q == 1 else int(rng.integers(0, w - n + 1)))
+            c = np.arange(f, f + n)
+            if q % 16 == 5 and q // 16 < scattered:
+                c = np.unique(np.array([lo, lo + w // 2, lo + w - 1]))
+            br.append(np.full(c.size, nb)); bc.append(c); ar.append(i); ac.append(nb)
+            nb += 1
+    b_r, b_c = np.concatenate(br), np.concatenate(bc)
+    B = gen.from_coo(nb, 5000, b_r, b_c, rng.integers(-4, 5, b_r.size).astype(np.float64))
+    A = gen.from_coo(10, nb, np.array(ar), np.array(ac), rng.integers(-4, 5, len(ar)).astype(np.float64))
+    ref = oracle_mod.spgemm(A, B)
+    Ad, Bd = (spg.CSR.from_host(M, dtype=dtype) for M in (A, B))
+    plan = spg.Plan(Ad, Bd, dense_min_u=513)
+    plan.numeric()
+    assert plan.stats()["rows_dense"] == 10
+    for scale in (1.0, 3.0):
+        if scale > 1.0:
+            Ad.val.mul_(scale)
+            plan.replay()
+        C = plan.numeric()
+        plan.check()
+        rp, col, val = C.to_host()
+        assert np.array_equal(rp, ref.row_ptr) and np.array_equal(col, ref.col)
+        assert np.array_equal(val.astype(np.float64), scale * ref.val)
+
+
 def _clip(ncols, span):
     """The same rows folded into a B of ncols columns (slices narrower than 1,024)."""
     A, B = _matrices(5000, seed=ncols + span)
