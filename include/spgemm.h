@@ -166,12 +166,10 @@ typedef struct spgemm_opts {
                                 the column range its products can reach (first to last column of
                                 the B rows it selects); negative = never.  Off with SPGEMM_MERGE_PATH,
                                 SPGEMM_LONG_ROWS_LEVEL1 and when B needs more than 64 slices */
-    int32_t dense_span;      /* widest dense slice in columns (0 = 131,072, at least 1,024).  A slice
-                                narrow enough for one sum and one flag per column in shared memory
-                                (about 21,900 columns in double) is filled in one pass over its
-                                products; a wider one keeps a bitmap of its columns, its rank
-                                directory and one sum per column of the result */
-    int32_t dense_span_div;  /* with dense_min_u = 0: the divisor of the rule above (0 = 8) */
+    int32_t dense_span;      /* widest dense slice in columns (0 = 131,072, at least 1,024) */
+    int32_t dense_span_div;  /* with dense_min_u = 0: the divisor of the rule above (0 = 32 for a row of at least
+                                1,024 products, 8 for a range of at most 16,384 columns, 512 for a
+                                row of more than 8,192 products) */
     const void *predictor;   /* spgemm_predictor* for SPGEMM_ALLOC_LEARNED, else NULL; it must
                                 not be freed before spgemm_symbolic (or spgemm_galerkin) has
                                 returned, since its weights are read by that call's kernels */
@@ -179,13 +177,14 @@ typedef struct spgemm_opts {
     int32_t dense_pred_min;  /* learned policy: a bin-37 row whose predicted nnz(c_i) is at least this
                                 is computed by the dense-slice kernels (the network's choice of
                                 kernel as well as of size); 0 = off */
-    int32_t dense_keep;      /* slices too wide for the single-pass fill (about 21,900 columns in
-                                double, 40,000 in float), which the compact form fills: the counting
-                                pass leaves every (row, slice)'s column bitmap in device memory (ceil(W / 32) + 1 words, rounded up to 4, per
-                                (row, slice), released when spgemm_numeric returns) and the fill reads
-                                it back instead of marking the columns again from the products.
+    int32_t dense_keep;      /* the slices' counting pass leaves every (row, slice)'s column bitmap in
+                                device memory (ceil(W / 32) + 1 words, rounded up to 4, per (row, slice)
+                                of the rows that reach more than 1,024 columns, released when
+                                spgemm_numeric returns) and the fill reads it back instead of marking
+                                the columns again.
                                 0 = kept by the hybrid, upper-bound and learned policies when the
-                                bitmaps take at most a quarter of the free device memory, never by the
+                                bitmaps take at most a quarter of the free device memory and hold no
+                                more words than twice the products, never by the
                                 precise policy (whose peak stays C plus O(rows) tables); positive = the
                                 same test under every policy; negative = never.  Products sized on the
                                 device never keep them (their tables are sized for every row) */

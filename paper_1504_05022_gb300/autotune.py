@@ -18,8 +18,7 @@ measured device time, over the parameters the library exposes for that choice:
 * initial_cap  - the first bin-37 row size of the plain (hybrid) policy;
 * predictor_margin - the safety factor of the learned policy;
 * dense_min_u, dense_span_div - which bin-37 rows the dense column slices take;
-* dense_span   - the slices' width (and with it their form: one sum per column of a
-                 narrow slice, or a bitmap with compact sums for a wide one);
+* dense_span   - the slices' width;
 * dense_pred_min - the learned policy's choice of kernel: rows predicted at least this
                  long go to the dense column slices;
 * dense_keep   - whether the slices' counting pass leaves its column bitmaps for the
@@ -63,12 +62,10 @@ SPACE = {
     "initial_cap": [256, 512, 1024],
     "predictor_margin": [None, 1.15, 1.5, 2.0],  # None = the margin stored with the weights
     "dense_min_u": [0, 16384, 8192, 4096, 2048, 1024, -1],  # 0 = the rule of dense_span_div, -1 = no slice rows
-    "dense_span": [0, 65536, 32768, 21856, 16384, 10912],  # 0 = 131,072-column slices (bitmap, compact
-                                                           # sums); narrow enough for a sum per column
-                                                           # (21,856 and below in double): single-pass
-    "dense_span_div": [0, 16, 4, 64],     # 0 = 8: dense when 8 u_i >= the row's column range
+    "dense_span": [0, 65536, 32768, 21856, 16384, 10912],  # 0 = 131,072-column slices
+    "dense_span_div": [0, 8, 64, 256],    # 0 = the default line (32; 8 and 512 for short ranges and long rows)
     "dense_pred_min": [0, 12288, 6144, 3072],  # learned: predicted nnz(c_i) that sends a row to the slices
-    "dense_keep": [0, -1],                # 0 = the count leaves its bitmaps for the compact fill, -1 = never
+    "dense_keep": [0, -1],                # 0 = the count leaves its bitmaps for the fill, -1 = never
 }
 POLICY_PARAMS = {
     "hybrid": ["heap_max_u", "heap_block", "merge_batch", "smem_cap_max", "merge_wide_above", "merge_miss",

@@ -90,12 +90,17 @@ struct BoundOut {
     uint8_t *flag;
     int32_t *lo, *hi;
     int64_t dmin;  // a bin-37 row is dense when u_i >= dmin (dmin > 0),
-    int div;       // else when div u_i >= the width of its column range
+    int div;       // else when div u_i >= the width of its column range and u_i >= floor,
+    int floor;
+    int div_short; // div_short (and no floor) for a range of at most DENSE_SHORT_RANGE columns,
+    int div_long;  // div_long for u_i > DENSE_LONG_U
     int small_u;   // as MergeLaunch::small_u
     int32_t *hist;
     int64_t *part;
     int64_t *err;
 };
+constexpr int64_t DENSE_LONG_U = 8192;  // = MERGE_SMALL_U: longer rows are the batched merge kernel's
+constexpr int64_t DENSE_SHORT_RANGE = 16384;
 int64_t bin_blocks(int64_t m, int64_t nnzA);
 cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, const BoundOut &O, cudaStream_t st);
 // Stage 2: the rows grouped by bin, C~'s row offsets, and the summary (also into `host`, pinned

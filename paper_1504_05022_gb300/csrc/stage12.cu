@@ -165,9 +165,20 @@ SPG_DEV bool dense_row(int b, int64_t i, const CapPolicy &P) {
 // range [lo, hi) (first and last column of every B row they select) and the flag that sends them
 // to the dense-slice kernels: u_i >= dmin (dmin > 0), else div u_i >= hi - lo -- their products
 // cover at least a div-th of the columns they can reach, so the accumulator's O(hi - lo) clearing
-// and write-out are small beside them.  Latency-bound (two dependent gathers per nonzero): the
-// 27-point operator on 64^3 (6.9 M nonzeros) takes 45 us here (cold caches) and took 113 us as a
-// prefix sum, a marking pass and a histogram pass.
+// and write-out are small beside them.  By default div = 32 up to DENSE_LONG_U products, where
+// the register merge kernel is the other way, and 512 above, where it is the batched one.  The
+// product by hybrid / learned plans, ms, at div 8, 32 and 64: R-MAT 2^16 x 16 4.70, 3.64, 3.53 /
+// 3.84, 3.52, 3.55, 2^17 x 8 9.23, 4.38, 3.95 / 5.09, 3.74, 3.73, 2^18 x 8 37.9, 14.6, 10.7 / 27.0,
+// 10.7, 9.78 (at 64 the learned plan, at its peak there, no longer needs less memory than the
+// bound's).  Rows of uniformly random columns are the slices' worst case, merge against slices:
+// u = 2,500 of 200,000 columns (div 80) 18.7, 16.0, u = 1,600 (125) 11.7, 13.8, u = 4,096 of
+// 500,000 (122) 3.86, 5.28; above the line u = 9,216 of 4,000,000 (434) 46.7, 34.3.
+// Rows of fewer than 1,024 products stay with the register merge, where hubs leave it little to
+// gain (R-MAT 2^16 x 16: 3.54 / 3.56), and ranges of at most DENSE_SHORT_RANGE columns at an
+// eighth, the line that small products were always given (R-MAT 2^13 x 16: 0.57 against 0.47).
+// Latency-bound (two dependent gathers per nonzero): the 27-point
+// operator on 64^3 (6.9 M nonzeros) takes 45 us here (cold caches) and took 113 us as a prefix
+// sum, a marking pass and a histogram pass.
 template <int G>
 __global__ void __launch_bounds__(BOUND_NT, 3)
 k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int factor, int64_t nblk) {
@@ -228,7 +239,9 @@ k_bound(DevCSR A, DevCSR B, CapPolicy P, BoundOut O, int R, int factor, int64_t 
         if (P.dense != nullptr) {
             if (b == BIN_MERGE) {
                 const int64_t span = (int64_t)cmax - cmin + 1;  // u > 0, so some B row is not empty
-                dense = O.dmin > 0 ? u >= O.dmin : (int64_t)O.div * u >= span;
+                const int div = u > DENSE_LONG_U ? O.div_long : span > DENSE_SHORT_RANGE ? O.div : O.div_short;
+                dense = O.dmin > 0 ? u >= O.dmin
+                                   : (int64_t)div * u >= span && (span <= DENSE_SHORT_RANGE || u >= O.floor);
                 O.lo[i] = cmin;
                 O.hi[i] = cmax + 1;
             }
@@ -455,7 +468,7 @@ cudaError_t launch_cap_rescan(int64_t m, const int64_t *u, const uint8_t *bin, C
 
 cudaError_t launch_bound(const DevCSR &A, const DevCSR &B, const CapPolicy &P, const BoundOut &O, cudaStream_t st) {
     const int64_t nblk = bin_blocks(A.nrows, A.nnz);
-    if (P.dense != nullptr && O.div < 1) return cudaErrorInvalidValue;
+    if (P.dense != nullptr && (O.div < 1 || O.div_short < 1 || O.div_long < 1)) return cudaErrorInvalidValue;
     if (nblk <= 0) return cudaMemsetAsync(O.err, 0, sizeof(int64_t), st);
     const int64_t rows = bound_rows(A.nrows, A.nnz);
     const int factor = (int)(bin_rows_per_block(A.nrows, A.nnz) / rows);
