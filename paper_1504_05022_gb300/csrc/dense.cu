@@ -625,8 +625,10 @@ k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_co
 // warp holds a sum per column in shared memory and takes the B rows one after another, 32
 // entries at a time: their columns are distinct, so plain fused multiply-adds suffice, and no
 // barrier wider than the warp is needed.  A*A of a band matrix of 50,021 rows and width 40 (80 M
-// products, single precision) takes 73 + 293 us for the count and the sums; a CTA per row
-// took 3.08 ms, and 1.45 ms with the product walk above.  Bound by shared memory and, in double precision, the FP64 pipe.
+// products, single precision) takes 404 us as a whole, 73 of them for the count; 490 us with all
+// sums in shared memory, 3.39 ms with a CTA per row and 1.75 ms with the product walk above.
+// Bound by shared memory (issue where registers hold the sums) and, in double precision, the
+// FP64 pipe.
 // The columns are a bitmap, a word per lane.  A B row whose entries are consecutive columns
 // (last - first + 1 = length, as in a band or a block) sets its bits and finds its columns
 // without reading them, and 32 such rows (a window of A) are summed in registers: lane l holds
