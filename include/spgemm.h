@@ -179,7 +179,7 @@ typedef struct spgemm_opts {
                                 kernel as well as of size); 0 = off */
     int32_t dense_keep;      /* the slices' counting pass leaves every (row, slice)'s column bitmap in
                                 device memory (ceil(W / 32) + 1 words, rounded up to 4, per (row, slice)
-                                of the rows that reach more than 1,024 columns, released when
+                                of the rows that take a CTA per slice, released when
                                 spgemm_numeric returns) and the fill reads it back instead of marking
                                 the columns again.
                                 0 = kept by the hybrid, upper-bound and learned policies when the

@@ -54,44 +54,89 @@ cudaError_t launch_dense_bounds(const DevCSR &B, int K, int W, int32_t *bnd, cud
 }
 
 // ---- selection of the dense rows among the bin-37 rows ----
-// Bucket g = 63 - floor(log2 u) (the leading zeros of u) for a dense row, so that
-// larger rows come first; then the rows that reach few columns (a warp each), in two buckets
-// by width; DENSE_BUCKETS for the others.  order[0..nd) lists the dense items,
-// order[nd..n37) the rest.
+// A dense row's bucket is 64 kind + the leading zeros of u, so that larger rows come first.  Kind 0
+// takes a CTA per slice: the rows of more than DENSE_MID_W columns, and narrower ones whose parts
+// (products per entry of A) a warp would take one by one with most lanes idle, or whose parts are
+// long but scattered.  Kinds 1 and 2, more and at most DENSE_NARROW_W columns, take a warp per row, but
+// for the rows that would outlast the others (k_dense_select_starts).  DENSE_BUCKETS for the rows
+// that are not dense.  order[0..nd) lists the dense items, order[nd..n37) the rest.
+//
+// Product of 30,000 rows by a warp each / by CTAs, ms.  Double, consecutive parts in ranges of 200
+// columns: parts of 2, u = 600 1.44 / 0.92, u = 32,000 66.6 / 16.2; of 8, u = 600 0.55 / 0.75, u = 2,000
+// 1.30 / 0.93; of 16, u = 4,500 1.60 / 1.48 (single precision 1.26 / 1.51), u = 8,000 2.68 / 2.00; of 32
+// and 80, u = 32,000 5.2 / 6.6 and 4.4 / 6.2.  Single precision, scattered parts of 80, u = 2,000, 8,000 and
+// 32,000: of 200 columns 0.84 / 0.97, 2.65 / 1.92 and 9.5 / 5.8, of 1,000 0.69 / 0.97, 1.83 / 1.84 and 5.84 / 5.22.
 
-constexpr int DENSE_BUCKETS = 66;
-SPG_DEV int dense_bucket(int64_t u, int32_t width) {
-    return width > DENSE_MID_W ? __clzll((long long)u) : (width > DENSE_NARROW_W ? 64 : 65);
+constexpr int DENSE_BUCKETS = 3 * 64;
+constexpr int64_t DENSE_SCATTERED = 32;  // products per column from which scattered parts take a CTA
+SPG_DEV int dense_bucket(const DevCSR &A, const DevCSR &B, int row, int64_t u, int32_t width) {
+    const int c = __clzll((long long)u);
+    if (width > DENSE_MID_W) return c;
+    const int64_t a0 = A.rp[row], nA = A.rp[row + 1] - a0;
+    if (u < 4 * nA || (u >= 1536 && u < 12 * nA) || (u >= 6144 && u < 18 * nA)) return c;
+    if (u >= 4096 && u >= DENSE_SCATTERED * width) {  // the part in the middle stands for all
+        const int32_t k = A.col[a0 + nA / 2];
+        const int64_t b0 = B.rp[k], b1 = B.rp[k + 1];
+        if (b1 > b0 && B.col[b1 - 1] - B.col[b0] != b1 - b0 - 1) return c;
+    }
+    return (width > DENSE_NARROW_W ? 64 : 128) + c;
 }
 
-__global__ void k_dense_select_count(const int32_t *bin_rows, int64_t m, const BinSummary *summary, const int64_t *u,
-                                     const uint8_t *flag, const int32_t *lo, const int32_t *hi, int32_t *cls_of,
-                                     int32_t *count) {
+__global__ void k_dense_select_count(DevCSR A, DevCSR B, const int32_t *bin_rows, int64_t m, const BinSummary *summary,
+                                     const int64_t *u, const uint8_t *flag, const int32_t *lo, const int32_t *hi,
+                                     int32_t *cls_of, int32_t *count) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t n37 = summary->bin_count[BIN_MERGE];
     if (j >= n37) return;
     const int32_t row = bin_rows[m - n37 + j];
     const int64_t uu = u[row];
-    const int g = flag[row] ? dense_bucket(uu, hi[row] - lo[row]) : DENSE_BUCKETS;
+    const int g = flag[row] ? dense_bucket(A, B, row, uu, hi[row] - lo[row]) : DENSE_BUCKETS;
     cls_of[j] = g;
     // one add per bucket and warp: most rows fall into few buckets
     const unsigned peers = __match_any_sync(__activemask(), g);
     if (lane_id() == __ffs(peers) - 1) atomicAdd(&count[g], __popc(peers));
 }
 
-__global__ void k_dense_select_starts(const int32_t *count, int32_t *start, int32_t *cursor, BinSummary *summary) {
-    __shared__ int32_t c[DENSE_BUCKETS + 1];
-    if (threadIdx.x <= DENSE_BUCKETS) {
-        c[threadIdx.x] = count[threadIdx.x];
-        cursor[threadIdx.x] = 0;
+// The buckets' places, a thread per size.  A warp per row is as fast as the chip is full of them,
+// about DENSE_FEW_ROWS of equal length.  A row of 2^DENSE_FEW_LOG products or more that is longer than
+// a DENSE_FEW_ROWS-th of all such rows' products takes a CTA per slice.  Product of R rows of u products
+// in parts of 80 consecutive columns out of 200 by a warp each / by CTAs, ms, double: R = 150, u = 2,000 0.15 /
+// 0.19, u = 8,000 0.21 / 0.21, u = 128,000 2.03 / 0.57; R = 1,000 0.15 / 0.19, 0.25 / 0.24 and 2.03 / 1.27; R = 3,000
+// 0.17 / 0.26, 0.28 / 0.39 and 2.06 / 2.69.  A^T A of 10^6 x 64 with 8 entries a row: 97 / 6.3.
+constexpr int DENSE_FEW_ROWS = 2048, DENSE_FEW_LOG = 13;
+
+__global__ void __launch_bounds__(64)
+k_dense_select_starts(const int32_t *count, int32_t *start, int32_t *cursor, BinSummary *summary) {
+    __shared__ int64_t scratch[3];
+    __shared__ double narrow[2];
+    const int z = threadIdx.x;
+    int32_t n[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        n[k] = count[64 * k + z];
+        cursor[64 * k + z] = 0;
     }
+    const double size = ldexp(1.0, 63 - z);
+    const double t = warp_reduce_sum(size * (n[1] + n[2]));
+    if (lane_id() == 0) narrow[warp_id()] = t;
     __syncthreads();
-    if (threadIdx.x <= DENSE_BUCKETS) {
-        int32_t s = 0;
-        for (int g = 0; g < (int)threadIdx.x; ++g) s += c[g];
-        start[threadIdx.x] = s;
-        if (threadIdx.x == DENSE_BUCKETS) summary->dense_count = s;
-        else if (threadIdx.x >= 64) summary->dense_end[threadIdx.x - 64] = s;
+    const bool cta = 63 - z >= DENSE_FEW_LOG && DENSE_FEW_ROWS * size > narrow[0] + narrow[1];
+    // kind 0 (with the moved rows), then kind 1, then kind 2
+    const int64_t w = (int64_t)n[0] + (cta ? n[1] + n[2] : 0);
+    const int64_t rest = cta ? 0 : ((int64_t)n[1] << 32) | n[2];
+    int64_t nw, nr;
+    const int32_t pw = (int32_t)block_exclusive_scan<64>(w, scratch, nw);
+    const int64_t pr = block_exclusive_scan<64>(rest, scratch, nr);
+    const int32_t e0 = (int32_t)nw, e1 = e0 + (int32_t)(nr >> 32), e2 = e1 + (int32_t)(nr & 0xffffffff);
+    start[z] = pw;
+    start[64 + z] = cta ? pw + n[0] : e0 + (int32_t)(pr >> 32);
+    start[128 + z] = cta ? pw + n[0] + n[1] : e1 + (int32_t)(pr & 0xffffffff);
+    if (z == 0) {
+        start[DENSE_BUCKETS] = e2;
+        cursor[DENSE_BUCKETS] = 0;
+        summary->dense_count = e2;
+        summary->dense_end[0] = e0;
+        summary->dense_end[1] = e1;
     }
 }
 
@@ -118,17 +163,18 @@ __global__ void k_dense_select_scatter(const int32_t *bin_rows, int64_t m, const
 
 int64_t dense_select_scratch(int64_t m) { return 3 * (DENSE_BUCKETS + 1) + m; }
 
-cudaError_t launch_dense_select(const int32_t *bin_rows, int64_t m, BinSummary *summary, const int64_t *u,
-                                const uint8_t *flag, const int32_t *lo, const int32_t *hi, int32_t *scratch,
-                                int32_t *order, int32_t *rows, int32_t *rlo, int32_t *rhi, cudaStream_t st) {
+cudaError_t launch_dense_select(const DevCSR &A, const DevCSR &B, const int32_t *bin_rows, BinSummary *summary,
+                                const int64_t *u, const uint8_t *flag, const int32_t *lo, const int32_t *hi,
+                                int32_t *scratch, int32_t *order, int32_t *rows, int32_t *rlo, int32_t *rhi, cudaStream_t st) {
+    const int64_t m = A.nrows;
     if (m <= 0) return cudaSuccess;
     int32_t *count = scratch, *start = count + DENSE_BUCKETS + 1, *cursor = start + DENSE_BUCKETS + 1,
             *cls_of = cursor + DENSE_BUCKETS + 1;
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int32_t) * (DENSE_BUCKETS + 1), st);
     if (e != cudaSuccess) return e;
     const unsigned g = (unsigned)((m + 255) / 256);
-    k_dense_select_count<<<g, 256, 0, st>>>(bin_rows, m, summary, u, flag, lo, hi, cls_of, count);
-    k_dense_select_starts<<<1, 96, 0, st>>>(count, start, cursor, summary);
+    k_dense_select_count<<<g, 256, 0, st>>>(A, B, bin_rows, m, summary, u, flag, lo, hi, cls_of, count);
+    k_dense_select_starts<<<1, 64, 0, st>>>(count, start, cursor, summary);
     k_dense_select_scatter<<<g, 256, 0, st>>>(bin_rows, m, summary, cls_of, start, cursor, lo, hi, order, rows, rlo,
                                               rhi);
     return cudaGetLastError();

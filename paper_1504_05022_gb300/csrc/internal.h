@@ -32,7 +32,8 @@ struct DevCSR {
 };
 
 // Host-visible summary written by stage 2 (copied back in one transfer).
-// Rows of the dense-slice kernels that reach at most so many columns take a warp each.
+// Rows of the dense-slice kernels that reach at most so many columns take a warp each, unless they
+// are long or of short parts (dense_bucket).
 constexpr int DENSE_MID_W = 1024, DENSE_NARROW_W = 256;
 constexpr int NUM_LAUNCH_CLASSES = 8;  // learned: shared-memory classes of bin-37 rows
 
@@ -44,8 +45,8 @@ struct BinSummary {
     int64_t merge_batched;  // bin-37 rows, not flagged dense by stage 1, that k_merge_small cannot take
     int64_t class_count[NUM_LAUNCH_CLASSES];  // learned: bin-37 rows per launch class
     int64_t dense_count;                      // bin-37 rows computed by the dense-slice kernels
-    int64_t dense_end[2];                     // of these, the first [0] reach more than DENSE_MID_W columns,
-                                              // the next up to [1] more than DENSE_NARROW_W
+    int64_t dense_end[2];                     // of these, the first [0] take a CTA per slice, the next up
+                                              // to [1] a warp and reach more than DENSE_NARROW_W columns
     int64_t bin_start[NUM_BINS + 1];          // offsets of the bins in bin_rows (for launches sized on the device)
 };
 
@@ -239,8 +240,8 @@ struct DenseArgs {
     const int32_t *rows;   // their rows of A
     const int32_t *clo;    // and the column range [clo, chi) that each row's products can reach
     const int32_t *chi;
-    int64_t n;             // number of dense items: the first n_wide reach more than DENSE_MID_W
-    int64_t n_wide, n_mid; // columns, those up to n_mid more than DENSE_NARROW_W
+    int64_t n;             // number of dense items: the first n_wide take a CTA per slice, the others a
+    int64_t n_wide, n_mid; // warp per row (those up to n_mid reach more than DENSE_NARROW_W columns)
     int K;                 // column slices of B
     int W;                 // slice width (a multiple of 32); slice s holds columns [s W, (s + 1) W)
     const int32_t *bnd;    // K > 1: per B row, K + 1 offsets of the slices' first entries in the row
@@ -260,9 +261,9 @@ int64_t dense_select_scratch(int64_t m);
 // order[0..nd) = items of the flagged bin-37 rows (the wide ones, larger u first, then the
 // narrow ones), order[nd..n37) = the rest; rows, rlo, rhi [0..nd) = their rows and column
 // ranges; nd and the ends of the wide ones go to the summary
-cudaError_t launch_dense_select(const int32_t *bin_rows, int64_t m, BinSummary *summary, const int64_t *u,
-                                const uint8_t *flag, const int32_t *lo, const int32_t *hi, int32_t *scratch,
-                                int32_t *order, int32_t *rows, int32_t *rlo, int32_t *rhi, cudaStream_t st);
+cudaError_t launch_dense_select(const DevCSR &A, const DevCSR &B, const int32_t *bin_rows, BinSummary *summary,
+                                const int64_t *u, const uint8_t *flag, const int32_t *lo, const int32_t *hi,
+                                int32_t *scratch, int32_t *order, int32_t *rows, int32_t *rlo, int32_t *rhi, cudaStream_t st);
 // counts the columns of every (row, slice) into D.cnt (reads no work-item table, so it
 // may run beside the merge launches)
 cudaError_t launch_dense_count(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t *err, cudaStream_t st);

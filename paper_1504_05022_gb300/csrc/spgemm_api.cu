@@ -943,8 +943,8 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
                 SPG_TRY(p->alloc_n(&p->dense_rows, m));
                 SPG_TRY(p->alloc_n(&p->dense_clo, m));
                 SPG_TRY(p->alloc_n(&p->dense_chi, m));
-                SPG_TRY(launch_dense_select(p->bin_rows, m, p->d_summary, p->u, p->dense_flag, p->dense_lo, p->dense_hi,
-                                            scratch, p->dense_order, p->dense_rows, p->dense_clo, p->dense_chi, p->st));
+                SPG_TRY(launch_dense_select(p->A, p->B, p->bin_rows, p->d_summary, p->u, p->dense_flag, p->dense_lo,
+                                            p->dense_hi, scratch, p->dense_order, p->dense_rows, p->dense_clo, p->dense_chi, p->st));
                 p->count(SPGEMM_K_OTHER, 3);
             }
             SPG_TRY(p->d2h(&p->h_summary, p->d_summary, sizeof(BinSummary)));  // class and slice counts
@@ -2213,7 +2213,7 @@ static cudaError_t precise_count(spgemm_plan *p, bool dev) {
         const cudaStream_t ds = p->stream();
         if (dev) {
             // the slice rows of this run, and B's slice boundaries
-            if ((e = launch_dense_select(p->bin_rows, p->A.nrows, p->d_summary, p->u, p->dense_flag, p->dense_lo,
+            if ((e = launch_dense_select(p->A, p->B, p->bin_rows, p->d_summary, p->u, p->dense_flag, p->dense_lo,
                                          p->dense_hi, p->d_select, p->dense_order, p->dense_rows, p->dense_clo,
                                          p->dense_chi, ds)) != cudaSuccess)
                 return e;
