@@ -226,14 +226,15 @@ spgemm_status spgemm_numeric(spgemm_plan *plan, spgemm_csr_out *C_out);
    the plan itself.  NULL is accepted. */
 spgemm_status spgemm_free(spgemm_plan *plan);
 
-/* Every plan allocates from two stream-ordered memory pools per device (results, temporaries).
-   Blocks freed by earlier plans are kept for reuse: up to half of the device's memory by size,
-   the rest in the pools (no release threshold), so a process that ran a large product keeps
-   holding that device memory.  This returns the unused memory
-   on `device` to the system, keeping at most keep_bytes (cudaMemPoolTrimTo).  Synchronise
-   the streams of the plans freed on that device first: blocks whose stream-ordered free has
-   not run yet are still in use.  SPGEMM_ERR_INVALID_ARG for a negative device or
-   keep_bytes; no-op for a device the library has not allocated on. */
+/* Plans allocate from stream-ordered memory pools of the library (no release threshold).  Freed
+   memory stays in them for later plans, so a process that ran a large product keeps holding that device
+   memory: at most half of the device's beside what plans use.  Any allocation of the process that finds
+   the device full gets the unused memory back from the driver, but for small blocks of 1/256 of the
+   device's memory in all.  This call returns unused memory on `device` to the system until the pools
+   hold at most keep_bytes.  It waits for nothing: synchronise the streams of the plans freed on
+   that device first, since blocks whose stream-ordered free has not run yet are still in use.
+   SPGEMM_ERR_INVALID_ARG for a negative device or keep_bytes; no-op for a device the library has
+   not allocated on. */
 spgemm_status spgemm_pool_trim(int32_t device, int64_t keep_bytes);
 
 /* The bounds-checked build (libspgemm_check.so: the same sources with SPGEMM_CHECK defined).

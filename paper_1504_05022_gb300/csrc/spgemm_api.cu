@@ -2,17 +2,17 @@
 //
 // The host side decides which per-bin kernels run (only non-empty bins), sizes
 // and allocates the temporary matrix C~ and the result C, and drives the
-// progressive relaunch loop of bin 37.  Device memory comes from a
-// library-owned stream-ordered pool (cudaMallocAsync), so every buffer is
+// progressive relaunch loop of bin 37.  Device memory comes from the
+// library's stream-ordered pools (device_memory.h), so every buffer is
 // ordered on the plan's stream and its high-water mark is the peak memory of
 // a call.
 #include "spgemm.h"
 #include "internal.h"
+#include "device_memory.h"
 
 #include <algorithm>
 #include <chrono>
 #include <cstring>
-#include <map>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -21,190 +21,7 @@ using namespace spg;
 
 namespace {
 
-// Two pools per device: what a plan keeps (results and the O(rows) tables) and its temporaries.
-// A large block carved out of freed memory of other sizes makes the pool map it anew, which
-// holds up the host for 0.7 ms per GB: in one pool, C of R-MAT 2^20 x 8 (43 GB) was placed over the
-// slice bitmaps and temporary rows of the call before it (21 GB) and the other way round, 30 ms a
-// product.  Apart, a repeated product finds its own blocks again.
-struct DevicePool {
-    int device;
-    cudaMemPool_t kept, temp;
-    size_t cache_limit;  // bytes of freed blocks kept: half of the device's memory
-};
-
-std::mutex g_pool_mu;
-std::vector<DevicePool> g_pools;
-
-cudaError_t make_pool(int device, cudaMemPool_t *out) {
-    cudaMemPoolProps props;
-    std::memset(&props, 0, sizeof(props));
-    props.allocType = cudaMemAllocationTypePinned;
-    props.handleTypes = cudaMemHandleTypeNone;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = device;
-    cudaError_t e = cudaMemPoolCreate(out, &props);
-    if (e != cudaSuccess) return e;
-    uint64_t thr = UINT64_MAX;  // keep freed blocks for reuse by later calls
-    e = cudaMemPoolSetAttribute(*out, cudaMemPoolAttrReleaseThreshold, &thr);
-    if (e != cudaSuccess) cudaMemPoolDestroy(*out);
-    return e;
-}
-
-cudaError_t get_pools(int device, DevicePool *out) {
-    std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (auto &p : g_pools)
-        if (p.device == device) {
-            *out = p;
-            return cudaSuccess;
-        }
-    DevicePool p{device, nullptr, nullptr, 0};
-    size_t free_b = 0, total_b = 0;
-    cudaError_t e = cudaMemGetInfo(&free_b, &total_b);  // the device is current
-    if (e != cudaSuccess) return e;
-    p.cache_limit = total_b / 2;
-    e = make_pool(device, &p.kept);
-    if (e != cudaSuccess) return e;
-    e = make_pool(device, &p.temp);
-    if (e != cudaSuccess) {
-        cudaMemPoolDestroy(p.kept);
-        return e;
-    }
-    g_pools.push_back(p);
-    *out = p;
-    return cudaSuccess;
-}
-
-// Freed blocks kept for the next call, above the pools: a pool that holds free memory of other
-// sizes maps a large block anew (see above), and a sequence of different products leaves it just
-// that; a batch of 20 pairs after a product with 6 GB of C spent 3.8 of 11.6 ms in it on every
-// call.  A block is taken again by a request of its size (at most an eighth less), on any
-// stream: every block carries an event recorded when it was freed, which the new owner's stream
-// waits for -- at once on the stream that freed it, and on another one only when it has passed,
-// so that streams do not come to wait for each other.  Bounded: CACHE_BLOCKS blocks and half of the
-// device's memory, the longest unused go back to the pool first; all of it goes back when an
-// allocation fails and when the pools are trimmed.
-struct Block {
-    void *ptr = nullptr;
-    size_t bytes = 0;
-    cudaEvent_t freed = nullptr;
-    cudaStream_t st = nullptr;  // where it was freed
-    uint64_t stamp = 0;         // when
-};
-// Per device and pool, by size.
-struct BlockCache {
-    int device;
-    bool temp;
-    std::multimap<size_t, Block> blocks;
-    size_t total;  // their bytes
-};
-constexpr size_t CACHE_BLOCKS = 4096;  // a batch of 512 pairs in 64 waves holds about 2,600
-std::mutex g_cache_mu;
-std::vector<BlockCache> g_caches;
-uint64_t g_cache_clock = 0;
-
-BlockCache &cache_of(int device, bool temp) {  // under g_cache_mu
-    for (BlockCache &c : g_caches)
-        if (c.device == device && c.temp == temp) return c;
-    g_caches.push_back(BlockCache{device, temp, {}, 0});
-    return g_caches.back();
-}
-
-// Sizes in steps of a sixteenth to a thirty-second, so that nearly equal requests share blocks.
-size_t block_size(size_t bytes) {
-    size_t step = 4096;
-    while (step * 32 < bytes) step *= 2;
-    return (bytes + step - 1) / step * step;
-}
-
-// A cached block of `bytes` (a block_size) or a little more for stream st, or false.
-bool cache_take(int device, bool temp, size_t bytes, cudaStream_t st, Block *out) {
-    std::lock_guard<std::mutex> lk(g_cache_mu);
-    BlockCache &cache = cache_of(device, temp);
-    auto &m = cache.blocks;
-    for (auto i = m.lower_bound(bytes); i != m.end() && i->first <= bytes + bytes / 8; ++i) {
-        if (i->second.st != st && cudaEventQuery(i->second.freed) != cudaSuccess) {
-            cudaGetLastError();  // not passed yet
-            continue;
-        }
-        if (cudaStreamWaitEvent(st, i->second.freed, 0) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        *out = i->second;
-        cache.total -= i->first;
-        m.erase(i);
-        return true;
-    }
-    return false;
-}
-
-// Back to the pool, ordered on st.
-void block_free(const Block &b, cudaStream_t st) {
-    cudaStreamWaitEvent(st, b.freed, 0);
-    cudaEventDestroy(b.freed);
-    cudaFreeAsync(b.ptr, st);
-}
-
-// Blocks whose last use is enqueued on st go into the cache; what exceeds the bounds leaves it.
-void cache_put(std::vector<Block> &blocks, int device, bool temp, cudaStream_t st, size_t limit) {
-    std::lock_guard<std::mutex> lk(g_cache_mu);
-    for (Block &b : blocks) {
-        if (b.freed == nullptr && cudaEventCreateWithFlags(&b.freed, cudaEventDisableTiming) != cudaSuccess)
-            b.freed = nullptr;
-        if (b.freed == nullptr || cudaEventRecord(b.freed, st) != cudaSuccess) {
-            cudaGetLastError();
-            if (b.freed) cudaEventDestroy(b.freed);
-            cudaFreeAsync(b.ptr, st);
-            continue;
-        }
-        b.st = st;
-        b.stamp = ++g_cache_clock;
-        BlockCache &c = cache_of(device, temp);
-        c.blocks.emplace(b.bytes, b);
-        c.total += b.bytes;
-    }
-    while (true) {
-        size_t count = 0, total = 0;
-        for (const BlockCache &c : g_caches) {
-            if (c.device != device) continue;
-            count += c.blocks.size();
-            total += c.total;
-        }
-        if (count <= CACHE_BLOCKS && total <= limit) return;
-        BlockCache *from = nullptr;
-        std::multimap<size_t, Block>::iterator oldest;
-        for (BlockCache &c : g_caches) {
-            if (c.device != device) continue;
-            for (auto i = c.blocks.begin(); i != c.blocks.end(); ++i) {
-                if (from != nullptr && i->second.stamp >= oldest->second.stamp) continue;
-                from = &c;
-                oldest = i;
-            }
-        }
-        block_free(oldest->second, st);
-        from->total -= oldest->first;
-        from->blocks.erase(oldest);
-    }
-}
-
-// Every cached block of the device (the current one) back to its pool.
-void cache_drop(int device, cudaStream_t st) {
-    std::lock_guard<std::mutex> lk(g_cache_mu);
-    for (BlockCache &c : g_caches) {
-        if (c.device != device) continue;
-        for (auto &i : c.blocks) block_free(i.second, st);
-        c.blocks.clear();
-        c.total = 0;
-    }
-}
-
-size_t cache_bytes(int device) {
-    std::lock_guard<std::mutex> lk(g_cache_mu);
-    size_t total = 0;
-    for (const BlockCache &c : g_caches)
-        if (c.device == device) total += c.total;
-    return total;
-}
+DeviceMemory g_memory;
 
 // Small pinned host blocks for the few device->host size reads of a call, mapped into the
 // device's address space: a kernel stores the sizes there, so the reads do not go through a
@@ -318,7 +135,6 @@ struct spgemm_plan {
     int device = 0;
     cudaStream_t st = nullptr;
     spgemm_opts opts{};
-    DevicePool pools{};
     DevCSR A{}, B{};
     // Device memory by lifetime (symbolic: stage-1 and binning scratch; numeric: C~, merge pools
     // and lists; plan: the rest).  Small arrays share blocks of CHUNK bytes: a product on a few
@@ -455,25 +271,8 @@ struct spgemm_plan {
     }
     cudaError_t alloc_block(void **p, size_t bytes, int life) {
         const auto t0 = std::chrono::steady_clock::now();
-        const bool temp = life != LIFE_PLAN;
         Block b;
-        cudaError_t e = cudaSuccess;
-        bytes = block_size(bytes);
-        if (!cache_take(device, temp, bytes, st, &b)) {
-            b.bytes = bytes;
-            const cudaMemPool_t pool = temp ? pools.temp : pools.kept;
-            e = cudaMallocFromPoolAsync(&b.ptr, bytes, pool, st);
-            if (e == cudaErrorMemoryAllocation) {
-                // cached blocks and the other pool may hold unused memory: give it back, try once more
-                cudaGetLastError();
-                cache_drop(device, st);
-                if (cudaStreamSynchronize(st) == cudaSuccess) {
-                    cudaMemPoolTrimTo(pools.kept, 0);
-                    cudaMemPoolTrimTo(pools.temp, 0);
-                    e = cudaMallocFromPoolAsync(&b.ptr, bytes, pool, st);
-                }
-            }
-        }
+        const cudaError_t e = g_memory.alloc(device, life != LIFE_PLAN, bytes, false, st, &b);
         stats.alloc_host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         stats.allocs += 1;
         if (e != cudaSuccess) {
@@ -501,7 +300,7 @@ struct spgemm_plan {
     }
     void free_memory(int life) {
         Memory &m = mem[life];
-        if (!m.blocks.empty()) cache_put(m.blocks, device, life != LIFE_PLAN, st, pools.cache_limit);
+        for (const Block &b : m.blocks) g_memory.free(device, b, life != LIFE_PLAN, st);
         bytes_held -= m.bytes;
         m = Memory{};
     }
@@ -792,7 +591,6 @@ static spgemm_status plan_begin(const spgemm_opts *opts, spgemm_stream_t stream,
     spgemm_status status = SPGEMM_OK;
     {
         SPG_TRY(cudaGetDevice(&p->device));
-        SPG_TRY(get_pools(p->device, &p->pools));
         SPG_TRY(cudaDeviceGetAttribute(&p->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
         p->pinned = get_pinned();
         if (!p->pinned) {
@@ -1251,16 +1049,13 @@ static void alloc_dense_keep(spgemm_plan *p) {
     const int64_t words = p->dense_wide * p->dense_K * (int64_t)kw;
     if (words / 2 > p->stats.sum_u) return;
     size_t free_b = 0, total_b = 0;
-    uint64_t reserved = 0, used = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
-        cudaMemPoolGetAttribute(p->pools.temp, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
-        cudaMemPoolGetAttribute(p->pools.temp, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
-    // the pool's unused memory and the cached blocks are free to the plan
-    free_b += (size_t)(reserved - std::min(used, reserved)) + cache_bytes(p->device);
-    if ((uint64_t)words * sizeof(uint32_t) > free_b / 4) return;
+    // the pools' unused memory is free to the plan
+    const uint64_t most = (uint64_t)words * sizeof(uint32_t);
+    if (most > free_b / 4 && most > (free_b + g_memory.unused(p->device)) / 4) return;
     if (p->alloc_n(&p->dense_keep, words, LIFE_NUMERIC) != cudaSuccess) {
         p->dense_keep = nullptr;
         return;
@@ -1642,23 +1437,7 @@ extern "C" spgemm_status spgemm_check_status(int64_t *code_out, int32_t reset) {
 
 extern "C" spgemm_status spgemm_pool_trim(int32_t device, int64_t keep_bytes) {
     if (device < 0 || keep_bytes < 0) return SPGEMM_ERR_INVALID_ARG;
-    DevicePool pools{};
-    {
-        std::lock_guard<std::mutex> lk(g_pool_mu);
-        for (auto &q : g_pools)
-            if (q.device == device) pools = q;
-    }
-    if (pools.kept == nullptr) return SPGEMM_OK;
-    int before = 0;
-    cudaError_t e = cudaGetDevice(&before);
-    if (e == cudaSuccess && before != device) e = cudaSetDevice(device);
-    if (e != cudaSuccess) return from_cuda(e);
-    cache_drop(device, nullptr);
-    e = cudaStreamSynchronize(nullptr);
-    if (e == cudaSuccess) e = cudaMemPoolTrimTo(pools.temp, 0);
-    if (e == cudaSuccess) e = cudaMemPoolTrimTo(pools.kept, (size_t)keep_bytes);
-    if (before != device) cudaSetDevice(before);
-    return from_cuda(e);
+    return from_cuda(g_memory.trim(device, (size_t)keep_bytes));
 }
 
 extern "C" spgemm_status spgemm_free(spgemm_plan *p) {

@@ -345,7 +345,7 @@ class BatchPlan(Plan):
 def pool_trim(device: int = 0, keep_bytes: int = 0) -> None:
     """Returns the device memory that the libraries' pools (double and single precision) keep
     for reuse on `device` to the system, down to keep_bytes each (synchronises the device
-    first)."""
+    first; the call itself waits for nothing)."""
     torch.cuda.synchronize(device)
     for dt in ("f64", "f32"):
         _lib.check(_lib.load(dtype=dt).spgemm_pool_trim(int(device), int(keep_bytes)), "spgemm_pool_trim")
