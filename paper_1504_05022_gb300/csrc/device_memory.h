@@ -17,7 +17,7 @@
 // once on the stream that freed it, on another one only when it has passed, so that streams do
 // not come to wait for each other.
 //
-// Host code only; the plan's device is made current where memory is allocated or trimmed.
+// Host code only; the plan's device is made current for every call.
 #pragma once
 
 #include <cuda_runtime_api.h>
@@ -104,10 +104,11 @@ class DeviceMemory {
 
     // Stream-ordered on st, where the block's last use is.
     void free(int device, Block b, bool temp, cudaStream_t st) {
+        DeviceGuard g(device);
         std::lock_guard<std::mutex> lk(mu_);
         Device &d = devices_[device];
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (b.bytes < CLASS_MIN && b.bytes == block_size(b.bytes) &&
+        if (b.bytes < CLASS_MIN && b.bytes == block_size(b.bytes) && g.error() == cudaSuccess &&
             cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
             (b.freed != nullptr || cudaEventCreateWithFlags(&b.freed, cudaEventDisableTiming) == cudaSuccess) &&
             cudaEventRecord(b.freed, st) == cudaSuccess) {

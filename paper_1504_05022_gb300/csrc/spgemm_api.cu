@@ -393,6 +393,7 @@ struct spgemm_plan {
         return cudaSuccess;
     }
     void release() {
+        DeviceGuard g(device);  // a finaliser runs with any device current, and the default stream is per device
         if (dense_count_done) {
             cudaStreamWaitEvent(st, dense_count_done, 0);
             cudaEventDestroy(dense_count_done);

@@ -189,6 +189,19 @@ static int small_blocks_follow_their_event() {
     return 0;
 }
 
+static int the_plans_device_is_current() {
+    reset();
+    DeviceMemory m;
+    Block a = get(m, 100000, nullptr, false, 1), b = get(m, GB, nullptr, false, 1);
+    CHECK(g_device == 0);
+    m.free(1, a, false, nullptr);  // as a finaliser does, with device 0 current
+    m.free(1, b, false, nullptr);
+    CHECK(g_device == 0 && g_event_errors == 0);
+    CHECK(reinterpret_cast<FakeEvent *>(get(m, 100000, nullptr, false, 1).freed)->device == 1);
+    CHECK(m.trim(1, 0) == cudaSuccess && g_device == 0);
+    return 0;
+}
+
 static int kept_blocks_are_bounded() {
     reset();
     DeviceMemory m;
@@ -293,6 +306,7 @@ int main() {
 #define CASE(f) {#f, f}
         CASE(large_blocks_go_back_to_the_driver),
         CASE(small_blocks_follow_their_event),
+        CASE(the_plans_device_is_current),
         CASE(kept_blocks_are_bounded),
         CASE(a_full_device_is_tried_once_more),
         CASE(trim_waits_for_nothing_and_keeps_what_it_may),
