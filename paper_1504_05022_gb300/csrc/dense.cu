@@ -24,6 +24,7 @@
 // u_i >= 8,192, kept: 129.8 -> 75.9 ms (14.6 -> 25 G B-entries/s through both passes).
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 
 #include <algorithm>
 #include <type_traits>
@@ -913,7 +914,7 @@ static cudaError_t launch_narrow(const DevCSR &A, const DevCSR &B, const DenseAr
     if (n <= 0) return cudaSuccess;
     auto kern = k_dense_narrow<W, FILL, REPLAY>;
     const int smem = FILL ? DN_WARPS * W * (int)sizeof(val_t) : 0;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     const int64_t need = (n + DN_WARPS - 1) / DN_WARPS;
@@ -1006,7 +1007,7 @@ cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs 
     if (e != cudaSuccess) return e;
     // a persistent grid of nt threads per CTA over the items with counts in (cmin, cmax]
     auto go = [&](auto kern, int nt, int smem, int vcap, unsigned long long *q, int cmin, int cmax) -> cudaError_t {
-        cudaError_t x = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t x = allow_dynamic_smem((const void *)kern, smem);
         if (x == cudaSuccess) x = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         if (x != cudaSuccess) return x;
         const int grid = persistent_blocks((const void *)kern, nt, smem, nb);

@@ -9,6 +9,7 @@
 // a warp touch 32 consecutive words and never conflict on a bank.
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 
 namespace spg {
 
@@ -109,7 +110,7 @@ cudaError_t launch_heap_set(const StageArgs &a, const RowSet &R, int slots, int 
     const int64_t need = (R.n + nt - 1) / nt;
     auto go = [&](auto kern) -> cudaError_t {
         if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = allow_dynamic_smem((const void *)kern, (int)smem);
             if (e != cudaSuccess) return e;
         }
         const int64_t grid = R.dev_lo ? persistent_blocks((const void *)kern, nt, smem, need) : need;

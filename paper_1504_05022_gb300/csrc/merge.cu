@@ -27,6 +27,7 @@
 // other sum is taken in a fixed order.
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 #include "scan.cuh"
 
 #include <algorithm>
@@ -626,7 +627,7 @@ template <int NT, int MINB>
 static cudaError_t launch_merge_nt(const StageArgs &a, const MergeItems &s, const MergeLaunch &L, int smem,
                                   cudaStream_t st) {
     auto kern = k_merge<NT, MINB>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;

@@ -28,6 +28,7 @@
 // split; level-1 launches use k_merge.
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 
 #include <algorithm>
 #include <type_traits>
@@ -597,7 +598,7 @@ template <int NT, int MINB, bool TWO>
 static cudaError_t launch_bm_nt(const StageArgs &a, const MergeItems &s, const MergeLaunch &L, int smem,
                                 cudaStream_t st) {
     auto kern = k_merge_bm<NT, MINB, TWO>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;

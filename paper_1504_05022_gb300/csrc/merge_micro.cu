@@ -12,6 +12,7 @@
 // and merge path); the bitonic network does not keep that order.
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 
 #include <type_traits>
 
@@ -113,7 +114,7 @@ static cudaError_t micro_launch(int method, const int32_t *keys, const void *val
     const int smem = merge_micro_smem(l, VB);
     auto kern = method == 0 ? k_merge_micro<NT, VB, 0> : (method == 1 ? k_merge_micro<NT, VB, 1>
                                                                       : k_merge_micro<NT, VB, 2>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)groups, NT, smem, st>>>(keys, vals, l, okeys, ovals);
     return cudaGetLastError();

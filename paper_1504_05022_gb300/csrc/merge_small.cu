@@ -22,6 +22,7 @@
 // products because 512 threads of 16 are the most that share an SM twice.
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 
 namespace spg {
 
@@ -242,7 +243,7 @@ template <int NT, int MINB>
 static cudaError_t launch_ms(const StageArgs &a, const MergeItems &s, const MergeLaunch &L, cudaStream_t st) {
     auto kern = k_merge_small<NT, MINB>;
     const int smem = ms_smem(NT, a.B.ncols);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)L.nwork, NT, smem, st>>>(a, s, L, ms_words(a.B.ncols));

@@ -10,6 +10,7 @@
 #include "spgemm.h"
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 
 #include <new>
 
@@ -614,8 +615,7 @@ extern "C" spgemm_status spgemm_mlp_loss_grad(const float *params, const float *
     const int ctas = (int)(tiles < MLP_MAX_CTAS ? tiles : MLP_MAX_CTAS);
     static_assert((int64_t)MLP_TILE * MLP_WORK >= 2 * MLP_PART, "the partials of n > MLP_TILE samples fit");
     if (ctas > 1 && reinterpret_cast<uintptr_t>(work) % 8 != 0) work += 1;  // 4-byte aligned: one float is spare
-    if (cudaFuncSetAttribute(k_mlp_loss_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(MlpShared)) !=
-        cudaSuccess)
+    if (allow_dynamic_smem((const void *)k_mlp_loss_grad, (int)sizeof(MlpShared)) != cudaSuccess)
         return SPGEMM_ERR_CUDA;
     k_mlp_loss_grad<<<ctas, MLP_NT, sizeof(MlpShared), st>>>(params, X, cls, y, n, work, grad, loss);
     if (ctas > 1) k_mlp_grad_sum<<<(SPGEMM_MLP_NUM_PARAMS + 63) / 64, 512, 0, st>>>(work, ctas, grad, loss);

@@ -9,6 +9,7 @@
 // graph.
 #include "internal.h"
 #include "common.cuh"
+#include "dynamic_smem.h"
 
 namespace spg {
 
@@ -233,7 +234,7 @@ template <int NT>
 static cudaError_t launch_replay_nt(const StageArgs &a, const ReplayLeaves &lv, const int32_t *order, int64_t n,
                                    int32_t *c_col, val_t *c_val, int64_t *err, int smem, cudaStream_t st) {
     auto kern = k_replay<NT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)n, NT, smem, st>>>(a, lv, order, c_col, c_val, err);
     return cudaGetLastError();
@@ -244,7 +245,7 @@ static cudaError_t launch_replay_bm_nt(const StageArgs &a, const ReplayLeaves &l
                                       int nwords, int32_t *c_col, val_t *c_val, int64_t *err, int smem,
                                       cudaStream_t st) {
     auto kern = k_replay_bm<NT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)n, NT, smem, st>>>(a, lv, order, nwords, c_col, c_val, err);
     return cudaGetLastError();
