@@ -188,8 +188,9 @@ typedef struct spgemm_opts {
                                 precise policy (whose peak stays C plus O(rows) tables); positive = the
                                 same test under every policy; negative = never.  Products sized on the
                                 device never keep them (their tables are sized for every row) */
-    int64_t max_bytes;       /* device bytes the plan may hold at once (0 = no limit): an allocation
-                                that would exceed it fails as if the device were full and the call
+    int64_t max_bytes;       /* device bytes the plan may hold at once (0 = no limit; with one, every
+                                array is a block of just its bytes, which costs a small product some
+                                time): an allocation that would exceed it fails as if the device were full and the call
                                 returns SPGEMM_ERR_OOM (the kept bitmaps of dense_keep are skipped
                                 instead).  A failed spgemm_symbolic leaves nothing allocated; a
                                 failed spgemm_numeric leaves its temporaries with the plan until
@@ -273,11 +274,13 @@ typedef struct spgemm_stats {
     int64_t rows_split;         /* column splits of long rows (SPGEMM_LONG_ROWS_SPLIT) */
     int64_t rows_fallback;      /* rows recomputed because a prediction was too small */
     int64_t bytes_ctilde;       /* device bytes allocated for temporary rows (all rounds) */
-    int64_t peak_bytes;         /* high-water mark of the device bytes held by the plan (temporaries
-                                   and C) from spgemm_symbolic on */
+    int64_t peak_bytes;         /* high-water mark of the device bytes of the plan's arrays (temporaries
+                                   and C) from spgemm_symbolic on.  Without max_bytes the blocks that
+                                   hold them are up to 1/16 larger (reused ones below 128 MB up to
+                                   1/8), and arrays of up to 64 KB share blocks of 512 KB */
     int32_t launches[SPGEMM_K_COUNT];  /* kernels launched per class */
     float kernel_ms[SPGEMM_K_COUNT];   /* summed event time per class (record_timing = 1) */
-    int64_t held_bytes;         /* device bytes the plan holds now: stage-1/2 scratch is released
+    int64_t held_bytes;         /* device bytes of the plan's arrays now: stage-1/2 scratch is released
                                    when spgemm_symbolic returns and C~ with the merge pools when
                                    spgemm_numeric returns (stream-ordered), so after the product
                                    this is C plus the O(rows) tables that values-only replay uses */

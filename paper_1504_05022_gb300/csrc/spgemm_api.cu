@@ -125,9 +125,6 @@ const struct {
 constexpr int64_t ENTRY_BYTES = sizeof(int32_t) + sizeof(val_t);
 
 // Lifetimes of plan allocations.
-constexpr int LIFE_SYMBOLIC = 0;  // released when spgemm_symbolic returns
-constexpr int LIFE_NUMERIC = 1;   // released when spgemm_numeric returns
-constexpr int LIFE_PLAN = 2;      // released by spgemm_free
 
 }  // namespace
 
@@ -136,20 +133,8 @@ struct spgemm_plan {
     cudaStream_t st = nullptr;
     spgemm_opts opts{};
     DevCSR A{}, B{};
-    // Device memory by lifetime (symbolic: stage-1 and binning scratch; numeric: C~, merge pools
-    // and lists; plan: the rest).  Small arrays share blocks of CHUNK bytes: a product on a few
-    // thousand rows makes 5 allocations instead of 21, which had taken a sixth of its time.
-    struct Memory {
-        std::vector<Block> blocks;
-        int64_t bytes = 0;        // requested
-        char *open = nullptr;     // rest of the last shared block
-        size_t room = 0;
-    };
-    Memory mem[3];
-    static constexpr size_t CHUNK = 512 * 1024, SMALL = 64 * 1024;
+    PlanMemory mem;
     int64_t bytes_ctilde = 0;
-    int64_t bytes_held = 0;  // device bytes the plan holds now
-    int64_t bytes_peak = 0;  // largest bytes_held so far
     // stage 1-2 buffers
     int64_t *u = nullptr, *ctil_rp = nullptr, *scan_partial = nullptr;
     uint8_t *bin = nullptr;
@@ -235,54 +220,16 @@ struct spgemm_plan {
     int smem_optin = 0;
 
     cudaError_t alloc(void **p, size_t bytes, int life = LIFE_PLAN) {
-        if (bytes == 0) bytes = 16;
-        if (opts.max_bytes > 0 && bytes_held + (int64_t)bytes > opts.max_bytes) {
-            *p = nullptr;
-            return cudaErrorMemoryAllocation;
-        }
-        Memory &m = mem[life];
-        const size_t need = (bytes + 255) & ~size_t(255);
-        cudaError_t e = cudaSuccess;
-        if (need > SMALL) {
-            e = alloc_block(p, bytes, life);
-        } else {
-            if (m.room < need) {
-                void *q = nullptr;
-                e = alloc_block(&q, CHUNK, life);
-                if (e == cudaSuccess) {
-                    m.open = static_cast<char *>(q);
-                    m.room = CHUNK;
-                }
-            }
-            if (e == cudaSuccess) {
-                *p = m.open;
-                m.open += need;
-                m.room -= need;
-            }
-        }
-        if (e != cudaSuccess) {
-            *p = nullptr;
-            return e;
-        }
-        m.bytes += (int64_t)bytes;
-        bytes_held += (int64_t)bytes;
-        bytes_peak = std::max(bytes_peak, bytes_held);
-        return cudaSuccess;
-    }
-    cudaError_t alloc_block(void **p, size_t bytes, int life) {
         const auto t0 = std::chrono::steady_clock::now();
-        Block b;
-        const cudaError_t e = g_memory.alloc(device, life != LIFE_PLAN, bytes, false, st, &b);
-        stats.alloc_host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-        stats.allocs += 1;
-        if (e != cudaSuccess) {
-            *p = nullptr;
-            cudaGetLastError();
-            return e;
+        const int64_t before = mem.blocks;
+        mem.limit = opts.max_bytes;
+        const cudaError_t e = mem.alloc(g_memory, device, st, bytes, life, p);
+        if (e != cudaSuccess) cudaGetLastError();
+        if (mem.blocks != before) {
+            stats.allocs += mem.blocks - before;
+            stats.alloc_host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
-        *p = b.ptr;
-        mem[life].blocks.push_back(b);
-        return cudaSuccess;
+        return e;
     }
     template <typename T>
     cudaError_t alloc_n(T **p, int64_t n, int life = LIFE_PLAN) {
@@ -298,12 +245,7 @@ struct spgemm_plan {
         *col = q ? reinterpret_cast<int32_t *>(static_cast<char *>(q) + vb) : nullptr;
         return e;
     }
-    void free_memory(int life) {
-        Memory &m = mem[life];
-        for (const Block &b : m.blocks) g_memory.free(device, b, life != LIFE_PLAN, st);
-        bytes_held -= m.bytes;
-        m = Memory{};
-    }
+    void free_memory(int life) { mem.release(g_memory, device, st, life); }
     // Frees (stream-ordered) every temporary whose life ends at or before `life`.
     void release_temps(int life) {
         for (int l = 0; l <= life && l < LIFE_PLAN; ++l) free_memory(l);
@@ -413,7 +355,6 @@ struct spgemm_plan {
         timers.clear();
         drop_branches();
         for (int l = 0; l < 3; ++l) free_memory(l);
-        bytes_held = 0;
         put_pinned(pinned);
         pinned = nullptr;
     }
@@ -1459,8 +1400,8 @@ extern "C" spgemm_status spgemm_plan_stats(spgemm_plan *p, spgemm_stats *out) {
             if (t.a && t.b && cudaEventElapsedTime(&ms, t.a, t.b) == cudaSuccess) p->stats.kernel_ms[t.kind] += ms;
         }
     }
-    p->stats.peak_bytes = p->bytes_peak;
-    p->stats.held_bytes = p->bytes_held;
+    p->stats.peak_bytes = p->mem.peak;
+    p->stats.held_bytes = p->mem.held;
     *out = p->stats;
     for (spgemm_plan *w : p->waves) {  // wave mode: sums over the waves
         spgemm_stats ws;
@@ -1672,7 +1613,7 @@ static spgemm_status batched_numeric_waves(spgemm_plan *p, spgemm_csr_out *C_out
     spgemm_opts o = p->opts;
     o.wave_mproducts = -1;
     int64_t held_before = 0;
-    for (spgemm_plan *w : p->waves) held_before += w->bytes_held;
+    for (spgemm_plan *w : p->waves) held_before += w->mem.held;
     const int nw = (int)p->wave_start.size() - 1;
     std::vector<spgemm_csr_out> outs(p->npairs);
     for (int w = 0; w < nw; ++w) {
@@ -1686,8 +1627,8 @@ static spgemm_status batched_numeric_waves(spgemm_plan *p, spgemm_csr_out *C_out
             p->waves.push_back(sub);
             st = spgemm_batched_numeric(sub, outs.data() + s0);
             if (st != SPGEMM_OK) return st;
-            p->bytes_peak = std::max(p->bytes_peak, held_before + sub->bytes_peak);
-            held_before += sub->bytes_held;
+            p->mem.peak = std::max(p->mem.peak, held_before + sub->mem.peak);
+            held_before += sub->mem.held;
         } else {
             st = spgemm_batched_numeric(p->waves[w], outs.data() + s0);  // finished earlier
             if (st != SPGEMM_OK) return st;
@@ -2378,7 +2319,7 @@ extern "C" spgemm_status spgemm_dplan_result(spgemm_dplan *d, spgemm_csr_out *C_
 
 extern "C" spgemm_status spgemm_dplan_bytes(spgemm_dplan *d, int64_t *bytes) {
     if (!d || !d->p || !bytes) return SPGEMM_ERR_INVALID_ARG;
-    *bytes = d->p->bytes_held;
+    *bytes = d->p->mem.held;
     return SPGEMM_OK;
 }
 

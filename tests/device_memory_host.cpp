@@ -298,6 +298,57 @@ static int exact_blocks_are_of_just_their_bytes() {
     return 0;
 }
 
+static size_t live_bytes() {
+    size_t n = 0;
+    for (auto &a : g_allocs) n += a.second.bytes;
+    return n;
+}
+
+// A plan's arrays: several small ones, a middling and a large one, per lifetime.
+static const size_t kArrays[] = {16, 4000, 64 * 1024, 64 * 1024 + 1, 700001, 3 * MB + 5, 300 * MB + 77};
+
+static int a_plans_limit_is_of_the_memory_itself() {
+    reset();
+    DeviceMemory m;
+    spg::PlanMemory warm;  // leaves kept blocks of nearly these sizes, some a little larger
+    void *p = nullptr;
+    for (int life = 0; life < 3; ++life)
+        for (size_t n : kArrays) CHECK(warm.alloc(m, 0, S(1), n + n / 16, life, &p) == cudaSuccess);
+    for (int life = 0; life < 3; ++life) warm.release(m, 0, S(1), life);
+    CHECK(warm.held == 0);
+    const size_t idle = live_bytes();
+    size_t all = 0;
+    for (size_t n : kArrays) all += 3 * n;
+    spg::PlanMemory plan;
+    plan.limit = (int64_t)all;  // fits exactly
+    for (int life = 0; life < 3; ++life)
+        for (size_t n : kArrays) {
+            CHECK(plan.alloc(m, 0, S(1), n, life, &p) == cudaSuccess && p != nullptr);
+            CHECK(live_bytes() - idle <= (size_t)plan.limit && (size_t)plan.held == live_bytes() - idle);
+        }
+    CHECK(plan.alloc(m, 0, S(1), 1, 0, &p) == cudaErrorMemoryAllocation && p == nullptr);
+    plan.release(m, 0, S(1), 0);
+    CHECK(plan.alloc(m, 0, S(1), all / 3, 1, &p) == cudaSuccess && plan.peak == plan.limit);
+    spg::PlanMemory tiny;  // less than a shared block
+    tiny.limit = 10000;
+    const size_t before = live_bytes();
+    CHECK(tiny.alloc(m, 0, S(1), 4000, 2, &p) == cudaSuccess && tiny.alloc(m, 0, S(1), 4000, 0, &p) == cudaSuccess);
+    CHECK(live_bytes() - before <= 10000);
+    return 0;
+}
+
+static int without_a_limit_blocks_are_little_larger() {
+    reset();
+    DeviceMemory m;
+    spg::PlanMemory plan;
+    void *p = nullptr;
+    for (int k = 0; k < 40; ++k)
+        for (int life = 0; life < 3; ++life) CHECK(plan.alloc(m, 0, S(1), kArrays[k % 7], life, &p) == cudaSuccess);
+    CHECK(live_bytes() <= (size_t)plan.held + (size_t)plan.held / 16 + 3 * 512 * 1024 + 120 * 4096);
+    CHECK(plan.blocks < 90);  // the small ones share
+    return 0;
+}
+
 int main() {
     const struct {
         const char *name;
@@ -313,6 +364,8 @@ int main() {
         CASE(pools_hold_at_most_half_for_others),
         CASE(a_free_inside_a_capture_keeps_nothing),
         CASE(exact_blocks_are_of_just_their_bytes),
+        CASE(a_plans_limit_is_of_the_memory_itself),
+        CASE(without_a_limit_blocks_are_little_larger),
     };
     for (auto &c : cases) {
         g_case = c.name;

@@ -1,6 +1,7 @@
 """The plans' device memory (csrc/device_memory.h) on a fake CUDA runtime, compiled for the host:
 which freed memory the driver gets back at once, which small blocks are kept and for whom, the
-bounds and the order of eviction, a full device, trimming, and another device being current."""
+bounds and the order of eviction, a full device, trimming, another device being current, and that a
+plan's limit bounds the memory it really holds."""
 import os
 import shutil
 import subprocess
@@ -23,4 +24,4 @@ def test_on_a_fake_runtime(tmp_path):
     assert r.returncode == 0, r.stderr[-3000:]
     r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
-    assert r.stdout.count(": ok") == 9
+    assert r.stdout.count(": ok") == 11
