@@ -83,7 +83,7 @@ SPG_DEV int dense_bucket(const DevCSR &A, const DevCSR &B, int row, int64_t u, i
     return (width > DENSE_NARROW_W ? 64 : 128) + c;
 }
 
-__global__ void k_dense_select_count(DevCSR A, DevCSR B, const int32_t *bin_rows, int64_t m, const BinSummary *summary,
+__global__ void k_dense_select_count(DevCSR A, DevCSR B, const int32_t *bin_rows, int64_t m, BinSummary *summary,
                                      const int64_t *u, const uint8_t *flag, const int32_t *lo, const int32_t *hi,
                                      int32_t *cls_of, int32_t *count) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -94,8 +94,14 @@ __global__ void k_dense_select_count(DevCSR A, DevCSR B, const int32_t *bin_rows
     const int g = flag[row] ? dense_bucket(A, B, row, uu, hi[row] - lo[row]) : DENSE_BUCKETS;
     cls_of[j] = g;
     // one add per bucket and warp: most rows fall into few buckets
-    const unsigned peers = __match_any_sync(__activemask(), g);
+    const unsigned act = __activemask();
+    const unsigned peers = __match_any_sync(act, g);
     if (lane_id() == __ffs(peers) - 1) atomicAdd(&count[g], __popc(peers));
+    // A's entries in the rows of kind 0 (fewer than 2^31 in a row: summed in halves of 16 bits)
+    const uint32_t nA = g < 64 ? (uint32_t)(A.rp[row + 1] - A.rp[row]) : 0u;
+    const uint32_t low = __reduce_add_sync(act, nA & 0xffffu), high = __reduce_add_sync(act, nA >> 16);
+    if (lane_id() == __ffs(act) - 1 && (low | high) != 0u)
+        atomicAdd((unsigned long long *)&summary->dense_entries, ((unsigned long long)high << 16) + low);
 }
 
 // The buckets' places, a thread per size.  A warp per row is as fast as the chip is full of them,
@@ -206,7 +212,7 @@ struct DenseWin {
 // Builds the table of the entries [e, min(e + NT, a1)); returns the number of products (a
 // part has at most DENSE_W_MAX entries, so the window's products fit 32 bits).  Its first
 // barrier ends the use of the previous window; the table is ready when it returns.
-template <int NT, bool VALS>
+template <int NT, bool VALS, bool TAB>
 SPG_DEV int dense_window(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int s, int64_t e, int64_t a1,
                          DenseWin<NT> &w) {
     static_assert((int64_t)NT * DENSE_W_MAX < INT32_MAX, "products of a window");
@@ -218,11 +224,16 @@ SPG_DEV int dense_window(const DevCSR &A, const DevCSR &B, const DenseArgs &D, i
         const int32_t k = A.col[i];
         if (VALS) av = A.val[i];
         const int64_t rs = B.rp[k];
-        if (D.K > 1) {
+        if (TAB && D.K > 1) {
             const int32_t *bk = D.bnd + (int64_t)k * (D.K + 1) + s;
             const int32_t b0 = bk[0];
             bs = rs + b0;
             len = bk[1] - b0;
+        } else if (!TAB) {  // the part is searched for
+            const int n = (int)(B.rp[k + 1] - rs);
+            const int b0 = s > 0 ? lower_bound_i32(B.col + rs, n, (int32_t)((int64_t)s * D.W)) : 0;
+            bs = rs + b0;
+            len = s + 1 < D.K ? lower_bound_i32(B.col + bs, n - b0, (int32_t)((int64_t)(s + 1) * D.W)) : n - b0;
         } else {
             bs = rs;
             len = (int)(B.rp[k + 1] - rs);
@@ -323,13 +334,13 @@ SPG_DEV int dense_span(const DevCSR &B, const DenseArgs &D, int64_t d, int s, in
 // Marks the column offset x of every product of the row in the slice with mark(x).  Returns
 // whether a column lay outside [lo, lo + span) (cannot happen: the slice boundaries select
 // the columns); a barrier must follow before the marks are read.
-template <int NT, typename M>
+template <int NT, bool TAB, typename M>
 SPG_DEV bool dense_mark_columns(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int row, int s, int64_t lo,
                                 int span, DenseWin<NT> &win, M mark) {
     bool bad = false;
     const int64_t a0 = A.rp[row], a1 = A.rp[row + 1];
     for (int64_t e = a0; e < a1; e += NT) {
-        const int T = dense_window<NT, false>(A, B, D, s, e, a1, win);
+        const int T = dense_window<NT, false, TAB>(A, B, D, s, e, a1, win);
         dense_walk<NT, false>(win, T, [&](const int64_t *p, const val_t *, const bool *ok, auto full) {
             int32_t c[DENSE_UN];
 #pragma unroll
@@ -350,7 +361,7 @@ SPG_DEV bool dense_mark_columns(const DevCSR &A, const DevCSR &B, const DenseArg
 // ---- pass 1: the number of columns of every (row, slice) ----
 // Shared memory: the slice's column bitmap (one bit per column), then its popcount.  Bound by
 // the gather of B's columns and the shared atomics on the bitmap.
-template <int NT>
+template <int NT, bool TAB>
 SPG_DEV void dense_count_item(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t b, int64_t *err) {
     extern __shared__ __align__(16) uint32_t dc_bm[];
     __shared__ DenseWin<NT> win;
@@ -367,7 +378,7 @@ SPG_DEV void dense_count_item(const DevCSR &A, const DevCSR &B, const DenseArgs 
     uint4 *b4 = reinterpret_cast<uint4 *>(dc_bm);
     for (int q = threadIdx.x; q < ng; q += NT) b4[q] = make_uint4(0u, 0u, 0u, 0u);
     // (the first window's barriers come before the first mark)
-    const bool bad = dense_mark_columns<NT>(A, B, D, D.rows[d], s, lo, span, win,
+    const bool bad = dense_mark_columns<NT, TAB>(A, B, D, D.rows[d], s, lo, span, win,
                                             [&](int x) { atomicOr(&dc_bm[x >> 5], 1u << (x & 31)); });
     __syncthreads();
     int n = 0;
@@ -382,14 +393,14 @@ SPG_DEV void dense_count_item(const DevCSR &A, const DevCSR &B, const DenseArgs 
     if (threadIdx.x == 0) D.cnt[b] = n;
 }
 
-template <int NT>
+template <int NT, bool TAB>
 __global__ void __launch_bounds__(NT, 1536 / NT)
 k_dense_count(DevCSR A, DevCSR B, DenseArgs D, int64_t *err) {
     __shared__ int64_t s_b;
     unsigned long long *q = D.dev_end != nullptr ? D.queue : nullptr;
     const int64_t nb = dense_items(D);
     for (int64_t b = dense_next(q, 0, true, &s_b); b < nb; b = dense_next(q, b, false, &s_b))
-        dense_count_item<NT>(A, B, D, b, err);
+        dense_count_item<NT, TAB>(A, B, D, b, err);
 }
 
 // One thread per dense item: the slices' offsets inside the row and the row's length.
@@ -475,7 +486,7 @@ SPG_DEV bool dense_index(uint2 *idx, int nwords, int32_t *scan32, S src, E enter
 
 // REPLAY: values-only replay; C's columns are already in place, so the bitmap is built
 // from the slice's known entries of C and only the values are written.
-template <int NT, bool REPLAY, bool SHV>
+template <int NT, bool REPLAY, bool SHV, bool TAB>
 SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &D, int64_t b, const int64_t *c_rp,
                              int32_t *c_col, val_t *c_val, int64_t *err, int vcap) {
     extern __shared__ __align__(16) unsigned char df_smem[];
@@ -508,7 +519,7 @@ SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &
                 else bad = true;  // C's columns were changed since the product
             }
         } else {
-            bad = dense_mark_columns<NT>(A, B, D, row, s, lo, span, win, mark);
+            bad = dense_mark_columns<NT, TAB>(A, B, D, row, s, lo, span, win, mark);
         }
         __syncthreads();
     }
@@ -576,7 +587,7 @@ SPG_DEV void dense_fill_item(const DevCSR &A, const DevCSR &B, const DenseArgs &
         }
         const int x0 = w0 << 5, x1 = min(span, w1 << 5);
         for (int64_t e = a0; e < a1; e += NT) {
-            const int T = dense_window<NT, true>(A, B, D, s, e, a1, win);
+            const int T = dense_window<NT, true, TAB>(A, B, D, s, e, a1, win);
             dense_walk<NT, true>(win, T, [&](const int64_t *p, const val_t *a, const bool *ok, auto full) {
                 int32_t c[DENSE_UN];
                 val_t v[DENSE_UN];
@@ -627,7 +638,7 @@ SPG_DEV int64_t dense_run(int64_t t, int64_t ctas, int &len) {
 // A persistent grid over the items whose count lies in (cmin, cmax].  A CTA takes a run of
 // consecutive items from the work counter, looks at all their counts at once and fills the
 // ones that are its own.
-template <int NT, int MINB, bool REPLAY, bool SHV>
+template <int NT, int MINB, bool REPLAY, bool SHV, bool TAB>
 __global__ void __launch_bounds__(NT, MINB)
 k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_col, val_t *c_val, int64_t *err,
              const int64_t *gate, int vcap, unsigned long long *counter, int cmin, int cmax) {
@@ -660,7 +671,7 @@ k_dense_fill(DevCSR A, DevCSR B, DenseArgs D, const int64_t *c_rp, int32_t *c_co
             // way into L2 while this item is filled
             if (threadIdx.x == 0 && !REPLAY && D.keep != nullptr && mask)
                 prefetch_l2(D.keep + (base + __ffs(mask) - 1) * (int64_t)D.keep_words, 4u * (uint32_t)D.keep_words);
-            dense_fill_item<NT, REPLAY, SHV>(A, B, D, b, c_rp, c_col, c_val, err, vcap);
+            dense_fill_item<NT, REPLAY, SHV, TAB>(A, B, D, b, c_rp, c_col, c_val, err, vcap);
             __syncthreads();  // the item's shared memory is free
         }
         __syncthreads();  // every thread has read the run before the next one
@@ -951,6 +962,9 @@ __global__ void k_dense_rowsum(DenseArgs D, int32_t *nnzc) {
 constexpr int DENSE_NT = 256;
 constexpr int DENSE_FEW = 4096;  // entries of a (row, slice) filled by the smaller CTAs in double
 
+// The parts' places come from the table (or one slice holds whole rows), else from searches.
+static bool dense_tabled(const DenseArgs &D) { return D.K == 1 || D.bnd != nullptr; }
+
 int dense_keep_words(int W) { return dense_nw4(W); }  // a multiple of 4: every item's bitmap starts on a 16-byte boundary
 
 static cudaError_t dense_check(const DevCSR &B, const DenseArgs &D) {
@@ -967,7 +981,7 @@ cudaError_t launch_dense_count(const DevCSR &A, const DevCSR &B, const DenseArgs
     if (e == cudaSuccess) e = launch_narrow_rows<false, false>(A, B, D, nullptr, nullptr, nullptr, err, nullptr, st);
     if (e != cudaSuccess || nb <= 0) return e;
     const int smem = (int)(sizeof(uint32_t) * dense_nw4(D.W));
-    auto kern = k_dense_count<DENSE_NT>;
+    auto kern = dense_tabled(D) ? k_dense_count<DENSE_NT, true> : k_dense_count<DENSE_NT, false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     int64_t grid = nb;
@@ -993,9 +1007,9 @@ cudaError_t launch_dense_rows(const MergeItems &it, const DenseArgs &D, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs &D, const int64_t *c_rp,
-                              int32_t *c_col, val_t *c_val, int64_t *err, cudaStream_t st, bool replay,
-                              const int64_t *gate) {
+template <bool TAB>
+static cudaError_t launch_fill(const DevCSR &A, const DevCSR &B, const DenseArgs &D, const int64_t *c_rp, int32_t *c_col,
+                               val_t *c_val, int64_t *err, cudaStream_t st, bool replay, const int64_t *gate) {
     if (D.n <= 0) return cudaSuccess;
     cudaError_t e = dense_check(B, D);
     if (e == cudaSuccess)
@@ -1021,11 +1035,11 @@ cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs 
         // in flight, since their sums must stay in L2 while they are added to (16 k entries per
         // row, R-MAT 2^16 x 16: 1.62 ms at 304 CTAs, 2.34 at 608, 2.90 at 760; 3.2 k entries, 2^18 x
         // 8: 10.2 ms at 304, 8.8 at 608)
-        e = replay ? go(k_dense_fill<256, 4, true, false>, 256, index, 0, D.queue + 1, 0, DENSE_FEW)
-                   : go(k_dense_fill<256, 4, false, false>, 256, index, 0, D.queue + 1, 0, DENSE_FEW);
+        e = replay ? go(k_dense_fill<256, 4, true, false, TAB>, 256, index, 0, D.queue + 1, 0, DENSE_FEW)
+                   : go(k_dense_fill<256, 4, false, false, TAB>, 256, index, 0, D.queue + 1, 0, DENSE_FEW);
         if (e != cudaSuccess || D.W <= DENSE_FEW) return e;  // a slice has at most W entries
-        return replay ? go(k_dense_fill<512, 2, true, false>, 512, index, 0, D.queue + 2, DENSE_FEW, INT32_MAX)
-                      : go(k_dense_fill<512, 2, false, false>, 512, index, 0, D.queue + 2, DENSE_FEW, INT32_MAX);
+        return replay ? go(k_dense_fill<512, 2, true, false, TAB>, 512, index, 0, D.queue + 2, DENSE_FEW, INT32_MAX)
+                      : go(k_dense_fill<512, 2, false, false, TAB>, 512, index, 0, D.queue + 2, DENSE_FEW, INT32_MAX);
     } else {
         // sums in shared memory: the items whose entries fit a quarter of an SM's shared memory at
         // four CTAs of 256 threads per SM, those that fit a half at two of 512, the rest at one of 1,024
@@ -1037,17 +1051,24 @@ cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs 
         const int v4 = room(4, 256), v2 = room(2, 512), v1 = room(1, 1024);
         if (v4 < 32) return cudaErrorInvalidValue;
         const int fs = (int)sizeof(val_t);
-        e = replay ? go(k_dense_fill<256, 4, true, true>, 256, index + v4 * fs, v4, D.queue + 1, 0, v4)
-                   : go(k_dense_fill<256, 4, false, true>, 256, index + v4 * fs, v4, D.queue + 1, 0, v4);
+        e = replay ? go(k_dense_fill<256, 4, true, true, TAB>, 256, index + v4 * fs, v4, D.queue + 1, 0, v4)
+                   : go(k_dense_fill<256, 4, false, true, TAB>, 256, index + v4 * fs, v4, D.queue + 1, 0, v4);
         if (e != cudaSuccess) return e;
         if (D.W <= v4) return e;  // a slice has at most W entries
-        e = replay ? go(k_dense_fill<512, 2, true, true>, 512, index + v2 * fs, v2, D.queue + 2, v4, v2)
-                   : go(k_dense_fill<512, 2, false, true>, 512, index + v2 * fs, v2, D.queue + 2, v4, v2);
+        e = replay ? go(k_dense_fill<512, 2, true, true, TAB>, 512, index + v2 * fs, v2, D.queue + 2, v4, v2)
+                   : go(k_dense_fill<512, 2, false, true, TAB>, 512, index + v2 * fs, v2, D.queue + 2, v4, v2);
         if (e != cudaSuccess) return e;
         if (D.W <= v2) return e;
-        return replay ? go(k_dense_fill<1024, 1, true, true>, 1024, index + v1 * fs, v1, D.queue + 3, v2, INT32_MAX)
-                      : go(k_dense_fill<1024, 1, false, true>, 1024, index + v1 * fs, v1, D.queue + 3, v2, INT32_MAX);
+        return replay ? go(k_dense_fill<1024, 1, true, true, TAB>, 1024, index + v1 * fs, v1, D.queue + 3, v2, INT32_MAX)
+                      : go(k_dense_fill<1024, 1, false, true, TAB>, 1024, index + v1 * fs, v1, D.queue + 3, v2, INT32_MAX);
     }
+}
+
+cudaError_t launch_dense_fill(const DevCSR &A, const DevCSR &B, const DenseArgs &D, const int64_t *c_rp,
+                              int32_t *c_col, val_t *c_val, int64_t *err, cudaStream_t st, bool replay,
+                              const int64_t *gate) {
+    return dense_tabled(D) ? launch_fill<true>(A, B, D, c_rp, c_col, c_val, err, st, replay, gate)
+                           : launch_fill<false>(A, B, D, c_rp, c_col, c_val, err, st, replay, gate);
 }
 
 }  // namespace spg

@@ -45,6 +45,7 @@ struct BinSummary {
     int64_t merge_batched;  // bin-37 rows, not flagged dense by stage 1, that k_merge_small cannot take
     int64_t class_count[NUM_LAUNCH_CLASSES];  // learned: bin-37 rows per launch class
     int64_t dense_count;                      // bin-37 rows computed by the dense-slice kernels
+    int64_t dense_entries;                    // A's entries in those that reach far (kind 0 of dense_bucket)
     int64_t dense_end[2];                     // of these, the first [0] take a CTA per slice, the next up
                                               // to [1] a warp and reach more than DENSE_NARROW_W columns
     int64_t bin_start[NUM_BINS + 1];          // offsets of the bins in bin_rows (for launches sized on the device)
@@ -244,7 +245,8 @@ struct DenseArgs {
     int64_t n_wide, n_mid; // warp per row (those up to n_mid reach more than DENSE_NARROW_W columns)
     int K;                 // column slices of B
     int W;                 // slice width (a multiple of 32); slice s holds columns [s W, (s + 1) W)
-    const int32_t *bnd;    // K > 1: per B row, K + 1 offsets of the slices' first entries in the row
+    const int32_t *bnd;    // K > 1: per B row, K + 1 offsets of the slices' first entries in the row; null:
+                           // the kernels search the rows
     int32_t *cnt;          // n K columns per (row, slice)
     int32_t *soff;         // n K offsets of the slices inside their row of C
     const int64_t *dev_n = nullptr;  // when set: the number of dense items is *dev_n (<= n), and n_wide

@@ -575,6 +575,21 @@ static BoundOut bound_out(const spgemm_plan *p) {
     return o;
 }
 
+// Whether B's slice boundaries are tabled; the slice kernels search the rows without.  The table
+// takes K searches per row of B, the search two per slice and selected B row in the count and in
+// the fill: it pays from a quarter as many selected rows as B has.  (A square matrix of 4,190,000
+// columns with 4 rows of 16,000 products: 4.8 -> 4.2 ms without the table of 553 MB, 8,000,000 columns: 10.3 ->
+// 8.0 ms and 2 GB less held; R-MAT 2^20 x 8 takes 77.3 ms with and 91.8 without, 2^18 x 8, precise, 11.8 and
+// 13.0.)  Under a limit of the plan only when everything still to come fits beside it.
+static bool wants_bounds(const spgemm_plan *p) {
+    if (p->B.nrows > 4 * p->h_summary.dense_entries) return false;
+    if (p->opts.max_bytes <= 0) return true;
+    const int64_t table = (int64_t)sizeof(int32_t) * p->B.nrows * (p->dense_K + 1);
+    const int64_t slices = 2 * (int64_t)sizeof(int32_t) * p->dense_n * p->dense_K;
+    const int64_t most = (p->h_summary.sum_cap + p->h_summary.sum_u) * ENTRY_BYTES + (p->A.nrows + 1) * (int64_t)sizeof(int64_t);
+    return p->mem.held + table + slices + most + (1 << 20) <= p->opts.max_bytes;
+}
+
 // Stages 1 and 2 on the plan's A and B (int64 row pointers on the device).
 static spgemm_status plan_symbolic_core(spgemm_plan *p) {
     spgemm_status status = SPGEMM_OK;
@@ -701,10 +716,14 @@ static spgemm_status plan_symbolic_core(spgemm_plan *p) {
         p->stats.dense_slices = p->dense_n > 0 ? p->dense_K : 0;
         if (p->dense_n > 0) {
             // kept for values-only replay: the slice boundaries, counts and offsets
-            if (p->dense_K > 1 && p->dense_wide > 0) {
-                SPG_TRY(p->alloc_n(&p->dense_bnd, p->B.nrows * (p->dense_K + 1)));
-                SPG_TRY(launch_dense_bounds(p->B, p->dense_K, p->dense_W, p->dense_bnd, p->st));
-                p->count(SPGEMM_K_OTHER);
+            if (p->dense_K > 1 && p->dense_wide > 0 && wants_bounds(p)) {
+                const cudaError_t e = p->alloc_n(&p->dense_bnd, p->B.nrows * (p->dense_K + 1));
+                if (e == cudaSuccess) {
+                    SPG_TRY(launch_dense_bounds(p->B, p->dense_K, p->dense_W, p->dense_bnd, p->st));
+                    p->count(SPGEMM_K_OTHER);
+                } else if (e != cudaErrorMemoryAllocation) {
+                    SPG_TRY(e);
+                }
             }
             SPG_TRY(p->alloc_n(&p->dense_cnt, p->dense_n * p->dense_K));
             SPG_TRY(p->alloc_n(&p->dense_soff, p->dense_n * p->dense_K));

@@ -398,7 +398,7 @@ k_bin_scan(int64_t m, int32_t *hist, int64_t nblk, int64_t *part, int64_t *ctil_
             S->sum_cap = total[NUM_BINS];
             S->sum_u = total[NUM_BINS + 1];
             S->merge_batched = total[NUM_BINS + 2];
-            S->dense_count = 0;
+            S->dense_count = S->dense_entries = 0;
             S->dense_end[0] = S->dense_end[1] = 0;
         }
     }
