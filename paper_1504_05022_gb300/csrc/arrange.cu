@@ -108,6 +108,71 @@ cudaError_t launch_arrange_short(const StageArgs &a, const RowSet &R, const uint
     return go(k_arrange_short<32>, 32);
 }
 
+// The rows of bin 1 alone (a replay, the precise method): the one entry of A that selects a row of B that is not
+// empty is searched by G lanes, one entry each at first, several in a row that turns out long.  Bound by
+// the gathers of B's row pointers, so few registers and many warps.  A launch on rows of bin 1 among 200,000 rows
+// of A of 256 and of 3 entries, 100 rows of 200,000: by four lanes with the copy's registers 100 us, 64 us and 13.1 ms,
+// here 69 us, 51 us and 0.83 ms (a warp per row: 69 us, 264 us and 1.5 ms).
+template <int G>
+__global__ void __launch_bounds__(ARR_NT, 8)
+k_single(StageArgs a, RowSet R, const int64_t *__restrict__ c_rp, int32_t *__restrict__ c_col,
+         val_t *__restrict__ c_val) {
+    if (gated(a.gate)) return;
+    const int32_t *rows;
+    int64_t nrows;
+    rowset_range(R, rows, nrows);
+    constexpr int UN = 4;
+    const int gl = threadIdx.x & (G - 1);
+    const unsigned gm = G == 32 ? SPG_FULL : ((1u << (G & 31)) - 1u) << (lane_id() & ~(G - 1));
+    for (int64_t wg = ((int64_t)blockIdx.x * ARR_NT + threadIdx.x) / G; wg < nrows;
+         wg += (int64_t)gridDim.x * (ARR_NT / G)) {
+        const int row = rows[wg];
+        const int64_t a0 = a.A.rp[row], a1 = a.A.rp[row + 1];
+        auto hit = [&](int32_t j) { return a.B.rp[j + 1] > a.B.rp[j]; };
+        int64_t p = -1;
+        for (int64_t base = a0 + gl; base - gl < a1;) {
+            if (base - a0 < 16 * G) {
+                if (base < a1 && hit(a.A.col[base])) p = base;
+                base += G;
+            } else {
+                int32_t j[UN];
+#pragma unroll
+                for (int u = 0; u < UN; ++u)
+                    if (base + u * G < a1) j[u] = a.A.col[base + u * G];
+#pragma unroll
+                for (int u = 0; u < UN; ++u)
+                    if (base + u * G < a1 && hit(j[u])) p = base + u * G;
+                base += UN * G;
+            }
+            if (__any_sync(gm, p >= 0)) break;
+        }
+        if (p >= 0) {
+            const int64_t o = c_rp[row], b0 = a.B.rp[a.A.col[p]];
+            if (SPG_IN(o < c_rp[row + 1], 116)) {
+                c_col[o] = a.B.col[b0];
+                c_val[o] = a.A.val[p] * a.B.val[b0];
+            }
+        }
+    }
+}
+
+cudaError_t launch_single(const StageArgs &a, const RowSet &R, const int64_t *c_rp, int32_t *c_col, val_t *c_val,
+                          cudaStream_t st) {
+    if (R.n <= 0) return cudaSuccess;
+    auto go = [&](auto kern, int g) {
+        const int64_t need = (R.n * g + ARR_NT - 1) / ARR_NT;
+        const int64_t grid = R.dev_lo ? persistent_blocks((const void *)kern, ARR_NT, 0, need) : need;
+        if (grid <= 0) return cudaErrorInvalidValue;
+        kern<<<(unsigned)grid, ARR_NT, 0, st>>>(a, R, c_rp, c_col, c_val);
+        return cudaGetLastError();
+    };
+    const int64_t half = a.A.nnz / (2 * (a.A.nrows > 0 ? a.A.nrows : 1));  // of an average row of A
+    if (half <= 4) return go(k_single<4>, 4);
+    if (half <= 12) return go(k_single<8>, 8);
+    if (half <= 24) return go(k_single<16>, 16);
+    return go(k_single<32>, 32);
+}
+
 // One thread: whether C (c_rp[m] entries) fits the cap entries allocated for it.
 __global__ void k_gate(const int64_t *c_rp, int64_t m, int64_t cap, int64_t *gate, int64_t *err) {
     const bool over = c_rp[m] > cap;

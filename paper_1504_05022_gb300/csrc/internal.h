@@ -333,6 +333,9 @@ cudaError_t launch_row_scan(int64_t m, const int32_t *nnzc, int64_t *c_rp, int64
 // copies the rows of C~ into C; avg_nnz: entries of an average row of C (sets the lanes per row)
 cudaError_t launch_arrange_short(const StageArgs &a, const RowSet &R, const uint8_t *bin, const int64_t *c_rp,
                                  int32_t *c_col, val_t *c_val, int64_t avg_nnz, cudaStream_t st);
+// the rows of bin 1 (one product each) alone
+cudaError_t launch_single(const StageArgs &a, const RowSet &R, const int64_t *c_rp, int32_t *c_col, val_t *c_val,
+                          cudaStream_t st);
 // *gate = 1, *err = 8 and every c_rp[0..m] = 0 (C empty) when the result of m rows (c_rp[m]
 // entries) exceeds cap entries, else *gate = 0
 cudaError_t launch_gate(int64_t *c_rp, int64_t m, int64_t cap, int64_t *gate, int64_t *err, cudaStream_t st);

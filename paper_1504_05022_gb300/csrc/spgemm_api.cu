@@ -1786,8 +1786,7 @@ extern "C" spgemm_status spgemm_numeric_replay(spgemm_plan *p) {
         // bin 1: the single product of each row
         {
             const int64_t s0 = p->bin_start[1], s1 = p->bin_start[2];
-            SPG_TRY(launch_arrange_short(a, host_rows(p->bin_rows + s0, s1 - s0), p->bin, p->C.row_ptr, p->C.col_idx,
-                                         p->C.val, 1, p->st));
+            SPG_TRY(launch_single(a, host_rows(p->bin_rows + s0, s1 - s0), p->C.row_ptr, p->C.col_idx, p->C.val, p->st));
         }
         // bin 37: every leaf fuses its products into its known columns
         int64_t off = 0;
@@ -1981,7 +1980,7 @@ static cudaError_t precise_fill(spgemm_plan *p, bool dev, const int64_t *gate) {
     // bin 1: the single product of each row
     const RowSet r1 = bin_range(p, 1, 1, dev);
     if (!dev) p->time_begin(SPGEMM_K_ARRANGE);
-    e = launch_arrange_short(a, r1, p->bin, p->C.row_ptr, p->C.col_idx, p->C.val, 1, p->stream());
+    e = launch_single(a, r1, p->C.row_ptr, p->C.col_idx, p->C.val, p->stream());
     if (!dev) {
         p->time_end();
         if (r1.n > 0) p->count(SPGEMM_K_ARRANGE);
