@@ -277,14 +277,14 @@ SPG_DEV int bm_merge_misses(const BmSmem &s, Index &ix, int rlen, int nm, int32_
     for (int m = threadIdx.x; m < nm; m += NT) {
         const int32_t c = s.Mk[m];
         const int t = ix.lookup(c - lo);
-        if (!SPG_IN(t >= 0 && t < fnew, 108)) continue;
+        if (!SPG_IN(t >= 0 && t < fnew, 118)) continue;
         s.Rk[t] = c;
         s.Rv[t] = 0.0;
     }
     __syncthreads();
     for (int m = threadIdx.x; m < nm; m += NT) {
         const int t = ix.lookup(s.Mk[m] - lo);
-        if (SPG_IN(t >= 0 && t < fnew, 108)) atomicAdd(&s.Rv[t], s.Mv[m]);
+        if (SPG_IN(t >= 0 && t < fnew, 119)) atomicAdd(&s.Rv[t], s.Mv[m]);
     }
     __syncthreads();
     return fnew;

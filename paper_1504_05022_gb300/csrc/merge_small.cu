@@ -223,7 +223,7 @@ k_merge_small(StageArgs a, MergeItems it, MergeLaunch L, int nw1) {
 #pragma unroll
             for (int u = 0; u < UN; ++u) {
                 const int k = k0 + u;
-                if (c[k] < 0 || !SPG_IN(pos[k] < nnz, 114)) continue;
+                if (c[k] < 0 || !SPG_IN(pos[k] < nnz, 117)) continue;
                 atomicAdd(&V[pos[k]], av[u] * v[u]);
                 dst_col[pos[k]] = c[k];  // the same column from every product of the position
             }
