@@ -5,21 +5,24 @@
 // registers while they find their places: a bitmap of the occupied 32-column words of
 // B (one bit per word) and its rank directory number the words; a bitmap per occupied word and
 // the ranks over those give every column its position in the row.  Then the values are read and
-// added into one sum per column.  Eight barriers in all, and no capacity to outgrow before the
+// added into one sum per column.  Fifteen barriers in all, and no capacity to outgrow before the
 // size is known: a row longer than its home is listed as overflowed with its exact size (its
 // length in the work-item table) before any value is read, and later rounds pass it on until
 // their capacity fits.
 //
 // The batched kernel (merge_bm.cu) searches each product's B row in a table, buffers the products
 // whose columns are new and merges them by rank, with a barrier per batch and a dozen per merge;
-// at 230 KB of shared memory per CTA it leaves 16 warps on an SM.  Here a CTA needs at most 8
-// bytes per product: 28 to 32 warps per SM.  Shared-memory latency
+// at 230 KB of shared memory per CTA it leaves 16 warps on an SM.  Here a CTA needs 8 bytes per
+// product and per 1,024 columns of B: 28 to 32 warps per SM up to 1.2 million columns (3.5 million for
+// the CTAs of 512 threads), 16 to 24 at the 4,194,304 that the index takes.  Shared-memory latency
 // and instruction issue bound it.
 //
 // Measured (kernel time of all bin-37 merge launches, one GB300, before -> after): R-MAT 2^20 x 8, its
 // 180 k rows of 513..8,191 products, 23.3 -> 9.2 ms; R-MAT 2^16 x 16 1.68 -> 1.19 ms; R-MAT 30,011 x 8
-// in single precision under the hybrid policy (five rounds) 0.89 -> 0.70 ms.  The line lies at 8,192
-// products because 512 threads of 16 are the most that share an SM twice.
+// in single precision under the hybrid policy (five rounds) 0.89 -> 0.70 ms.  50,000 rows of 576 and of 2,025
+// products, the whole product by the upper-bound policy: B of 200,000 columns 3.92 -> 1.34 and 5.85 ->
+// 2.04 ms, of 4,194,304 4.45 -> 2.23 and 6.53 -> 3.10.  The line lies at 8,192 products because 512
+// threads of 16 are the most that share an SM twice.
 #include "internal.h"
 #include "common.cuh"
 #include "dynamic_smem.h"

@@ -151,7 +151,7 @@ __global__ void k_mlp_forward(const float *__restrict__ params, const float *__r
 // loss), which k_mlp_grad_sum adds in a fixed order: the result does not depend on timing.
 // Each neuron's sum runs over its inputs in ascending order from the bias, as in
 // mlp_forward_one.  Bound by shared-memory reads and latency (two CTAs per SM at 8,192 samples).
-// A step of 8,192 samples with its Adam update takes 23 us; it took 118 us when one thread ran a
+// A step of 8,192 samples with its Adam update takes 26 us; it took 118 us when one thread ran a
 // whole sample and wrote a 612-byte record of it, which the reduction read with a stride.
 constexpr int MLP_TILE = 64;
 constexpr int MLP_NT = 4 * MLP_TILE;

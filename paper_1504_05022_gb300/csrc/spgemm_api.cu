@@ -389,8 +389,8 @@ static void merge_limits(spgemm_plan *p) {
     p->capmax = capmax;
     p->small_u = p->bm_words > 0 ? std::min(MERGE_SMALL_U, capmax) : 0;
     // dense column slices: B's columns cut into equal slices of at most DENSE_W_MAX columns
-    // (a multiple of 32); a fill CTA holds the slice's bitmap and rank directory and a
-    // compact buffer of sums, one per column of the result; dense_span narrows the slices
+    // (a multiple of 32); a fill CTA holds the slice's bitmap and its ranks, and in single
+    // precision a buffer of sums; dense_span narrows the slices
     p->dense_K = 0;
     p->dense_W = 0;
     p->dense_min_u = 0;
@@ -993,10 +993,9 @@ fail:
 }
 
 // The column bitmaps that the slices' counting pass leaves for the fill (opts.dense_keep):
-// only where the count builds bitmaps and the fill is the compact form, never by default in
-// the precise method, and only while they take at most a quarter of the free device memory
-// and no more than twice as many words as there are products: a sparser row's products are marked again for
-// less than its bitmap's traffic (A*A of the 27-point operator on 40^3, 2,004 words and 729
+// never by default in the precise method, and only while they take at most a quarter of the free
+// device memory and no more than twice as many words as there are products: a sparser row's
+// products are marked again for less than its bitmap's traffic (A*A of the 27-point operator on 40^3, 2,004 words and 729
 // products a row: 1.22 ms and 570 MB with, 1.37 ms and 130 MB without; R-MAT 2^18 x 8, 16 k
 // products a row: 10.7 and 11.9 ms).
 // Released with the other numeric temporaries; without them the fill marks the columns again.
