@@ -55,6 +55,20 @@ class DeviceGuard {
     cudaError_t err_ = cudaSuccess;
 };
 
+// While one lives, the thread's event queries and frees are no concern of a stream capture that this
+// thread or another one has begun: they touch no capturing stream, but would invalidate a capture in
+// the global mode (torch's), into which a finaliser may free a plan.
+class OutsideCapture {
+  public:
+    OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    ~OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    OutsideCapture(const OutsideCapture &) = delete;
+    OutsideCapture &operator=(const OutsideCapture &) = delete;
+
+  private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
+
 constexpr size_t CLASS_MIN = size_t(128) << 20;
 constexpr size_t CACHE_BLOCKS = 4096;  // a batch of 512 pairs in 64 waves holds about 2,600
 constexpr size_t CACHE_SHARE = 256;
@@ -107,6 +121,7 @@ class DeviceMemory {
     // Stream-ordered on st, where the block's last use is.
     void free(int device, Block b, bool temp, cudaStream_t st) {
         DeviceGuard g(device);
+        OutsideCapture relaxed;
         std::lock_guard<std::mutex> lk(mu_);
         Device &d = devices_[device];
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;

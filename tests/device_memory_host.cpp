@@ -32,6 +32,8 @@ std::vector<FakePool *> g_pools;
 std::vector<std::pair<cudaStream_t, cudaEvent_t>> g_waits;
 int g_syncs = 0, g_frees_async = 0, g_frees = 0, g_mallocs = 0, g_event_errors = 0;
 std::set<cudaStream_t> g_capturing;
+cudaStreamCaptureMode g_mode = cudaStreamCaptureModeGlobal;
+int g_invalidated = 0;  // captures that a call of the thread would have ended
 uintptr_t g_next = 0x1000;
 
 size_t reserved_all() {
@@ -92,12 +94,17 @@ cudaError_t cudaFreeAsync(void *ptr, cudaStream_t) {
     if (g_allocs.count(ptr) && g_allocs[ptr].pool->device != g_device) ++g_event_errors;
     return release(ptr);
 }
-cudaError_t cudaFree(void *ptr) { ++g_frees; return release(ptr); }
+cudaError_t cudaFree(void *ptr) {
+    ++g_frees;
+    if (!g_capturing.empty() && g_mode != cudaStreamCaptureModeRelaxed) ++g_invalidated;
+    return release(ptr);
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t st) { ++g_syncs; g_ran[st] = g_issued[st]; return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t st, cudaStreamCaptureStatus *s) {
     *s = g_capturing.count(st) ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *m) { std::swap(*m, g_mode); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) {
     *e = reinterpret_cast<cudaEvent_t>(new FakeEvent{g_device});
     return cudaSuccess;
@@ -114,6 +121,7 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st) {
     return cudaSuccess;
 }
 cudaError_t cudaEventQuery(cudaEvent_t e) {
+    if (!g_capturing.empty() && g_mode != cudaStreamCaptureModeRelaxed) ++g_invalidated;
     return event_passed(reinterpret_cast<FakeEvent *>(e)) ? cudaSuccess : cudaErrorNotReady;
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned) { g_waits.emplace_back(st, e); return cudaSuccess; }
@@ -144,7 +152,7 @@ static void reset() {
     g_ran.clear();
     g_waits.clear();
     g_capturing.clear();
-    g_syncs = g_frees_async = g_frees = g_mallocs = g_event_errors = 0;
+    g_syncs = g_frees_async = g_frees = g_mallocs = g_event_errors = g_invalidated = 0;
     g_device = 0;
     g_room = g_total;
 }
@@ -287,6 +295,19 @@ static int a_free_inside_a_capture_keeps_nothing() {
     return 0;
 }
 
+static int a_free_beside_a_capture_leaves_it_valid() {
+    reset();
+    DeviceMemory m;
+    std::vector<Block> v;
+    for (size_t i = 0; i < spg::CACHE_BLOCKS + 10; ++i) v.push_back(get(m, 8192, S(1)));
+    for (size_t i = 0; i < spg::CACHE_BLOCKS; ++i) m.free(0, v[i], false, S(1));
+    g_ran[S(1)] = g_issued[S(1)];
+    g_capturing.insert(S(2));
+    for (size_t i = spg::CACHE_BLOCKS; i < v.size(); ++i) m.free(0, v[i], false, S(1));  // with evictions
+    CHECK(g_frees == 10 && g_invalidated == 0 && g_mode == cudaStreamCaptureModeGlobal);
+    return 0;
+}
+
 static int exact_blocks_are_of_just_their_bytes() {
     reset();
     DeviceMemory m;
@@ -363,6 +384,7 @@ int main() {
         CASE(trim_waits_for_nothing_and_keeps_what_it_may),
         CASE(pools_hold_at_most_half_for_others),
         CASE(a_free_inside_a_capture_keeps_nothing),
+        CASE(a_free_beside_a_capture_leaves_it_valid),
         CASE(exact_blocks_are_of_just_their_bytes),
         CASE(a_plans_limit_is_of_the_memory_itself),
         CASE(without_a_limit_blocks_are_little_larger),

@@ -24,4 +24,4 @@ def test_on_a_fake_runtime(tmp_path):
     assert r.returncode == 0, r.stderr[-3000:]
     r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
-    assert r.stdout.count(": ok") == 11
+    assert r.stdout.count(": ok") == 12

@@ -58,3 +58,25 @@ def test_trim_to_a_size():
     assert free0 - torch.cuda.mem_get_info()[0] <= keep + (64 << 20)  # pools hold memory in pieces of 32 MB
     spg.pool_trim()
     assert torch.cuda.mem_get_info()[0] >= free0 - (8 << 20)
+
+
+def test_plans_freed_inside_a_capture_leave_it_valid():
+    """A finaliser may run while a graph is captured: plans of other streams go, the graph stays good."""
+    import paper_1504_05022_gb300 as spg
+    A = _uniform(3000, 3000, 9, 6)
+    side = torch.cuda.Stream()
+    Cs = [spg.spgemm(A, A) for _ in range(3)]
+    with torch.cuda.stream(side):
+        Cs += [spg.spgemm(A, A) for _ in range(3)]
+    want = Cs[0].val.clone()
+    x = torch.ones(1000, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        y = x * 2
+        del Cs
+        y = y + 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert y[0].item() == 3.0
+    assert torch.equal(spg.spgemm(A, A).val, want)
