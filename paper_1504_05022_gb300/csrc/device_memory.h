@@ -118,27 +118,39 @@ class DeviceMemory {
         return e;
     }
 
-    // Stream-ordered on st, where the block's last use is.
-    void free(int device, Block b, bool temp, cudaStream_t st) {
+    // Stream-ordered on st, where the blocks' last use is.
+    void free(int device, const Block *blocks, size_t n, bool temp, cudaStream_t st) {
+        if (n == 0) return;
         DeviceGuard g(device);
         OutsideCapture relaxed;
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        // inside a capture of st itself nothing is kept: an event of the capture orders nothing outside
+        cudaError_t e = g.error();
+        if (e == cudaSuccess) e = cudaStreamIsCapturing(st, &capture);
+        bool may_keep = e == cudaSuccess && capture == cudaStreamCaptureStatusNone;
         std::lock_guard<std::mutex> lk(mu_);
         Device &d = devices_[device];
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (b.bytes < CLASS_MIN && b.bytes == block_size(b.bytes) && g.error() == cudaSuccess &&
-            cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
-            (b.freed != nullptr || cudaEventCreateWithFlags(&b.freed, cudaEventDisableTiming) == cudaSuccess) &&
-            cudaEventRecord(b.freed, st) == cudaSuccess) {
-            b.st = st;
-            b.stamp = ++clock_;
-            d.oldest.emplace(b.stamp, std::make_pair(&d.kept[temp], d.kept[temp].emplace(b.bytes, b)));
-            d.kept_bytes += b.bytes;
-            while ((d.oldest.size() > CACHE_BLOCKS || d.kept_bytes > d.limit / (CACHE_SHARE / 2)) && drop_oldest(d, st)) {
+        for (size_t k = 0; k < n; ++k) {
+            Block b = blocks[k];
+            const bool keep = may_keep && b.bytes < CLASS_MIN && b.bytes == block_size(b.bytes);
+            if (keep && b.freed == nullptr) {
+                e = cudaEventCreateWithFlags(&b.freed, cudaEventDisableTiming);
+                if (e != cudaSuccess) b.freed = nullptr;
             }
-            return;
+            if (keep && e == cudaSuccess) e = cudaEventRecord(b.freed, st);
+            if (keep && e == cudaSuccess) {
+                b.st = st;
+                b.stamp = ++clock_;
+                d.oldest.emplace(b.stamp, std::make_pair(&d.kept[temp], d.kept[temp].emplace(b.bytes, b)));
+                d.kept_bytes += b.bytes;
+                while ((d.oldest.size() > CACHE_BLOCKS || d.kept_bytes > d.limit / (CACHE_SHARE / 2)) && drop_oldest(d, st)) {
+                }
+                continue;
+            }
+            may_keep = may_keep && e == cudaSuccess;
+            give(b, [&] { cudaFreeAsync(b.ptr, st); });
         }
-        cudaGetLastError();
-        give(b, [&] { cudaFreeAsync(b.ptr, st); });
+        if (e != cudaSuccess) cudaGetLastError();  // of these calls only
     }
 
     // Unused memory back to the system until the device's pools hold at most `keep` bytes; waits
@@ -384,7 +396,7 @@ class PlanMemory {
     // Stream-ordered on st.
     void release(DeviceMemory &m, int device, cudaStream_t st, int life) {
         Life &l = life_[life];
-        for (const Block &b : l.blocks) m.free(device, b, life != LIFE_PLAN, st);
+        m.free(device, l.blocks.data(), l.blocks.size(), life != LIFE_PLAN, st);
         held -= l.bytes;
         l = Life{};
     }

@@ -166,8 +166,8 @@ static int large_blocks_go_back_to_the_driver() {
     CHECK(a.ptr && b.ptr && t.ptr && c.ptr);
     CHECK(a.from == b.from && a.from != t.from && a.from != c.from);  // by size and use
     CHECK(a.bytes >= 40 * GB && a.bytes <= 40 * GB + 40 * GB / 16);
-    m.free(0, a, false, S(1));
-    m.free(0, c, false, S(1));
+    m.free(0, &a, 1, false, S(1));
+    m.free(0, &c, 1, false, S(1));
     CHECK(g_frees_async == 2 && g_allocs.count(a.ptr) == 0);  // the driver has them: any allocation can get that memory
     Block d = get(m, 40 * GB - 1000, S(2));  // a nearly equal request finds the same pool
     CHECK(d.from == b.from && g_waits.empty());
@@ -178,7 +178,7 @@ static int small_blocks_follow_their_event() {
     reset();
     DeviceMemory m;
     Block a = get(m, 100000, S(1));
-    m.free(0, a, false, S(1));
+    m.free(0, &a, 1, false, S(1));
     CHECK(g_frees_async == 0);
     Block b = get(m, 99000, S(2));  // another stream, the last use has not run
     CHECK(b.ptr != a.ptr && g_waits.empty());
@@ -186,12 +186,12 @@ static int small_blocks_follow_their_event() {
     CHECK(t.ptr != a.ptr);
     Block c = get(m, 99000, S(1));  // the same stream: at once, in order
     CHECK(c.ptr == a.ptr && g_waits.size() == 1 && g_waits[0].first == S(1));
-    m.free(0, c, false, S(1));
+    m.free(0, &c, 1, false, S(1));
     g_ran[S(1)] = g_issued[S(1)];
     Block d = get(m, 99000, S(2));  // now it has run
     CHECK(d.ptr == a.ptr);
     Block e = get(m, 60000, S(2)), f = get(m, 2 * MB, S(2));
-    m.free(0, f, false, S(2));
+    m.free(0, &f, 1, false, S(2));
     Block g = get(m, MB, S(2));  // not a block twice as large
     CHECK(g.ptr != f.ptr && e.ptr);
     return 0;
@@ -202,8 +202,8 @@ static int the_plans_device_is_current() {
     DeviceMemory m;
     Block a = get(m, 100000, nullptr, false, 1), b = get(m, GB, nullptr, false, 1);
     CHECK(g_device == 0);
-    m.free(1, a, false, nullptr);  // as a finaliser does, with device 0 current
-    m.free(1, b, false, nullptr);
+    m.free(1, &a, 1, false, nullptr);  // as a finaliser does, with device 0 current
+    m.free(1, &b, 1, false, nullptr);
     CHECK(g_device == 0 && g_event_errors == 0);
     CHECK(reinterpret_cast<FakeEvent *>(get(m, 100000, nullptr, false, 1).freed)->device == 1);
     CHECK(m.trim(1, 0) == cudaSuccess && g_device == 0);
@@ -215,7 +215,7 @@ static int kept_blocks_are_bounded() {
     DeviceMemory m;
     std::vector<Block> v;
     for (size_t i = 0; i < spg::CACHE_BLOCKS + 10; ++i) v.push_back(get(m, 8192, S(1)));
-    for (auto &b : v) m.free(0, b, false, S(1));
+    for (auto &b : v) m.free(0, &b, 1, false, S(1));
     CHECK(g_frees_async + g_frees == 10 && g_allocs.size() == spg::CACHE_BLOCKS);
     for (int i = 0; i < 10; ++i) CHECK(g_allocs.count(v[i].ptr) == 0);  // the longest unused
     reset();
@@ -223,14 +223,14 @@ static int kept_blocks_are_bounded() {
     const size_t most = g_total / spg::CACHE_SHARE;
     v.clear();
     for (size_t k = 0; k < most / (64 * MB) + 5; ++k) v.push_back(get(n, 64 * MB, S(1)));
-    for (auto &b : v) n.free(0, b, false, S(1));
+    for (auto &b : v) n.free(0, &b, 1, false, S(1));
     CHECK(g_allocs.size() * 64 * MB <= most);
     // blocks whose last use is on another stream and has not run stay: nothing waits for them
     v.clear();
     g_waits.clear();
     const size_t before = g_allocs.size();
     for (int k = 0; k < 8; ++k) v.push_back(get(n, 100 * MB, S(2)));
-    for (auto &b : v) n.free(0, b, false, S(2));
+    for (auto &b : v) n.free(0, &b, 1, false, S(2));
     for (auto &w : g_waits) CHECK(w.first == reinterpret_cast<FakeEvent *>(w.second)->st || w.first == S(2));
     CHECK(before > 0);
     return 0;
@@ -240,15 +240,15 @@ static int a_full_device_is_tried_once_more() {
     reset();
     DeviceMemory m;
     Block small = get(m, MB, S(1)), big = get(m, 100 * GB, S(1), true);
-    m.free(0, small, false, S(1));
-    m.free(0, big, true, S(1));
+    m.free(0, &small, 1, false, S(1));
+    m.free(0, &big, 1, true, S(1));
     g_room = 120 * GB;
     Block a = get(m, 119 * GB, S(1));  // rounded it would not fit, and the other pool holds 100 GB
     CHECK(a.ptr && a.bytes == 119 * GB && g_syncs == 1);
     CHECK(g_allocs.count(small.ptr) == 0);
     Block b = get(m, 2 * GB, S(1));
     CHECK(!b.ptr && g_allocs.size() == 1);
-    m.free(0, a, false, S(1));
+    m.free(0, &a, 1, false, S(1));
     CHECK(get(m, 100 * GB, S(1)).ptr);  // a failure leaves nothing behind
     return 0;
 }
@@ -258,11 +258,11 @@ static int trim_waits_for_nothing_and_keeps_what_it_may() {
     DeviceMemory m;
     CHECK(m.trim(0, 0) == cudaSuccess && g_pools.empty());  // a device never used
     Block a = get(m, GB, S(1)), b = get(m, 2 * GB, S(1), true), held = get(m, 3 * GB, S(1)), s = get(m, MB, S(1)), p = get(m, MB, S(2));
-    m.free(0, a, false, S(1));
-    m.free(0, b, true, S(1));
-    m.free(0, s, false, S(1));
+    m.free(0, &a, 1, false, S(1));
+    m.free(0, &b, 1, true, S(1));
+    m.free(0, &s, 1, false, S(1));
     g_ran[S(1)] = g_issued[S(1)];
-    m.free(0, p, false, S(2));  // its stream has not got there
+    m.free(0, &p, 1, false, S(2));  // its stream has not got there
     const size_t all = reserved_all();
     CHECK(m.trim(0, all) == cudaSuccess && reserved_all() == all);
     CHECK(m.trim(0, all - GB) == cudaSuccess && reserved_all() == all - GB);
@@ -279,7 +279,7 @@ static int pools_hold_at_most_half_for_others() {
     for (size_t k = 0; k < 12; ++k) {  // sizes that share no pool
         Block b = get(m, (20 + 2 * k) * GB, S(1));
         CHECK(b.ptr);
-        m.free(0, b, false, S(1));
+        m.free(0, &b, 1, false, S(1));
         CHECK(reserved_all() <= std::max(g_total / 2, b.bytes));
     }
     return 0;
@@ -290,7 +290,7 @@ static int a_free_inside_a_capture_keeps_nothing() {
     DeviceMemory m;
     Block a = get(m, 100000, S(1));
     g_capturing.insert(S(1));
-    m.free(0, a, false, S(1));
+    m.free(0, &a, 1, false, S(1));
     CHECK(g_frees_async == 1 && g_allocs.empty());
     return 0;
 }
@@ -300,10 +300,10 @@ static int a_free_beside_a_capture_leaves_it_valid() {
     DeviceMemory m;
     std::vector<Block> v;
     for (size_t i = 0; i < spg::CACHE_BLOCKS + 10; ++i) v.push_back(get(m, 8192, S(1)));
-    for (size_t i = 0; i < spg::CACHE_BLOCKS; ++i) m.free(0, v[i], false, S(1));
+    for (size_t i = 0; i < spg::CACHE_BLOCKS; ++i) m.free(0, &v[i], 1, false, S(1));
     g_ran[S(1)] = g_issued[S(1)];
     g_capturing.insert(S(2));
-    for (size_t i = spg::CACHE_BLOCKS; i < v.size(); ++i) m.free(0, v[i], false, S(1));  // with evictions
+    for (size_t i = spg::CACHE_BLOCKS; i < v.size(); ++i) m.free(0, &v[i], 1, false, S(1));  // with evictions
     CHECK(g_frees == 10 && g_invalidated == 0 && g_mode == cudaStreamCaptureModeGlobal);
     return 0;
 }
@@ -313,8 +313,8 @@ static int exact_blocks_are_of_just_their_bytes() {
     DeviceMemory m;
     Block a = get(m, 100001, S(1), false, 0, true), b = get(m, GB + 1, S(1), false, 0, true);
     CHECK(a.bytes == 100001 && b.bytes == GB + 1);
-    m.free(0, a, false, S(1));
-    m.free(0, b, false, S(1));
+    m.free(0, &a, 1, false, S(1));
+    m.free(0, &b, 1, false, S(1));
     CHECK(g_frees_async == 2);
     return 0;
 }
